@@ -217,3 +217,118 @@ def tolerance(case):
     # single difference is a dQ element of the first rows, where dP - D cancels: 0.098 of the tensor's root mean square
     # (0.06 for an element of the loss head's dW).
     return {"rel": 1e-2, "max": 0.25 if case["kind"] == "lce" else 0.4}
+
+
+# ---- the same outputs from the definitions, in 64 bits ----
+
+def _attend64(q, pos, k, v, window, own=None, do=None):
+    """Rows q [R, G, d] at positions `pos` [R] over the visible keys of one KV head: clean keys k, v [n, d] with
+    j < lim[r] and pos[r] - j < window, and the rows' own blocks.  `own` = (lim [R], k [R, d], v [R, d], block of each
+    row [R]) for corrupted rows; clean rows see the keys up to their own position.  Returns o, lse and, with `do`, dq,
+    (dk, dv) of the clean keys and (dk, dv) of the own keys."""
+    d = q.shape[-1]
+    j = torch.arange(k.shape[0], device=q.device)
+    lim = pos + 1 if own is None else own[0]
+    seen = j[None, :] < lim[:, None]
+    if window > 0:
+        seen &= pos[:, None] - j[None, :] < window
+    keys, vals = k, v
+    if own is not None:
+        keys, vals = torch.cat([k, own[1]]), torch.cat([v, own[2]])
+        seen = torch.cat([seen, own[3][:, None] == own[3][None, :]], dim=1)
+    s = torch.einsum("rgd,nd->grn", q, keys) / math.sqrt(d)
+    s.masked_fill_(~seen, -math.inf)
+    lse = torch.logsumexp(s, dim=-1)                       # [G, R]
+    p = s.sub_(lse[..., None]).exp_()
+    o = torch.einsum("grn,nd->rgd", p, vals)
+    if do is None:
+        return o, lse, None, None, None
+    dv = torch.einsum("grn,rgd->nd", p, do)
+    ds = torch.einsum("rgd,nd->grn", do, vals).sub_((do * o).sum(-1).T[..., None]).mul_(p).div_(math.sqrt(d))
+    dq = torch.einsum("grn,nd->rgd", ds, keys)
+    dk = torch.einsum("grn,rgd->nd", ds, q)
+    n = k.shape[0]
+    return o, lse, dq, (dk[:n], dv[:n]), (dk[n:], dv[n:])
+
+
+def _stream64(q, k, v, do, pos, window, lim=None, M=1, kn=None, vn=None):
+    """One query stream over the clean keys in position order (and its own blocks, with `lim`): o, lse, dq, dk and dv of
+    the clean keys, dk and dv of the own keys."""
+    batch, rows, H, d = q.shape
+    H_kv, G = k.shape[2], H // k.shape[2]
+    f = lambda *s: torch.zeros(*s, dtype=torch.float64, device=q.device)
+    o, lse, dq = f(*q.shape), f(batch, H, rows), f(*q.shape)
+    dk, dv = f(*k.shape), f(*k.shape)
+    dkn, dvn = (f(*kn.shape), f(*kn.shape)) if lim is not None else (None, None)
+    step = M * max(1, 1024 // M)
+    for b in range(batch):
+        for hk in range(H_kv):
+            h = slice(hk * G, hk * G + G)
+            kd, vd = k[b, :, hk].double(), v[b, :, hk].double()
+            for r0 in range(0, rows, step):
+                r = slice(r0, min(rows, r0 + step))
+                n = int(lim[r].max()) if lim is not None else int(pos[r].max()) + 1
+                own = None
+                if lim is not None:
+                    own = (lim[r], kn[b, r, hk].double(), vn[b, r, hk].double(), torch.arange(r.start, r.stop, device=q.device) // M)
+                got = _attend64(q[b, r, h].double(), pos[r], kd[:n], vd[:n], window, own, None if do is None else do[b, r, h].double())
+                o[b, r, h], lse[b, h, r] = got[0], got[1]
+                if do is not None:
+                    dq[b, r, h] = got[2]
+                    dk[b, :n, hk] += got[3][0]
+                    dv[b, :n, hk] += got[3][1]
+                    if lim is not None:
+                        dkn[b, r, hk], dvn[b, r, hk] = got[4]
+    return o, lse, dq, dk, dv, dkn, dvn
+
+
+def _exact_lce(s):
+    h, w, y, wt = s["h"].double(), s["w"].double(), s["labels"].long(), s["weight"].double()
+    nll, lse = torch.zeros_like(wt), torch.zeros_like(wt)
+    dh, dw = torch.zeros_like(h), torch.zeros_like(w)
+    for t0 in range(0, h.shape[0], 2048):
+        t = slice(t0, t0 + 2048)
+        z = h[t] @ w.T
+        lse[t] = torch.logsumexp(z, dim=-1)
+        at, on = y[t].clamp(min=0)[:, None], y[t] >= 0
+        nll[t] = torch.where(on, lse[t] - z.gather(1, at)[:, 0], 0.0)
+        z = z.sub_(lse[t][:, None]).exp_()
+        z.scatter_add_(1, at, torch.full_like(at, -1, dtype=torch.float64))
+        z.mul_((wt[t] * on)[:, None])
+        dh[t] = z @ w
+        dw += z.T @ h[t]
+    return (wt * nll).sum().reshape(1), nll, lse, dh, dw
+
+
+def exact(case, seed):
+    if work(case)["flops"] > 8.0e13:   # over about 20 seconds
+        return None
+    s = prepare(case, seed)
+    if case["kind"] == "lce":
+        return _exact_lce(s)
+    M, L, window, dev = case["M"], case["L"], case.get("window", 0), s["k_clean"].device
+    k, v = s["k_clean"], s["v_clean"]
+    at = lambda p0, p1: torch.arange(p0, p1, device=dev)
+    rows = s["q_noisy"].shape[1]
+    block = at(0, rows) // M
+    prefix = (s["block_prefix"].long() if "block_prefix" in s else at(0, L // M) * M)[block]
+    noisy = lambda kc, vc: _stream64(s["q_noisy"], kc, vc, s.get("do_noisy"), prefix + at(0, rows) % M, window, prefix, M,
+                                     s["k_noisy"], s["v_noisy"])
+    if case["kind"] == "rank":
+        chunk, positions = s["kv_chunks"]
+        where = torch.cat([at(p, p + chunk) for p in positions])     # position of each stored row
+        by_pos = torch.argsort(where)
+        k, v = k[:, by_pos], v[:, by_pos]
+        n = noisy(k, v)
+        (p0, q0, do0), (p1, q1, do1) = s["runs"]
+        c0, c1 = (_stream64(q, k, v, do, at(p, p + q.shape[1]), 0) for p, q, do in ((p0, q0, do0), (p1, q1, do1)))
+        return ((c0[0], c0[1], n[0], n[1]), (c1[0], c1[1], None, None),
+                (c0[2], (c0[3] + n[3])[:, where], (c0[4] + n[4])[:, where], n[2], n[5], n[6]),
+                (c1[2], c1[3][:, where], c1[4][:, where], None, None, None))
+    n = noisy(k, v)
+    if case["kind"] == "packed":
+        return (None, None, n[0], n[1]), (None, n[3], n[4], n[2], n[5], n[6])
+    c = _stream64(s["q_clean"], k, v, s.get("do_clean"), at(0, L), window)
+    if case["kind"] == "shards":
+        return (c[0], c[1]), (n[0], n[1])
+    return (c[0], c[1], n[0], n[1]), (c[2], c[3] + n[3], c[4] + n[4], n[2], n[5], n[6])
