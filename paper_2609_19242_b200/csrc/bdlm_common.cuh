@@ -142,14 +142,14 @@ int device_sm_count();
 //                    first over the whole launch.  Chosen by the launchers when the heaviest tile is a sizeable part of
 //                    the ideal duration of the launch (short sequences), where the first order would start the heavy
 //                    tiles of the second and later batch elements too late.
-struct TileGrid { int nx, ny, nz, tile_major; };
-__device__ __forceinline__ void tile_grid_decode(const TileGrid& g, int& x, int& y, int& z) {
-  int i = blockIdx.x;
+// parts: CTAs that share one unit (the backward's key tiles: a cluster of that size), index i = unit * parts + part.
+struct TileGrid { int nx, ny, nz, tile_major, parts; };
+__device__ __forceinline__ void tile_grid_decode(const TileGrid& g, int i, int& x, int& y, int& z) {
   if (!g.tile_major) { x = i % g.nx; i /= g.nx; y = i % g.ny; z = i / g.ny; }
   else { const int c = g.ny * g.nz; x = i / c; i -= x * c; y = i % g.ny; z = i / g.ny; }
 }
 inline TileGrid make_tile_grid(int nx, int ny, int nz) {
-  TileGrid g = {nx, ny, nz, 0};
+  TileGrid g = {nx, ny, nz, 0, 1};
   // heaviest tile ~ nx units, whole launch ~ ny nz nx (nx + 1) / 2 units over the device's SMs: tile-major when the
   // heaviest tile exceeds a fifth of the ideal duration
   g.tile_major = (10LL * device_sm_count() > (long long)ny * nz * (nx + 1)) ? 1 : 0;

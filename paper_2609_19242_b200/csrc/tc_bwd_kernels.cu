@@ -86,27 +86,117 @@ struct QStep { int qs, h, q0; };
 // L2 between the CTAs that share them.  (Alternating the two streams tile by tile as well was measured and is
 // slower: 4.7 against 3.3 ms on the sliding-window workload.)  Counters only, no division; the order is fixed, so
 // dK / dV stay bitwise reproducible.
+//
+// When a key tile is split over a cluster (see ClusterSplit), its steps are dealt out one by one: CTA `part` of `parts`
+// takes steps part, part + parts, ... of the same order.
 struct StepWalk {
-  int a0, a1, b0, b1, G, h_first, qs_a, rows;
-  int t, seg, hh;
-  __device__ __forceinline__ int count() const { return ((a1 - a0) + (b1 - b0)) * G; }
-  __device__ __forceinline__ void init(int a0_, int na, int b0_, int nb, int G_, int h_first_, int qs_a_, int rows_) {
-    a0 = a0_; a1 = a0_ + na; b0 = b0_; b1 = b0_ + nb; G = G_; h_first = h_first_; qs_a = qs_a_; rows = rows_;
-    hh = 0;
-    if (a1 > a0) { seg = 0; t = a1 - 1; } else { seg = 1; t = b1 - 1; }
+  int a1, na, b1, nb, G, h_first, qs_a, rows, part, parts;
+  int t, hh;   // tile counter over both segments, head within the group
+  __device__ __forceinline__ int total() const { return (na + nb) * G; }
+  __device__ __forceinline__ int count() const { return max(0, (total() - part + parts - 1) / parts); }
+  __device__ __forceinline__ void init(int a0, int na_, int b0, int nb_, int G_, int h_first_, int qs_a_, int rows_, int part_, int parts_) {
+    na = na_; nb = nb_; a1 = a0 + na_ - 1; b1 = b0 + nb_ - 1; G = G_; h_first = h_first_; qs_a = qs_a_; rows = rows_;
+    part = part_; parts = parts_;
+    t = 0; hh = part_;
+    while (hh >= G) { hh -= G; ++t; }
   }
   __device__ __forceinline__ QStep cur() const {
     QStep s;
-    s.h = h_first + hh; s.qs = seg == 0 ? qs_a : NOISY; s.q0 = t * rows;
+    s.h = h_first + hh;
+    if (t < na) { s.qs = qs_a; s.q0 = (a1 - t) * rows; }
+    else { s.qs = NOISY; s.q0 = (b1 - (t - na)) * rows; }
     return s;
   }
   __device__ __forceinline__ void next() {
-    if (++hh < G) return;
-    hh = 0;
-    --t;
-    if (seg == 0 && t < a0) { seg = 1; t = b1 - 1; }
+    hh += parts;
+    while (hh >= G) { hh -= G; ++t; }
   }
 };
+
+// ---------------------------------------------------------------- key tiles split over a cluster
+// Short sequences have few key tiles and the first of them carries twice the mean work: with one CTA per key tile the
+// launch lasts as long as that one CTA (L = 2048, H = 32: 256 steps against a mean of 125 per SM).  A cluster of 2 or 4
+// CTAs then shares a clean key tile: each takes every second or fourth step and accumulates its own dV / dK; at the end
+// the partial tiles go to shared memory, each CTA adds up a share of the rows over its peers through distributed
+// shared memory, in the order of their ranks (so the sums stay reproducible), and stores it.  Noisy key tiles have a
+// few steps only (their own block's queries): in such a launch each CTA of a cluster takes one of its own.
+struct KeyUnit { int bx, hk, ks, b, part, parts; bool none; };
+__device__ __forceinline__ KeyUnit key_unit(const TileGrid& tg) {
+  KeyUnit u;
+  int bz;
+  u.parts = tg.parts;
+  u.part = tg.parts == 1 ? 0 : blockIdx.x % tg.parts;
+  tile_grid_decode(tg, tg.parts == 1 ? blockIdx.x : blockIdx.x / tg.parts, u.bx, u.hk, bz);
+  u.ks = bz & 1; u.b = bz >> 1;
+  u.none = false;
+  if (u.ks == NOISY && tg.parts > 1) {
+    u.bx = u.bx * tg.parts + u.part;
+    u.none = u.bx >= tg.nx;
+    u.part = 0; u.parts = 1;
+  }
+  return u;
+}
+__device__ __forceinline__ void cluster_sync() {
+  asm volatile("barrier.cluster.arrive.release;\n\tbarrier.cluster.wait.acquire;" ::: "memory");
+}
+__device__ __forceinline__ float4 ld_peer(uint32_t addr, int rank) {
+  float4 v;
+  asm volatile(
+      "{\n\t.reg .b32 p;\n\t"
+      "mapa.shared::cluster.u32 p, %4, %5;\n\t"
+      "ld.shared::cluster.v4.f32 {%0, %1, %2, %3}, [p];\n\t}"
+      : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "r"(addr), "r"(rank) : "memory");
+  return v;
+}
+// A thread's accumulator row (D columns from `tacc`) as the partial tile `which` (0 dV, 1 dK) at the start of shared
+// memory, 16-byte pieces of 128 rows one after the other: neighbouring lanes write neighbouring pieces.
+template <int D>
+__device__ __forceinline__ void put_partial(uint8_t* sm, int which, int r, uint32_t tacc) {
+  float4* dst = reinterpret_cast<float4*>(sm + which * TILE * D * 4) + r;
+#pragma unroll
+  for (int c = 0; c < D / 32; ++c) {
+    uint32_t v[32];
+    tmem_ld32(tacc + c * 32, v);
+    tmem_wait_ld();
+#pragma unroll
+    for (int q = 0; q < 8; ++q)
+      dst[(c * 8 + q) * TILE] = make_float4(__uint_as_float(v[4 * q]), __uint_as_float(v[4 * q + 1]),
+                                            __uint_as_float(v[4 * q + 2]), __uint_as_float(v[4 * q + 3]));
+  }
+}
+// Warp `wi` (0..7): a quarter of the columns of dV (0..3) or dK (4..7), for this CTA's share of the 128 rows.
+// `have` peers took at least one step; a tile no query sees is written as zeros.
+template <int D>
+__device__ __forceinline__ void sum_partials(const uint8_t* sm, int wi, int lane, int part, int parts, int have, bf16* dst0,
+                                             int64_t row_stride, int rows_left, float scale) {
+  constexpr int NQ = D / 16;                          // 16-byte pieces of a quarter row
+  const int which = wi >> 2, cq0 = (wi & 3) * NQ;
+  const int share = TILE / parts;
+  for (int r = part * share + lane; r < (part + 1) * share; r += 32) {
+    const uint8_t* own = sm + which * (TILE * D * 4) + (cq0 * TILE + r) * 16;
+    const uint32_t at = smem_u32(own);
+    float4 acc[NQ];
+#pragma unroll
+    for (int q = 0; q < NQ; ++q) acc[q] = make_float4(0.f, 0.f, 0.f, 0.f);
+    for (int p = 0; p < have; ++p) {
+      float4 u[NQ];   // a peer's pieces all in flight at once
+#pragma unroll
+      for (int q = 0; q < NQ; ++q) u[q] = p == part ? *reinterpret_cast<const float4*>(own + q * TILE * 16) : ld_peer(at + q * TILE * 16, p);
+#pragma unroll
+      for (int q = 0; q < NQ; ++q) { acc[q].x += u[q].x; acc[q].y += u[q].y; acc[q].z += u[q].z; acc[q].w += u[q].w; }
+    }
+    if (r < rows_left) {
+      bf16* dst = dst0 + r * row_stride + cq0 * 4;
+#pragma unroll
+      for (int q = 0; q < NQ; q += 2) {
+        uint4 o;
+        o.x = pack_bf16(acc[q].x * scale, acc[q].y * scale); o.y = pack_bf16(acc[q].z * scale, acc[q].w * scale);
+        o.z = pack_bf16(acc[q + 1].x * scale, acc[q + 1].y * scale); o.w = pack_bf16(acc[q + 1].z * scale, acc[q + 1].w * scale);
+        *reinterpret_cast<uint4*>(dst + q * 4) = o;
+      }
+    }
+  }
+}
 
 template <bool TR, int D>
 __global__ void __launch_bounds__(DKDV_THREADS, 1)
@@ -126,14 +216,13 @@ tc_dkdv_kernel(const __grid_constant__ BwdMaps maps, const KArgs a, const TileGr
   volatile uint32_t* tmem_slot = reinterpret_cast<volatile uint32_t*>(sm + DKDV_BARS + 128);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(sm + DKDV_BARS + 136);
 
-  int bx, by, bz;
-  tile_grid_decode(tg, bx, by, bz);
-  const int ks = bz & 1, b = bz >> 1, hk = by;
-  const int k0_row = bx * TILE;   // the tile's first key in memory; key tile 0 has the most query tiles: started first
+  const KeyUnit unit = key_unit(tg);
+  const int ks = unit.ks, b = unit.b, hk = unit.hk, part = unit.part, parts = unit.parts;
+  const int k0_row = unit.bx * TILE;   // the tile's first key in memory; key tile 0 has the most query tiles: started first
   const int k0 = ks == CLEAN ? clean_key_pos(a, k0_row) : k0_row;   // and its position
   const int warp = __shfl_sync(0xffffffffu, threadIdx.x >> 5, 0), lane = threadIdx.x & 31;   // warp index, provably uniform
   const int L = rows_k(a, ks), M = a.M;   // rows of this stream's K/V tensors
-  if (k0_row >= L || a.dk[ks] == nullptr) return;
+  if (unit.none || k0_row >= L || a.dk[ks] == nullptr) return;
 
   // query tiles that see this key tile: segment A (clean queries; noisy ones for a noisy key tile), then
   // segment B (noisy queries of a clean key tile), for each head of the group.  The visible-query interval of
@@ -157,8 +246,8 @@ tc_dkdv_kernel(const __grid_constant__ BwdMaps maps, const KArgs a, const TileGr
   }
   // the steps are walked in the same order by every role (see StepWalk)
   StepWalk walk;
-  walk.init(tA0, nA, tB0, nB, a.G, hk * a.G, ks == NOISY ? NOISY : CLEAN, TILE);
-  const int nsteps = walk.count();
+  walk.init(tA0, nA, tB0, nB, a.G, hk * a.G, ks == NOISY ? NOISY : CLEAN, TILE, part, parts);
+  const int nsteps = walk.count(), walk_total = walk.total();
   auto step_cur = [&]() { return walk.cur(); };
   auto step_next = [&]() { walk.next(); };
 
@@ -461,7 +550,10 @@ tc_dkdv_kernel(const __grid_constant__ BwdMaps maps, const KArgs a, const TileGr
       ok = mbar_wait_abortable(bar_done, 0, abort_flag);
       ok = __all_sync(0xffffffffu, ok);
     }
-    if (ok) {
+    if (ok && parts > 1) {
+      tc_fence_after();
+      if (nsteps > 0) put_partial<D>(sm, w, r, tl + 256 + w * 128);
+    } else if (ok) {
       tc_fence_after();
       constexpr int EW = 256 / DKDV_NWG;                       // accumulator columns per thread
       const int acol = w * EW;                                 // first of them, in [0, 256)
@@ -483,6 +575,13 @@ tc_dkdv_kernel(const __grid_constant__ BwdMaps maps, const KArgs a, const TileGr
   }
   tc_fence_before();
   __syncthreads();
+  if (parts > 1) {   // as in the fused kernel
+    cluster_sync();
+    if (warp < 8)
+      sum_partials<D>(sm, warp, lane, part, parts, min(parts, walk_total), (warp < 4 ? a.dv[ks] : a.dk[ks]) +
+                      (((int64_t)b * L + k0_row) * a.Hkv + hk) * D, (int64_t)a.Hkv * D, L - k0_row, warp < 4 ? 1.f : a.scale);
+    cluster_sync();
+  }
   if (threadIdx.x == 0 && *abort_flag) atomicExch(status, (int)BDLM_ERR_DEVICE_TIMEOUT);
   if (warp == DKDV_PRODUCER) tmem_dealloc(tmem, 512);
 }
@@ -531,7 +630,7 @@ tc_dq_kernel(const __grid_constant__ BwdMaps maps, const KArgs a, const TileGrid
   volatile int* abort_flag = reinterpret_cast<volatile int*>(sm + DQ_BARS + 152);
 
   int bx, by, bz;
-  tile_grid_decode(tg, bx, by, bz);
+  tile_grid_decode(tg, blockIdx.x, bx, by, bz);
   const int qs = bz & 1, b = bz >> 1, h = by, hk = h / a.G;
   const int q0 = (tg.nx - 1 - bx) * TILE;
   const int warp = __shfl_sync(0xffffffffu, threadIdx.x >> 5, 0), lane = threadIdx.x & 31;   // warp index, provably uniform
@@ -854,14 +953,13 @@ tc_bwdf_kernel(const __grid_constant__ BwdMaps maps, const KArgs a, const TileGr
   volatile uint32_t* tmem_slot = reinterpret_cast<volatile uint32_t*>(sm + BF_BARS + 208);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(sm + BF_BARS + 216);
 
-  int bx, by, bz;
-  tile_grid_decode(tg, bx, by, bz);
-  const int ks = bz & 1, b = bz >> 1, hk = by;
-  const int k0_row = bx * TILE;   // the tile's first key in memory; key tile 0 has the most query tiles: started first
+  const KeyUnit unit = key_unit(tg);
+  const int ks = unit.ks, b = unit.b, hk = unit.hk, part = unit.part, parts = unit.parts;
+  const int k0_row = unit.bx * TILE;   // the tile's first key in memory; key tile 0 has the most query tiles: started first
   const int k0 = ks == CLEAN ? clean_key_pos(a, k0_row) : k0_row;   // and its position
   const int warp = __shfl_sync(0xffffffffu, threadIdx.x >> 5, 0), lane = threadIdx.x & 31;   // warp index, provably uniform
   const int L = rows_k(a, ks), M = a.M;
-  if (k0_row >= L || a.dk[ks] == nullptr) return;
+  if (unit.none || k0_row >= L || a.dk[ks] == nullptr) return;
 
   // 64-row query tiles that see this key tile: segment A (clean queries; noisy ones for a noisy key tile),
   // then segment B (noisy queries of a clean key tile), for each head of the group
@@ -883,8 +981,8 @@ tc_bwdf_kernel(const __grid_constant__ BwdMaps maps, const KArgs a, const TileGr
     tA0 = lo / HT; nA = (hi + HT - 1) / HT - tA0;
   }
   StepWalk walk;
-  walk.init(tA0, nA, tB0, nB, a.G, hk * a.G, ks == NOISY ? NOISY : CLEAN, HT);
-  const int nsteps = walk.count();
+  walk.init(tA0, nA, tB0, nB, a.G, hk * a.G, ks == NOISY ? NOISY : CLEAN, HT, part, parts);
+  const int nsteps = walk.count(), walk_total = walk.total();
   auto step_cur = [&]() { return walk.cur(); };
   auto step_next = [&]() { walk.next(); };
 
@@ -1269,7 +1367,10 @@ tc_bwdf_kernel(const __grid_constant__ BwdMaps maps, const KArgs a, const TileGr
       ok = mbar_wait_abortable(bar_done, 0, abort_flag);
       ok = __all_sync(0xffffffffu, ok);
     }
-    if (ok) {
+    if (ok && parts > 1) {
+      tc_fence_after();
+      if (nsteps > 0) put_partial<D>(sm, w, r, tl + 256 + w * 128);
+    } else if (ok) {
       tc_fence_after();
       bf16* dst = (w == 0 ? a.dv[ks] : a.dk[ks]) + (((int64_t)b * L + k0_row + r) * a.Hkv + hk) * D;
       const float sc = (w == 0) ? 1.f : a.scale;
@@ -1287,6 +1388,13 @@ tc_bwdf_kernel(const __grid_constant__ BwdMaps maps, const KArgs a, const TileGr
   }
   tc_fence_before();
   __syncthreads();
+  if (parts > 1) {   // every CTA of the cluster gets here: all waits above are bounded
+    cluster_sync();
+    if (warp < 8)
+      sum_partials<D>(sm, warp, lane, part, parts, min(parts, walk_total), (warp < 4 ? a.dv[ks] : a.dk[ks]) +
+                      (((int64_t)b * L + k0_row) * a.Hkv + hk) * D, (int64_t)a.Hkv * D, L - k0_row, warp < 4 ? 1.f : a.scale);
+    cluster_sync();   // no CTA leaves while a peer still reads its shared memory
+  }
   if (threadIdx.x == 0 && *abort_flag) atomicExch(status, (int)BDLM_ERR_DEVICE_TIMEOUT);
   if (warp == 8) tmem_dealloc(tmem, 512);
 }
@@ -1347,6 +1455,56 @@ size_t tc_bwd_fused_workspace(const bdlm_params* p, const bdlm_packed_geometry* 
   return (pad64(rows_c) + pad64(rows_n)) * p->batch * p->H * 128 * sizeof(float);
 }
 
+// How many CTAs share a clean key tile (1, 2 or 4), from two estimates in steps of `rows` query rows: `heavy` for the
+// first clean key tile and `mean` per SM; with a prefix table the blocks are taken to be spread evenly over the keys.
+// A launch cannot end before its heaviest CTA, so a split pays when that is well above the mean; below, longest-first
+// start order fills the chip and the exchange of the partial tiles (about 4 steps per CTA) is a loss.  Clusters of four
+// only reach 132 of the 148 SMs.  Fused backward with 1 / 2 / 4 CTAs per tile (us, all kernels of the call):
+//   L = 2048, H = 32 / 8        heavy 1.9 means    386 /  308 /  343
+//   L = 1024, H = 32 / 8        heavy 3.4 means    236 /  176 /  174
+//   L = 8192, H = 8 / 1         heavy 4.4 means   2097 / 1098 /  740
+//   L = 16384, H = 8 / 1        heavy 2.3 means   4284 / 2717 / 2919
+//   L = 4096, H = 32 / 8        heavy 1.06 means   914 /  920 / 1050
+//   L = 8192, H = 32 / 8        heavy 0.55 means  2755 / 3122 / 4237
+// Under MIN_HEAVY steps the exchange eats what the split gives (L = 256: 37 / 36 / 36).
+constexpr double MIN_HEAVY = 24, SPLIT_2 = 1.2, SPLIT_4 = 3.0;
+static int split_key_tiles(const KArgs& a, int rows) {
+  const double W = a.window > 0 ? a.window : 0;
+  double heavy = 0, total = 0;
+  for (int qs = CLEAN; qs <= NOISY; ++qs) {
+    if (a.q[qs] == nullptr) continue;
+    const double nq = (rows_q(a, qs) + rows - 1) / rows;
+    const double seen = qs == CLEAN ? a.cq_pos0 + 0.5 * a.Lqc : 0.5 * a.L;   // keys a query sees on average
+    heavy += W > 0 ? min(nq, (W + TILE) / rows + 1) : nq;
+    total += nq * ((W > 0 ? min(W, seen) : seen) / TILE + 1);
+  }
+  heavy *= a.G;
+  const double mean = total * a.G * a.Hkv * a.batch / device_sm_count();
+  if (heavy < MIN_HEAVY || heavy < SPLIT_2 * mean) return 1;
+  return heavy < SPLIT_4 * mean ? 2 : 4;
+}
+
+// One CTA, or one cluster of tg.parts CTAs, per unit of the grid.
+template <class Kern>
+static cudaError_t launch_units(Kern kern, const TileGrid& tg, int threads, size_t smem, cudaStream_t st, const BwdMaps& maps,
+                                const KArgs& a, int* status) {
+  const long long blocks = (long long)tile_grid_blocks(tg) * tg.parts;
+  if (blocks == 0 || blocks > 0x7fffffffLL) return cudaErrorInvalidValue;
+  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  if (e != cudaSuccess) return e;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)blocks);
+  cfg.blockDim = dim3(threads);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cudaLaunchAttribute attr = {};
+  attr.id = cudaLaunchAttributeClusterDimension;
+  attr.val.clusterDim.x = tg.parts; attr.val.clusterDim.y = 1; attr.val.clusterDim.z = 1;
+  cfg.attrs = &attr;
+  cfg.numAttrs = tg.parts > 1 ? 1 : 0;
+  return cudaLaunchKernelEx(&cfg, kern, maps, a, tg, status);
+}
+
 template <int D>
 static cudaError_t launch_tc_bwd_d(const KArgs& a_in, void* extra_ws, int passes, cudaStream_t st) {
   KArgs a = a_in;
@@ -1376,11 +1534,9 @@ static cudaError_t launch_tc_bwd_d(const KArgs& a_in, void* extra_ws, int passes
     if (passes & BDLM_BWD_PASS_DKDV) {
       if ((e = cudaMemsetAsync(a.dq32[0], 0, (dq32_elems[0] + dq32_elems[1]) * sizeof(float), st)) != cudaSuccess) return e;
       auto kern = a.trace ? tc_bwdf_kernel<true, D> : tc_bwdf_kernel<false, D>;
-      if ((e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, BF_SMEM)) != cudaSuccess) return e;
-      const TileGrid tg = make_tile_grid((max(a.L, a.k[NOISY] != nullptr ? a.Ln : 0) + TILE - 1) / TILE, a.Hkv, a.batch * 2);
-      if (tile_grid_blocks(tg) == 0) return cudaErrorInvalidValue;
-      kern<<<tile_grid_blocks(tg), BF_THREADS, BF_SMEM, st>>>(maps, a, tg, status);
-      if ((e = cudaGetLastError()) != cudaSuccess) return e;
+      TileGrid tg = make_tile_grid((max(a.L, a.k[NOISY] != nullptr ? a.Ln : 0) + TILE - 1) / TILE, a.Hkv, a.batch * 2);
+      tg.parts = split_key_tiles(a, HT);
+      if ((e = launch_units(kern, tg, BF_THREADS, BF_SMEM, st, maps, a, status)) != cudaSuccess) return e;
       for (int s2 = 0; s2 < 2; ++s2) {
         if (dq32_elems[s2] == 0) continue;
         dq_convert_kernel<D><<<device_sm_count() * 16, 256, 0, st>>>(a.dq32[s2], a.dq[s2], a.batch, a.H, rows_q(a, s2), a.dq32_rows[s2]);
@@ -1391,11 +1547,9 @@ static cudaError_t launch_tc_bwd_d(const KArgs& a_in, void* extra_ws, int passes
   }
   if (passes & BDLM_BWD_PASS_DKDV) {
     auto kern = a.trace ? tc_dkdv_kernel<true, D> : tc_dkdv_kernel<false, D>;
-    if ((e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, DKDV_SMEM)) != cudaSuccess) return e;
-    const TileGrid tg = make_tile_grid((max(a.L, a.k[NOISY] != nullptr ? a.Ln : 0) + TILE - 1) / TILE, a.Hkv, a.batch * 2);
-    if (tile_grid_blocks(tg) == 0) return cudaErrorInvalidValue;
-    kern<<<tile_grid_blocks(tg), DKDV_THREADS, DKDV_SMEM, st>>>(maps, a, tg, status);
-    if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    TileGrid tg = make_tile_grid((max(a.L, a.k[NOISY] != nullptr ? a.Ln : 0) + TILE - 1) / TILE, a.Hkv, a.batch * 2);
+    tg.parts = split_key_tiles(a, TILE);
+    if ((e = launch_units(kern, tg, DKDV_THREADS, DKDV_SMEM, st, maps, a, status)) != cudaSuccess) return e;
   }
   if (passes & BDLM_BWD_PASS_DQ) {
     auto kern = a.trace ? tc_dq_kernel<true, D> : tc_dq_kernel<false, D>;

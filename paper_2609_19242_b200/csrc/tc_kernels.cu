@@ -146,7 +146,7 @@ tc_fwdr_kernel(const __grid_constant__ FwdMaps maps, const KArgs a, const TileGr
   volatile int* abort_flag = reinterpret_cast<volatile int*>(sm + FWDR_BARS + 136);
 
   int bx, by, bz;
-  tile_grid_decode(tg, bx, by, bz);
+  tile_grid_decode(tg, blockIdx.x, bx, by, bz);
   const int qs = bz & 1, b = bz >> 1;
   if (a.q[qs] == nullptr) return;
   // warpgroup w works on head h0 + w * HSTEP, query rows q0 + w * QSTEP ...

@@ -1,0 +1,32 @@
+"""Backward calls short enough that a cluster of CTAs shares each clean key tile: the partial dK / dV tiles are added up
+through distributed shared memory.  Two and four CTAs per tile, step counts that the CTAs do not divide, ragged last
+tiles, one head per group, key tiles only some of the CTAs have steps for (sliding window), both kernel paths."""
+import pytest
+import torch
+
+from paper_2609_19242_b200 import binding, synth
+from paper_2609_19242_b200.synth import Workload
+
+import parity_util as pu
+
+pytestmark = pytest.mark.gpu
+
+CASES = [
+    Workload("two", 4, 16, 8, 128, 512, 32, seed=1),               # heaviest tile 1.6 times the mean load per SM
+    Workload("two_ragged_d64", 4, 24, 8, 64, 440, 40, seed=2),
+    Workload("four", 1, 4, 1, 128, 640, 64, seed=3),
+    Workload("four_one_head", 1, 1, 1, 128, 1000, 40, seed=4),     # the CTAs of a cluster take different query tiles
+    Workload("four_three_heads_d64", 1, 3, 1, 64, 776, 8, seed=5),
+    Workload("four_window", 1, 4, 1, 128, 1024, 16, window=130, seed=6),
+]
+
+
+@pytest.mark.parametrize("single_pass", [True, False], ids=["fused", "two_pass"])
+@pytest.mark.parametrize("w", CASES, ids=lambda w: w.name)
+def test_split_key_tiles_match_the_oracle_and_are_reproducible(w, single_pass):
+    pu.check_full(w, binding.IMPL_TCGEN05, single_pass=single_pass)
+    g = synth.make_inputs(w, "cuda")
+    out = pu.gpu_fwd(g, w.block_size, window=w.window)
+    a, b = (pu.gpu_bwd(g, out, w.block_size, window=w.window, single_pass=single_pass) for _ in range(2))
+    for i in (1, 2, 4, 5):   # dK, dV of both streams: a fixed order of summation
+        assert torch.equal(a[i], b[i])
