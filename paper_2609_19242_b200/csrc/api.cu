@@ -227,11 +227,11 @@ static int bwd_impl(const bdlm_params* p, const bdlm_packed_geometry* g,
                    workspace_bytes >= need_fused) ? 1 : 0;
   const int passes = p->bwd_passes ? p->bwd_passes : 7;
   cudaError_t e = cudaSuccess;
-  if (passes & BDLM_BWD_PASS_DSUM) e = launch_dsum(a, ds_c, ds_n, st);
+  if (a.single_pass) tc_bwd_place_dq(a, static_cast<char*>(workspace) + 2 * dsum_bytes(p, g));
+  if (passes & BDLM_BWD_PASS_DSUM) e = launch_bwd_prepare(a, ds_c, ds_n, a.single_pass && (passes & BDLM_BWD_PASS_DKDV), st);
   if (e != cudaSuccess) return BDLM_ERR_CUDA;
   if (tc_ok && p->impl != 1) {
-    void* extra = static_cast<char*>(workspace) + 2 * dsum_bytes(p, g);
-    e = launch_tc_bwd(a, extra, passes, st);
+    e = launch_tc_bwd(a, passes, st);
   } else {
     e = launch_portable_bwd(a, passes, st);
   }

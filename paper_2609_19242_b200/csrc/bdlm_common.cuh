@@ -50,7 +50,7 @@ struct KArgs {
   __nv_bfloat16* dv[2];
   unsigned long long* trace;   // optional cycle counters (bdlm_set_trace_buffer), else nullptr
   int single_pass;             // backward: the fused kernel forms dQ^T per step and adds it into dq32 by TMA bulk add-reductions
-  float* dq32[2];              // fp32 dQ accumulators [batch, H, dq32_rows, 128] (fused backward), else nullptr
+  float* dq32[2];              // fp32 dQ accumulators [batch, H, dq32_rows, d] (fused backward), else nullptr
   int dq32_rows[2];            // their row counts: the stream's query rows rounded up to the 64-row step of the fused kernel
 };
 
@@ -169,7 +169,8 @@ __device__ __forceinline__ uint32_t pack_bf16(float lo, float hi) {
 // Launchers (host).  Each enqueues on `st` and returns the launch's cudaError_t.
 cudaError_t launch_portable_fwd(const KArgs& a, cudaStream_t st);
 cudaError_t launch_portable_bwd(const KArgs& a, int passes, cudaStream_t st);
-cudaError_t launch_dsum(const KArgs& a, float* dsum_clean, float* dsum_noisy, cudaStream_t st);
+// D rows of both query streams; with zero_dq the fused backward's accumulators a.dq32 are cleared in the same launch.
+cudaError_t launch_bwd_prepare(const KArgs& a, float* dsum_clean, float* dsum_noisy, bool zero_dq, cudaStream_t st);
 cudaError_t launch_merge(int n, int batch, int L, int H, int d, const void* const* o_parts,
                          const float* const* lse_parts, int dtype, void* o_out, float* lse_out,
                          cudaStream_t st);

@@ -107,102 +107,85 @@ __global__ void __launch_bounds__(256, 3) merge_kernel(MergeArgs ma, int64_t tot
   }
 }
 
-// D = sum over d of dO * O, fp32.  D / 8 lanes per (batch, row, head) with 16-byte loads, four rows per lane group in
-// flight (the kernel is a pure stream over dO and O: enough bytes in flight per thread to keep HBM busy).
+// What the backward needs before its first key tile, for both query streams in one launch: D = sum over d of dO * O
+// (fp32), and the fp32 dQ accumulators of the fused kernel set to zero.  A block takes PREP_ROWS consecutive rows of
+// PREP_HEADS heads; dO and O are read as they lie ([batch, L, H, d]), the sums go through shared memory and leave as
+// 128-byte runs along L of the [batch, H, L] result (written straight from the reading lanes they would be 4-byte stores
+// H*4 apart).  A pure stream: bound by memory at large sizes (32K rows, H = 32: 2.15 GB in 340 us = 6.3 TB/s), by the
+// number of blocks at small ones, hence the split over the heads too.
+// Against one launch per stream over all heads of a row tile plus a memset: L = 2048, H = 32 (64 blocks a launch, now
+// 1024) 78 -> 23 us; 32K 472 -> 340 us.
+constexpr int PREP_ROWS = 32, PREP_HEADS = 4;
+struct PrepArgs {
+  const bf16* dout[2];
+  const bf16* o[2];
+  float* dsum[2];      // nullptr: the stream has no queries
+  float* dq32[2];      // nullptr: nothing to zero
+  int rows[2], dq32_rows[2];
+  int blocks_clean, H;
+};
 template <int D>
-__global__ void __launch_bounds__(256) dsum_kernel(const bf16* __restrict__ dout, const bf16* __restrict__ o,
-                                                   float* __restrict__ dsum, int64_t nrows, int L, int H) {
-  constexpr int LPR = D / 8;            // lanes per row: 16 (d = 128) or 8 (d = 64)
-  constexpr int RPW = 32 / LPR;         // rows per warp and pass
-  constexpr int UNROLL = 4;
-  const int lane = threadIdx.x & 31, sub = lane / LPR, c = lane % LPR;
-  const int64_t warp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-  const int64_t base = warp * (RPW * UNROLL);
-  uint4 ua[UNROLL], ub[UNROLL];
-#pragma unroll
-  for (int j = 0; j < UNROLL; ++j) {
-    const int64_t w = base + j * RPW + sub;
-    if (w < nrows) {
-      ua[j] = *reinterpret_cast<const uint4*>(dout + w * D + c * 8);
-      ub[j] = *reinterpret_cast<const uint4*>(o + w * D + c * 8);
-    } else {
-      ua[j] = make_uint4(0u, 0u, 0u, 0u); ub[j] = ua[j];
-    }
-  }
-#pragma unroll
-  for (int j = 0; j < UNROLL; ++j) {
-    const uint32_t* pa = reinterpret_cast<const uint32_t*>(&ua[j]);
-    const uint32_t* pb = reinterpret_cast<const uint32_t*>(&ub[j]);
-    float acc = 0.f;
-#pragma unroll
-    for (int e = 0; e < 4; ++e) {
-      const float2 x = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&pa[e]));
-      const float2 y = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&pb[e]));
-      acc = fmaf(x.x, y.x, fmaf(x.y, y.y, acc));
-    }
-#pragma unroll
-    for (int sft = LPR / 2; sft > 0; sft >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, sft);
-    const int64_t w = base + j * RPW + sub;
-    if (c == 0 && w < nrows) {
-      // w indexes [batch, L, H]; D is stored [batch, H, L]
-      const int h = (int)(w % H);
-      const int64_t row = w / H;
-      const int64_t bidx = row / L;
-      const int i = (int)(row % L);
-      dsum[(bidx * H + h) * L + i] = acc;
-    }
-  }
-}
-
-// The same sums for a tile of 32 consecutive rows x all H heads per block: dO and O are read as they lie
-// ([batch, L, H, d]: the tile is one contiguous piece), the sums go through shared memory and leave as 128-byte runs
-// along L of the [batch, H, L] result (written straight from the reading lanes they would be 4-byte stores H*4 apart).
-constexpr int DS_LB = 32;
-template <int D>
-__global__ void __launch_bounds__(256) dsum_tile_kernel(const bf16* __restrict__ dout, const bf16* __restrict__ o,
-                                                        float* __restrict__ dsum, int L, int H, int tiles_per_batch) {
-  extern __shared__ float sums[];          // [H][DS_LB + 1]
+__global__ void __launch_bounds__(256) bwd_prepare_kernel(const PrepArgs pa) {
+  __shared__ float sums[PREP_HEADS][PREP_ROWS + 1];
   constexpr int LPR = D / 8;               // lanes per row
   constexpr int RPP = 256 / LPR;           // rows per pass of the block
   constexpr int UNROLL = 4;
-  const int b = blockIdx.x / tiles_per_batch, l0 = (blockIdx.x % tiles_per_batch) * DS_LB;
-  const int nl = min(DS_LB, L - l0);
-  const int nrows = nl * H;                // rows of the tile: r = li * H + h
-  const int64_t base = ((int64_t)b * L + l0) * H;
+  const int s = (int)blockIdx.x < pa.blocks_clean ? CLEAN : NOISY;
+  auto of = [&](const auto& x) { return s == CLEAN ? x[0] : x[1]; };   // (an index computed at run time would copy the arguments to local memory)
+  const int L = of(pa.rows), H = pa.H;
+  int i = blockIdx.x - (s == CLEAN ? 0 : pa.blocks_clean);
+  const int hgroups = (H + PREP_HEADS - 1) / PREP_HEADS, tiles = (L + PREP_ROWS - 1) / PREP_ROWS;
+  const int h0 = (i % hgroups) * PREP_HEADS;   // neighbouring blocks read neighbouring heads of the same rows
+  i /= hgroups;
+  const int l0 = (i % tiles) * PREP_ROWS, b = i / tiles;
+  const int nl = min(PREP_ROWS, L - l0), nh = min(PREP_HEADS, H - h0);
+  const int64_t base = ((int64_t)b * L + l0) * H + h0;
   const int sub = threadIdx.x / LPR, c = threadIdx.x % LPR;
-  for (int r0 = 0; r0 < nrows; r0 += RPP * UNROLL) {
+  const bf16 *dout = of(pa.dout), *o = of(pa.o);
+  float* dq32 = of(pa.dq32);
+  const int dq32_rows = of(pa.dq32_rows);
+  constexpr int NROWS = PREP_ROWS * PREP_HEADS;   // r = li * PREP_HEADS + hi
+#pragma unroll 1
+  for (int r0 = 0; r0 < NROWS; r0 += RPP * UNROLL) {
     uint4 ua[UNROLL], ub[UNROLL];
 #pragma unroll
     for (int j = 0; j < UNROLL; ++j) {
-      const int r = r0 + j * RPP + sub;
-      if (r < nrows) {
-        ua[j] = *reinterpret_cast<const uint4*>(dout + (base + r) * D + c * 8);
-        ub[j] = *reinterpret_cast<const uint4*>(o + (base + r) * D + c * 8);
+      const int r = r0 + j * RPP + sub, li = r / PREP_HEADS, hi = r % PREP_HEADS;
+      if (li < nl && hi < nh) {
+        const int64_t at = (base + (int64_t)li * H + hi) * D + c * 8;
+        ua[j] = *reinterpret_cast<const uint4*>(dout + at);
+        ub[j] = *reinterpret_cast<const uint4*>(o + at);
       } else {
         ua[j] = make_uint4(0u, 0u, 0u, 0u); ub[j] = ua[j];
       }
     }
+    if (r0 == 0 && dq32 != nullptr) {   // the stores go out under the first loads
+      for (int hi = 0; hi < nh; ++hi) {
+        float4* z = reinterpret_cast<float4*>(dq32 + (((int64_t)b * H + h0 + hi) * dq32_rows + l0) * D);
+        for (int e = threadIdx.x; e < nl * D / 4; e += 256) z[e] = make_float4(0.f, 0.f, 0.f, 0.f);
+      }
+    }
 #pragma unroll
     for (int j = 0; j < UNROLL; ++j) {
-      const uint32_t* pa = reinterpret_cast<const uint32_t*>(&ua[j]);
-      const uint32_t* pb = reinterpret_cast<const uint32_t*>(&ub[j]);
+      const uint32_t* pa_ = reinterpret_cast<const uint32_t*>(&ua[j]);
+      const uint32_t* pb_ = reinterpret_cast<const uint32_t*>(&ub[j]);
       float acc = 0.f;
 #pragma unroll
       for (int e = 0; e < 4; ++e) {
-        const float2 x = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&pa[e]));
-        const float2 y = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&pb[e]));
+        const float2 x = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&pa_[e]));
+        const float2 y = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&pb_[e]));
         acc = fmaf(x.x, y.x, fmaf(x.y, y.y, acc));
       }
 #pragma unroll
       for (int sft = LPR / 2; sft > 0; sft >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, sft);
       const int r = r0 + j * RPP + sub;
-      if (c == 0 && r < nrows) sums[(r % H) * (DS_LB + 1) + r / H] = acc;
+      if (c == 0) sums[r % PREP_HEADS][r / PREP_HEADS] = acc;
     }
   }
   __syncthreads();
-  for (int idx = threadIdx.x; idx < H * DS_LB; idx += 256) {
-    const int h = idx / DS_LB, li = idx % DS_LB;
-    if (li < nl) dsum[((int64_t)b * H + h) * L + l0 + li] = sums[h * (DS_LB + 1) + li];
+  if (threadIdx.x < NROWS) {
+    const int hi = threadIdx.x / PREP_ROWS, li = threadIdx.x % PREP_ROWS;
+    if (hi < nh && li < nl) of(pa.dsum)[((int64_t)b * H + h0 + hi) * L + l0 + li] = sums[hi][li];
   }
 }
 
@@ -245,35 +228,25 @@ cudaError_t launch_merge(int n, int batch, int L, int H, int d, const void* cons
   return cudaGetLastError();
 }
 
-cudaError_t launch_dsum(const KArgs& a, float* dsum_clean, float* dsum_noisy, cudaStream_t st) {
+cudaError_t launch_bwd_prepare(const KArgs& a, float* dsum_clean, float* dsum_noisy, bool zero_dq, cudaStream_t st) {
+  PrepArgs pa = {};
   float* out[2] = {dsum_clean, dsum_noisy};
+  long long blocks[2] = {0, 0};
+  pa.H = a.H;
   for (int s = 0; s < 2; ++s) {
     if (a.q[s] == nullptr) continue;   // a stream without queries has no D rows
-    const int rows = rows_q(a, s);
-    const size_t tile_smem = (size_t)a.H * (DS_LB + 1) * sizeof(float);
-    if (tile_smem <= 48 * 1024 && rows > 0) {   // the tiled form: coalesced on both sides
-      const int tpb = (rows + DS_LB - 1) / DS_LB;
-      const int64_t nblk = (int64_t)a.batch * tpb;
-      if (nblk <= 0x7fffffff) {
-        if (a.d == 128) dsum_tile_kernel<128><<<(int)nblk, 256, tile_smem, st>>>(a.dout[s], a.o[s], out[s], rows, a.H, tpb);
-        else dsum_tile_kernel<64><<<(int)nblk, 256, tile_smem, st>>>(a.dout[s], a.o[s], out[s], rows, a.H, tpb);
-        cudaError_t e = cudaGetLastError();
-        if (e != cudaSuccess) return e;
-        continue;
-      }
-    }
-    const int64_t nrows = (int64_t)a.batch * rows * a.H;
-    const int rows_per_block = 8 * (32 / (a.d / 8)) * 4;   // 8 warps, 32 / (d / 8) rows per warp and pass, 4 passes
-    const int blocks = (int)((nrows + rows_per_block - 1) / rows_per_block);
-    if (blocks == 0) continue;
-    if (a.d == 128)
-      dsum_kernel<128><<<blocks, 256, 0, st>>>(a.dout[s], a.o[s], out[s], nrows, rows, a.H);
-    else
-      dsum_kernel<64><<<blocks, 256, 0, st>>>(a.dout[s], a.o[s], out[s], nrows, rows, a.H);
-    cudaError_t e = cudaGetLastError();
-    if (e != cudaSuccess) return e;
+    pa.dout[s] = a.dout[s]; pa.o[s] = a.o[s]; pa.dsum[s] = out[s];
+    pa.dq32[s] = zero_dq ? a.dq32[s] : nullptr;
+    pa.rows[s] = rows_q(a, s); pa.dq32_rows[s] = a.dq32_rows[s];
+    blocks[s] = (long long)a.batch * ((pa.rows[s] + PREP_ROWS - 1) / PREP_ROWS) * ((a.H + PREP_HEADS - 1) / PREP_HEADS);
   }
-  return cudaSuccess;
+  const long long n = blocks[0] + blocks[1];
+  if (n == 0) return cudaSuccess;
+  if (n > 0x7fffffffLL) return cudaErrorInvalidValue;
+  pa.blocks_clean = (int)blocks[0];
+  if (a.d == 128) bwd_prepare_kernel<128><<<(unsigned)n, 256, 0, st>>>(pa);
+  else bwd_prepare_kernel<64><<<(unsigned)n, 256, 0, st>>>(pa);
+  return cudaGetLastError();
 }
 
 }  // namespace bdlm

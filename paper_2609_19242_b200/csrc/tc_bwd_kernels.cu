@@ -903,8 +903,8 @@ tc_dq_kernel(const __grid_constant__ BwdMaps maps, const KArgs a, const TileGrid
 //                  MN-major B operand of dQ^T = K^T dS^T (K, resident, is the MN-major A operand).
 //   dQ             a fourth warpgroup copies each dQ^T tile (lane = head-dim index, column = query) into a
 //                  [64 query x 128] fp32 staging tile, and one of its threads hands it to the TMA engine as
-//                  a bulk add-reduction into the fp32 dQ accumulator [batch, H, rows, 128] (32 KB
-//                  contiguous).  The compute warps never touch dQ; the reduction runs behind the GEMMs.
+//                  a bulk add-reduction into the fp32 dQ accumulator [batch, H, rows, D] (32 KB
+//                  contiguous for D = 128).  The compute warps never touch dQ; the reduction runs behind the GEMMs.
 // dQ depends on the order in which the key tiles' reductions arrive (fp32 rounding only).
 // Shared memory: K, V, a 3-stage Q ring and a 2-stage dO ring of 64-row tiles (+ LSE, D rows, fetched one step
 // ahead by the producer), dS^T, 2 dQ staging tiles of 64 query rows: one reduction per step, the next step's tile
@@ -931,8 +931,8 @@ __host__ __device__ constexpr uint32_t koff_h(int kk) { return (kk >> 2) * HPANE
 __device__ __forceinline__ uint32_t desc_lo_mn_h(uint32_t addr) { return ((addr & 0x3FFFFu) >> 4) | (HPANEL_LO << 16); }
 
 // D = head dimension.  With D = 64 the operand tiles are one panel wide, the contractions over the head dimension take
-// four k-slices and dV / dK have 64 columns; dQ^T keeps its 128 lanes (the upper 64 hold nothing of value and land in
-// the unused half of the 128-wide fp32 accumulator rows).
+// four k-slices and dV / dK have 64 columns; dQ^T keeps its 128 lanes (the upper 64 hold nothing of value and
+// are not read out).
 template <bool TR, int D>
 __global__ void __launch_bounds__(BF_THREADS, 1)
 tc_bwdf_kernel(const __grid_constant__ BwdMaps maps, const KArgs a, const TileGrid tg, int* __restrict__ status) {
@@ -1184,7 +1184,7 @@ tc_bwdf_kernel(const __grid_constant__ BwdMaps maps, const KArgs a, const TileGr
       }
       const long long t0 = tick<TR>();
       if (ok) tc_fence_after();
-      float* dst = a.dq32[st.qs] + (((int64_t)b * a.H + st.h) * a.dq32_rows[st.qs] + st.q0) * 128;
+      float* dst = a.dq32[st.qs] + (((int64_t)b * a.H + st.h) * a.dq32_rows[st.qs] + st.q0) * D;
       uint32_t v[64];
       if (ok) {   // the whole tile into registers first: the tensor core gets its columns back at once
         uint32_t (*c)[32] = reinterpret_cast<uint32_t (*)[32]>(v);
@@ -1200,7 +1200,7 @@ tc_bwdf_kernel(const __grid_constant__ BwdMaps maps, const KArgs a, const TileGr
       if (ok) {
         float* sg = reinterpret_cast<float*>(sm + BF_STG + (i & 1) * STG_BYTES) + dd;
 #pragma unroll
-        for (int e = 0; e < HT; ++e) sg[e * 128] = __uint_as_float(v[e]) * a.scale;
+        for (int e = 0; e < HT; ++e) if (D == 128 || dd < D) sg[e * D] = __uint_as_float(v[e]);   // D = 64: the upper lanes hold nothing
         fence_async_smem();
       }
       // the second meeting also takes the decision to leave, for all 128 threads at once (a flag raised between two
@@ -1214,7 +1214,7 @@ tc_bwdf_kernel(const __grid_constant__ BwdMaps maps, const KArgs a, const TileGr
           : "=r"(leave) : "r"(*abort_flag) : "memory");
       if (leave) break;
       if (leader) {
-        bulk_reduce_add_f32(dst, sSTG + (i & 1) * STG_BYTES, STG_BYTES);
+        bulk_reduce_add_f32(dst, sSTG + (i & 1) * STG_BYTES, HT * D * 4);
         bulk_commit();
       }
       c_ro += tick<TR>() - t0;
@@ -1399,43 +1399,49 @@ tc_bwdf_kernel(const __grid_constant__ BwdMaps maps, const KArgs a, const TileGr
   if (warp == 8) tmem_dealloc(tmem, 512);
 }
 
-// fp32 dQ accumulator [batch, H, rows, 128] -> bf16 dQ [batch, rows, H, D]; one warp per row (D = 64: the first 64
-// of the accumulator row's 128 floats)
+// fp32 dQ accumulators [batch, H, rows, D] -> bf16 dQ [batch, rows, H, D] with the softmax scale, both query streams in
+// one launch.  A block takes 64 rows of one (batch, head), a warp 8 of them, all their loads in flight at once: the
+// kernel is a pure stream (32K rows, H = 32: 1.6 GB in 251 us = 6.4 TB/s; one launch per stream and an index division
+// per row took 311), and index arithmetic is paid once per block.
+struct ConvertArgs {
+  const float* src[2];
+  bf16* dst[2];
+  int rows[2], src_rows[2];
+  int blocks_clean, H;
+  float scale;
+};
 template <int D>
-__global__ void __launch_bounds__(256) dq_convert_kernel(const float* __restrict__ src, bf16* __restrict__ dst, int batch, int H, int rows,
-                                                         int src_rows) {
-  constexpr int U = 4;   // rows per warp in flight: the kernel is a pure stream
-  const int lane = threadIdx.x & 31;
-  const int64_t n = (int64_t)batch * rows * H;
-  const int64_t warps = (int64_t)gridDim.x * 8;
-  for (int64_t o0 = ((int64_t)blockIdx.x * 8 + (threadIdx.x >> 5)) * U; o0 < n; o0 += warps * U) {
-    float4 u4[U];
-    float2 u2[U];
+__global__ void __launch_bounds__(256) dq_convert_kernel(const ConvertArgs ca) {
+  constexpr int U = 8;
+  const int s = (int)blockIdx.x < ca.blocks_clean ? CLEAN : NOISY;
+  int i = blockIdx.x - (s == CLEAN ? 0 : ca.blocks_clean);
+  auto of = [&](const auto& x) { return s == CLEAN ? x[0] : x[1]; };
+  const int rows = of(ca.rows), H = ca.H, src_rows = of(ca.src_rows), tiles = src_rows / 64;
+  const int h = i % H;
+  i /= H;
+  const int l0 = (i % tiles) * 64 + (threadIdx.x >> 5) * U, b = i / tiles, lane = threadIdx.x & 31;
+  const float* src = of(ca.src) + (((int64_t)b * H + h) * src_rows + l0) * D;
+  bf16* dst = of(ca.dst) + (((int64_t)b * rows + l0) * H + h) * D;
+  const int n = min(U, rows - l0);
+  if (D == 128) {
+    float4 u[U];
+#pragma unroll
+    for (int j = 0; j < U; ++j) if (j < n) u[j] = __ldcs(reinterpret_cast<const float4*>(src + j * D) + lane);
 #pragma unroll
     for (int j = 0; j < U; ++j) {
-      const int64_t o = o0 + j;
-      if (o < n) {
-        const int h = (int)(o % H);
-        const int64_t bl = o / H;
-        const int l = (int)(bl % rows), b = (int)(bl / rows);
-        const float* row = src + (((int64_t)b * H + h) * src_rows + l) * 128;
-        if (D == 128) u4[j] = reinterpret_cast<const float4*>(row)[lane];
-        else u2[j] = reinterpret_cast<const float2*>(row)[lane];
+      if (j < n) {
+        uint2 v;
+        v.x = pack_bf16(u[j].x * ca.scale, u[j].y * ca.scale); v.y = pack_bf16(u[j].z * ca.scale, u[j].w * ca.scale);
+        reinterpret_cast<uint2*>(dst + (int64_t)j * H * D)[lane] = v;
       }
     }
+  } else {
+    float2 u[U];
 #pragma unroll
-    for (int j = 0; j < U; ++j) {
-      const int64_t o = o0 + j;
-      if (o < n) {
-        if (D == 128) {
-          uint2 v;
-          v.x = pack_bf16(u4[j].x, u4[j].y); v.y = pack_bf16(u4[j].z, u4[j].w);
-          reinterpret_cast<uint2*>(dst + o * D)[lane] = v;
-        } else {
-          reinterpret_cast<uint32_t*>(dst + o * D)[lane] = pack_bf16(u2[j].x, u2[j].y);
-        }
-      }
-    }
+    for (int j = 0; j < U; ++j) if (j < n) u[j] = __ldcs(reinterpret_cast<const float2*>(src + j * D) + lane);
+#pragma unroll
+    for (int j = 0; j < U; ++j)
+      if (j < n) reinterpret_cast<uint32_t*>(dst + (int64_t)j * H * D)[lane] = pack_bf16(u[j].x * ca.scale, u[j].y * ca.scale);
   }
 }
 
@@ -1446,13 +1452,21 @@ static size_t pad64(size_t rows) { return (rows + 63) / 64 * 64; }
 bool tc_bwd_supported(const KArgs& a) {
   return (a.d == 128 || a.d == 64) && tc_rows_ok(a) && tc_encoder_available();
 }
-// fp32 dQ accumulators of the fused backward: one [batch, H, rows, 128] tensor per query stream
+// fp32 dQ accumulators of the fused backward: one [batch, H, rows, d] tensor per query stream
 size_t tc_bwd_fused_workspace(const bdlm_params* p, const bdlm_packed_geometry* g) {
   if ((p->d != 128 && p->d != 64) || p->impl == 1) return 0;
   const size_t rows_c = g != nullptr ? (size_t)g->Lq_clean : (size_t)p->L;
   const size_t rows_n = g != nullptr ? (size_t)g->n_blocks * p->block_size : (size_t)p->L;
   // rows rounded up to the kernel's 64-row steps: a reduction always covers a whole step
-  return (pad64(rows_c) + pad64(rows_n)) * p->batch * p->H * 128 * sizeof(float);
+  return (pad64(rows_c) + pad64(rows_n)) * p->batch * p->H * p->d * sizeof(float);
+}
+void tc_bwd_place_dq(KArgs& a, void* extra_ws) {
+  float* at = static_cast<float*>(extra_ws);
+  for (int s = 0; s < 2; ++s) {
+    a.dq32_rows[s] = a.q[s] != nullptr ? (int)pad64(rows_q(a, s)) : 0;
+    a.dq32[s] = at;
+    at += (size_t)a.batch * a.H * a.dq32_rows[s] * a.d;
+  }
 }
 
 // How many CTAs share a clean key tile (1, 2 or 4), from two estimates in steps of `rows` query rows: `heavy` for the
@@ -1506,15 +1520,7 @@ static cudaError_t launch_units(Kern kern, const TileGrid& tg, int threads, size
 }
 
 template <int D>
-static cudaError_t launch_tc_bwd_d(const KArgs& a_in, void* extra_ws, int passes, cudaStream_t st) {
-  KArgs a = a_in;
-  a.dq32_rows[CLEAN] = a.q[CLEAN] != nullptr ? (int)pad64(a.Lqc) : 0;
-  a.dq32_rows[NOISY] = a.q[NOISY] != nullptr ? (int)pad64(a.Ln) : 0;
-  const size_t dq32_elems[2] = {(size_t)a.batch * a.H * a.dq32_rows[CLEAN] * 128, (size_t)a.batch * a.H * a.dq32_rows[NOISY] * 128};
-  if (a.single_pass) {
-    a.dq32[0] = static_cast<float*>(extra_ws);
-    a.dq32[1] = a.dq32[0] + dq32_elems[0];
-  }
+static cudaError_t launch_tc_bwd_d(const KArgs& a, int passes, cudaStream_t st) {
   BwdMaps maps;
   for (int s = 0; s < 2; ++s) {
     // a stream that is left out gets the other stream's tensors as placeholders: its maps are never used
@@ -1532,16 +1538,25 @@ static cudaError_t launch_tc_bwd_d(const KArgs& a_in, void* extra_ws, int passes
   if (a.single_pass) {
     // one kernel produces dK, dV and (through fp32 add-reductions) dQ; it runs for the DKDV pass bit, the DQ bit is a no-op
     if (passes & BDLM_BWD_PASS_DKDV) {
-      if ((e = cudaMemsetAsync(a.dq32[0], 0, (dq32_elems[0] + dq32_elems[1]) * sizeof(float), st)) != cudaSuccess) return e;
+      if (!(passes & BDLM_BWD_PASS_DSUM)) {   // otherwise the launch that forms the D rows has cleared the accumulators
+        const size_t rows = (size_t)a.dq32_rows[CLEAN] + a.dq32_rows[NOISY];
+        if ((e = cudaMemsetAsync(a.dq32[CLEAN], 0, rows * a.batch * a.H * D * sizeof(float), st)) != cudaSuccess) return e;
+      }
       auto kern = a.trace ? tc_bwdf_kernel<true, D> : tc_bwdf_kernel<false, D>;
       TileGrid tg = make_tile_grid((max(a.L, a.k[NOISY] != nullptr ? a.Ln : 0) + TILE - 1) / TILE, a.Hkv, a.batch * 2);
       tg.parts = split_key_tiles(a, HT);
       if ((e = launch_units(kern, tg, BF_THREADS, BF_SMEM, st, maps, a, status)) != cudaSuccess) return e;
+      ConvertArgs ca = {};
+      long long blocks[2];
       for (int s2 = 0; s2 < 2; ++s2) {
-        if (dq32_elems[s2] == 0) continue;
-        dq_convert_kernel<D><<<device_sm_count() * 16, 256, 0, st>>>(a.dq32[s2], a.dq[s2], a.batch, a.H, rows_q(a, s2), a.dq32_rows[s2]);
-        if ((e = cudaGetLastError()) != cudaSuccess) return e;
+        ca.src[s2] = a.dq32[s2]; ca.dst[s2] = a.dq[s2];
+        ca.rows[s2] = rows_q(a, s2); ca.src_rows[s2] = a.dq32_rows[s2];
+        blocks[s2] = (long long)a.batch * a.H * (a.dq32_rows[s2] / 64);
       }
+      if (blocks[0] + blocks[1] > 0x7fffffffLL) return cudaErrorInvalidValue;
+      ca.blocks_clean = (int)blocks[0]; ca.H = a.H; ca.scale = a.scale;
+      dq_convert_kernel<D><<<(unsigned)(blocks[0] + blocks[1]), 256, 0, st>>>(ca);
+      return cudaGetLastError();
     }
     return cudaSuccess;
   }
@@ -1562,8 +1577,8 @@ static cudaError_t launch_tc_bwd_d(const KArgs& a_in, void* extra_ws, int passes
   return cudaSuccess;
 }
 
-cudaError_t launch_tc_bwd(const KArgs& a, void* extra_ws, int passes, cudaStream_t st) {
-  return a.d == 64 ? launch_tc_bwd_d<64>(a, extra_ws, passes, st) : launch_tc_bwd_d<128>(a, extra_ws, passes, st);
+cudaError_t launch_tc_bwd(const KArgs& a, int passes, cudaStream_t st) {
+  return a.d == 64 ? launch_tc_bwd_d<64>(a, passes, st) : launch_tc_bwd_d<128>(a, passes, st);
 }
 
 }  // namespace bdlm

@@ -23,6 +23,8 @@ bool tc_bwd_supported(const KArgs& a);
 // Bytes of the fused backward's fp32 dQ accumulators for these sizes (0 when the fused kernel cannot take them).
 size_t tc_bwd_fused_workspace(const bdlm_params* p, const bdlm_packed_geometry* g);
 cudaError_t launch_tc_fwd(const KArgs& a, cudaStream_t st);
-cudaError_t launch_tc_bwd(const KArgs& a, void* extra_ws, int passes, cudaStream_t st);
+// Lays the fused backward's dQ accumulators out in the workspace (a.dq32, a.dq32_rows).
+void tc_bwd_place_dq(KArgs& a, void* extra_ws);
+cudaError_t launch_tc_bwd(const KArgs& a, int passes, cudaStream_t st);
 
 }  // namespace bdlm
