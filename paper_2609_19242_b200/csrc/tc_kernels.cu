@@ -13,7 +13,7 @@ using namespace tc;
 using bf16 = __nv_bfloat16;
 
 struct FwdMaps {
-  CUtensorMap q[2], k[2], v[2];
+  CUtensorMap q[2], k[2], v[2], o[2];
 };
 
 // ---------------------------------------------------------------- host: tensor maps
@@ -109,7 +109,7 @@ struct TileSched {
 };
 
 // ---------------------------------------------------------------- forward, warp-specialised
-// One CTA = one 128-row query tile of TWO query heads of the same KV group (same stream, same rows, so
+// A unit is one 128-row query tile of TWO query heads of the same KV group (same stream, same rows, so
 // the same key tiles and the same masks).  Warp 8 loads Q of both heads once and streams K/V tiles through
 // a 2-stage ring; warp 9 issues tcgen05.mma (QK^T from shared memory, PV with P as a TMEM operand: the whole
 // warp walks the loop, one elected lane issues); warps 0-7 run the online softmax, one warpgroup per head and
@@ -119,14 +119,33 @@ struct TileSched {
 // the S columns it was computed from; O is rescaled only when the running maximum grew by more than 2^8 (the
 // stale maximum is exact in the final LSE and normalisation).
 // With an odd number of query heads per KV head (PAIRQ) the two warpgroups take two consecutive query tiles of
-// ONE head instead: the CTA walks the union of their key tiles (the later tile's list contains the earlier
+// ONE head instead: the unit walks the union of their key tiles (the later tile's list contains the earlier
 // one's except for noisy diagonal tiles), a tile that one of them does not see at all is masked out for it
 // like any other hidden key, and a second tile past the end of the tensor stays masked and is not written.
 // TMEM columns: [0,128) S/P head A   [128,256) S/P head B   [256,384) O head A   [384,512) O head B
+//
+// A CTA works on one unit after another: the grid has a CTA per unit, and a running CTA takes over the next one that
+// has not started (cluster launch control), so the start order still decides who goes first.  Tensor memory,
+// barriers and the K/V ring carry over, the next unit's Q is loaded once the last Q K^T has read the old one, its first
+// Q K^T runs under the previous unit's last P V and output, and O leaves through a 4 KB staging tile per warp and
+// TMA stores.  With one unit per CTA, 16k of the 43k clk of a 1024-key window's unit were not tile work: set-up
+// 2k, first scores 4.5k, 16-byte row stores 3.9k (each a memory line of its own), exit and start of the next CTA 4.2k.
+// Forward: L = 2048, H = 32 82 -> 69 us, windowed 32K 1.46 -> 1.26 ms, 2 x 8K, H = 16 1.05 -> 1.01 ms, 32K 15.0 -> 14.7 ms.
 constexpr int FWDR_THREADS = 384;                            // 8 softmax warps, producer warp, MMA warp, two idle ones
 constexpr int FWDR_REGS_SOFTMAX = 224, FWDR_REGS_REST = 56;  // 256 x 224 + 128 x 56 = 384 x 168, what the block is launched with
-constexpr int FWDR_BARS = 6 * TILE_BYTES;                    // after Q (2 tiles) and the K/V ring (2 stages x 2 tiles)
-constexpr int FWDR_SMEM = FWDR_BARS + 256 + 1024;
+constexpr int FWDR_STG = 6 * TILE_BYTES;                     // after Q (2 tiles) and the K/V ring (2 stages x 2 tiles)
+constexpr int FWDR_STG_WARP = 32 * 128;                      // per softmax warp: 32 rows x 64 columns of O
+constexpr int FWDR_BARS = FWDR_STG + 8 * FWDR_STG_WARP;
+constexpr int FWDR_SMEM = FWDR_BARS + 512 + 1024;
+
+// What a CTA knows about a unit; written to shared memory by the producer, two slots in turn.
+struct FwdUnit {
+  int more;                // 0: no unit left
+  int qs, b, h0, q0;
+  TileSched sch;
+};
+constexpr int FWD_UNIT_BYTES = 64;
+static_assert(sizeof(FwdUnit) <= FWD_UNIT_BYTES, "unit slot");
 
 // D = head dimension (128 or 64).  With D = 64 a tile is one 64-column panel: the second panel of every shared-memory
 // tile stays unused, Q K^T contracts over four k-slices and P V produces 64 output columns.
@@ -135,92 +154,140 @@ __global__ void __launch_bounds__(FWDR_THREADS, 1)
 tc_fwdr_kernel(const __grid_constant__ FwdMaps maps, const KArgs a, const TileGrid tg, int* __restrict__ status) {
   constexpr uint32_t IDESC_PV = make_idesc(128, D, false, true);
   constexpr int OPER_BYTES = TILE_BYTES * D / 128;   // bytes TMA delivers per operand tile
+  // warpgroup w works on head h0 + w * HSTEP, query rows q0 + w * QSTEP ...
+  constexpr int HSTEP = PAIRQ ? 0 : 1, QSTEP = PAIRQ ? TILE : 0, QROWS = PAIRQ ? 2 * TILE : TILE;
   extern __shared__ uint8_t smem_raw[];
   const uint32_t base = (smem_u32(smem_raw) + 1023u) & ~1023u;
   uint8_t* sm = smem_raw + (base - smem_u32(smem_raw));
   const uint32_t sQ = base, sK0 = base + 2 * TILE_BYTES;   // stage s: K at sK0 + s*2*TILE, V after it
   const uint32_t bars = base + FWDR_BARS;
   const uint32_t bar_q = bars, bar_k_full = bars + 8 /*[2]*/, bar_v_full = bars + 24 /*[2]*/, bar_kv_empty = bars + 40 /*[2]*/,
-                 bar_s = bars + 56 /*[2]*/, bar_o = bars + 72 /*[2]*/, bar_p = bars + 88 /*[head][key half]*/;
-  volatile uint32_t* tmem_slot = reinterpret_cast<volatile uint32_t*>(sm + FWDR_BARS + 128);
-  volatile int* abort_flag = reinterpret_cast<volatile int*>(sm + FWDR_BARS + 136);
-
-  int bx, by, bz;
-  tile_grid_decode(tg, blockIdx.x, bx, by, bz);
-  const int qs = bz & 1, b = bz >> 1;
-  if (a.q[qs] == nullptr) return;
-  // warpgroup w works on head h0 + w * HSTEP, query rows q0 + w * QSTEP ...
-  constexpr int HSTEP = PAIRQ ? 0 : 1, QSTEP = PAIRQ ? TILE : 0, QROWS = PAIRQ ? 2 * TILE : TILE;
-  const int h0 = PAIRQ ? by : by * 2, hk = h0 / a.G;
-  const int q0 = (tg.nx - 1 - bx) * QROWS;   // the last query tile sees the most keys: started first
-  const int Lq = rows_q(a, qs);
-  if (q0 >= Lq) return;
+                 bar_s = bars + 56 /*[2]*/, bar_o = bars + 72 /*[2]*/, bar_p = bars + 88 /*[head][key half]*/,
+                 bar_q_empty = bars + 120, bar_unit_full = bars + 128 /*[2]*/, bar_unit_empty = bars + 144 /*[2]*/,
+                 bar_clc = bars + 160, clc_slot = bars + 176;
+  volatile uint32_t* tmem_slot = reinterpret_cast<volatile uint32_t*>(sm + FWDR_BARS + 192);
+  volatile int* abort_flag = reinterpret_cast<volatile int*>(sm + FWDR_BARS + 200);
+  auto unit_slot = [&](int k) { return reinterpret_cast<FwdUnit*>(sm + FWDR_BARS + 256 + (k & 1) * FWD_UNIT_BYTES); };
   const int warp = __shfl_sync(0xffffffffu, threadIdx.x >> 5, 0), lane = threadIdx.x & 31;   // warp index, provably uniform
 
-  TileSched sch;
-  sch.init(qs, q0, min(q0 + QROWS, Lq) - 1, a);
-  const int nt = sch.nt0 + sch.nt1;
-  auto tile_ks = [&](int t) { return t < sch.nt0 ? 0 : 1; };
-  auto tile_k0 = [&](int t) { return t < sch.nt0 ? sch.lo0 + t * TILE : sch.lo1 + (t - sch.nt0) * TILE; };
+  auto tile_ks = [](const TileSched& sch, int t) { return t < sch.nt0 ? 0 : 1; };
+  auto tile_k0 = [](const TileSched& sch, int t) { return t < sch.nt0 ? sch.lo0 + t * TILE : sch.lo1 + (t - sch.nt0) * TILE; };
 
-  if (threadIdx.x == 0) {
-    mbar_init(bar_q, 1);
-    for (int i = 0; i < 2; ++i) {
-      mbar_init(bar_k_full + 8 * i, 1); mbar_init(bar_v_full + 8 * i, 1); mbar_init(bar_kv_empty + 8 * i, 1);
-      mbar_init(bar_s + 8 * i, 1); mbar_init(bar_o + 8 * i, 1);
-      mbar_init(bar_p + 16 * i, 128); mbar_init(bar_p + 16 * i + 8, 128);
+  // The producer starts loading as soon as the barriers are set up; everyone else also needs tensor memory.
+  if (warp == 8) {
+    if (lane == 0) {
+      mbar_init(bar_q, 1); mbar_init(bar_q_empty, 1); mbar_init(bar_clc, 1);
+      for (int i = 0; i < 2; ++i) {
+        mbar_init(bar_k_full + 8 * i, 1); mbar_init(bar_v_full + 8 * i, 1); mbar_init(bar_kv_empty + 8 * i, 1);
+        mbar_init(bar_s + 8 * i, 1); mbar_init(bar_o + 8 * i, 1);
+        mbar_init(bar_p + 16 * i, 128); mbar_init(bar_p + 16 * i + 8, 128);
+        mbar_init(bar_unit_full + 8 * i, 1); mbar_init(bar_unit_empty + 8 * i, 9);   // read by the MMA warp and 8 softmax warps
+      }
+      *abort_flag = 0;
+      fence_mbar_init();
+      fence_async_smem();   // this thread issues its first loads without a block barrier in between
     }
-    *abort_flag = 0;
-    fence_mbar_init();
+    __syncwarp();
+    asm volatile("barrier.cta.arrive 1, 384;" ::: "memory");
+  } else {
+    if (warp == 9) tmem_alloc(smem_u32(const_cast<uint32_t*>(tmem_slot)), 512);
+    tc_fence_before();
+    asm volatile("barrier.cta.sync 1, 384;" ::: "memory");
+    tc_fence_after();
   }
-  if (warp == 8) tmem_alloc(smem_u32(const_cast<uint32_t*>(tmem_slot)), 512);
-  tc_fence_before();
-  __syncthreads();
-  tc_fence_after();
-  const uint32_t tmem = __shfl_sync(0xffffffffu, *tmem_slot, 0);   // broadcast: provably warp-uniform
-  // TMEM columns: [0,128) S/P head A   [128,256) S/P head B   [256,384) O head A   [384,512) O head B
 
   if (warp >= 8) {
     reg_dec<FWDR_REGS_REST>();
     if (warp == 8) {
-    if (lane == 0 && nt > 0) {
-      mbar_expect_tx(bar_q, 2 * OPER_BYTES);
-      tma_load_3d(sQ, &maps.q[qs], bar_q, h0 * D, q0, b);
-      if (D == 128) tma_load_3d(sQ + PANEL_BYTES, &maps.q[qs], bar_q, h0 * D + 64, q0, b);
-      // (rows past the end of the tensor are filled with zeros)
-      tma_load_3d(sQ + TILE_BYTES, &maps.q[qs], bar_q, (h0 + HSTEP) * D, q0 + QSTEP, b);
-      if (D == 128) tma_load_3d(sQ + TILE_BYTES + PANEL_BYTES, &maps.q[qs], bar_q, (h0 + HSTEP) * D + 64, q0 + QSTEP, b);
-      bool ok = true;
-      for (int t = 0; t < nt && ok; ++t) {
-        const int s = t & 1;
-        if (t >= 2) ok = mbar_wait_abortable(bar_kv_empty + 8 * s, ((t >> 1) - 1) & 1, abort_flag);
-        if (!ok) break;
-        const int ks = tile_ks(t), k0 = tile_k0(t);
-        const uint32_t dK = sK0 + s * 2 * TILE_BYTES, dV = dK + TILE_BYTES;
-        mbar_expect_tx(bar_k_full + 8 * s, OPER_BYTES);
-        const int krow = ks == CLEAN ? clean_key_row(a, k0) : k0;   // where the tile's first key is stored
-        tma_load_3d(dK, &maps.k[ks], bar_k_full + 8 * s, hk * D, krow, b);
-        if (D == 128) tma_load_3d(dK + PANEL_BYTES, &maps.k[ks], bar_k_full + 8 * s, hk * D + 64, krow, b);
-        mbar_expect_tx(bar_v_full + 8 * s, OPER_BYTES);
-        tma_load_3d(dV, &maps.v[ks], bar_v_full + 8 * s, hk * D, krow, b);
-        if (D == 128) tma_load_3d(dV + PANEL_BYTES, &maps.v[ks], bar_v_full + 8 * s, hk * D + 64, krow, b);
+      // ------------------------------------------------------------------ producer
+      if (lane == 0) {
+        const bool two = a.q[CLEAN] != nullptr && a.q[NOISY] != nullptr;
+        int index = blockIdx.x, g = 0, n_units = 0, n_q = 0, n_clc = 0;   // g: K/V tiles loaded so far
+        bool ok = true, asked = false;
+        while (ok) {
+          clc_request(clc_slot, bar_clc);   // answered while this unit is loaded
+          asked = true;
+          int bx, by, bz;
+          tile_grid_decode(tg, index, bx, by, bz);
+          const int qs = two ? bz & 1 : (a.q[CLEAN] != nullptr ? CLEAN : NOISY), b = two ? bz >> 1 : bz;
+          const int h0 = PAIRQ ? by : by * 2, hk = h0 / a.G;
+          const int q0 = (tg.nx - 1 - bx) * QROWS;   // the last query tile sees the most keys: started first
+          const int Lq = rows_q(a, qs);
+          if (q0 < Lq) {
+            TileSched sch;
+            sch.init(qs, q0, min(q0 + QROWS, Lq) - 1, a);
+            if (n_units >= 2) ok = mbar_wait_abortable(bar_unit_empty + 8 * (n_units & 1), ((n_units >> 1) - 1) & 1, abort_flag);
+            if (!ok) break;
+            FwdUnit* slot = unit_slot(n_units);
+            slot->more = 1; slot->qs = qs; slot->b = b; slot->h0 = h0; slot->q0 = q0; slot->sch = sch;
+            mbar_arrive(bar_unit_full + 8 * (n_units & 1));
+            ++n_units;
+            const int nt = sch.nt0 + sch.nt1;
+            if (nt > 0) {
+              if (n_q > 0) ok = mbar_wait_abortable(bar_q_empty, (n_q - 1) & 1, abort_flag);
+              if (!ok) break;
+              ++n_q;
+              mbar_expect_tx(bar_q, 2 * OPER_BYTES);
+              tma_load_3d(sQ, &maps.q[qs], bar_q, h0 * D, q0, b);
+              if (D == 128) tma_load_3d(sQ + PANEL_BYTES, &maps.q[qs], bar_q, h0 * D + 64, q0, b);
+              // (rows past the end of the tensor are filled with zeros)
+              tma_load_3d(sQ + TILE_BYTES, &maps.q[qs], bar_q, (h0 + HSTEP) * D, q0 + QSTEP, b);
+              if (D == 128) tma_load_3d(sQ + TILE_BYTES + PANEL_BYTES, &maps.q[qs], bar_q, (h0 + HSTEP) * D + 64, q0 + QSTEP, b);
+            }
+            for (int t = 0; t < nt; ++t, ++g) {
+              const int s = g & 1;
+              if (g >= 2) ok = mbar_wait_abortable(bar_kv_empty + 8 * s, ((g >> 1) - 1) & 1, abort_flag);
+              if (!ok) break;
+              const int ks = tile_ks(sch, t), k0 = tile_k0(sch, t);
+              const uint32_t dK = sK0 + s * 2 * TILE_BYTES, dV = dK + TILE_BYTES;
+              mbar_expect_tx(bar_k_full + 8 * s, OPER_BYTES);
+              const int krow = ks == CLEAN ? clean_key_row(a, k0) : k0;   // where the tile's first key is stored
+              tma_load_3d(dK, &maps.k[ks], bar_k_full + 8 * s, hk * D, krow, b);
+              if (D == 128) tma_load_3d(dK + PANEL_BYTES, &maps.k[ks], bar_k_full + 8 * s, hk * D + 64, krow, b);
+              mbar_expect_tx(bar_v_full + 8 * s, OPER_BYTES);
+              tma_load_3d(dV, &maps.v[ks], bar_v_full + 8 * s, hk * D, krow, b);
+              if (D == 128) tma_load_3d(dV + PANEL_BYTES, &maps.v[ks], bar_v_full + 8 * s, hk * D + 64, krow, b);
+            }
+            if (!ok) break;
+          }
+          ok = mbar_wait_abortable(bar_clc, n_clc & 1, abort_flag);
+          if (!ok) break;
+          asked = false;
+          ++n_clc;
+          const bool more = clc_answer(clc_slot, index);
+          if (!more) break;
+          fence_async_smem();   // the answer has been read before the next request may overwrite it
+        }
+        if (!ok && asked) {   // leaving early: not before the answer on its way has landed (bounded)
+          const long long t0 = clock64();
+          while (!mbar_try_wait(bar_clc, n_clc & 1) && clock64() - t0 < WAIT_LIMIT_TICKS) {}
+        }
+        if (ok && n_units >= 2) ok = mbar_wait_abortable(bar_unit_empty + 8 * (n_units & 1), ((n_units >> 1) - 1) & 1, abort_flag);
+        if (ok) {
+          unit_slot(n_units)->more = 0;
+          mbar_arrive(bar_unit_full + 8 * (n_units & 1));
+        }
       }
-    }
-  } else if (warp == 9) {
-    // the whole warp walks the MMA loop; one elected lane issues (see elect_one)
-    if (nt > 0) {
+    } else if (warp == 9) {
+      // ------------------------------------------------------------------ MMA issuer
+      // the whole warp walks the MMA loop; one elected lane issues (see elect_one).  A wait that fails only clears `ok`:
+      // the lanes of the warp stay together (later waits return at once when the abort flag is up) and leave with the
+      // next unit, whose tile count is broadcast so that the loop is provably uniform.
+      const uint32_t tmem = __shfl_sync(0xffffffffu, *tmem_slot, 0);   // broadcast: provably warp-uniform
       const uint32_t el = elect_one();
       const uint32_t qa_lo = desc_lo_k(sQ), qb_lo = qa_lo + TILE_LO;
       const uint32_t k_lo0 = desc_lo_k(sK0), v_lo0 = desc_lo_mn(sK0 + TILE_BYTES);
-      bool ok = mbar_wait_abortable(bar_q, 0, abort_flag);
-      ok = ok && mbar_wait_abortable(bar_k_full, 0, abort_flag);
-      if (ok) {
-        tc_fence_after();
-        gemm_ss_e<D / 16>(tmem, qa_lo, k_lo0, IDESC_QK, 0u, el);
-        mma_commit_e(bar_s, el);
-        gemm_ss_e<D / 16>(tmem + 128, qb_lo, k_lo0, IDESC_QK, 0u, el);
-        mma_commit_e(bar_s + 8, el);
-      }
+      int n_units = 0;
+      bool ok = true;
+      // tiles of the next unit (0: it sees no key), -1 when none is left
+      auto next_unit = [&]() {
+        ok = mbar_wait_abortable(bar_unit_full + 8 * (n_units & 1), (n_units >> 1) & 1, abort_flag) && ok;
+        const volatile FwdUnit* u = unit_slot(n_units);
+        const int n = __shfl_sync(0xffffffffu, ok && u->more ? u->sch.nt0 + u->sch.nt1 : -1, 0);
+        if (lane == 0) mbar_arrive(bar_unit_empty + 8 * (n_units & 1));
+        ++n_units;
+        return n;
+      };
       // O += P V over key half j of the tile: four k-slices of 16 keys
       auto pv_half = [&](uint32_t d, uint32_t p_tmem, uint32_t v_lo, int j, uint32_t acc_first) {
 #pragma unroll
@@ -229,200 +296,255 @@ tc_fwdr_kernel(const __grid_constant__ FwdMaps maps, const KArgs a, const TileGr
       };
       long long w_p = 0, w_v = 0, w_k = 0;
       const long long tm0 = tick<TR>();
-      for (int t = 0; t < nt && ok; ++t) {
-        const int s = t & 1;
-        const uint32_t cv_lo = v_lo0 + s * 2 * TILE_LO;
-        const uint32_t nk_lo = k_lo0 + (s ^ 1) * 2 * TILE_LO;
-        const uint32_t acc = t > 0 ? 1u : 0u;
-        // head A: P arrives in two halves of the keys (bf16 pairs at columns [0,32) and [32,64) of the head's S
-        // region), so P V over the first 64 keys runs while the softmax is still in the exponentials of the rest
-        ok = mbar_wait_timed<TR>(bar_p, t & 1, abort_flag, w_p);
-        ok = ok && mbar_wait_timed<TR>(bar_v_full + 8 * s, (t >> 1) & 1, abort_flag, w_v);
-        if (!ok) break;
-        tc_fence_after();
-        pv_half(tmem + 256, tmem, cv_lo, 0, acc);
-        ok = mbar_wait_timed<TR>(bar_p + 8, t & 1, abort_flag, w_p);
-        if (!ok) break;
-        tc_fence_after();
-        pv_half(tmem + 256, tmem, cv_lo, 1, 1u);
-        mma_commit_e(bar_o, el);
-        if (t + 1 < nt) {
-          ok = mbar_wait_timed<TR>(bar_k_full + 8 * (s ^ 1), ((t + 1) >> 1) & 1, abort_flag, w_k);
-          if (!ok) break;
+      int nt = 0, g = 0, n_q = 0;   // g: tiles done so far, n_q: units whose Q has been waited for
+      while (nt >= 0) {
+        if (nt == 0) {   // the first unit, and after units that see no key: nothing in flight to overlap with
+          nt = next_unit();
+          if (nt <= 0) continue;
+          ok = mbar_wait_abortable(bar_q, n_q & 1, abort_flag) && ok;
+          ok = mbar_wait_abortable(bar_k_full + 8 * (g & 1), (g >> 1) & 1, abort_flag) && ok;
+          ++n_q;
           tc_fence_after();
-          gemm_ss_e<D / 16>(tmem, qa_lo, nk_lo, IDESC_QK, 0u, el);
+          const uint32_t k_lo = k_lo0 + (g & 1) * 2 * TILE_LO;
+          gemm_ss_e<D / 16>(tmem, qa_lo, k_lo, IDESC_QK, 0u, el);
           mma_commit_e(bar_s, el);
-        }
-        // head B
-        ok = mbar_wait_timed<TR>(bar_p + 16, t & 1, abort_flag, w_p);
-        if (!ok) break;
-        tc_fence_after();
-        pv_half(tmem + 384, tmem + 128, cv_lo, 0, acc);
-        ok = mbar_wait_timed<TR>(bar_p + 24, t & 1, abort_flag, w_p);
-        if (!ok) break;
-        tc_fence_after();
-        pv_half(tmem + 384, tmem + 128, cv_lo, 1, 1u);
-        mma_commit_e(bar_o + 8, el);
-        mma_commit_e(bar_kv_empty + 8 * s, el);
-        if (t + 1 < nt) {
-          gemm_ss_e<D / 16>(tmem + 128, qb_lo, nk_lo, IDESC_QK, 0u, el);
+          gemm_ss_e<D / 16>(tmem + 128, qb_lo, k_lo, IDESC_QK, 0u, el);
           mma_commit_e(bar_s + 8, el);
+          if (nt == 1) mma_commit_e(bar_q_empty, el);
         }
+        int nt_next = 0;
+        for (int t = 0; t < nt; ++t, ++g) {
+          const int s = g & 1;
+          const uint32_t cv_lo = v_lo0 + s * 2 * TILE_LO;
+          const uint32_t nk_lo = k_lo0 + (s ^ 1) * 2 * TILE_LO;
+          const uint32_t acc = t > 0 ? 1u : 0u;
+          // head A: P arrives in two halves of the keys (bf16 pairs at columns [0,32) and [32,64) of the head's S
+          // region), so P V over the first 64 keys runs while the softmax is still in the exponentials of the rest
+          ok = mbar_wait_timed<TR>(bar_p, g & 1, abort_flag, w_p) && ok;
+          ok = mbar_wait_timed<TR>(bar_v_full + 8 * s, (g >> 1) & 1, abort_flag, w_v) && ok;
+          tc_fence_after();
+          pv_half(tmem + 256, tmem, cv_lo, 0, acc);
+          ok = mbar_wait_timed<TR>(bar_p + 8, g & 1, abort_flag, w_p) && ok;
+          tc_fence_after();
+          pv_half(tmem + 256, tmem, cv_lo, 1, 1u);
+          mma_commit_e(bar_o, el);
+          // the next tile's scores: this unit's, or the first of the next unit (whose Q has been loaded meanwhile).
+          // Only one unit ahead: the one after it is announced when the softmax warps have left this one, and they
+          // still wait for head B's P V below.
+          bool more = t + 1 < nt, q_done = t + 2 == nt;   // q_done: they are the last that read Q
+          if (!more) {
+            nt_next = next_unit();
+            if (nt_next > 0) {
+              ok = mbar_wait_timed<TR>(bar_q, n_q & 1, abort_flag, w_k) && ok;
+              ++n_q;
+              more = true;
+              q_done = nt_next == 1;
+            }
+          }
+          if (more) {
+            ok = mbar_wait_timed<TR>(bar_k_full + 8 * (s ^ 1), ((g + 1) >> 1) & 1, abort_flag, w_k) && ok;
+            tc_fence_after();
+            gemm_ss_e<D / 16>(tmem, qa_lo, nk_lo, IDESC_QK, 0u, el);
+            mma_commit_e(bar_s, el);
+          }
+          // head B
+          ok = mbar_wait_timed<TR>(bar_p + 16, g & 1, abort_flag, w_p) && ok;
+          tc_fence_after();
+          pv_half(tmem + 384, tmem + 128, cv_lo, 0, acc);
+          ok = mbar_wait_timed<TR>(bar_p + 24, g & 1, abort_flag, w_p) && ok;
+          tc_fence_after();
+          pv_half(tmem + 384, tmem + 128, cv_lo, 1, 1u);
+          mma_commit_e(bar_o + 8, el);
+          mma_commit_e(bar_kv_empty + 8 * s, el);
+          if (more) {
+            gemm_ss_e<D / 16>(tmem + 128, qb_lo, nk_lo, IDESC_QK, 0u, el);
+            mma_commit_e(bar_s + 8, el);
+            if (q_done) mma_commit_e(bar_q_empty, el);
+          }
+        }
+        nt = nt_next;
       }
       if (lane == 0) {
         trace_add(a.trace, 8, tick<TR>() - tm0); trace_add(a.trace, 9, w_p); trace_add(a.trace, 10, w_v); trace_add(a.trace, 11, w_k);
       }
-    }
+    } else if (lane < 2 && warp == 10) {
+      prefetch_tmap(&maps.k[lane]); prefetch_tmap(&maps.v[lane]); prefetch_tmap(&maps.o[lane]);
     }
   } else {
+    // ------------------------------------------------------------------ softmax: one warpgroup per head, one thread per query row
     reg_inc<FWDR_REGS_SOFTMAX>();
-    const int w = warp >> 2;                               // head: one warpgroup per head, one thread per query row
+    const uint32_t tmem = __shfl_sync(0xffffffffu, *tmem_slot, 0);
+    const int w = warp >> 2;
     const int r = (warp & 3) * 32 + lane;
-    const int row = q0 + w * QSTEP + r;
-    const int h = h0 + w * HSTEP;
-    const bool row_ok = row < Lq;                            // PAIRQ: the second tile may lie past the end
     const uint32_t lane_base = (uint32_t)((warp & 3) * 32) << 16;
     const uint32_t tS = tmem + lane_base + w * 128;          // this row's 128 score columns
     const uint32_t tO = tmem + lane_base + 256 + w * 128;    // and its 128 output columns
-    int rlo0 = 0, rhi0 = 0, rlo1 = 0, rhi1 = 0;
-    if (row_ok) {
-      visible_interval(a, qs, 0, row, rlo0, rhi0);
-      visible_interval(a, qs, 1, row, rlo1, rhi1);
-    }
-    float m_ref = -INFINITY, l = 0.f;
+    const uint32_t stg = base + FWDR_STG + warp * FWDR_STG_WARP;
     bool ok = true;
+    int g = 0;   // tiles done so far
     long long w_s = 0, c_ld = 0, c_max = 0, c_exp = 0;
     const long long t_begin = tick<TR>();
-    for (int t = 0; t < nt && ok; ++t) {
-      const int ks = tile_ks(t), k0 = tile_k0(t);
-      ok = mbar_wait_timed<TR>(bar_s + 8 * w, t & 1, abort_flag, w_s);
+    for (int k = 0; ok; ++k) {
+      ok = mbar_wait_abortable(bar_unit_full + 8 * (k & 1), (k >> 1) & 1, abort_flag);
       ok = __all_sync(0xffffffffu, ok);
       if (!ok) break;
-      tc_fence_after();
-      const bool need_mask = sch.need_mask(ks, k0) || q0 + QROWS > Lq;   // rows past the end of the tensor see nothing
-      const int vlo = (ks == 0 ? rlo0 : rlo1) - k0, vhi = (ks == 0 ? rhi0 : rhi1) - k0;
-      // the whole row of the tile in registers: one pass over S.  The softmax warps are bound by instruction issue and
-      // by the exponential unit, so the arithmetic is packed two to an instruction where it can be (scaling, sums,
-      // three-input maxima) and hidden keys are cleared by bit masks: 3330 -> 2900 clk per key tile of two heads,
-      // 5750 -> 3900 for a masked first one; forward at L = 2048, H = 32: 88.8 -> 82.1 us, windowed 32K layer
-      // 1.57 -> 1.46 ms.  Long sequences run into the power cap: 32K 15.2 -> 15.0 ms.
-      const long long tp0 = tick<TR>();
-      uint32_t v[128];
-      {
-        uint32_t (*c)[32] = reinterpret_cast<uint32_t (*)[32]>(v);
-        tmem_ld32(tS, c[0]); tmem_ld32(tS + 32, c[1]); tmem_ld32(tS + 64, c[2]); tmem_ld32(tS + 96, c[3]);
-        tmem_wait_ld();
+      const FwdUnit un = *unit_slot(k);
+      __syncwarp();
+      if (lane == 0) mbar_arrive(bar_unit_empty + 8 * (k & 1));
+      if (!un.more) break;
+      const TileSched sch = un.sch;
+      const int qs = un.qs, b = un.b, nt = sch.nt0 + sch.nt1;
+      const int Lq = rows_q(a, qs), row = un.q0 + w * QSTEP + r, h = un.h0 + w * HSTEP;
+      const bool row_ok = row < Lq;                            // PAIRQ: the second tile may lie past the end
+      int rlo0 = 0, rhi0 = 0, rlo1 = 0, rhi1 = 0;
+      if (row_ok) {
+        visible_interval(a, qs, 0, row, rlo0, rhi0);
+        visible_interval(a, qs, 1, row, rlo1, rhi1);
       }
-      const long long tp1 = tick<TR>();
-      if (need_mask) {
-#pragma unroll
-        for (int g = 0; g < 4; ++g) {   // -inf on hidden keys: one bit per key, so an element costs one test and one select
-          const uint32_t seen = interval_bits(vlo - 32 * g, vhi - 32 * g);
-#pragma unroll
-          for (int e = 0; e < 32; ++e) v[32 * g + e] = (seen >> e) & 1u ? v[32 * g + e] : 0xff800000u;
+      float m_ref = -INFINITY, l = 0.f;
+      for (int t = 0; t < nt; ++t, ++g) {
+        const int ks = tile_ks(sch, t), k0 = tile_k0(sch, t);
+        ok = mbar_wait_timed<TR>(bar_s + 8 * w, g & 1, abort_flag, w_s);
+        ok = __all_sync(0xffffffffu, ok);
+        if (!ok) break;
+        tc_fence_after();
+        const bool need_mask = sch.need_mask(ks, k0) || un.q0 + QROWS > Lq;   // rows past the end of the tensor see nothing
+        const int vlo = (ks == 0 ? rlo0 : rlo1) - k0, vhi = (ks == 0 ? rhi0 : rhi1) - k0;
+        // the whole row of the tile in registers: one pass over S.  The softmax warps are bound by instruction issue and
+        // by the exponential unit, so the arithmetic is packed two to an instruction where it can be (scaling, sums,
+        // three-input maxima) and hidden keys are cleared by bit masks: 3330 -> 2900 clk per key tile of two heads,
+        // 5750 -> 3900 for a masked first one; forward at L = 2048, H = 32: 88.8 -> 82.1 us, windowed 32K layer
+        // 1.57 -> 1.46 ms.  Long sequences run into the power cap: 32K 15.2 -> 15.0 ms.
+        const long long tp0 = tick<TR>();
+        uint32_t v[128];
+        {
+          uint32_t (*c)[32] = reinterpret_cast<uint32_t (*)[32]>(v);
+          tmem_ld32(tS, c[0]); tmem_ld32(tS + 32, c[1]); tmem_ld32(tS + 64, c[2]); tmem_ld32(tS + 96, c[3]);
+          tmem_wait_ld();
         }
-      }
-      float mx0 = -INFINITY, mx1 = -INFINITY, mx2 = -INFINITY, mx3 = -INFINITY;
+        const long long tp1 = tick<TR>();
+        if (need_mask) {
 #pragma unroll
-      for (int e = 0; e < 32; e += 2) {
-        mx0 = max3(mx0, __uint_as_float(v[e]), __uint_as_float(v[e + 1]));
-        mx1 = max3(mx1, __uint_as_float(v[32 + e]), __uint_as_float(v[33 + e]));
-        mx2 = max3(mx2, __uint_as_float(v[64 + e]), __uint_as_float(v[65 + e]));
-        mx3 = max3(mx3, __uint_as_float(v[96 + e]), __uint_as_float(v[97 + e]));
-      }
-      const float mx = fmaxf(fmaxf(mx0, mx1), fmaxf(mx2, mx3)) * a.scale_log2;
-      const float m_new = fmaxf(m_ref, mx);
-      const bool grow = m_new > m_ref + 8.0f;
-      if (__any_sync(0xffffffffu, grow)) {
-        const float mb_new = (m_new == -INFINITY) ? 0.f : m_new;
-        const float corr = exp2f(m_ref - mb_new);
-        m_ref = m_new;
-        l *= corr;
-        if (t > 0) {
-          ok = mbar_wait_abortable(bar_o + 8 * w, (t - 1) & 1, abort_flag);
-          ok = __all_sync(0xffffffffu, ok);
-          if (!ok) break;
-          tc_fence_after();
+          for (int j = 0; j < 4; ++j) {   // -inf on hidden keys: one bit per key, so an element costs one test and one select
+            const uint32_t seen = interval_bits(vlo - 32 * j, vhi - 32 * j);
+#pragma unroll
+            for (int e = 0; e < 32; ++e) v[32 * j + e] = (seen >> e) & 1u ? v[32 * j + e] : 0xff800000u;
+          }
+        }
+        float mx0 = -INFINITY, mx1 = -INFINITY, mx2 = -INFINITY, mx3 = -INFINITY;
+#pragma unroll
+        for (int e = 0; e < 32; e += 2) {
+          mx0 = max3(mx0, __uint_as_float(v[e]), __uint_as_float(v[e + 1]));
+          mx1 = max3(mx1, __uint_as_float(v[32 + e]), __uint_as_float(v[33 + e]));
+          mx2 = max3(mx2, __uint_as_float(v[64 + e]), __uint_as_float(v[65 + e]));
+          mx3 = max3(mx3, __uint_as_float(v[96 + e]), __uint_as_float(v[97 + e]));
+        }
+        const float mx = fmaxf(fmaxf(mx0, mx1), fmaxf(mx2, mx3)) * a.scale_log2;
+        const float m_new = fmaxf(m_ref, mx);
+        const bool grow = m_new > m_ref + 8.0f;
+        if (__any_sync(0xffffffffu, grow)) {
+          const float mb_new = (m_new == -INFINITY) ? 0.f : m_new;
+          const float corr = exp2f(m_ref - mb_new);
+          m_ref = m_new;
+          l *= corr;
+          if (t > 0) {
+            ok = mbar_wait_abortable(bar_o + 8 * w, (g - 1) & 1, abort_flag);
+            ok = __all_sync(0xffffffffu, ok);
+            if (!ok) break;
+            tc_fence_after();
 #pragma unroll 1
-          for (int c = 0; c < D / 32; ++c) {
-            uint32_t o[32];
-            tmem_ld32(tO + c * 32, o);
-            tmem_wait_ld();
+            for (int c = 0; c < D / 32; ++c) {
+              uint32_t o[32];
+              tmem_ld32(tO + c * 32, o);
+              tmem_wait_ld();
 #pragma unroll
-            for (int e = 0; e < 32; ++e) o[e] = __float_as_uint(__uint_as_float(o[e]) * corr);
-            tmem_st32(tO + c * 32, o);
+              for (int e = 0; e < 32; ++e) o[e] = __float_as_uint(__uint_as_float(o[e]) * corr);
+              tmem_st32(tO + c * 32, o);
+            }
           }
         }
-      }
-      const float mb = (m_ref == -INFINITY) ? 0.f : m_ref;
-      const long long tp2 = tick<TR>();
-      // p = exp2(s * scale - m) (exp2(-inf) = 0 on hidden keys); bf16 pairs over the first 64 columns
-      uint64_t ps0 = 0, ps1 = 0;
-      const uint64_t sc2 = pack_f32x2(a.scale_log2, a.scale_log2), nm2 = pack_f32x2(-mb, -mb);
+        const float mb = (m_ref == -INFINITY) ? 0.f : m_ref;
+        const long long tp2 = tick<TR>();
+        // p = exp2(s * scale - m) (exp2(-inf) = 0 on hidden keys); bf16 pairs over the first 64 columns
+        uint64_t ps0 = 0, ps1 = 0;
+        const uint64_t sc2 = pack_f32x2(a.scale_log2, a.scale_log2), nm2 = pack_f32x2(-mb, -mb);
 #pragma unroll
-      for (int half = 0; half < 2; ++half) {
-        uint32_t pk[32];
+        for (int half = 0; half < 2; ++half) {
+          uint32_t pk[32];
 #pragma unroll
-        for (int e = 0; e < 16; ++e) {
-          if (half == 1 && e == 4) {   // the first half's store has landed by now: hand it over without stalling for it
-            tmem_wait_st();
-            tc_fence_before();
-            mbar_arrive(bar_p + 16 * w);
+          for (int e = 0; e < 16; ++e) {
+            if (half == 1 && e == 4) {   // the first half's store has landed by now: hand it over without stalling for it
+              tmem_wait_st();
+              tc_fence_before();
+              mbar_arrive(bar_p + 16 * w);
+            }
+            const int c = 64 * half + 4 * e;
+            float p0, p1, p2, p3;
+            unpack_f32x2(fma_f32x2(pack_f32x2(__uint_as_float(v[c]), __uint_as_float(v[c + 1])), sc2, nm2), p0, p1);
+            unpack_f32x2(fma_f32x2(pack_f32x2(__uint_as_float(v[c + 2]), __uint_as_float(v[c + 3])), sc2, nm2), p2, p3);
+            p0 = exp2f(p0); p1 = exp2f(p1); p2 = exp2f(p2); p3 = exp2f(p3);
+            ps0 = add_f32x2(ps0, pack_f32x2(p0, p1));
+            ps1 = add_f32x2(ps1, pack_f32x2(p2, p3));
+            pk[2 * e] = pack_bf16(p0, p1);
+            pk[2 * e + 1] = pack_bf16(p2, p3);
           }
-          const int c = 64 * half + 4 * e;
-          float p0, p1, p2, p3;
-          unpack_f32x2(fma_f32x2(pack_f32x2(__uint_as_float(v[c]), __uint_as_float(v[c + 1])), sc2, nm2), p0, p1);
-          unpack_f32x2(fma_f32x2(pack_f32x2(__uint_as_float(v[c + 2]), __uint_as_float(v[c + 3])), sc2, nm2), p2, p3);
-          p0 = exp2f(p0); p1 = exp2f(p1); p2 = exp2f(p2); p3 = exp2f(p3);
-          ps0 = add_f32x2(ps0, pack_f32x2(p0, p1));
-          ps1 = add_f32x2(ps1, pack_f32x2(p2, p3));
-          pk[2 * e] = pack_bf16(p0, p1);
-          pk[2 * e + 1] = pack_bf16(p2, p3);
+          tmem_st32(tS + 32 * half, pk);
         }
-        tmem_st32(tS + 32 * half, pk);
+        tmem_wait_st();
+        tc_fence_before();
+        mbar_arrive(bar_p + 16 * w + 8);
+        float l0, l1;
+        unpack_f32x2(add_f32x2(ps0, ps1), l0, l1);
+        l += l0 + l1;
+        c_ld += tp1 - tp0; c_max += tp2 - tp1; c_exp += tick<TR>() - tp2;
       }
-      tmem_wait_st();
-      tc_fence_before();
-      mbar_arrive(bar_p + 16 * w + 8);
-      float l0, l1;
-      unpack_f32x2(add_f32x2(ps0, ps1), l0, l1);
-      l += l0 + l1;
-      c_ld += tp1 - tp0; c_max += tp2 - tp1; c_exp += tick<TR>() - tp2;
-    }
-    if (warp == 0 && lane == 0) { trace_add(a.trace, 0, nt); trace_add(a.trace, 1, w_s); trace_add(a.trace, 6, tick<TR>() - t_begin);
-      trace_add(a.trace, 3, c_ld); trace_add(a.trace, 4, c_max); trace_add(a.trace, 5, c_exp); }
-    if (ok && nt > 0) {
-      ok = mbar_wait_abortable(bar_o + 8 * w, (nt - 1) & 1, abort_flag);
-      ok = __all_sync(0xffffffffu, ok);
-    }
-    if (ok) {
+      if (TR && warp == 0 && lane == 0) trace_add(a.trace, 0, nt);
+      if (ok && nt > 0) {
+        ok = mbar_wait_abortable(bar_o + 8 * w, (g - 1) & 1, abort_flag);
+        ok = __all_sync(0xffffffffu, ok);
+      }
+      if (!ok) break;
+      // O leaves 64 columns at a time: TMEM -> registers -> the warp's staging tile -> TMA store of its 32 rows.  (The next
+      // unit's P V may overwrite O once this thread has handed over the next P, i.e. after it has read O here.)
       tc_fence_after();
       const float inv = l > 0.f ? 1.f / l : 0.f;
-      bf16* orow = a.o[qs] + (((int64_t)b * Lq + row) * a.H + h) * D;
 #pragma unroll 1
-      for (int c = 0; c < D / 32; ++c) {
-        uint32_t o[32];
-        if (nt > 0) { tmem_ld32(tO + c * 32, o); tmem_wait_ld(); }
+      for (int c = 0; c < D / 64; ++c) {
+        uint32_t pk[32];
+        if (nt > 0) {
+          uint32_t o[64];
+          uint32_t (*oc)[32] = reinterpret_cast<uint32_t (*)[32]>(o);
+          tmem_ld32(tO + c * 64, oc[0]); tmem_ld32(tO + c * 64 + 32, oc[1]);
+          tmem_wait_ld();
 #pragma unroll
-        for (int e8 = 0; e8 < 4; ++e8) {
-          uint4 vv;
-          uint32_t* pv = reinterpret_cast<uint32_t*>(&vv);
+          for (int e = 0; e < 32; ++e) pk[e] = pack_bf16(__uint_as_float(o[2 * e]) * inv, __uint_as_float(o[2 * e + 1]) * inv);
+        } else {
 #pragma unroll
-          for (int e = 0; e < 4; ++e) {
-            const float x0 = nt > 0 ? __uint_as_float(o[e8 * 8 + 2 * e]) * inv : 0.f;
-            const float x1 = nt > 0 ? __uint_as_float(o[e8 * 8 + 2 * e + 1]) * inv : 0.f;
-            pv[e] = pack_bf16(x0, x1);
-          }
-          if (row_ok) *reinterpret_cast<uint4*>(orow + c * 32 + e8 * 8) = vv;
+          for (int e = 0; e < 32; ++e) pk[e] = 0u;
+        }
+        if (lane == 0) bulk_wait_read0();   // the store before this one has read the staging tile
+        __syncwarp();
+        uint8_t* mine = sm + FWDR_STG + warp * FWDR_STG_WARP + lane * 128;
+#pragma unroll
+        for (int c8 = 0; c8 < 8; ++c8)
+          *reinterpret_cast<uint4*>(mine + ((c8 ^ (lane & 7)) << 4)) = make_uint4(pk[4 * c8], pk[4 * c8 + 1], pk[4 * c8 + 2], pk[4 * c8 + 3]);
+        fence_async_smem();
+        __syncwarp();
+        if (lane == 0 && row < Lq) {   // lane 0 has the warp's first row; rows past the end are clipped
+          tma_store_3d(&maps.o[qs], stg, h * D + c * 64, row, b);
+          bulk_commit();
         }
       }
       if (row_ok) a.lse[qs][((int64_t)b * a.H + h) * Lq + row] = l > 0.f ? (m_ref + log2f(l)) * LN2 : -INFINITY;
     }
+    if (lane == 0) bulk_wait_all();
+    if (warp == 0 && lane == 0) { trace_add(a.trace, 1, w_s); trace_add(a.trace, 6, tick<TR>() - t_begin);
+      trace_add(a.trace, 3, c_ld); trace_add(a.trace, 4, c_max); trace_add(a.trace, 5, c_exp); }
   }
   tc_fence_before();
   __syncthreads();
   if (threadIdx.x == 0 && *abort_flag) atomicExch(status, (int)BDLM_ERR_DEVICE_TIMEOUT);
-  if (warp == 8) tmem_dealloc(tmem, 512);
+  if (warp == 9) tmem_dealloc(*tmem_slot, 512);
 }
 
 }  // namespace
@@ -448,11 +570,13 @@ static cudaError_t launch_tc_fwd_d(const KArgs& a, cudaStream_t st) {
     // a stream that is left out gets the other stream's tensors as placeholders: its maps are never used
     const int sq = a.q[s] ? s : 1 - s;
     if (!tc_make_map(&maps.q[s], a.q[sq], a.H, rows_q(a, sq), a.batch, TILE, D)) return cudaErrorInvalidValue;
+    if (!tc_make_map(&maps.o[s], a.o[sq], a.H, rows_q(a, sq), a.batch, 32, D)) return cudaErrorInvalidValue;
     const int sk = (s == NOISY && (a.q[NOISY] == nullptr || a.Ln == 0 || !a.diag)) ? CLEAN : s;
     if (!tc_make_map(&maps.k[s], a.k[sk], a.Hkv, rows_k(a, sk), a.batch, TILE, D)) return cudaErrorInvalidValue;
     if (!tc_make_map(&maps.v[s], a.v[sk], a.Hkv, rows_k(a, sk), a.batch, TILE, D)) return cudaErrorInvalidValue;
   }
   const int qrows = max(a.q[CLEAN] != nullptr ? a.Lqc : 0, a.q[NOISY] != nullptr ? a.Ln : 0);
+  const int streams = (a.q[CLEAN] != nullptr) + (a.q[NOISY] != nullptr);
   int* status = device_status_ptr();
   if (status == nullptr) return cudaErrorUnknown;
   cudaError_t e;
@@ -460,7 +584,7 @@ static cudaError_t launch_tc_fwd_d(const KArgs& a, cudaStream_t st) {
     auto kern = a.trace ? tc_fwdr_kernel<true, false, D> : tc_fwdr_kernel<false, false, D>;
     e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, FWDR_SMEM);
     if (e != cudaSuccess) return e;
-    const TileGrid tg = make_tile_grid((qrows + TILE - 1) / TILE, a.H / 2, a.batch * 2);
+    const TileGrid tg = make_tile_grid((qrows + TILE - 1) / TILE, a.H / 2, a.batch * streams);
     if (tile_grid_blocks(tg) == 0) return cudaErrorInvalidValue;
     kern<<<tile_grid_blocks(tg), FWDR_THREADS, FWDR_SMEM, st>>>(maps, a, tg, status);
     return cudaGetLastError();
@@ -469,7 +593,7 @@ static cudaError_t launch_tc_fwd_d(const KArgs& a, cudaStream_t st) {
   auto kern = a.trace ? tc_fwdr_kernel<true, true, D> : tc_fwdr_kernel<false, true, D>;
   e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, FWDR_SMEM);
   if (e != cudaSuccess) return e;
-  const TileGrid tg = make_tile_grid(((qrows + TILE - 1) / TILE + 1) / 2, a.H, a.batch * 2);
+  const TileGrid tg = make_tile_grid(((qrows + TILE - 1) / TILE + 1) / 2, a.H, a.batch * streams);
   if (tile_grid_blocks(tg) == 0) return cudaErrorInvalidValue;
   kern<<<tile_grid_blocks(tg), FWDR_THREADS, FWDR_SMEM, st>>>(maps, a, tg, status);
   return cudaGetLastError();
