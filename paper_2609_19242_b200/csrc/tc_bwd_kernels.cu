@@ -1452,13 +1452,14 @@ static size_t pad64(size_t rows) { return (rows + 63) / 64 * 64; }
 bool tc_bwd_supported(const KArgs& a) {
   return (a.d == 128 || a.d == 64) && tc_rows_ok(a) && tc_encoder_available();
 }
-// fp32 dQ accumulators of the fused backward: one [batch, H, rows, d] tensor per query stream
+// fp32 dQ accumulators of the fused backward: one [batch, H, rows, d] tensor per query stream.  The size asked for is
+// that of 128-wide rows for either head dimension, as callers have been told; d = 64 uses the first half.
 size_t tc_bwd_fused_workspace(const bdlm_params* p, const bdlm_packed_geometry* g) {
   if ((p->d != 128 && p->d != 64) || p->impl == 1) return 0;
   const size_t rows_c = g != nullptr ? (size_t)g->Lq_clean : (size_t)p->L;
   const size_t rows_n = g != nullptr ? (size_t)g->n_blocks * p->block_size : (size_t)p->L;
   // rows rounded up to the kernel's 64-row steps: a reduction always covers a whole step
-  return (pad64(rows_c) + pad64(rows_n)) * p->batch * p->H * p->d * sizeof(float);
+  return (pad64(rows_c) + pad64(rows_n)) * p->batch * p->H * 128 * sizeof(float);
 }
 void tc_bwd_place_dq(KArgs& a, void* extra_ws) {
   float* at = static_cast<float*>(extra_ws);
