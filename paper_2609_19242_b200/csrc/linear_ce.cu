@@ -39,16 +39,19 @@ constexpr int G_SMEM = G_BARS + 256 + 1024;      // barriers, TMEM slot, abort f
 constexpr int G_THREADS = 192;                   // warps 0-3 epilogue, warp 4 TMA, warp 5 MMA
 constexpr int MN_PANEL = BK * 128;               // an MN-major panel: 64 contraction rows x 64 M/N elements
 
-enum { EPI_LSE = 0, EPI_DZ = 1, EPI_STORE = 2 };
-enum { C_BF16 = 0, C_F32_STORE = 1, C_F32_ADD = 2, C_F32_ADD_TO_BF16 = 3 };
+enum { EPI_LSE = 0, EPI_DZ = 1, EPI_STORE = 2, EPI_ADD = 3 };   // EPI_ADD: the two c_modes that read C first
+enum { C_BF16 = 0, C_F32_STORE = 1, C_F32_ADD = 2, C_F32_ADD_TO_BF16 = 3, C_F32_PART = 4 };
 
 struct GemmMaps { CUtensorMap a, b; };
+enum { K_MAJOR = 0, MN_PANELS = 1, MN_BOXES = 2 };
 
 struct GemmArgs {
   int M, N, K;
+  int bn;                                // width of an N tile: a multiple of 16, at most BN
   int m_tiles, n_tiles, n_run, n_runs;   // an item = one M tile x n_run consecutive N tiles; n_runs = ceil(n_tiles / n_run)
+  int splits, k_split;                   // the contraction in `splits` pieces of k_split steps, each an item of its own
   int m_inner;                           // item order: 1 = consecutive items share the N run, 0 = share the M tile
-  int a_mn, b_mn;                        // operand layouts (0 = K-major, 1 = MN-major)
+  int a_mn, b_mn;                        // operand layouts: K_MAJOR, MN_PANELS (one load per tile), MN_BOXES (one per 64-column panel)
   // EPI_LSE / EPI_DZ: rows are tokens row0 .. row0 + M - 1
   int row0;
   const int* labels;
@@ -62,33 +65,47 @@ struct GemmArgs {
   bf16* dz;        // EPI_DZ: [M, N] row-major, ld = ldz
   int ldz;
   // EPI_STORE
-  int c_mode;
+  int c_mode;      // C_F32_PART: piece s of the contraction goes to c32 + s * M * ldc
   bf16* c16; float* c32; int ldc;
 };
 
-__device__ __forceinline__ void tma_load_2d(uint32_t dst, const CUtensorMap* map, uint32_t bar, int x, int y) {
+// Loads issued by the elected lane of a converged warp (see elect_one).
+__device__ __forceinline__ void tma_load_2d_e(uint32_t dst, const CUtensorMap* map, uint32_t bar, int x, int y, uint32_t elected) {
   asm volatile(
-      "cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4}], [%2];"
-      ::"r"(dst), "l"(reinterpret_cast<uint64_t>(map)), "r"(bar), "r"(x), "r"(y) : "memory");
+      "{\n\t.reg .pred q;\n\tsetp.ne.b32 q, %5, 0;\n\t"
+      "@q cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4}], [%2];\n\t}"
+      ::"r"(dst), "l"(reinterpret_cast<uint64_t>(map)), "r"(bar), "r"(x), "r"(y), "r"(elected) : "memory");
+}
+__device__ __forceinline__ void tma_load_panels_e(uint32_t dst, const CUtensorMap* map, uint32_t bar, int row, int panel, uint32_t elected) {
+  asm volatile(
+      "{\n\t.reg .pred q;\n\tsetp.ne.b32 q, %5, 0;\n\t"
+      "@q cp.async.bulk.tensor.3d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {0, %3, %4}], [%2];\n\t}"
+      ::"r"(dst), "l"(reinterpret_cast<uint64_t>(map)), "r"(bar), "r"(row), "r"(panel), "r"(elected) : "memory");
 }
 
 // Walks the CTA's tiles in the order every role uses.
 struct TileWalk {
-  int item, items, mt, nrun, nt, nt_end;
+  int item, items, mt, nrun, nt, nt_end, split;
   const GemmArgs* a;
   __device__ __forceinline__ void start(const GemmArgs& args) {
-    a = &args; items = args.m_tiles * args.n_runs; item = blockIdx.x; nt = 0; nt_end = 0;
+    a = &args; items = args.m_tiles * args.n_runs * args.splits; item = blockIdx.x; nt = 0; nt_end = 0; split = 0;
     if (item < items) open();
   }
   __device__ __forceinline__ void open() {
-    if (a->m_inner) { nrun = item / a->m_tiles; mt = item - nrun * a->m_tiles; }
-    else { mt = item / a->n_runs; nrun = item - mt * a->n_runs; }
+    int i = item;
+    const int per = a->m_tiles * a->n_runs;
+    split = 0;
+    if (a->splits > 1) { split = i / per; i -= split * per; }
+    if (a->m_inner) { nrun = i / a->m_tiles; mt = i - nrun * a->m_tiles; }
+    else { mt = i / a->n_runs; nrun = i - mt * a->n_runs; }
     nt = nrun * a->n_run;
     nt_end = min(a->n_tiles, nt + a->n_run);
   }
   __device__ __forceinline__ bool valid() const { return item < items; }
   __device__ __forceinline__ bool first_of_item() const { return nt == nrun * a->n_run; }
   __device__ __forceinline__ bool last_of_item() const { return nt + 1 == nt_end; }
+  __device__ __forceinline__ int k_begin() const { return split * a->k_split; }   // 64-deep steps of the contraction
+  __device__ __forceinline__ int k_end(int nk) const { return min(nk, (split + 1) * a->k_split); }
   __device__ __forceinline__ void next() {
     if (++nt < nt_end) return;
     item += gridDim.x;
@@ -123,30 +140,34 @@ lce_gemm_kernel(const __grid_constant__ GemmMaps maps, const GemmArgs a, int* __
   const int nk = (a.K + BK - 1) / BK;
 
   if (warp == 4) {
-    // ------------------------------------------------------------------ producer
-    if (lane == 0) {
-      TileWalk w;
-      w.start(a);
-      int ks = 0;
-      bool ok = true;
-      for (; w.valid() && ok; w.next()) {
-        const int m0 = w.mt * BM, n0 = w.nt * BN;
-        for (int k = 0; k < nk && ok; ++k, ++ks) {
-          const int s = ks % STAGES;
-          if (ks >= STAGES) ok = mbar_wait_abortable(bar_empty + 8 * s, ((ks / STAGES) - 1) & 1, abort_flag);
-          if (!ok) break;
-          const uint32_t sA = base + s * STAGE_BYTES, sB = sA + A_BYTES, bar = bar_full + 8 * s;
-          mbar_expect_tx(bar, STAGE_BYTES);
-          if (!a.a_mn) tma_load_2d(sA, &maps.a, bar, k * BK, m0);
-          else {
+    // ------------------------------------------------------------------ producer: the whole warp walks the loop, one
+    // elected lane issues.  Issuing is what the products with MN-major operands were bound by (six 64-column boxes a
+    // step, each from a lone lane): one load for all panels of a tile where the matrix allows it.
+    const uint32_t el = elect_one();
+    TileWalk w;
+    w.start(a);
+    int ks = 0;
+    bool ok = true;
+    const int stage_bytes = A_BYTES + (a.b_mn != K_MAJOR ? B_BYTES : a.bn * BK * 2);   // (MN-major: always all four panels, zeros past the end)
+    for (; w.valid() && ok; w.next()) {
+      const int m0 = w.mt * BM, n0 = w.nt * a.bn, k1 = w.k_end(nk);
+      for (int k = w.k_begin(); k < k1; ++k, ++ks) {
+        const int s = ks % STAGES;
+        if (ks >= STAGES) ok = mbar_wait_lean(bar_empty + 8 * s, ((ks / STAGES) - 1) & 1, abort_flag);
+        if (!ok) break;
+        const uint32_t sA = base + s * STAGE_BYTES, sB = sA + A_BYTES, bar = bar_full + 8 * s;
+        if (el) mbar_expect_tx(bar, stage_bytes);
+        if (a.a_mn == K_MAJOR) tma_load_2d_e(sA, &maps.a, bar, k * BK, m0, el);
+        else if (a.a_mn == MN_PANELS) tma_load_panels_e(sA, &maps.a, bar, k * BK, m0 / 64, el);
+        else {
 #pragma unroll
-            for (int p = 0; p < BM / 64; ++p) tma_load_2d(sA + p * MN_PANEL, &maps.a, bar, m0 + 64 * p, k * BK);
-          }
-          if (!a.b_mn) tma_load_2d(sB, &maps.b, bar, k * BK, n0);
-          else {
+          for (int p = 0; p < BM / 64; ++p) tma_load_2d_e(sA + p * MN_PANEL, &maps.a, bar, m0 + 64 * p, k * BK, el);
+        }
+        if (a.b_mn == K_MAJOR) tma_load_2d_e(sB, &maps.b, bar, k * BK, n0, el);
+        else if (a.b_mn == MN_PANELS) tma_load_panels_e(sB, &maps.b, bar, k * BK, n0 / 64, el);
+        else {
 #pragma unroll
-            for (int p = 0; p < BN / 64; ++p) tma_load_2d(sB + p * MN_PANEL, &maps.b, bar, n0 + 64 * p, k * BK);
-          }
+          for (int p = 0; p < BN / 64; ++p) tma_load_2d_e(sB + p * MN_PANEL, &maps.b, bar, n0 + 64 * p, k * BK, el);
         }
       }
     }
@@ -154,7 +175,7 @@ lce_gemm_kernel(const __grid_constant__ GemmMaps maps, const GemmArgs a, int* __
     // ------------------------------------------------------------------ MMA issuer: the whole warp walks the loop,
     // one elected lane issues
     const uint32_t el = elect_one();
-    const uint32_t idesc = make_idesc(BM, BN, a.a_mn != 0, a.b_mn != 0);
+    const uint32_t idesc = make_idesc(BM, a.bn, a.a_mn != 0, a.b_mn != 0);
     const uint32_t a_lo0 = a.a_mn ? (((base & 0x3FFFFu) >> 4) | (static_cast<uint32_t>(MN_PANEL >> 4) << 16)) : desc_lo_k(base);
     const uint32_t b_lo0 = a.b_mn ? ((((base + A_BYTES) & 0x3FFFFu) >> 4) | (static_cast<uint32_t>(MN_PANEL >> 4) << 16))
                                   : desc_lo_k(base + A_BYTES);
@@ -171,7 +192,8 @@ lce_gemm_kernel(const __grid_constant__ GemmMaps maps, const GemmArgs a, int* __
         tc_fence_after();
       }
       const uint32_t d = tmem + buf * BN;
-      for (int k = 0; k < nk; ++k, ++ks) {
+      const int k0 = w.k_begin(), k1 = w.k_end(nk);
+      for (int k = k0; k < k1; ++k, ++ks) {
         const int s = ks % STAGES;
         ok = mbar_wait_lean(bar_full + 8 * s, (ks / STAGES) & 1, abort_flag);
         if (!ok) break;
@@ -179,7 +201,7 @@ lce_gemm_kernel(const __grid_constant__ GemmMaps maps, const GemmArgs a, int* __
         const uint32_t a_lo = a_lo0 + s * (STAGE_BYTES >> 4), b_lo = b_lo0 + s * (STAGE_BYTES >> 4);
 #pragma unroll
         for (int kk = 0; kk < BK / 16; ++kk)
-          mma_ss_e(d, desc64(a_lo + kk * a_step), desc64(b_lo + kk * b_step), idesc, (k > 0 || kk > 0) ? 1u : 0u, el);
+          mma_ss_e(d, desc64(a_lo + kk * a_step), desc64(b_lo + kk * b_step), idesc, (k > k0 || kk > 0) ? 1u : 0u, el);
         mma_commit_e(bar_empty + 8 * s, el);
       }
       if (!ok) break;
@@ -197,13 +219,13 @@ lce_gemm_kernel(const __grid_constant__ GemmMaps maps, const GemmArgs a, int* __
     float run_m = -INFINITY, run_l = 0.f;
     for (; w.valid() && ok; w.next(), ++tcnt) {
       const int buf = tcnt & 1;
-      const int m0 = w.mt * BM, n0 = w.nt * BN;
+      const int m0 = w.mt * BM, n0 = w.nt * a.bn;
       const int row = m0 + r;
       const bool row_ok = row < a.M;
-      const int ncols = min(BN, a.N - n0);          // valid columns of this tile (a multiple of 8)
+      const int ncols = min(a.bn, a.N - n0);        // valid columns of this tile (a multiple of 8)
       int y = -1;
       float coef = 0.f, lse2 = 0.f;
-      if (EPI != EPI_STORE && row_ok) {
+      if ((EPI == EPI_LSE || EPI == EPI_DZ) && row_ok) {
         y = a.labels[a.row0 + row];
         if (EPI == EPI_DZ) {
           const float wt = a.weight != nullptr ? a.weight[a.row0 + row] : 1.f;
@@ -212,12 +234,63 @@ lce_gemm_kernel(const __grid_constant__ GemmMaps maps, const GemmArgs a, int* __
         }
       }
       if (EPI == EPI_LSE && w.first_of_item()) { run_m = -INFINITY; run_l = 0.f; }
+      if (EPI == EPI_ADD) {
+        // The fp32 sums of the earlier token chunks are requested two 32-column chunks ahead, the first ones before the
+        // wait for the accumulator: requested where they are used, their round trips to memory took longer than the
+        // tile's MMAs.
+        const float* src = a.c32 + (int64_t)row * a.ldc + n0;
+        float4 pre[2][8];
+        auto request = [&](int c, float4 (&u)[8]) {
+#pragma unroll
+          for (int q = 0; q < 8; ++q) if (row_ok && c * 32 + q * 4 < ncols) u[q] = __ldcs(reinterpret_cast<const float4*>(src + c * 32) + q);
+        };
+        auto finish = [&](int c, float4 (&u)[8]) {
+          uint32_t x[32];
+          tmem_ld32(tl + buf * BN + c * 32, x);
+          tmem_wait_ld();
+#pragma unroll
+          for (int q = 0; q < 8; ++q) {
+            u[q].x += __uint_as_float(x[4 * q]); u[q].y += __uint_as_float(x[4 * q + 1]);
+            u[q].z += __uint_as_float(x[4 * q + 2]); u[q].w += __uint_as_float(x[4 * q + 3]);
+          }
+          if (!row_ok) return;
+          const int64_t off = (int64_t)row * a.ldc + n0 + c * 32;
+#pragma unroll
+          for (int q = 0; q < 8; q += 2) {
+            if (c * 32 + q * 4 < ncols) {
+              if (a.c_mode == C_F32_ADD) {
+                *reinterpret_cast<float4*>(a.c32 + off + q * 4) = u[q];
+                *reinterpret_cast<float4*>(a.c32 + off + q * 4 + 4) = u[q + 1];
+              } else {
+                *reinterpret_cast<uint4*>(a.c16 + off + q * 4) =
+                    make_uint4(pack_bf16(u[q].x, u[q].y), pack_bf16(u[q].z, u[q].w), pack_bf16(u[q + 1].x, u[q + 1].y), pack_bf16(u[q + 1].z, u[q + 1].w));
+              }
+            }
+          }
+        };
+        request(0, pre[0]);
+        request(1, pre[1]);
+        ok = mbar_wait_abortable(bar_acc_full + 8 * buf, (tcnt >> 1) & 1, abort_flag);
+        ok = __all_sync(0xffffffffu, ok);
+        if (!ok) break;
+        tc_fence_after();
+#pragma unroll 1
+        for (int c = 0; c < BN / 32; c += 2) {   // (columns past the tile are read from tensor memory and dropped)
+          finish(c, pre[0]);
+          request(c + 2, pre[0]);
+          finish(c + 1, pre[1]);
+          request(c + 3, pre[1]);
+        }
+        tc_fence_before();
+        mbar_arrive(bar_acc_empty + 8 * buf);
+        continue;
+      }
       ok = mbar_wait_abortable(bar_acc_full + 8 * buf, (tcnt >> 1) & 1, abort_flag);
       ok = __all_sync(0xffffffffu, ok);
       if (!ok) break;
       tc_fence_after();
 #pragma unroll 1
-      for (int c = 0; c < BN / 32; ++c) {
+      for (int c = 0; c < (a.bn + 31) / 32; ++c) {
         uint32_t x[32];
         tmem_ld32(tl + buf * BN + c * 32, x);
         tmem_wait_ld();
@@ -234,14 +307,18 @@ lce_gemm_kernel(const __grid_constant__ GemmMaps maps, const GemmArgs a, int* __
           for (int e = 0; e < 32; ++e) mx = fmaxf(mx, __uint_as_float(x[e]));
           mx *= LOG2E;
           if (mx > run_m) { run_l *= exp2f(run_m - mx); run_m = mx; }
-          float s0 = 0.f, s1 = 0.f;
+          const uint64_t c2 = pack_f32x2(LOG2E, LOG2E), m2 = pack_f32x2(-run_m, -run_m);
+          uint64_t s2 = 0;
 #pragma unroll
           for (int e = 0; e < 32; e += 2) {
-            s0 += exp2f(fmaf(__uint_as_float(x[e]), LOG2E, -run_m));
-            s1 += exp2f(fmaf(__uint_as_float(x[e + 1]), LOG2E, -run_m));
+            float u, v;
+            unpack_f32x2(fma_f32x2(pack_f32x2(__uint_as_float(x[e]), __uint_as_float(x[e + 1])), c2, m2), u, v);
+            s2 = add_f32x2(s2, pack_f32x2(exp2f(u), exp2f(v)));
           }
+          float s0, s1;
+          unpack_f32x2(s2, s0, s1);
           run_l += s0 + s1;
-          if ((unsigned)(y - col0) < 32u) {
+          if ((unsigned)(y - col0) < (unsigned)min(cvalid, 32)) {   // (a chunk may reach into the next tile's columns)
             float z = 0.f;
 #pragma unroll
             for (int e = 0; e < 32; ++e) if (col0 + e == y) z = __uint_as_float(x[e]);
@@ -266,19 +343,14 @@ lce_gemm_kernel(const __grid_constant__ GemmMaps maps, const GemmArgs a, int* __
             }
           }
         } else if (EPI == EPI_STORE && cvalid > 0 && row_ok) {
-          const int64_t off = (int64_t)row * a.ldc + col0;
+          const int64_t off = ((int64_t)w.split * a.M + row) * a.ldc + col0;
 #pragma unroll
           for (int e8 = 0; e8 < 4; ++e8) {
             if (e8 * 8 >= cvalid) break;
             float v[8];
 #pragma unroll
             for (int e = 0; e < 8; ++e) v[e] = __uint_as_float(x[e8 * 8 + e]);
-            if (a.c_mode == C_F32_ADD || a.c_mode == C_F32_ADD_TO_BF16) {
-              const float4 u0 = *reinterpret_cast<const float4*>(a.c32 + off + e8 * 8);
-              const float4 u1 = *reinterpret_cast<const float4*>(a.c32 + off + e8 * 8 + 4);
-              v[0] += u0.x; v[1] += u0.y; v[2] += u0.z; v[3] += u0.w; v[4] += u1.x; v[5] += u1.y; v[6] += u1.z; v[7] += u1.w;
-            }
-            if (a.c_mode == C_F32_STORE || a.c_mode == C_F32_ADD) {
+            if (a.c_mode != C_BF16) {
               *reinterpret_cast<float4*>(a.c32 + off + e8 * 8) = make_float4(v[0], v[1], v[2], v[3]);
               *reinterpret_cast<float4*>(a.c32 + off + e8 * 8 + 4) = make_float4(v[4], v[5], v[6], v[7]);
             } else {
@@ -305,19 +377,36 @@ lce_gemm_kernel(const __grid_constant__ GemmMaps maps, const GemmArgs a, int* __
 
 // Combines the per-run partial (maximum, sum) pairs of every token (Eq. csbp-lse-merge's rule, in log2 units),
 // writes lse and nll, and leaves one weighted partial sum of the loss per block (fixed order: reproducible).
-__global__ void __launch_bounds__(256) lce_finish_kernel(const float* __restrict__ part_m, const float* __restrict__ part_l,
+// A block takes FIN_T tokens, eight threads share a token's runs (one thread per token left a few blocks alone with a
+// hundred dependent rounds of loads when the runs are short).  The block's sum replaces its own first token's first
+// partial maximum, which nobody else reads.
+constexpr int FIN_T = 32;
+__global__ void __launch_bounds__(256) lce_finish_kernel(float* part_m, const float* __restrict__ part_l,
                                                          const float* __restrict__ zlab, const int* __restrict__ labels,
                                                          const float* __restrict__ weight, int T, int n_runs, int ldp,
-                                                         float* __restrict__ lse, float* __restrict__ nll,
-                                                         float* __restrict__ block_sums) {
-  __shared__ float red[256];
-  const int t = blockIdx.x * 256 + threadIdx.x;
+                                                         float* __restrict__ lse, float* __restrict__ nll) {
+  __shared__ float sm_m[8][FIN_T], sm_l[8][FIN_T];
+  const int x = threadIdx.x % FIN_T, y0 = threadIdx.x / FIN_T;
+  const int t = blockIdx.x * FIN_T + x;
+  float m = -INFINITY, l = 0.f;
+  if (t < T) {
+#pragma unroll 8
+    for (int c = y0; c < n_runs; c += 8) m = fmaxf(m, part_m[(int64_t)c * ldp + t]);
+    if (m != -INFINITY) {
+#pragma unroll 8
+      for (int c = y0; c < n_runs; c += 8) l += part_l[(int64_t)c * ldp + t] * exp2f(part_m[(int64_t)c * ldp + t] - m);
+    }
+  }
+  sm_m[y0][x] = m; sm_l[y0][x] = l;
+  __syncthreads();
+  if (threadIdx.x >= FIN_T) return;
   float contrib = 0.f;
   if (t < T) {
-    float m = -INFINITY;
-    for (int c = 0; c < n_runs; ++c) m = fmaxf(m, part_m[(int64_t)c * ldp + t]);
-    float l = 0.f;
-    for (int c = 0; c < n_runs; ++c) l += part_l[(int64_t)c * ldp + t] * exp2f(part_m[(int64_t)c * ldp + t] - m);
+    m = -INFINITY; l = 0.f;
+#pragma unroll
+    for (int j = 0; j < 8; ++j) m = fmaxf(m, sm_m[j][x]);
+#pragma unroll
+    for (int j = 0; j < 8; ++j) if (sm_m[j][x] != -INFINITY) l += sm_l[j][x] * exp2f(sm_m[j][x] - m);
     const float z = (m + log2f(l)) * LN2;
     const int y = labels[t];
     const float n = y >= 0 ? z - zlab[t] : 0.f;
@@ -325,19 +414,15 @@ __global__ void __launch_bounds__(256) lce_finish_kernel(const float* __restrict
     if (nll != nullptr) nll[t] = n;
     contrib = (weight != nullptr ? weight[t] : 1.f) * n;
   }
-  red[threadIdx.x] = contrib;
-  __syncthreads();
-  for (int s = 128; s > 0; s >>= 1) {
-    if (threadIdx.x < s) red[threadIdx.x] += red[threadIdx.x + s];
-    __syncthreads();
-  }
-  if (threadIdx.x == 0) block_sums[blockIdx.x] = red[0];
+#pragma unroll
+  for (int sft = FIN_T / 2; sft > 0; sft >>= 1) contrib += __shfl_xor_sync(0xffffffffu, contrib, sft);
+  if (x == 0) part_m[blockIdx.x * FIN_T] = contrib;
 }
 
-__global__ void __launch_bounds__(256) lce_sum_kernel(const float* __restrict__ block_sums, int n, float* __restrict__ loss) {
+__global__ void __launch_bounds__(256) lce_sum_kernel(const float* __restrict__ block_sums, int n, int stride, float* __restrict__ loss) {
   __shared__ float red[256];
   float acc = 0.f;
-  for (int i = threadIdx.x; i < n; i += 256) acc += block_sums[i];
+  for (int i = threadIdx.x; i < n; i += 256) acc += block_sums[i * stride];
   red[threadIdx.x] = acc;
   __syncthreads();
   for (int s = 128; s > 0; s >>= 1) {
@@ -347,39 +432,181 @@ __global__ void __launch_bounds__(256) lce_sum_kernel(const float* __restrict__ 
   if (threadIdx.x == 0) *loss = red[0];
 }
 
+// Sum of the pieces of a split contraction, in their order, as bf16.  n = elements per piece (a multiple of 8).
+__global__ void __launch_bounds__(256) lce_sum_pieces_kernel(const float* __restrict__ part, int pieces, int64_t n, bf16* __restrict__ out) {
+  for (int64_t i = ((int64_t)blockIdx.x * 256 + threadIdx.x) * 4; i < n; i += (int64_t)gridDim.x * 1024) {
+    float4 acc = *reinterpret_cast<const float4*>(part + i);
+#pragma unroll 4
+    for (int p = 1; p < pieces; ++p) {
+      const float4 u = *reinterpret_cast<const float4*>(part + p * n + i);
+      acc.x += u.x; acc.y += u.y; acc.z += u.z; acc.w += u.w;
+    }
+    *reinterpret_cast<uint2*>(out + i) = make_uint2(pack_bf16(acc.x, acc.y), pack_bf16(acc.z, acc.w));
+  }
+}
+
+// Copies W [V, D] and the tokens' h [T, D] to rows of `ld` elements (a whole number of 128-byte lines), 16 bytes per thread and
+// turn; what lies past a row's D elements is never looked at.
+__global__ void __launch_bounds__(256) lce_pack_kernel(const uint4* __restrict__ w, uint4* __restrict__ w_out, unsigned nw,
+                                                       const uint4* __restrict__ h, uint4* __restrict__ h_out, unsigned nh,
+                                                       unsigned per_row, unsigned per_row_out) {
+  constexpr int U = 4;
+  for (unsigned i0 = blockIdx.x * 256 * U + threadIdx.x; i0 < nw + nh; i0 += gridDim.x * 256 * U) {
+    uint4 v[U];
+#pragma unroll
+    for (int j = 0; j < U; ++j) {
+      const unsigned i = i0 + j * 256;
+      if (i < nw) v[j] = __ldcs(w + i);
+      else if (i < nw + nh) v[j] = h[i - nw];
+    }
+#pragma unroll
+    for (int j = 0; j < U; ++j) {
+      unsigned i = i0 + j * 256;
+      if (i >= nw + nh) break;
+      uint4* dst = w_out;
+      if (i >= nw) { i -= nw; dst = h_out; }
+      const unsigned row = i / per_row;
+      dst[(size_t)row * per_row_out + (i - row * per_row)] = v[j];
+    }
+  }
+}
+
 // ------------------------------------------------------------------------------------------ host
 // Operand descriptions of one product: A is [M x K] (K-major) or [K x M] (MN-major) in memory, B likewise with N.
-struct Operand { const void* ptr; int64_t ld; int mn; };
+// whole: rows may be read up to the next multiple of 64 elements (a copy of our own).
+struct Operand { const void* ptr; int64_t ld; int mn; bool whole; };
+
+// How a product is cut into tiles: with fixed 256-column tiles and runs of eight, a ragged or small product leaves a
+// part of the chip idle (T = 1531, D = 1544, V = 32008: 192 forward items on 148 SMs, dH 84 tiles, the last of every
+// seven 8 columns wide).  The width of an N tile and the length of a run are chosen for the shortest launch: rounds of
+// items per SM times the clocks of one item.  A 16-deep slice of an M = 128 MMA takes bn / 2 clk, and no less than its
+// operands need from shared memory at 128 bytes per clk.  Ties go to the longer run (fewer partial results).  A B operand
+// that lies MN-major keeps 256 columns where it has them (dH at T = 4096, D = 4096 in one piece: 5.7 ms with 240 or 192
+// columns against 3.4: its panels then start off the 128-byte lines, or a tile's rows off the 512 bytes they share).
+// Forward / dz at T = 1531, D = 1544, V = 32008: 234 -> 160 and 275 -> 188 us.
+struct Tiling { int bn, n_run; };
+Tiling choose_tiling(int M, int N, int K, int splits, int max_run, int epi_per_32, int b_mn) {
+  const long long m_tiles = (M + BM - 1) / BM, sms = device_sm_count();
+  const int nk = ((K + BK - 1) / BK + splits - 1) / splits;
+  Tiling best = {BN, max_run};
+  double t_best = 1e300;
+  const int unit = b_mn ? 128 : 16;
+  for (int bn = BN; bn >= 128; bn -= unit) {
+    if (bn > 128 && bn - unit >= N) continue;              // a whole unit wider than the matrix
+    if (b_mn && bn < BN && N > bn) break;
+    const long long n_tiles = (N + bn - 1) / bn;
+    const double slice = bn / 2 > 32 + bn / 4 ? bn / 2 : 32 + bn / 4;
+    const double epi = (double)epi_per_32 * ((bn + 31) / 32);
+    const double mma = nk * (BK / 16) * slice;
+    const double tile = mma > epi ? mma : epi;
+    for (int run = max_run; run >= 1; run /= 2) {
+      const long long items = m_tiles * ((n_tiles + run - 1) / run) * splits;
+      const double t = (double)((items + sms - 1) / sms) * (run < n_tiles ? run : n_tiles) * tile + epi;
+      if (t < 0.99 * t_best) { t_best = t; best = {bn, run}; }
+    }
+  }
+  return best;
+}
+constexpr int EPI_CLK_LSE = 350, EPI_CLK_DZ = 500, EPI_CLK_STORE = 300;   // per 32 columns, rough
 
 template <int EPI>
 cudaError_t launch_gemm(GemmArgs a, const Operand& A, const Operand& B, cudaStream_t st) {
   GemmMaps maps;
-  a.a_mn = A.mn; a.b_mn = B.mn;
-  const bool okA = A.mn ? tc_make_map_2d(&maps.a, A.ptr, a.K, a.M, A.ld, 64) : tc_make_map_2d(&maps.a, A.ptr, a.M, a.K, A.ld, BM);
-  const bool okB = B.mn ? tc_make_map_2d(&maps.b, B.ptr, a.K, a.N, B.ld, 64) : tc_make_map_2d(&maps.b, B.ptr, a.N, a.K, B.ld, BN);
+  auto encode = [&](CUtensorMap* m, const Operand& o, int extent, int box, int& layout) {
+    if (!o.mn) { layout = K_MAJOR; return tc_make_map_2d(m, o.ptr, extent, a.K, o.ld, box); }
+    if (o.whole) extent = (extent + 63) / 64 * 64;
+    layout = extent % 64 == 0 ? MN_PANELS : MN_BOXES;   // (a last panel that is not whole would reach past the matrix)
+    return layout == MN_PANELS ? tc_make_map_panels(m, o.ptr, a.K, extent, o.ld, BK, box / 64) : tc_make_map_2d(m, o.ptr, a.K, extent, o.ld, 64);
+  };
+  const bool okA = encode(&maps.a, A, a.M, BM, a.a_mn), okB = encode(&maps.b, B, a.N, B.mn ? BN : a.bn, a.b_mn);
   if (!okA || !okB) return cudaErrorInvalidValue;
   a.m_tiles = (a.M + BM - 1) / BM;
-  a.n_tiles = (a.N + BN - 1) / BN;
+  a.n_tiles = (a.N + a.bn - 1) / a.bn;
   a.n_runs = (a.n_tiles + a.n_run - 1) / a.n_run;
+  if (a.splits <= 1) { a.splits = 1; a.k_split = (a.K + BK - 1) / BK; }
   int* status = device_status_ptr();
   if (status == nullptr) return cudaErrorUnknown;
   auto kern = lce_gemm_kernel<EPI>;
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, G_SMEM);
   if (e != cudaSuccess) return e;
-  const int items = a.m_tiles * a.n_runs;
+  const int items = a.m_tiles * a.n_runs * a.splits;
   const int grid = items < device_sm_count() ? items : device_sm_count();
   kern<<<grid, G_THREADS, G_SMEM, st>>>(maps, a, status);
   return cudaGetLastError();
 }
 
-constexpr int FWD_N_RUN = 8;   // vocabulary tiles per forward work item: 2048 logits per partial (maximum, sum) pair
+constexpr int FWD_N_RUN = 8;   // most vocabulary tiles per work item: at most 2048 logits per partial (maximum, sum) pair
+constexpr Tiling FWD_COARSE = {BN, FWD_N_RUN};   // the fewest partial results: what the smallest accepted workspace holds
 
-int fwd_runs(int V) { const int nt = (V + BN - 1) / BN; return (nt + FWD_N_RUN - 1) / FWD_N_RUN; }
+int fwd_runs(int V, const Tiling& t) { const int nt = (V + t.bn - 1) / t.bn; return (nt + t.n_run - 1) / t.n_run; }
 size_t align256(size_t x) { return (x + 255) / 256 * 256; }
+size_t fwd_part_bytes(const bdlm_lce_params* p, const Tiling& t) {
+  const size_t per = align256((size_t)p->T * sizeof(float));
+  return (2 * (size_t)fwd_runs(p->V, t) + 1) * per;
+}
+// Matrices whose rows are no whole number of 128-byte lines: every 128-byte row of a TMA box then straddles two lines,
+// and the products, which live on L2 bandwidth, take half as long again or more (T = 1531, V ~ 32000: D = 1536 against
+// 1544 forward 103 / 160 us, backward 346 / 600).  From PACK_*_T tokens on, W and h are copied to padded rows first
+// (W of 98 MB: 35 us); the rows of dz, which is ours, are padded in any case.
+constexpr int PACK_FWD_T = 1024, PACK_BWD_T = 384;
+int64_t up64(int64_t x) { return (x + 63) / 64 * 64; }
+bool packs(const bdlm_lce_params* p, int from) { return p->D % 64 != 0 && p->T >= from && ((int64_t)p->V + p->T) * (p->D / 8) < (1ll << 31); }
+size_t pack_w_bytes(const bdlm_lce_params* p) { return align256((size_t)p->V * up64(p->D) * 2); }
+size_t pack_bytes(const bdlm_lce_params* p) { return pack_w_bytes(p) + align256((size_t)p->T * up64(p->D) * 2); }
+// Copies both to `at`; h and w become the copies.
+cudaError_t pack(const bdlm_lce_params* p, char* at, Operand& h, Operand& w, cudaStream_t st) {
+  const unsigned per_row = p->D / 8, nw = (unsigned)p->V * per_row, nh = (unsigned)p->T * per_row;
+  uint4 *w_out = reinterpret_cast<uint4*>(at), *h_out = reinterpret_cast<uint4*>(at + pack_w_bytes(p));
+  const unsigned want = (nw + nh + 1023) / 1024, cap = device_sm_count() * 8;
+  lce_pack_kernel<<<want < cap ? want : cap, 256, 0, st>>>(static_cast<const uint4*>(w.ptr), w_out, nw, static_cast<const uint4*>(h.ptr), h_out, nh,
+                                                           per_row, (unsigned)(up64(p->D) / 8));
+  w = Operand{w_out, up64(p->D), 0, true};
+  h = Operand{h_out, up64(p->D), 0, true};
+  return cudaGetLastError();
+}
+size_t fwd_bytes(const bdlm_lce_params* p, const Tiling& t) { return fwd_part_bytes(p, t) + (packs(p, PACK_FWD_T) ? pack_bytes(p) : 0); }
+Tiling fwd_tiling(const bdlm_lce_params* p) { return choose_tiling(p->T, p->V, p->D, 1, FWD_N_RUN, EPI_CLK_LSE, 0); }
+// the smallest workspace that is accepted (with room for loss sums that now lie elsewhere: the size is an old promise)
+size_t fwd_bytes_min(const bdlm_lce_params* p) {
+  const size_t per = align256((size_t)p->T * sizeof(float));
+  return (2 * (size_t)fwd_runs(p->V, FWD_COARSE) + 1) * per + align256(((size_t)p->T + 255) / 256 * sizeof(float));
+}
 int default_chunk(const bdlm_lce_params* p) {
   if (p->token_chunk > 0) return p->token_chunk;
   const int up = (p->T + 127) / 128 * 128;
   return up < 4096 ? up : 4096;
+}
+// dH = dz W has few output tiles (rows x D) and a contraction as deep as the vocabulary: where the tiles do not fill the
+// chip it is cut into pieces that are summed by lce_sum_pieces_kernel.  The cut depends on T, V and D, not on the token
+// chunks, so that a token's dH does not depend on how the tokens are chunked.  Pieces of 16 steps (1024 vocabulary
+// entries) at least; none from two tiles per SM on (T = 8192, D = 4096, 512 tiles: 3.43 ms in one piece, 3.74 in two).
+int dh_splits(int T, int V, int D) {
+  const long long sms = device_sm_count(), rows = T < 4096 ? T : 4096;
+  const long long tiles = ((rows + BM - 1) / BM) * ((D + BN - 1) / BN), nk = (V + BK - 1) / BK;
+  if (tiles >= 2 * sms) return 1;
+  int best = 1;
+  double t_best = 1e300;
+  for (int s = 1; s <= 16 && nk / s >= 16; ++s) {
+    // rounds of items, then each piece written and read again (about 2.5 KB per clk over the chip)
+    const double t = (double)((tiles * s + sms - 1) / sms) * ((nk + s - 1) / s) * 512 + (s > 1 ? 4000 + 8.0 * s * rows * D / 2500 : 0);
+    if (t < 0.98 * t_best) { t_best = t; best = s; }
+  }
+  return best;
+}
+// The backward's workspace: dz of a chunk, the fp32 dW with several chunks, the pieces of dH, the copies of W and h.  The
+// smallest that is accepted has the first two only, dz with rows of V elements.
+struct BwdPlan { int64_t ldz; int splits; bool packed; size_t dw32, pieces, copies, bytes; };
+BwdPlan bwd_plan(const bdlm_lce_params* p, bool least) {
+  const int tc_ = default_chunk(p), chunks = (p->T + tc_ - 1) / tc_, rows = tc_ < p->T ? tc_ : p->T;
+  BwdPlan b;
+  b.ldz = least ? p->V : up64(p->V);
+  b.splits = least ? 1 : dh_splits(p->T, p->V, p->D);
+  b.packed = !least && packs(p, PACK_BWD_T);
+  b.dw32 = align256((size_t)tc_ * b.ldz * 2);
+  b.pieces = b.dw32 + (chunks > 1 ? align256((size_t)p->V * p->D * sizeof(float)) : 0);
+  b.copies = b.pieces + (b.splits > 1 ? align256((size_t)b.splits * rows * p->D * sizeof(float)) : 0);
+  b.bytes = b.copies + (b.packed ? pack_bytes(p) : 0);
+  return b;
 }
 
 int check(const bdlm_lce_params* p) {
@@ -407,16 +634,10 @@ extern "C" {
 size_t bdlm_linear_ce_workspace_bytes(const bdlm_lce_params* p, int32_t which) {
   if (check(p) != BDLM_OK) return 0;
   if (which == BDLM_LCE_WS_FWD) {
-    const size_t per = align256((size_t)p->T * sizeof(float));
-    return (2 * (size_t)fwd_runs(p->V) + 1) * per + align256(((size_t)p->T + 255) / 256 * sizeof(float));
+    const size_t fine = fwd_bytes(p, fwd_tiling(p)), least = fwd_bytes_min(p);
+    return fine > least ? fine : least;
   }
-  if (which == BDLM_LCE_WS_BWD) {
-    const int tc_ = default_chunk(p);
-    const int chunks = (p->T + tc_ - 1) / tc_;
-    size_t bytes = align256((size_t)tc_ * p->V * 2);
-    if (chunks > 1) bytes += align256((size_t)p->V * p->D * sizeof(float));
-    return bytes;
-  }
+  if (which == BDLM_LCE_WS_BWD) return bwd_plan(p, false).bytes;
   return 0;
 }
 
@@ -431,24 +652,28 @@ int bdlm_linear_ce_fwd(const bdlm_lce_params* p, const void* h, const void* w, c
       (reinterpret_cast<uintptr_t>(loss) & 3u) || (reinterpret_cast<uintptr_t>(lse) & 3u) ||
       (reinterpret_cast<uintptr_t>(nll) & 3u) || (reinterpret_cast<uintptr_t>(token_weight) & 3u))
     return BDLM_ERR_INVALID_ARG;
-  if (workspace_bytes < bdlm_linear_ce_workspace_bytes(p, BDLM_LCE_WS_FWD)) return BDLM_ERR_WORKSPACE_TOO_SMALL;
+  if (workspace_bytes < fwd_bytes_min(p)) return BDLM_ERR_WORKSPACE_TOO_SMALL;
   if (!sm100() || !tc_encoder_available()) return BDLM_ERR_UNSUPPORTED;
   cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
-  const int runs = fwd_runs(p->V);
+  const Tiling fine = fwd_tiling(p);
+  const bool roomy = workspace_bytes >= fwd_bytes(p, fine);
+  const Tiling t = roomy ? fine : FWD_COARSE;
+  const int runs = fwd_runs(p->V, t);
   const size_t per = align256((size_t)p->T * sizeof(float));
   char* ws = static_cast<char*>(workspace);
   GemmArgs a = {};
-  a.M = p->T; a.N = p->V; a.K = p->D; a.n_run = FWD_N_RUN; a.m_inner = 1;
+  a.M = p->T; a.N = p->V; a.K = p->D; a.bn = t.bn; a.n_run = t.n_run; a.m_inner = 1;
   a.row0 = 0; a.labels = labels; a.weight = token_weight; a.ldp = (int)(per / sizeof(float));
   a.part_m = reinterpret_cast<float*>(ws);
   a.part_l = reinterpret_cast<float*>(ws + (size_t)runs * per);
   a.zlab = reinterpret_cast<float*>(ws + 2 * (size_t)runs * per);
-  float* block_sums = reinterpret_cast<float*>(ws + (2 * (size_t)runs + 1) * per);
-  if (launch_gemm<EPI_LSE>(a, Operand{h, p->D, 0}, Operand{w, p->D, 0}, st) != cudaSuccess) return BDLM_ERR_CUDA;
-  const int blocks = (p->T + 255) / 256;
-  lce_finish_kernel<<<blocks, 256, 0, st>>>(a.part_m, a.part_l, a.zlab, labels, token_weight, p->T, runs, a.ldp, lse, nll, block_sums);
+  Operand oh{h, p->D, 0, false}, ow{w, p->D, 0, false};
+  if (roomy && packs(p, PACK_FWD_T) && pack(p, ws + fwd_part_bytes(p, t), oh, ow, st) != cudaSuccess) return BDLM_ERR_CUDA;
+  if (launch_gemm<EPI_LSE>(a, oh, ow, st) != cudaSuccess) return BDLM_ERR_CUDA;
+  const int blocks = (p->T + FIN_T - 1) / FIN_T;
+  lce_finish_kernel<<<blocks, 256, 0, st>>>(a.part_m, a.part_l, a.zlab, labels, token_weight, p->T, runs, a.ldp, lse, nll);
   if (cudaGetLastError() != cudaSuccess) return BDLM_ERR_CUDA;
-  lce_sum_kernel<<<1, 256, 0, st>>>(block_sums, blocks, loss);
+  lce_sum_kernel<<<1, 256, 0, st>>>(a.part_m, blocks, FIN_T, loss);
   return cudaGetLastError() == cudaSuccess ? BDLM_OK : BDLM_ERR_CUDA;
 }
 
@@ -462,34 +687,55 @@ int bdlm_linear_ce_bwd(const bdlm_lce_params* p, const void* h, const void* w, c
   if (!al16(h) || !al16(w) || !al16(dh) || !al16(dw) || !al16(workspace) || (reinterpret_cast<uintptr_t>(labels) & 3u) ||
       (reinterpret_cast<uintptr_t>(lse) & 3u) || (reinterpret_cast<uintptr_t>(token_weight) & 3u))
     return BDLM_ERR_INVALID_ARG;
-  if (workspace_bytes < bdlm_linear_ce_workspace_bytes(p, BDLM_LCE_WS_BWD)) return BDLM_ERR_WORKSPACE_TOO_SMALL;
+  const bool roomy = workspace_bytes >= bwd_plan(p, false).bytes;
+  const BwdPlan plan = bwd_plan(p, !roomy);
+  if (workspace_bytes < plan.bytes) return BDLM_ERR_WORKSPACE_TOO_SMALL;
   if (!sm100() || !tc_encoder_available()) return BDLM_ERR_UNSUPPORTED;
   cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
   const int T = p->T, D = p->D, V = p->V;
   const int tc_ = default_chunk(p);
   const int chunks = (T + tc_ - 1) / tc_;
+  char* ws = static_cast<char*>(workspace);
   bf16* dz = static_cast<bf16*>(workspace);
-  float* dw32 = reinterpret_cast<float*>(static_cast<char*>(workspace) + align256((size_t)tc_ * V * 2));
-  const bf16* hb = static_cast<const bf16*>(h);
+  const int64_t ldz = plan.ldz;
+  const int splits = plan.splits;
+  float *dw32 = reinterpret_cast<float*>(ws + plan.dw32), *pieces = reinterpret_cast<float*>(ws + plan.pieces);
+  Operand oh{h, D, 0, false}, ow{w, D, 0, false};
+  if (plan.packed && pack(p, ws + plan.copies, oh, ow, st) != cudaSuccess) return BDLM_ERR_CUDA;
+  auto mn = [](Operand o) { o.mn = 1; return o; };
   for (int ci = 0; ci < chunks; ++ci) {
     const int t0 = ci * tc_, rows = (T - t0) < tc_ ? (T - t0) : tc_;
+    Operand oh_c = oh;
+    oh_c.ptr = static_cast<const bf16*>(oh.ptr) + (size_t)t0 * oh.ld;
+    const Operand odz{dz, ldz, 0, roomy};
     // dz of the chunk: logits again, softmax minus one-hot in the epilogue
     GemmArgs a = {};
-    a.M = rows; a.N = V; a.K = D; a.n_run = FWD_N_RUN; a.m_inner = 1;
+    const Tiling ta = choose_tiling(rows, V, D, 1, FWD_N_RUN, EPI_CLK_DZ, 0);
+    a.M = rows; a.N = V; a.K = D; a.bn = ta.bn; a.n_run = ta.n_run; a.m_inner = 1;
     a.row0 = t0; a.labels = labels; a.weight = token_weight; a.lse = lse; a.grad = p->grad_loss;
-    a.dz = dz; a.ldz = V;
-    if (launch_gemm<EPI_DZ>(a, Operand{hb + (size_t)t0 * D, D, 0}, Operand{w, D, 0}, st) != cudaSuccess) return BDLM_ERR_CUDA;
+    a.dz = dz; a.ldz = (int)ldz;
+    if (launch_gemm<EPI_DZ>(a, oh_c, ow, st) != cudaSuccess) return BDLM_ERR_CUDA;
     // dH of the chunk = dz W   (contraction over the vocabulary; W as it lies is the MN-major B operand)
     GemmArgs b = {};
-    b.M = rows; b.N = D; b.K = V; b.n_run = 1; b.m_inner = 1;
-    b.c_mode = C_BF16; b.c16 = static_cast<bf16*>(dh) + (size_t)t0 * D; b.ldc = D;
-    if (launch_gemm<EPI_STORE>(b, Operand{dz, V, 0}, Operand{w, D, 1}, st) != cudaSuccess) return BDLM_ERR_CUDA;
+    b.M = rows; b.N = D; b.K = V; b.bn = choose_tiling(rows, D, V, splits, 1, EPI_CLK_STORE, 1).bn; b.n_run = 1; b.m_inner = 1;
+    bf16* dh_c = static_cast<bf16*>(dh) + (size_t)t0 * D;
+    b.c_mode = splits > 1 ? C_F32_PART : C_BF16; b.c16 = dh_c; b.c32 = pieces; b.ldc = D;
+    b.k_split = ((V + BK - 1) / BK + splits - 1) / splits;
+    b.splits = ((V + BK - 1) / BK + b.k_split - 1) / b.k_split;   // no empty piece
+    if (launch_gemm<EPI_STORE>(b, odz, mn(ow), st) != cudaSuccess) return BDLM_ERR_CUDA;
+    if (splits > 1) {
+      const int64_t n = (int64_t)rows * D, want = (n / 4 + 255) / 256, cap = (int64_t)device_sm_count() * 8;
+      lce_sum_pieces_kernel<<<(unsigned)(want < cap ? want : cap), 256, 0, st>>>(pieces, b.splits, n, dh_c);
+      if (cudaGetLastError() != cudaSuccess) return BDLM_ERR_CUDA;
+    }
     // dW += dz^T H_c   (contraction over the chunk's tokens; both operands MN-major)
     GemmArgs c = {};
-    c.M = V; c.N = D; c.K = rows; c.n_run = 1; c.m_inner = 0;
+    c.M = V; c.N = D; c.K = rows; c.bn = choose_tiling(V, D, rows, 1, 1, EPI_CLK_STORE, 1).bn; c.n_run = 1; c.m_inner = 0;
     c.c16 = static_cast<bf16*>(dw); c.c32 = dw32; c.ldc = D;
     c.c_mode = chunks == 1 ? C_BF16 : (ci == 0 ? C_F32_STORE : (ci + 1 < chunks ? C_F32_ADD : C_F32_ADD_TO_BF16));
-    if (launch_gemm<EPI_STORE>(c, Operand{dz, V, 1}, Operand{hb + (size_t)t0 * D, D, 1}, st) != cudaSuccess) return BDLM_ERR_CUDA;
+    const Operand A = mn(odz), B = mn(oh_c);
+    const bool adds = c.c_mode == C_F32_ADD || c.c_mode == C_F32_ADD_TO_BF16;
+    if ((adds ? launch_gemm<EPI_ADD>(c, A, B, st) : launch_gemm<EPI_STORE>(c, A, B, st)) != cudaSuccess) return BDLM_ERR_CUDA;
   }
   return BDLM_OK;
 }

@@ -17,6 +17,10 @@ bool tc_make_map(CUtensorMap* m, const void* ptr, int heads, int L, int batch, i
 // `box_rows` rows, 128-byte swizzle, zero fill outside the matrix.
 bool tc_make_map_2d(CUtensorMap* m, const void* ptr, int64_t rows, int64_t cols, int64_t ld, int box_rows);
 
+// The same matrix as a stack of 64-column panels (cols a multiple of 64): one load brings `box_panels` neighbouring panels
+// of `box_rows` rows, one after the other.
+bool tc_make_map_panels(CUtensorMap* m, const void* ptr, int64_t rows, int64_t cols, int64_t ld, int box_rows, int box_panels);
+
 bool tc_rows_ok(const KArgs& a);
 bool tc_fwd_supported(const KArgs& a);
 bool tc_bwd_supported(const KArgs& a);

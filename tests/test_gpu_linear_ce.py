@@ -126,3 +126,39 @@ def test_all_positions_ignored_gives_zero_loss_and_zero_gradients():
     assert float(dh.float().abs().max()) == 0.0 and float(dw.float().abs().max()) == 0.0
     ref = lce.linear_ce_forward(synth.to_f64(inp["h"]), synth.to_f64(inp["w"]), labels.cpu().numpy())
     assert np.abs(synth.to_f64(lse) - ref[2]).max() <= TOL_LSE
+
+
+@pytest.mark.parametrize("w", [
+    LceWorkload("split_contraction", 150, 72, 8200),           # dH in eight pieces of the vocabulary, the last one short
+    LceWorkload("narrow_tiles", 520, 264, 9000),               # D one tile and 8 columns: tiles narrower than 256
+    LceWorkload("odd_half_chunks", 390, 512, 5000),            # 144-column tiles: the last 32-column chunk reaches past them
+    LceWorkload("many_short_runs", 260, 64, 20008),            # more partial (maximum, sum) pairs than one per 2048 logits
+], ids=lambda w: w.name)
+def test_tilings_and_split_contraction(w):
+    one = _check(w)
+    # dH does not depend on the token chunks; the smallest accepted workspace takes the coarse tiling and one piece
+    g = {k: v.cuda() for k, v in synth.make_lce_inputs(w, "cpu").items()}
+    dh, _ = binding.bdlm_linear_ce_bwd(g["h"], g["w"], g["labels"], one[2], g["weight"], token_chunk=128)
+    assert torch.equal(dh, one[3])
+    per = (w.T * 4 + 255) // 256 * 256
+    runs = (((w.V + 255) // 256) + 7) // 8
+    least = torch.empty((2 * runs + 1) * per + 256, dtype=torch.uint8, device="cuda")
+    loss, nll, lse = binding.bdlm_linear_ce_fwd(g["h"], g["w"], g["labels"], g["weight"], workspace=least)
+    least = torch.empty((w.T + 127) // 128 * 128 * w.V * 2, dtype=torch.uint8, device="cuda")
+    dh, dw = binding.bdlm_linear_ce_bwd(g["h"], g["w"], g["labels"], lse, g["weight"], workspace=least)
+    torch.cuda.synchronize()
+    assert float((lse - one[2]).abs().max()) <= TOL_LSE and abs(float(loss) - float(one[0])) <= TOL_LOSS_REL * abs(float(one[0]))
+    # another order of the fp32 sums, then one bf16 rounding (2^-9 of an element where it falls the other way)
+    assert _rel(synth.to_f64(dh), synth.to_f64(one[3])) <= 4e-3 and _rel(synth.to_f64(dw), synth.to_f64(one[4])) <= 4e-3
+
+
+@pytest.mark.parametrize("w", [
+    LceWorkload("copied_for_the_backward", 400, 72, 1032),
+    LceWorkload("copied_for_both", 1030, 200, 1544),
+    LceWorkload("copied_wide", 1100, 264, 1000),
+], ids=lambda w: w.name)
+def test_rows_that_are_no_whole_number_of_lines(w):
+    """From a number of tokens on, W and h are copied to padded rows (D no multiple of 64): one chunk and several."""
+    one = _check(w)
+    several = _check(w, token_chunk=256)
+    assert torch.equal(one[3], several[3])
