@@ -44,6 +44,47 @@ __device__ __forceinline__ void tma_tile(uint32_t dst, const CUtensorMap* map, u
   if (D == 128) tma_load_3d(dst + PANEL_BYTES, map, bar, head * D + 64, row0, b);
 }
 
+// The elementwise work of a tile, two elements per instruction where the arithmetic allows it: the compute warps are bound
+// by instruction issue beside the exponential unit (L = 2048, H = 32: fused kernel 192 -> 189 us, windowed 32K 2.95 -> 2.85 ms,
+// dQ pass at L = 16K, H = 8 1169 -> 1107 us; at the power cap, 32K, no change).  Scores x become P = exp2(x * scale - lse); hidden elements (bits of
+// [lo, hi) clear) become zero.  nlse: minus the LSE rows in log2 units, one per element (-inf where there is no row).
+template <int N>
+__device__ __forceinline__ void exp_tile(uint32_t (&x)[N], uint64_t scale2, const float* nlse) {
+#pragma unroll
+  for (int c = 0; c < N; c += 4) {
+    const ulonglong2 z = *reinterpret_cast<const ulonglong2*>(nlse + c);
+    float p0, p1, p2, p3;
+    unpack_f32x2(fma_f32x2(pack_f32x2(__uint_as_float(x[c]), __uint_as_float(x[c + 1])), scale2, z.x), p0, p1);
+    unpack_f32x2(fma_f32x2(pack_f32x2(__uint_as_float(x[c + 2]), __uint_as_float(x[c + 3])), scale2, z.y), p2, p3);
+    x[c] = __float_as_uint(exp2f(p0)); x[c + 1] = __float_as_uint(exp2f(p1));
+    x[c + 2] = __float_as_uint(exp2f(p2)); x[c + 3] = __float_as_uint(exp2f(p3));
+  }
+}
+template <int N>
+__device__ __forceinline__ void hide_tile(uint32_t (&x)[N], int lo, int hi) {
+#pragma unroll
+  for (int g = 0; g < N / 32; ++g) {
+    const uint32_t seen = interval_bits(lo - 32 * g, hi - 32 * g);
+#pragma unroll
+    for (int e = 0; e < 32; ++e) x[32 * g + e] = (seen >> e) & 1u ? x[32 * g + e] : 0u;
+  }
+}
+// dS = P * (dP - D) as bf16 pairs; nd: minus the D of each element.
+template <int N>
+__device__ __forceinline__ void ds_tile(uint32_t (&pk)[N / 2], const uint32_t (&x)[N], const uint32_t (&y)[N], const float* nd) {
+#pragma unroll
+  for (int c = 0; c < N; c += 4) {
+    const ulonglong2 d = *reinterpret_cast<const ulonglong2*>(nd + c);
+    float d0, d1, d2, d3;
+    unpack_f32x2(mul_f32x2(pack_f32x2(__uint_as_float(x[c]), __uint_as_float(x[c + 1])),
+                           add_f32x2(pack_f32x2(__uint_as_float(y[c]), __uint_as_float(y[c + 1])), d.x)), d0, d1);
+    unpack_f32x2(mul_f32x2(pack_f32x2(__uint_as_float(x[c + 2]), __uint_as_float(x[c + 3])),
+                           add_f32x2(pack_f32x2(__uint_as_float(y[c + 2]), __uint_as_float(y[c + 3])), d.y)), d2, d3);
+    pk[c / 2] = pack_bf16(d0, d1);
+    pk[c / 2 + 1] = pack_bf16(d2, d3);
+  }
+}
+
 // Write a thread's 128 accumulator columns (4 x 32) as bf16 to a global row, scaled.
 __device__ __forceinline__ void store_row_chunk(bf16* dst, const uint32_t (&v)[32], float scale) {
 #pragma unroll
@@ -206,8 +247,8 @@ tc_dkdv_kernel(const __grid_constant__ BwdMaps maps, const KArgs a, const TileGr
   extern __shared__ __align__(1024) uint8_t sm[];
   const uint32_t base = smem_u32(sm);
   const uint32_t sK = base, sV = base + TILE_BYTES, sQ0 = base + DKDV_Q0, sdO0 = base + DKDV_DO0, sP = base + DKDV_P;
-  float* lse_s = reinterpret_cast<float*>(sm + DKDV_ARR);          // [2][128], log2 units
-  float* d_s = lse_s + 256;                                        // [2][128]
+  float* lse_s = reinterpret_cast<float*>(sm + DKDV_ARR);          // [2][128], minus the LSE in log2 units
+  float* d_s = lse_s + 256;                                        // [2][128], minus D
   const uint32_t bars = base + DKDV_BARS;
   const uint32_t bar_kv = bars, bar_q_full = bars + 8 /*[2]*/, bar_q_empty = bars + 24 /*[2]*/,
                  bar_do_full = bars + 40 /*[2]*/, bar_do_empty = bars + 56 /*[2]*/,
@@ -325,10 +366,10 @@ tc_dkdv_kernel(const __grid_constant__ BwdMaps maps, const KArgs a, const TileGr
       }
       {
         float4 z2;
-        z2.x = isfinite(z.x) ? z.x * LOG2E : INFINITY; z2.y = isfinite(z.y) ? z.y * LOG2E : INFINITY;
-        z2.z = isfinite(z.z) ? z.z * LOG2E : INFINITY; z2.w = isfinite(z.w) ? z.w * LOG2E : INFINITY;
+        z2.x = isfinite(z.x) ? z.x * -LOG2E : -INFINITY; z2.y = isfinite(z.y) ? z.y * -LOG2E : -INFINITY;
+        z2.z = isfinite(z.z) ? z.z * -LOG2E : -INFINITY; z2.w = isfinite(z.w) ? z.w * -LOG2E : -INFINITY;
         reinterpret_cast<float4*>(lse_s + sd * 128)[lane] = z2;
-        reinterpret_cast<float4*>(d_s + sd * 128)[lane] = dd;
+        reinterpret_cast<float4*>(d_s + sd * 128)[lane] = make_float4(-dd.x, -dd.y, -dd.z, -dd.w);
       }
       __syncwarp();
       if (lane == 0) mbar_arrive(bar_do_full + 8 * sd);
@@ -429,6 +470,7 @@ tc_dkdv_kernel(const __grid_constant__ BwdMaps maps, const KArgs a, const TileGr
       vqn_lo = (j / M) * M; vqn_hi = vqn_lo + M;
       fulln_lo = ((k0 + TILE - 1) / M) * M; fulln_hi = (k0 / M) * M + M;
     }
+    const uint64_t scale2 = pack_f32x2(a.scale_log2, a.scale_log2);
     bool ok = true;
     long long w_st = 0, w_dpt = 0, w_pf = 0, c_exp = 0, c_ds = 0, c_ld = 0, c_math = 0;
     const long long t_begin = tick<TR>();
@@ -455,36 +497,9 @@ tc_dkdv_kernel(const __grid_constant__ BwdMaps maps, const KArgs a, const TileGr
       mbar_arrive(bar_sfree);   // S^T(i) is in registers: the tensor core may overwrite its columns
       const long long t0b = tick<TR>();
       c_ld += t0b - t0;
-      const float4* lz4 = reinterpret_cast<const float4*>(lse_s + sd * 128 + c0);
-      if (!need_mask) {
-#pragma unroll
-        for (int c8 = 0; c8 < CW / 8; ++c8) {
-          const float4 za = lz4[2 * c8], zb = lz4[2 * c8 + 1];
-          float* xf = reinterpret_cast<float*>(x) + 8 * c8;
-          xf[0] = exp2f(fmaf(xf[0], a.scale_log2, -za.x));
-          xf[1] = exp2f(fmaf(xf[1], a.scale_log2, -za.y));
-          xf[2] = exp2f(fmaf(xf[2], a.scale_log2, -za.z));
-          xf[3] = exp2f(fmaf(xf[3], a.scale_log2, -za.w));
-          xf[4] = exp2f(fmaf(xf[4], a.scale_log2, -zb.x));
-          xf[5] = exp2f(fmaf(xf[5], a.scale_log2, -zb.y));
-          xf[6] = exp2f(fmaf(xf[6], a.scale_log2, -zb.z));
-          xf[7] = exp2f(fmaf(xf[7], a.scale_log2, -zb.w));
-        }
-      } else {
-        // visible columns of this thread's key row inside the tile: [vlo, vhi)
-        const int vlo = (st.qs == CLEAN ? vqc_lo : vqn_lo) - st.q0 - c0, vhi = (st.qs == CLEAN ? vqc_hi : vqn_hi) - st.q0 - c0;
-#pragma unroll
-        for (int c4 = 0; c4 < CW / 4; ++c4) {
-          const float4 z = lz4[c4];
-          const float zz[4] = {z.x, z.y, z.z, z.w};
-#pragma unroll
-          for (int e = 0; e < 4; ++e) {
-            const int c = 4 * c4 + e;
-            const float p = exp2f(fmaf(__uint_as_float(x[c]), a.scale_log2, -zz[e]));
-            x[c] = __float_as_uint((c >= vlo && c < vhi) ? p : 0.f);
-          }
-        }
-      }
+      exp_tile<CW>(x, scale2, lse_s + sd * 128 + c0);
+      if (need_mask)   // visible columns of this thread's key row inside the tile
+        hide_tile<CW>(x, (st.qs == CLEAN ? vqc_lo : vqn_lo) - st.q0 - c0, (st.qs == CLEAN ? vqc_hi : vqn_hi) - st.q0 - c0);
       c_math += tick<TR>() - t0b;
       // P^T(i) as bf16 into the shared-memory tile, once dV(i-1) has finished reading P^T(i-1)
       if (i > 0) {
@@ -517,18 +532,8 @@ tc_dkdv_kernel(const __grid_constant__ BwdMaps maps, const KArgs a, const TileGr
 #pragma unroll
         for (int q = 0; q < CW / 32; ++q) tmem_ld32(tl + 128 + c0 + 32 * q, c[q]);
         tmem_wait_ld();
-        const float4* dz4 = reinterpret_cast<const float4*>(d_s + sd * 128 + c0);
         uint32_t pk[CW / 2];
-#pragma unroll
-        for (int c4 = 0; c4 < CW / 4; ++c4) {
-          const float4 dd = dz4[c4];
-          const float d0 = __uint_as_float(x[4 * c4 + 0]) * (__uint_as_float(y[4 * c4 + 0]) - dd.x);
-          const float d1 = __uint_as_float(x[4 * c4 + 1]) * (__uint_as_float(y[4 * c4 + 1]) - dd.y);
-          const float d2 = __uint_as_float(x[4 * c4 + 2]) * (__uint_as_float(y[4 * c4 + 2]) - dd.z);
-          const float d3 = __uint_as_float(x[4 * c4 + 3]) * (__uint_as_float(y[4 * c4 + 3]) - dd.w);
-          pk[2 * c4] = pack_bf16(d0, d1);
-          pk[2 * c4 + 1] = pack_bf16(d2, d3);
-        }
+        ds_tile<CW>(pk, x, y, d_s + sd * 128 + c0);
         if constexpr (CW == 64) tmem_st32(tl + 128 + c0, reinterpret_cast<uint32_t (&)[32]>(pk));
         else tmem_st16(tl + 128 + c0, reinterpret_cast<uint32_t (&)[16]>(pk));
         tmem_wait_st();
@@ -807,27 +812,16 @@ tc_dq_kernel(const __grid_constant__ BwdMaps maps, const KArgs a, const TileGrid
       sw.lap(c_ld);
       const bool need_mask = (ks == 0 ? (k0 < lo_last0 || k0 + TILE > hi_first0) : (k0 < lo_last1 || k0 + TILE > hi_first1)) ||
                              q0 + TILE > L;
-      if (!need_mask) {
+      {
+        const uint64_t scale2 = pack_f32x2(a.scale_log2, a.scale_log2), nlse2 = pack_f32x2(-lse2, -lse2);
 #pragma unroll
-        for (int c8 = 0; c8 < 8; ++c8) {
-          float* xf = reinterpret_cast<float*>(x) + 8 * c8;
-          xf[0] = exp2f(fmaf(xf[0], a.scale_log2, -lse2));
-          xf[1] = exp2f(fmaf(xf[1], a.scale_log2, -lse2));
-          xf[2] = exp2f(fmaf(xf[2], a.scale_log2, -lse2));
-          xf[3] = exp2f(fmaf(xf[3], a.scale_log2, -lse2));
-          xf[4] = exp2f(fmaf(xf[4], a.scale_log2, -lse2));
-          xf[5] = exp2f(fmaf(xf[5], a.scale_log2, -lse2));
-          xf[6] = exp2f(fmaf(xf[6], a.scale_log2, -lse2));
-          xf[7] = exp2f(fmaf(xf[7], a.scale_log2, -lse2));
-        }
-      } else {
-        const int vlo = (ks == 0 ? rlo0 : rlo1) - k0 - c0, vhi = (ks == 0 ? rhi0 : rhi1) - k0 - c0;
-#pragma unroll
-        for (int c = 0; c < 64; ++c) {
-          const float p = exp2f(fmaf(__uint_as_float(x[c]), a.scale_log2, -lse2));
-          x[c] = __float_as_uint((c >= vlo && c < vhi) ? p : 0.f);
+        for (int c = 0; c < 64; c += 2) {
+          float p0, p1;
+          unpack_f32x2(fma_f32x2(pack_f32x2(__uint_as_float(x[c]), __uint_as_float(x[c + 1])), scale2, nlse2), p0, p1);
+          x[c] = __float_as_uint(exp2f(p0)); x[c + 1] = __float_as_uint(exp2f(p1));
         }
       }
+      if (need_mask) hide_tile<64>(x, (ks == 0 ? rlo0 : rlo1) - k0 - c0, (ks == 0 ? rhi0 : rhi1) - k0 - c0);
       sw.lap(c_exp);
       ok = mbar_wait_timed<TR>(bar_dp, i & 1, abort_flag, w_dp);
       ok = __all_sync(0xffffffffu, ok);
@@ -840,10 +834,12 @@ tc_dq_kernel(const __grid_constant__ BwdMaps maps, const KArgs a, const TileGrid
         tmem_ld32(tl + C_DP + c0, c[0]); tmem_ld32(tl + C_DP + c0 + 32, c[1]);
         tmem_wait_ld();
         uint32_t pk[32];
+        const uint64_t nd2 = pack_f32x2(-dsum, -dsum);
 #pragma unroll
         for (int e = 0; e < 32; ++e) {
-          const float d0 = __uint_as_float(x[2 * e]) * (__uint_as_float(y[2 * e]) - dsum);
-          const float d1 = __uint_as_float(x[2 * e + 1]) * (__uint_as_float(y[2 * e + 1]) - dsum);
+          float d0, d1;
+          unpack_f32x2(mul_f32x2(pack_f32x2(__uint_as_float(x[2 * e]), __uint_as_float(x[2 * e + 1])),
+                                 add_f32x2(pack_f32x2(__uint_as_float(y[2 * e]), __uint_as_float(y[2 * e + 1])), nd2)), d0, d1);
           pk[e] = pack_bf16(d0, d1);
         }
         tmem_st32(tl + C_DP + c0, pk);
@@ -942,8 +938,8 @@ tc_bwdf_kernel(const __grid_constant__ BwdMaps maps, const KArgs a, const TileGr
   const uint32_t base = smem_u32(sm);
   const uint32_t sK = base, sV = base + TILE_BYTES, sQ0 = base + BF_Q0, sdO0 = base + BF_DO0, sDS = base + BF_DS,
                  sSTG = base + BF_STG;
-  float* lse_s = reinterpret_cast<float*>(sm + BF_ARR);            // [4][64], log2 units
-  float* d_s = lse_s + 256;                                        // [4][64]
+  float* lse_s = reinterpret_cast<float*>(sm + BF_ARR);            // [4][64], minus the LSE in log2 units
+  float* d_s = lse_s + 256;                                        // [4][64], minus D
   const uint32_t bars = base + BF_BARS;
   const uint32_t bar_kv = bars, bar_q_full = bars + 8 /*[4]*/, bar_q_empty = bars + 40 /*[4]*/,
                  bar_do_full = bars + 72 /*[3]*/, bar_do_empty = bars + 96 /*[3]*/,
@@ -1065,11 +1061,11 @@ tc_bwdf_kernel(const __grid_constant__ BwdMaps maps, const KArgs a, const TileGr
       if (!ok) break;
       if (lane < 16) {
         float4 z2;
-        z2.x = isfinite(rows.x) ? rows.x * LOG2E : INFINITY; z2.y = isfinite(rows.y) ? rows.y * LOG2E : INFINITY;
-        z2.z = isfinite(rows.z) ? rows.z * LOG2E : INFINITY; z2.w = isfinite(rows.w) ? rows.w * LOG2E : INFINITY;
+        z2.x = isfinite(rows.x) ? rows.x * -LOG2E : -INFINITY; z2.y = isfinite(rows.y) ? rows.y * -LOG2E : -INFINITY;
+        z2.z = isfinite(rows.z) ? rows.z * -LOG2E : -INFINITY; z2.w = isfinite(rows.w) ? rows.w * -LOG2E : -INFINITY;
         reinterpret_cast<float4*>(lse_s + sr * 64)[lane] = z2;
       } else {
-        reinterpret_cast<float4*>(d_s + sr * 64)[lane - 16] = rows;
+        reinterpret_cast<float4*>(d_s + sr * 64)[lane - 16] = make_float4(-rows.x, -rows.y, -rows.z, -rows.w);
       }
       __syncwarp();
       if (lane == 0) mbar_arrive(bar_rows_full + 8 * sr);
@@ -1252,6 +1248,7 @@ tc_bwdf_kernel(const __grid_constant__ BwdMaps maps, const KArgs a, const TileGr
       vqn_lo = (j / M) * M; vqn_hi = vqn_lo + M;
       fulln_lo = ((k0 + TILE - 1) / M) * M; fulln_hi = (k0 / M) * M + M;
     }
+    const uint64_t scale2 = pack_f32x2(a.scale_log2, a.scale_log2);
     bool ok = true;
     long long w_st = 0, w_dpt = 0, w_dsf = 0, c_exp = 0, c_ds = 0;
     const long long t_begin = tick<TR>();
@@ -1280,32 +1277,9 @@ tc_bwdf_kernel(const __grid_constant__ BwdMaps maps, const KArgs a, const TileGr
       uint32_t x[32];
       tmem_ld32(tl + c0, x);
       tmem_wait_ld();
-      const float4* lz4 = reinterpret_cast<const float4*>(lse_s + sr * 64 + c0);
-      if (!need_mask) {
-#pragma unroll
-        for (int c4 = 0; c4 < 8; ++c4) {
-          const float4 z = lz4[c4];
-          float* xf = reinterpret_cast<float*>(x) + 4 * c4;
-          xf[0] = exp2f(fmaf(xf[0], a.scale_log2, -z.x));
-          xf[1] = exp2f(fmaf(xf[1], a.scale_log2, -z.y));
-          xf[2] = exp2f(fmaf(xf[2], a.scale_log2, -z.z));
-          xf[3] = exp2f(fmaf(xf[3], a.scale_log2, -z.w));
-        }
-      } else {
-        // visible columns of this thread's key row inside the step: [vlo, vhi)
-        const int vlo = (st.qs == CLEAN ? vqc_lo : vqn_lo) - st.q0 - c0, vhi = (st.qs == CLEAN ? vqc_hi : vqn_hi) - st.q0 - c0;
-#pragma unroll
-        for (int c4 = 0; c4 < 8; ++c4) {
-          const float4 z = lz4[c4];
-          const float zz[4] = {z.x, z.y, z.z, z.w};
-#pragma unroll
-          for (int e = 0; e < 4; ++e) {
-            const int c = 4 * c4 + e;
-            const float p = exp2f(fmaf(__uint_as_float(x[c]), a.scale_log2, -zz[e]));
-            x[c] = __float_as_uint((c >= vlo && c < vhi) ? p : 0.f);
-          }
-        }
-      }
+      exp_tile<32>(x, scale2, lse_s + sr * 64 + c0);
+      if (need_mask)   // visible columns of this thread's key row inside the step
+        hide_tile<32>(x, (st.qs == CLEAN ? vqc_lo : vqn_lo) - st.q0 - c0, (st.qs == CLEAN ? vqc_hi : vqn_hi) - st.q0 - c0);
       {
         uint32_t pk[16];
 #pragma unroll
@@ -1330,17 +1304,7 @@ tc_bwdf_kernel(const __grid_constant__ BwdMaps maps, const KArgs a, const TileGr
         tmem_wait_ld();
         tc_fence_before();
         mbar_arrive(bar_dpfree);   // dP^T(i) is in registers: the tensor core may overwrite its columns
-        const float4* dz4 = reinterpret_cast<const float4*>(d_s + sr * 64 + c0);
-#pragma unroll
-        for (int c4 = 0; c4 < 8; ++c4) {
-          const float4 dz = dz4[c4];
-          const float d0 = __uint_as_float(x[4 * c4 + 0]) * (__uint_as_float(y[4 * c4 + 0]) - dz.x);
-          const float d1 = __uint_as_float(x[4 * c4 + 1]) * (__uint_as_float(y[4 * c4 + 1]) - dz.y);
-          const float d2 = __uint_as_float(x[4 * c4 + 2]) * (__uint_as_float(y[4 * c4 + 2]) - dz.z);
-          const float d3 = __uint_as_float(x[4 * c4 + 3]) * (__uint_as_float(y[4 * c4 + 3]) - dz.w);
-          pk[2 * c4] = pack_bf16(d0, d1);
-          pk[2 * c4 + 1] = pack_bf16(d2, d3);
-        }
+        ds_tile<32>(pk, x, y, d_s + sr * 64 + c0);
       }
       c_ds += tick<TR>() - t2;
       // dS^T(i) into the shared-memory tile, once dK and dQ^T of step i-1 have read dS^T(i-1)
