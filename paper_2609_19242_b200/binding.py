@@ -116,31 +116,24 @@ def make_params(batch, L, block_size, H, H_kv, d, scale=0.0, clean_mask_mode=0, 
                 include_noisy_diag=True, impl=IMPL_AUTO, bwd_passes=0, bwd_single_pass=None, window=0) -> BdlmParams:
     """`bwd_single_pass`: None = automatic (BDLM_BWD_AUTO: the fused kernel when the workspace has room for it),
     True = the fused kernel (BDLM_BWD_FUSED), False = the two-pass kernels (BDLM_BWD_TWO_PASS)."""
-    p = BdlmParams()
-    p.batch, p.L, p.block_size, p.H, p.H_kv, p.d = batch, L, block_size, H, H_kv, d
-    p.scale = float(scale)
-    p.clean_mask_mode = clean_mask_mode
-    if kv_range is None:
-        p.kv_begin, p.kv_end, p.kv_range_set = 0, 0, 0
-    else:
-        p.kv_begin, p.kv_end, p.kv_range_set = int(kv_range[0]), int(kv_range[1]), 1
-    p.include_noisy_diag = 1 if include_noisy_diag else 0
-    p.impl = impl
-    p.bwd_passes = bwd_passes
-    p.bwd_single_pass = BWD_AUTO if bwd_single_pass is None else (BWD_FUSED if bwd_single_pass else BWD_TWO_PASS)
-    p.window = int(window)
-    return p
+    # (one constructor call: assigning the sixteen fields one by one takes as long as a kernel launch)
+    begin, end = (0, 0) if kv_range is None else (int(kv_range[0]), int(kv_range[1]))
+    return BdlmParams(batch, L, block_size, H, H_kv, d, float(scale), clean_mask_mode, begin, end,
+                      0 if kv_range is None else 1, 1 if include_noisy_diag else 0, impl, bwd_passes,
+                      BWD_AUTO if bwd_single_pass is None else (BWD_FUSED if bwd_single_pass else BWD_TWO_PASS), int(window))
 
 
+# A small step (L = 256) is bound by this file: 45 pointer arguments and two stream look-ups.  ctypes takes plain integers
+# for void pointers, and the raw stream handle needs no Stream object.
 def _ptr(t):
     if t is None:
         return None
     assert t.is_cuda and t.is_contiguous(), "tensors must be contiguous CUDA tensors"
-    return ctypes.c_void_p(t.data_ptr())
+    return t.data_ptr()
 
 
 def _stream():
-    return ctypes.c_void_p(torch.cuda.current_stream().cuda_stream)
+    return torch._C._cuda_getCurrentRawStream(torch.cuda.current_device())
 
 
 def _shape_params(q, k, block_size, **kw):
@@ -248,10 +241,15 @@ def _packed_setup(q_clean, k_clean, q_noisy, block_size, block_prefix, clean_q_p
         inv = [0] * n
         for m, pos in enumerate(positions):
             inv[pos // chunk_len] = m
-        t_pos = torch.tensor(positions, dtype=torch.int32, device=k_clean.device)
-        t_inv = torch.tensor(inv, dtype=torch.int32, device=k_clean.device)
-        keep += [t_pos, t_inv]
-        g.kv_chunk_len, g.kv_chunk_pos, g.kv_pos_chunk = chunk_len, t_pos.data_ptr(), t_inv.data_ptr()
+        # both tables in one copy that does not wait for the stream (a pageable one would: the host fell behind by a
+        # whole backward per call).  Not under graph capture, where the pinned source would not outlive the replays:
+        # there the pageable copy refuses, as it always did.
+        tables = torch.tensor([positions, inv], dtype=torch.int32)
+        if not torch.cuda.is_current_stream_capturing():
+            tables = tables.pin_memory()
+        tables = tables.to(k_clean.device, non_blocking=tables.is_pinned())
+        keep.append(tables)
+        g.kv_chunk_len, g.kv_chunk_pos, g.kv_pos_chunk = chunk_len, tables.data_ptr(), tables.data_ptr() + 4 * n
     if q_noisy is not None:
         if q_noisy.shape[1] % block_size != 0:
             raise ValueError("packed noisy rows must be a whole number of blocks")
