@@ -161,6 +161,36 @@ inline unsigned tile_grid_blocks(const TileGrid& g) {
   return n > 0x7fffffffLL ? 0u : (unsigned)n;
 }
 
+// Launches of one call that follow one another are chained: a kernel started with launch_chained may be brought onto the
+// chip while its predecessor's last blocks still run (which hides about 2 us of launch latency per kernel: 11 of the 127 us
+// of a ragged d = 64 step were gaps), and every block of it first waits here until the predecessor has completed and its
+// writes are visible.  Data that the predecessor wrote must not be read through the read-only path (no __restrict__
+// const).  The first launch of a call is an ordinary one.
+__device__ __forceinline__ void wait_for_predecessor() {
+  asm volatile("griddepcontrol.wait;\n\tgriddepcontrol.launch_dependents;" ::: "memory");
+}
+template <class... P, class... A>
+cudaError_t launch_chained(void (*kern)(P...), bool chained, unsigned blocks, int threads, size_t smem, cudaStream_t st, int cluster, const A&... args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(blocks);
+  cfg.blockDim = dim3(threads);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cudaLaunchAttribute attr[2] = {};
+  int n = 0;
+  if (chained) {
+    attr[n].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[n++].val.programmaticStreamSerializationAllowed = 1;
+  }
+  if (cluster > 1) {
+    attr[n].id = cudaLaunchAttributeClusterDimension;
+    attr[n].val.clusterDim.x = cluster; attr[n].val.clusterDim.y = 1; attr[n++].val.clusterDim.z = 1;
+  }
+  cfg.attrs = attr;
+  cfg.numAttrs = n;
+  return cudaLaunchKernelEx(&cfg, kern, P(args)...);
+}
+
 __device__ __forceinline__ uint32_t pack_bf16(float lo, float hi) {
   __nv_bfloat162 v = __floats2bfloat162_rn(lo, hi);
   return *reinterpret_cast<uint32_t*>(&v);

@@ -127,6 +127,7 @@ struct PrepArgs {
 template <int D>
 __global__ void __launch_bounds__(256) bwd_prepare_kernel(const PrepArgs pa) {
   __shared__ float sums[PREP_HEADS][PREP_ROWS + 1];
+  wait_for_predecessor();
   constexpr int LPR = D / 8;               // lanes per row
   constexpr int RPP = 256 / LPR;           // rows per pass of the block
   constexpr int UNROLL = 4;

@@ -116,6 +116,7 @@ struct TileWalk {
 template <int EPI>
 __global__ void __launch_bounds__(G_THREADS, 1)
 lce_gemm_kernel(const __grid_constant__ GemmMaps maps, const GemmArgs a, int* __restrict__ status) {
+  wait_for_predecessor();
   extern __shared__ uint8_t smem_raw[];
   const uint32_t base = (smem_u32(smem_raw) + 1023u) & ~1023u;
   uint8_t* sm = smem_raw + (base - smem_u32(smem_raw));
@@ -381,11 +382,12 @@ lce_gemm_kernel(const __grid_constant__ GemmMaps maps, const GemmArgs a, int* __
 // hundred dependent rounds of loads when the runs are short).  The block's sum replaces its own first token's first
 // partial maximum, which nobody else reads.
 constexpr int FIN_T = 32;
-__global__ void __launch_bounds__(256) lce_finish_kernel(float* part_m, const float* __restrict__ part_l,
-                                                         const float* __restrict__ zlab, const int* __restrict__ labels,
+__global__ void __launch_bounds__(256) lce_finish_kernel(float* part_m, const float* part_l,
+                                                         const float* zlab, const int* __restrict__ labels,
                                                          const float* __restrict__ weight, int T, int n_runs, int ldp,
                                                          float* __restrict__ lse, float* __restrict__ nll) {
   __shared__ float sm_m[8][FIN_T], sm_l[8][FIN_T];
+  wait_for_predecessor();
   const int x = threadIdx.x % FIN_T, y0 = threadIdx.x / FIN_T;
   const int t = blockIdx.x * FIN_T + x;
   float m = -INFINITY, l = 0.f;
@@ -419,8 +421,9 @@ __global__ void __launch_bounds__(256) lce_finish_kernel(float* part_m, const fl
   if (x == 0) part_m[blockIdx.x * FIN_T] = contrib;
 }
 
-__global__ void __launch_bounds__(256) lce_sum_kernel(const float* __restrict__ block_sums, int n, int stride, float* __restrict__ loss) {
+__global__ void __launch_bounds__(256) lce_sum_kernel(const float* block_sums, int n, int stride, float* loss) {
   __shared__ float red[256];
+  wait_for_predecessor();
   float acc = 0.f;
   for (int i = threadIdx.x; i < n; i += 256) acc += block_sums[i * stride];
   red[threadIdx.x] = acc;
@@ -433,7 +436,8 @@ __global__ void __launch_bounds__(256) lce_sum_kernel(const float* __restrict__ 
 }
 
 // Sum of the pieces of a split contraction, in their order, as bf16.  n = elements per piece (a multiple of 8).
-__global__ void __launch_bounds__(256) lce_sum_pieces_kernel(const float* __restrict__ part, int pieces, int64_t n, bf16* __restrict__ out) {
+__global__ void __launch_bounds__(256) lce_sum_pieces_kernel(const float* part, int pieces, int64_t n, bf16* out) {
+  wait_for_predecessor();
   for (int64_t i = ((int64_t)blockIdx.x * 256 + threadIdx.x) * 4; i < n; i += (int64_t)gridDim.x * 1024) {
     float4 acc = *reinterpret_cast<const float4*>(part + i);
 #pragma unroll 4
@@ -451,6 +455,7 @@ __global__ void __launch_bounds__(256) lce_pack_kernel(const uint4* __restrict__
                                                        const uint4* __restrict__ h, uint4* __restrict__ h_out, unsigned nh,
                                                        unsigned per_row, unsigned per_row_out) {
   constexpr int U = 4;
+  wait_for_predecessor();
   for (unsigned i0 = blockIdx.x * 256 * U + threadIdx.x; i0 < nw + nh; i0 += gridDim.x * 256 * U) {
     uint4 v[U];
 #pragma unroll
@@ -510,7 +515,7 @@ Tiling choose_tiling(int M, int N, int K, int splits, int max_run, int epi_per_3
 constexpr int EPI_CLK_LSE = 350, EPI_CLK_DZ = 500, EPI_CLK_STORE = 300;   // per 32 columns, rough
 
 template <int EPI>
-cudaError_t launch_gemm(GemmArgs a, const Operand& A, const Operand& B, cudaStream_t st) {
+cudaError_t launch_gemm(GemmArgs a, const Operand& A, const Operand& B, cudaStream_t st, bool chained) {
   GemmMaps maps;
   auto encode = [&](CUtensorMap* m, const Operand& o, int extent, int box, int& layout) {
     if (!o.mn) { layout = K_MAJOR; return tc_make_map_2d(m, o.ptr, extent, a.K, o.ld, box); }
@@ -531,8 +536,7 @@ cudaError_t launch_gemm(GemmArgs a, const Operand& A, const Operand& B, cudaStre
   if (e != cudaSuccess) return e;
   const int items = a.m_tiles * a.n_runs * a.splits;
   const int grid = items < device_sm_count() ? items : device_sm_count();
-  kern<<<grid, G_THREADS, G_SMEM, st>>>(maps, a, status);
-  return cudaGetLastError();
+  return launch_chained(kern, chained, grid, G_THREADS, G_SMEM, st, 1, maps, a, status);
 }
 
 constexpr int FWD_N_RUN = 8;   // most vocabulary tiles per work item: at most 2048 logits per partial (maximum, sum) pair
@@ -668,13 +672,13 @@ int bdlm_linear_ce_fwd(const bdlm_lce_params* p, const void* h, const void* w, c
   a.part_l = reinterpret_cast<float*>(ws + (size_t)runs * per);
   a.zlab = reinterpret_cast<float*>(ws + 2 * (size_t)runs * per);
   Operand oh{h, p->D, 0, false}, ow{w, p->D, 0, false};
-  if (roomy && packs(p, PACK_FWD_T) && pack(p, ws + fwd_part_bytes(p, t), oh, ow, st) != cudaSuccess) return BDLM_ERR_CUDA;
-  if (launch_gemm<EPI_LSE>(a, oh, ow, st) != cudaSuccess) return BDLM_ERR_CUDA;
+  const bool packed = roomy && packs(p, PACK_FWD_T);
+  if (packed && pack(p, ws + fwd_part_bytes(p, t), oh, ow, st) != cudaSuccess) return BDLM_ERR_CUDA;
+  if (launch_gemm<EPI_LSE>(a, oh, ow, st, packed) != cudaSuccess) return BDLM_ERR_CUDA;
   const int blocks = (p->T + FIN_T - 1) / FIN_T;
-  lce_finish_kernel<<<blocks, 256, 0, st>>>(a.part_m, a.part_l, a.zlab, labels, token_weight, p->T, runs, a.ldp, lse, nll);
-  if (cudaGetLastError() != cudaSuccess) return BDLM_ERR_CUDA;
-  lce_sum_kernel<<<1, 256, 0, st>>>(a.part_m, blocks, FIN_T, loss);
-  return cudaGetLastError() == cudaSuccess ? BDLM_OK : BDLM_ERR_CUDA;
+  if (launch_chained(lce_finish_kernel, true, blocks, 256, 0, st, 1, a.part_m, a.part_l, a.zlab, labels, token_weight, p->T, runs, a.ldp, lse, nll) != cudaSuccess)
+    return BDLM_ERR_CUDA;
+  return launch_chained(lce_sum_kernel, true, 1, 256, 0, st, 1, a.part_m, blocks, FIN_T, loss) == cudaSuccess ? BDLM_OK : BDLM_ERR_CUDA;
 }
 
 int bdlm_linear_ce_bwd(const bdlm_lce_params* p, const void* h, const void* w, const int32_t* labels,
@@ -714,7 +718,7 @@ int bdlm_linear_ce_bwd(const bdlm_lce_params* p, const void* h, const void* w, c
     a.M = rows; a.N = V; a.K = D; a.bn = ta.bn; a.n_run = ta.n_run; a.m_inner = 1;
     a.row0 = t0; a.labels = labels; a.weight = token_weight; a.lse = lse; a.grad = p->grad_loss;
     a.dz = dz; a.ldz = (int)ldz;
-    if (launch_gemm<EPI_DZ>(a, oh_c, ow, st) != cudaSuccess) return BDLM_ERR_CUDA;
+    if (launch_gemm<EPI_DZ>(a, oh_c, ow, st, ci > 0 || plan.packed) != cudaSuccess) return BDLM_ERR_CUDA;
     // dH of the chunk = dz W   (contraction over the vocabulary; W as it lies is the MN-major B operand)
     GemmArgs b = {};
     b.M = rows; b.N = D; b.K = V; b.bn = choose_tiling(rows, D, V, splits, 1, EPI_CLK_STORE, 1).bn; b.n_run = 1; b.m_inner = 1;
@@ -722,11 +726,10 @@ int bdlm_linear_ce_bwd(const bdlm_lce_params* p, const void* h, const void* w, c
     b.c_mode = splits > 1 ? C_F32_PART : C_BF16; b.c16 = dh_c; b.c32 = pieces; b.ldc = D;
     b.k_split = ((V + BK - 1) / BK + splits - 1) / splits;
     b.splits = ((V + BK - 1) / BK + b.k_split - 1) / b.k_split;   // no empty piece
-    if (launch_gemm<EPI_STORE>(b, odz, mn(ow), st) != cudaSuccess) return BDLM_ERR_CUDA;
+    if (launch_gemm<EPI_STORE>(b, odz, mn(ow), st, true) != cudaSuccess) return BDLM_ERR_CUDA;
     if (splits > 1) {
       const int64_t n = (int64_t)rows * D, want = (n / 4 + 255) / 256, cap = (int64_t)device_sm_count() * 8;
-      lce_sum_pieces_kernel<<<(unsigned)(want < cap ? want : cap), 256, 0, st>>>(pieces, b.splits, n, dh_c);
-      if (cudaGetLastError() != cudaSuccess) return BDLM_ERR_CUDA;
+      if (launch_chained(lce_sum_pieces_kernel, true, (unsigned)(want < cap ? want : cap), 256, 0, st, 1, pieces, b.splits, n, dh_c) != cudaSuccess) return BDLM_ERR_CUDA;
     }
     // dW += dz^T H_c   (contraction over the chunk's tokens; both operands MN-major)
     GemmArgs c = {};
@@ -735,7 +738,7 @@ int bdlm_linear_ce_bwd(const bdlm_lce_params* p, const void* h, const void* w, c
     c.c_mode = chunks == 1 ? C_BF16 : (ci == 0 ? C_F32_STORE : (ci + 1 < chunks ? C_F32_ADD : C_F32_ADD_TO_BF16));
     const Operand A = mn(odz), B = mn(oh_c);
     const bool adds = c.c_mode == C_F32_ADD || c.c_mode == C_F32_ADD_TO_BF16;
-    if ((adds ? launch_gemm<EPI_ADD>(c, A, B, st) : launch_gemm<EPI_STORE>(c, A, B, st)) != cudaSuccess) return BDLM_ERR_CUDA;
+    if ((adds ? launch_gemm<EPI_ADD>(c, A, B, st, true) : launch_gemm<EPI_STORE>(c, A, B, st, true)) != cudaSuccess) return BDLM_ERR_CUDA;
   }
   return BDLM_OK;
 }

@@ -244,6 +244,7 @@ __global__ void __launch_bounds__(DKDV_THREADS, 1)
 tc_dkdv_kernel(const __grid_constant__ BwdMaps maps, const KArgs a, const TileGrid tg, int* __restrict__ status) {
   constexpr uint32_t IDESC_KM = idesc_km(D);
   constexpr int OPER_BYTES = TILE_BYTES * D / 128;   // bytes TMA delivers per operand tile (D = 64: one panel)
+  wait_for_predecessor();
   extern __shared__ __align__(1024) uint8_t sm[];
   const uint32_t base = smem_u32(sm);
   const uint32_t sK = base, sV = base + TILE_BYTES, sQ0 = base + DKDV_Q0, sdO0 = base + DKDV_DO0, sP = base + DKDV_P;
@@ -623,6 +624,7 @@ __global__ void __launch_bounds__(BWD_THREADS, 1)
 tc_dq_kernel(const __grid_constant__ BwdMaps maps, const KArgs a, const TileGrid tg, int* __restrict__ status) {
   constexpr uint32_t IDESC_KM = idesc_km(D);
   constexpr int OPER_BYTES = TILE_BYTES * D / 128;
+  wait_for_predecessor();
   extern __shared__ __align__(1024) uint8_t sm[];
   const uint32_t base = smem_u32(sm);
   const uint32_t sQ = base, sdO = base + TILE_BYTES, sK0 = base + DQ_K0, sV0 = base + DQ_V0;
@@ -934,6 +936,7 @@ __global__ void __launch_bounds__(BF_THREADS, 1)
 tc_bwdf_kernel(const __grid_constant__ BwdMaps maps, const KArgs a, const TileGrid tg, int* __restrict__ status) {
   constexpr uint32_t IDESC_KM = idesc_km(D);
   constexpr int OPER_BYTES = TILE_BYTES * D / 128, HOPER_BYTES = HT_BYTES * D / 128;   // bytes TMA delivers per 128- / 64-row tile
+  wait_for_predecessor();
   extern __shared__ __align__(1024) uint8_t sm[];
   const uint32_t base = smem_u32(sm);
   const uint32_t sK = base, sV = base + TILE_BYTES, sQ0 = base + BF_Q0, sdO0 = base + BF_DO0, sDS = base + BF_DS,
@@ -1376,6 +1379,7 @@ struct ConvertArgs {
 };
 template <int D>
 __global__ void __launch_bounds__(256) dq_convert_kernel(const ConvertArgs ca) {
+  wait_for_predecessor();
   constexpr int U = 8;
   const int s = (int)blockIdx.x < ca.blocks_clean ? CLEAN : NOISY;
   int i = blockIdx.x - (s == CLEAN ? 0 : ca.blocks_clean);
@@ -1466,22 +1470,12 @@ static int split_key_tiles(const KArgs& a, int rows) {
 // One CTA, or one cluster of tg.parts CTAs, per unit of the grid.
 template <class Kern>
 static cudaError_t launch_units(Kern kern, const TileGrid& tg, int threads, size_t smem, cudaStream_t st, const BwdMaps& maps,
-                                const KArgs& a, int* status) {
+                                const KArgs& a, int* status, bool chained) {
   const long long blocks = (long long)tile_grid_blocks(tg) * tg.parts;
   if (blocks == 0 || blocks > 0x7fffffffLL) return cudaErrorInvalidValue;
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3((unsigned)blocks);
-  cfg.blockDim = dim3(threads);
-  cfg.dynamicSmemBytes = smem;
-  cfg.stream = st;
-  cudaLaunchAttribute attr = {};
-  attr.id = cudaLaunchAttributeClusterDimension;
-  attr.val.clusterDim.x = tg.parts; attr.val.clusterDim.y = 1; attr.val.clusterDim.z = 1;
-  cfg.attrs = &attr;
-  cfg.numAttrs = tg.parts > 1 ? 1 : 0;
-  return cudaLaunchKernelEx(&cfg, kern, maps, a, tg, status);
+  return launch_chained(kern, chained, (unsigned)blocks, threads, smem, st, tg.parts, maps, a, tg, status);
 }
 
 template <int D>
@@ -1500,6 +1494,7 @@ static cudaError_t launch_tc_bwd_d(const KArgs& a, int passes, cudaStream_t st) 
   int* status = device_status_ptr();
   if (status == nullptr) return cudaErrorUnknown;
   cudaError_t e;
+  const bool after_rows = (passes & BDLM_BWD_PASS_DSUM) != 0;   // the launch that forms the D rows is this call's predecessor
   if (a.single_pass) {
     // one kernel produces dK, dV and (through fp32 add-reductions) dQ; it runs for the DKDV pass bit, the DQ bit is a no-op
     if (passes & BDLM_BWD_PASS_DKDV) {
@@ -1510,7 +1505,7 @@ static cudaError_t launch_tc_bwd_d(const KArgs& a, int passes, cudaStream_t st) 
       auto kern = a.trace ? tc_bwdf_kernel<true, D> : tc_bwdf_kernel<false, D>;
       TileGrid tg = make_tile_grid((max(a.L, a.k[NOISY] != nullptr ? a.Ln : 0) + TILE - 1) / TILE, a.Hkv, a.batch * 2);
       tg.parts = split_key_tiles(a, HT);
-      if ((e = launch_units(kern, tg, BF_THREADS, BF_SMEM, st, maps, a, status)) != cudaSuccess) return e;
+      if ((e = launch_units(kern, tg, BF_THREADS, BF_SMEM, st, maps, a, status, after_rows)) != cudaSuccess) return e;
       ConvertArgs ca = {};
       long long blocks[2];
       for (int s2 = 0; s2 < 2; ++s2) {
@@ -1520,8 +1515,7 @@ static cudaError_t launch_tc_bwd_d(const KArgs& a, int passes, cudaStream_t st) 
       }
       if (blocks[0] + blocks[1] > 0x7fffffffLL) return cudaErrorInvalidValue;
       ca.blocks_clean = (int)blocks[0]; ca.H = a.H; ca.scale = a.scale;
-      dq_convert_kernel<D><<<(unsigned)(blocks[0] + blocks[1]), 256, 0, st>>>(ca);
-      return cudaGetLastError();
+      return launch_chained(dq_convert_kernel<D>, true, (unsigned)(blocks[0] + blocks[1]), 256, 0, st, 1, ca);
     }
     return cudaSuccess;
   }
@@ -1529,15 +1523,13 @@ static cudaError_t launch_tc_bwd_d(const KArgs& a, int passes, cudaStream_t st) 
     auto kern = a.trace ? tc_dkdv_kernel<true, D> : tc_dkdv_kernel<false, D>;
     TileGrid tg = make_tile_grid((max(a.L, a.k[NOISY] != nullptr ? a.Ln : 0) + TILE - 1) / TILE, a.Hkv, a.batch * 2);
     tg.parts = split_key_tiles(a, TILE);
-    if ((e = launch_units(kern, tg, DKDV_THREADS, DKDV_SMEM, st, maps, a, status)) != cudaSuccess) return e;
+    if ((e = launch_units(kern, tg, DKDV_THREADS, DKDV_SMEM, st, maps, a, status, after_rows)) != cudaSuccess) return e;
   }
   if (passes & BDLM_BWD_PASS_DQ) {
     auto kern = a.trace ? tc_dq_kernel<true, D> : tc_dq_kernel<false, D>;
-    if ((e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, DQ_SMEM)) != cudaSuccess) return e;
     const TileGrid tg = make_tile_grid((max(a.q[CLEAN] != nullptr ? a.Lqc : 0, a.q[NOISY] != nullptr ? a.Ln : 0) + TILE - 1) / TILE, a.H, a.batch * 2);
-    if (tile_grid_blocks(tg) == 0) return cudaErrorInvalidValue;
-    kern<<<tile_grid_blocks(tg), BWD_THREADS, DQ_SMEM, st>>>(maps, a, tg, status);
-    if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    // (chained to whichever of this call's kernels came before)
+    if ((e = launch_units(kern, tg, BWD_THREADS, DQ_SMEM, st, maps, a, status, (passes & (BDLM_BWD_PASS_DSUM | BDLM_BWD_PASS_DKDV)) != 0)) != cudaSuccess) return e;
   }
   return cudaSuccess;
 }
