@@ -485,7 +485,9 @@ struct Operand { const void* ptr; int64_t ld; int mn; bool whole; };
 // part of the chip idle (T = 1531, D = 1544, V = 32008: 192 forward items on 148 SMs, dH 84 tiles, the last of every
 // seven 8 columns wide).  The width of an N tile and the length of a run are chosen for the shortest launch: rounds of
 // items per SM times the clocks of one item.  A 16-deep slice of an M = 128 MMA takes bn / 2 clk, and no less than its
-// operands need from shared memory at 128 bytes per clk.  Ties go to the longer run (fewer partial results).  A B operand
+// operands need from shared memory at 128 bytes per clk.  A
+// narrower tile or a shorter run has to promise 5 % (8192 x 4096 x 128256 would gain 3 % by this count and lost 1 %: more
+// partial results, and what bounds it is power).  A B operand
 // that lies MN-major keeps 256 columns where it has them (dH at T = 4096, D = 4096 in one piece: 5.7 ms with 240 or 192
 // columns against 3.4: its panels then start off the 128-byte lines, or a tile's rows off the 512 bytes they share).
 // Forward / dz at T = 1531, D = 1544, V = 32008: 234 -> 160 and 275 -> 188 us.
@@ -507,7 +509,7 @@ Tiling choose_tiling(int M, int N, int K, int splits, int max_run, int epi_per_3
     for (int run = max_run; run >= 1; run /= 2) {
       const long long items = m_tiles * ((n_tiles + run - 1) / run) * splits;
       const double t = (double)((items + sms - 1) / sms) * (run < n_tiles ? run : n_tiles) * tile + epi;
-      if (t < 0.99 * t_best) { t_best = t; best = {bn, run}; }
+      if (t < 0.95 * t_best) { t_best = t; best = {bn, run}; }
     }
   }
   return best;
