@@ -48,8 +48,12 @@ typedef struct {
 enum { BDLM_LCE_WS_FWD = 0, BDLM_LCE_WS_BWD = 1 };
 
 /* Scratch bytes of a call (0 for invalid parameters).  Forward: partial (maximum, sum) pairs per token and
- * vocabulary chunk.  Backward: one chunk of dz, bf16 [token_chunk, V], plus -- when T needs more than one
- * chunk -- an fp32 dW accumulator [V, D]. */
+ * vocabulary run.  Backward: one chunk of dz, bf16 [token_chunk, V], plus -- when T needs more than one
+ * chunk -- an fp32 dW accumulator [V, D].  Where the sizes call for it also: rows of dz padded to 128 bytes,
+ * partial sums of dH, copies of W and h with padded rows (D no multiple of 64).  Without those extras a call
+ * is still accepted and takes the plain path (same results up to the order of fp32 sums): forward
+ * (2 r + 1) * a(4 T) + a(4 ceil(T / 256)) bytes with r = ceil(ceil(V / 256) / 8) and a() = rounding up to 256;
+ * backward a(2 token_chunk V), plus a(4 V D) with several chunks. */
 size_t bdlm_linear_ce_workspace_bytes(const bdlm_lce_params* p, int32_t which);
 
 /*
