@@ -50,7 +50,7 @@ enum { BDLM_LCE_WS_FWD = 0, BDLM_LCE_WS_BWD = 1 };
 /* Scratch bytes of a call (0 for invalid parameters).  Forward: partial (maximum, sum) pairs per token and
  * vocabulary run.  Backward: one chunk of dz, bf16 [token_chunk, V], plus -- when T needs more than one
  * chunk -- an fp32 dW accumulator [V, D].  Where the sizes call for it also: rows of dz padded to 128 bytes,
- * partial sums of dH, copies of W and h with padded rows (D no multiple of 64).  Without those extras a call
+ * copies of W and h with padded rows (D no multiple of 64).  Without those extras a call
  * is still accepted and takes the plain path (same results up to the order of fp32 sums): forward
  * (2 r + 1) * a(4 T) + a(4 ceil(T / 256)) bytes with r = ceil(ceil(V / 256) / 8) and a() = rounding up to 256;
  * backward a(2 token_chunk V), plus a(4 V D) with several chunks. */
@@ -67,7 +67,8 @@ int bdlm_linear_ce_fwd(const bdlm_lce_params* p, const void* h, const void* w, c
 /*
  * Backward.  `lse` is the forward's.  Writes dh [T, D] bf16 and dw [V, D] bf16.  dz is rounded to bf16
  * before the two gradient GEMMs; sums over the vocabulary (dH) and over the tokens of a chunk (dW) are
- * accumulated in fp32, chunks are added in fp32 in a fixed order (bitwise reproducible).
+ * accumulated in fp32, chunks are added in fp32 in a fixed order (bitwise reproducible).  A token's dh depends on
+ * its own h, label, weight and lse only: not on the other tokens of the call, their number or the chunk size.
  */
 int bdlm_linear_ce_bwd(const bdlm_lce_params* p, const void* h, const void* w, const int32_t* labels,
                        const float* token_weight, const float* lse, void* dh, void* dw,

@@ -40,7 +40,7 @@ constexpr int G_THREADS = 192;                   // warps 0-3 epilogue, warp 4 T
 constexpr int MN_PANEL = BK * 128;               // an MN-major panel: 64 contraction rows x 64 M/N elements
 
 enum { EPI_LSE = 0, EPI_DZ = 1, EPI_STORE = 2, EPI_ADD = 3 };   // EPI_ADD: the two c_modes that read C first
-enum { C_BF16 = 0, C_F32_STORE = 1, C_F32_ADD = 2, C_F32_ADD_TO_BF16 = 3, C_F32_PART = 4 };
+enum { C_BF16 = 0, C_F32_STORE = 1, C_F32_ADD = 2, C_F32_ADD_TO_BF16 = 3 };
 
 struct GemmMaps { CUtensorMap a, b; };
 enum { K_MAJOR = 0, MN_PANELS = 1, MN_BOXES = 2 };
@@ -49,7 +49,6 @@ struct GemmArgs {
   int M, N, K;
   int bn;                                // width of an N tile: a multiple of 16, at most BN
   int m_tiles, n_tiles, n_run, n_runs;   // an item = one M tile x n_run consecutive N tiles; n_runs = ceil(n_tiles / n_run)
-  int splits, k_split;                   // the contraction in `splits` pieces of k_split steps, each an item of its own
   int m_inner;                           // item order: 1 = consecutive items share the N run, 0 = share the M tile
   int a_mn, b_mn;                        // operand layouts: K_MAJOR, MN_PANELS (one load per tile), MN_BOXES (one per 64-column panel)
   // EPI_LSE / EPI_DZ: rows are tokens row0 .. row0 + M - 1
@@ -65,7 +64,7 @@ struct GemmArgs {
   bf16* dz;        // EPI_DZ: [M, N] row-major, ld = ldz
   int ldz;
   // EPI_STORE
-  int c_mode;      // C_F32_PART: piece s of the contraction goes to c32 + s * M * ldc
+  int c_mode;
   bf16* c16; float* c32; int ldc;
 };
 
@@ -85,27 +84,21 @@ __device__ __forceinline__ void tma_load_panels_e(uint32_t dst, const CUtensorMa
 
 // Walks the CTA's tiles in the order every role uses.
 struct TileWalk {
-  int item, items, mt, nrun, nt, nt_end, split;
+  int item, items, mt, nrun, nt, nt_end;
   const GemmArgs* a;
   __device__ __forceinline__ void start(const GemmArgs& args) {
-    a = &args; items = args.m_tiles * args.n_runs * args.splits; item = blockIdx.x; nt = 0; nt_end = 0; split = 0;
+    a = &args; items = args.m_tiles * args.n_runs; item = blockIdx.x; nt = 0; nt_end = 0;
     if (item < items) open();
   }
   __device__ __forceinline__ void open() {
-    int i = item;
-    const int per = a->m_tiles * a->n_runs;
-    split = 0;
-    if (a->splits > 1) { split = i / per; i -= split * per; }
-    if (a->m_inner) { nrun = i / a->m_tiles; mt = i - nrun * a->m_tiles; }
-    else { mt = i / a->n_runs; nrun = i - mt * a->n_runs; }
+    if (a->m_inner) { nrun = item / a->m_tiles; mt = item - nrun * a->m_tiles; }
+    else { mt = item / a->n_runs; nrun = item - mt * a->n_runs; }
     nt = nrun * a->n_run;
     nt_end = min(a->n_tiles, nt + a->n_run);
   }
   __device__ __forceinline__ bool valid() const { return item < items; }
   __device__ __forceinline__ bool first_of_item() const { return nt == nrun * a->n_run; }
   __device__ __forceinline__ bool last_of_item() const { return nt + 1 == nt_end; }
-  __device__ __forceinline__ int k_begin() const { return split * a->k_split; }   // 64-deep steps of the contraction
-  __device__ __forceinline__ int k_end(int nk) const { return min(nk, (split + 1) * a->k_split); }
   __device__ __forceinline__ void next() {
     if (++nt < nt_end) return;
     item += gridDim.x;
@@ -151,8 +144,8 @@ lce_gemm_kernel(const __grid_constant__ GemmMaps maps, const GemmArgs a, int* __
     bool ok = true;
     const int stage_bytes = A_BYTES + (a.b_mn != K_MAJOR ? B_BYTES : a.bn * BK * 2);   // (MN-major: always all four panels, zeros past the end)
     for (; w.valid() && ok; w.next()) {
-      const int m0 = w.mt * BM, n0 = w.nt * a.bn, k1 = w.k_end(nk);
-      for (int k = w.k_begin(); k < k1; ++k, ++ks) {
+      const int m0 = w.mt * BM, n0 = w.nt * a.bn;
+      for (int k = 0; k < nk; ++k, ++ks) {
         const int s = ks % STAGES;
         if (ks >= STAGES) ok = mbar_wait_lean(bar_empty + 8 * s, ((ks / STAGES) - 1) & 1, abort_flag);
         if (!ok) break;
@@ -193,8 +186,7 @@ lce_gemm_kernel(const __grid_constant__ GemmMaps maps, const GemmArgs a, int* __
         tc_fence_after();
       }
       const uint32_t d = tmem + buf * BN;
-      const int k0 = w.k_begin(), k1 = w.k_end(nk);
-      for (int k = k0; k < k1; ++k, ++ks) {
+      for (int k = 0; k < nk; ++k, ++ks) {
         const int s = ks % STAGES;
         ok = mbar_wait_lean(bar_full + 8 * s, (ks / STAGES) & 1, abort_flag);
         if (!ok) break;
@@ -202,7 +194,7 @@ lce_gemm_kernel(const __grid_constant__ GemmMaps maps, const GemmArgs a, int* __
         const uint32_t a_lo = a_lo0 + s * (STAGE_BYTES >> 4), b_lo = b_lo0 + s * (STAGE_BYTES >> 4);
 #pragma unroll
         for (int kk = 0; kk < BK / 16; ++kk)
-          mma_ss_e(d, desc64(a_lo + kk * a_step), desc64(b_lo + kk * b_step), idesc, (k > k0 || kk > 0) ? 1u : 0u, el);
+          mma_ss_e(d, desc64(a_lo + kk * a_step), desc64(b_lo + kk * b_step), idesc, (k > 0 || kk > 0) ? 1u : 0u, el);
         mma_commit_e(bar_empty + 8 * s, el);
       }
       if (!ok) break;
@@ -344,7 +336,7 @@ lce_gemm_kernel(const __grid_constant__ GemmMaps maps, const GemmArgs a, int* __
             }
           }
         } else if (EPI == EPI_STORE && cvalid > 0 && row_ok) {
-          const int64_t off = ((int64_t)w.split * a.M + row) * a.ldc + col0;
+          const int64_t off = (int64_t)row * a.ldc + col0;
 #pragma unroll
           for (int e8 = 0; e8 < 4; ++e8) {
             if (e8 * 8 >= cvalid) break;
@@ -435,20 +427,6 @@ __global__ void __launch_bounds__(256) lce_sum_kernel(const float* block_sums, i
   if (threadIdx.x == 0) *loss = red[0];
 }
 
-// Sum of the pieces of a split contraction, in their order, as bf16.  n = elements per piece (a multiple of 8).
-__global__ void __launch_bounds__(256) lce_sum_pieces_kernel(const float* part, int pieces, int64_t n, bf16* out) {
-  wait_for_predecessor();
-  for (int64_t i = ((int64_t)blockIdx.x * 256 + threadIdx.x) * 4; i < n; i += (int64_t)gridDim.x * 1024) {
-    float4 acc = *reinterpret_cast<const float4*>(part + i);
-#pragma unroll 4
-    for (int p = 1; p < pieces; ++p) {
-      const float4 u = *reinterpret_cast<const float4*>(part + p * n + i);
-      acc.x += u.x; acc.y += u.y; acc.z += u.z; acc.w += u.w;
-    }
-    *reinterpret_cast<uint2*>(out + i) = make_uint2(pack_bf16(acc.x, acc.y), pack_bf16(acc.z, acc.w));
-  }
-}
-
 // Copies W [V, D] and the tokens' h [T, D] to rows of `ld` elements (a whole number of 128-byte lines), 16 bytes per thread and
 // turn; what lies past a row's D elements is never looked at.
 __global__ void __launch_bounds__(256) lce_pack_kernel(const uint4* __restrict__ w, uint4* __restrict__ w_out, unsigned nw,
@@ -492,9 +470,9 @@ struct Operand { const void* ptr; int64_t ld; int mn; bool whole; };
 // columns against 3.4: its panels then start off the 128-byte lines, or a tile's rows off the 512 bytes they share).
 // Forward / dz at T = 1531, D = 1544, V = 32008: 234 -> 160 and 275 -> 188 us.
 struct Tiling { int bn, n_run; };
-Tiling choose_tiling(int M, int N, int K, int splits, int max_run, int epi_per_32, int b_mn) {
+Tiling choose_tiling(int M, int N, int K, int max_run, int epi_per_32, int b_mn) {
   const long long m_tiles = (M + BM - 1) / BM, sms = device_sm_count();
-  const int nk = ((K + BK - 1) / BK + splits - 1) / splits;
+  const int nk = (K + BK - 1) / BK;
   Tiling best = {BN, max_run};
   double t_best = 1e300;
   const int unit = b_mn ? 128 : 16;
@@ -507,7 +485,7 @@ Tiling choose_tiling(int M, int N, int K, int splits, int max_run, int epi_per_3
     const double mma = nk * (BK / 16) * slice;
     const double tile = mma > epi ? mma : epi;
     for (int run = max_run; run >= 1; run /= 2) {
-      const long long items = m_tiles * ((n_tiles + run - 1) / run) * splits;
+      const long long items = m_tiles * ((n_tiles + run - 1) / run);
       const double t = (double)((items + sms - 1) / sms) * (run < n_tiles ? run : n_tiles) * tile + epi;
       if (t < 0.95 * t_best) { t_best = t; best = {bn, run}; }
     }
@@ -530,13 +508,12 @@ cudaError_t launch_gemm(GemmArgs a, const Operand& A, const Operand& B, cudaStre
   a.m_tiles = (a.M + BM - 1) / BM;
   a.n_tiles = (a.N + a.bn - 1) / a.bn;
   a.n_runs = (a.n_tiles + a.n_run - 1) / a.n_run;
-  if (a.splits <= 1) { a.splits = 1; a.k_split = (a.K + BK - 1) / BK; }
   int* status = device_status_ptr();
   if (status == nullptr) return cudaErrorUnknown;
   auto kern = lce_gemm_kernel<EPI>;
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, G_SMEM);
   if (e != cudaSuccess) return e;
-  const int items = a.m_tiles * a.n_runs * a.splits;
+  const int items = a.m_tiles * a.n_runs;
   const int grid = items < device_sm_count() ? items : device_sm_count();
   return launch_chained(kern, chained, grid, G_THREADS, G_SMEM, st, 1, maps, a, status);
 }
@@ -571,7 +548,7 @@ cudaError_t pack(const bdlm_lce_params* p, char* at, Operand& h, Operand& w, cud
   return cudaGetLastError();
 }
 size_t fwd_bytes(const bdlm_lce_params* p, const Tiling& t) { return fwd_part_bytes(p, t) + (packs(p, PACK_FWD_T) ? pack_bytes(p) : 0); }
-Tiling fwd_tiling(const bdlm_lce_params* p) { return choose_tiling(p->T, p->V, p->D, 1, FWD_N_RUN, EPI_CLK_LSE, 0); }
+Tiling fwd_tiling(const bdlm_lce_params* p) { return choose_tiling(p->T, p->V, p->D, FWD_N_RUN, EPI_CLK_LSE, 0); }
 // the smallest workspace that is accepted (with room for loss sums that now lie elsewhere: the size is an old promise)
 size_t fwd_bytes_min(const bdlm_lce_params* p) {
   const size_t per = align256((size_t)p->T * sizeof(float));
@@ -582,35 +559,20 @@ int default_chunk(const bdlm_lce_params* p) {
   const int up = (p->T + 127) / 128 * 128;
   return up < 4096 ? up : 4096;
 }
-// dH = dz W has few output tiles (rows x D) and a contraction as deep as the vocabulary: where the tiles do not fill the
-// chip it is cut into pieces that are summed by lce_sum_pieces_kernel.  The cut depends on T, V and D, not on the token
-// chunks, so that a token's dH does not depend on how the tokens are chunked.  Pieces of 16 steps (1024 vocabulary
-// entries) at least; none from two tiles per SM on (T = 8192, D = 4096, 512 tiles: 3.43 ms in one piece, 3.74 in two).
-int dh_splits(int T, int V, int D) {
-  const long long sms = device_sm_count(), rows = T < 4096 ? T : 4096;
-  const long long tiles = ((rows + BM - 1) / BM) * ((D + BN - 1) / BN), nk = (V + BK - 1) / BK;
-  if (tiles >= 2 * sms) return 1;
-  int best = 1;
-  double t_best = 1e300;
-  for (int s = 1; s <= 16 && nk / s >= 16; ++s) {
-    // rounds of items, then each piece written and read again (about 2.5 KB per clk over the chip)
-    const double t = (double)((tiles * s + sms - 1) / sms) * ((nk + s - 1) / s) * 512 + (s > 1 ? 4000 + 8.0 * s * rows * D / 2500 : 0);
-    if (t < 0.98 * t_best) { t_best = t; best = s; }
-  }
-  return best;
-}
-// The backward's workspace: dz of a chunk, the fp32 dW with several chunks, the pieces of dH, the copies of W and h.  The
-// smallest that is accepted has the first two only, dz with rows of V elements.
-struct BwdPlan { int64_t ldz; int splits; bool packed; size_t dw32, pieces, copies, bytes; };
+// The backward's workspace: dz of a chunk, the fp32 dW with several chunks, the copies of W and h.  The smallest that is
+// accepted has the first two only, dz with rows of V elements.
+// dH = dz W is one accumulation per element over the whole vocabulary, whatever the tile or the number of tokens, so that a
+// token's dH is the same bit for bit in every call it is part of.  (Cut into pieces where its tiles do not fill the chip --
+// T = 1531, D = 1544, V = 32008: 84 tiles -- forward and backward together took 674 us instead of 690, but a token's dH then
+// depended on how many others there were: 3.5e-4 of its norm.)
+struct BwdPlan { int64_t ldz; bool packed; size_t dw32, copies, bytes; };
 BwdPlan bwd_plan(const bdlm_lce_params* p, bool least) {
-  const int tc_ = default_chunk(p), chunks = (p->T + tc_ - 1) / tc_, rows = tc_ < p->T ? tc_ : p->T;
+  const int tc_ = default_chunk(p), chunks = (p->T + tc_ - 1) / tc_;
   BwdPlan b;
   b.ldz = least ? p->V : up64(p->V);
-  b.splits = least ? 1 : dh_splits(p->T, p->V, p->D);
   b.packed = !least && packs(p, PACK_BWD_T);
   b.dw32 = align256((size_t)tc_ * b.ldz * 2);
-  b.pieces = b.dw32 + (chunks > 1 ? align256((size_t)p->V * p->D * sizeof(float)) : 0);
-  b.copies = b.pieces + (b.splits > 1 ? align256((size_t)b.splits * rows * p->D * sizeof(float)) : 0);
+  b.copies = b.dw32 + (chunks > 1 ? align256((size_t)p->V * p->D * sizeof(float)) : 0);
   b.bytes = b.copies + (b.packed ? pack_bytes(p) : 0);
   return b;
 }
@@ -704,8 +666,7 @@ int bdlm_linear_ce_bwd(const bdlm_lce_params* p, const void* h, const void* w, c
   char* ws = static_cast<char*>(workspace);
   bf16* dz = static_cast<bf16*>(workspace);
   const int64_t ldz = plan.ldz;
-  const int splits = plan.splits;
-  float *dw32 = reinterpret_cast<float*>(ws + plan.dw32), *pieces = reinterpret_cast<float*>(ws + plan.pieces);
+  float* dw32 = reinterpret_cast<float*>(ws + plan.dw32);
   Operand oh{h, D, 0, false}, ow{w, D, 0, false};
   if (plan.packed && pack(p, ws + plan.copies, oh, ow, st) != cudaSuccess) return BDLM_ERR_CUDA;
   auto mn = [](Operand o) { o.mn = 1; return o; };
@@ -716,26 +677,19 @@ int bdlm_linear_ce_bwd(const bdlm_lce_params* p, const void* h, const void* w, c
     const Operand odz{dz, ldz, 0, roomy};
     // dz of the chunk: logits again, softmax minus one-hot in the epilogue
     GemmArgs a = {};
-    const Tiling ta = choose_tiling(rows, V, D, 1, FWD_N_RUN, EPI_CLK_DZ, 0);
+    const Tiling ta = choose_tiling(rows, V, D, FWD_N_RUN, EPI_CLK_DZ, 0);
     a.M = rows; a.N = V; a.K = D; a.bn = ta.bn; a.n_run = ta.n_run; a.m_inner = 1;
     a.row0 = t0; a.labels = labels; a.weight = token_weight; a.lse = lse; a.grad = p->grad_loss;
     a.dz = dz; a.ldz = (int)ldz;
     if (launch_gemm<EPI_DZ>(a, oh_c, ow, st, ci > 0 || plan.packed) != cudaSuccess) return BDLM_ERR_CUDA;
     // dH of the chunk = dz W   (contraction over the vocabulary; W as it lies is the MN-major B operand)
     GemmArgs b = {};
-    b.M = rows; b.N = D; b.K = V; b.bn = choose_tiling(rows, D, V, splits, 1, EPI_CLK_STORE, 1).bn; b.n_run = 1; b.m_inner = 1;
-    bf16* dh_c = static_cast<bf16*>(dh) + (size_t)t0 * D;
-    b.c_mode = splits > 1 ? C_F32_PART : C_BF16; b.c16 = dh_c; b.c32 = pieces; b.ldc = D;
-    b.k_split = ((V + BK - 1) / BK + splits - 1) / splits;
-    b.splits = ((V + BK - 1) / BK + b.k_split - 1) / b.k_split;   // no empty piece
+    b.M = rows; b.N = D; b.K = V; b.bn = choose_tiling(rows, D, V, 1, EPI_CLK_STORE, 1).bn; b.n_run = 1; b.m_inner = 1;
+    b.c_mode = C_BF16; b.c16 = static_cast<bf16*>(dh) + (size_t)t0 * D; b.ldc = D;
     if (launch_gemm<EPI_STORE>(b, odz, mn(ow), st, true) != cudaSuccess) return BDLM_ERR_CUDA;
-    if (splits > 1) {
-      const int64_t n = (int64_t)rows * D, want = (n / 4 + 255) / 256, cap = (int64_t)device_sm_count() * 8;
-      if (launch_chained(lce_sum_pieces_kernel, true, (unsigned)(want < cap ? want : cap), 256, 0, st, 1, pieces, b.splits, n, dh_c) != cudaSuccess) return BDLM_ERR_CUDA;
-    }
     // dW += dz^T H_c   (contraction over the chunk's tokens; both operands MN-major)
     GemmArgs c = {};
-    c.M = V; c.N = D; c.K = rows; c.bn = choose_tiling(V, D, rows, 1, 1, EPI_CLK_STORE, 1).bn; c.n_run = 1; c.m_inner = 0;
+    c.M = V; c.N = D; c.K = rows; c.bn = choose_tiling(V, D, rows, 1, EPI_CLK_STORE, 1).bn; c.n_run = 1; c.m_inner = 0;
     c.c16 = static_cast<bf16*>(dw); c.c32 = dw32; c.ldc = D;
     c.c_mode = chunks == 1 ? C_BF16 : (ci == 0 ? C_F32_STORE : (ci + 1 < chunks ? C_F32_ADD : C_F32_ADD_TO_BF16));
     const Operand A = mn(odz), B = mn(oh_c);

@@ -162,3 +162,16 @@ def test_rows_that_are_no_whole_number_of_lines(w):
     one = _check(w)
     several = _check(w, token_chunk=256)
     assert torch.equal(one[3], several[3])
+
+
+@pytest.mark.parametrize("D", [264, 256], ids=["copied_rows", "whole_rows"])
+def test_dh_of_a_token_does_not_depend_on_the_other_tokens(D):
+    """The same tokens by themselves and among many: every bit of their dH (one accumulation over the vocabulary)."""
+    g = {k: v.cuda() for k, v in synth.make_lce_inputs(LceWorkload("among_others", 1531, D, 9000), "cpu").items()}
+    _, _, lse = binding.bdlm_linear_ce_fwd(g["h"], g["w"], g["labels"], g["weight"])
+    dh, _ = binding.bdlm_linear_ce_bwd(g["h"], g["w"], g["labels"], lse, g["weight"])
+    for n in (1, 130, 700):
+        few = [g[k][:n].contiguous() for k in ("h", "labels", "weight")]
+        dh_n, _ = binding.bdlm_linear_ce_bwd(few[0], g["w"], few[1], lse[:n].contiguous(), few[2])
+        torch.cuda.synchronize()
+        assert torch.equal(dh_n, dh[:n]), n
