@@ -371,8 +371,9 @@ lce_gemm_kernel(const __grid_constant__ GemmMaps maps, const GemmArgs a, int* __
 // Combines the per-run partial (maximum, sum) pairs of every token (Eq. csbp-lse-merge's rule, in log2 units),
 // writes lse and nll, and leaves one weighted partial sum of the loss per block (fixed order: reproducible).
 // A block takes FIN_T tokens, eight threads share a token's runs (one thread per token left a few blocks alone with a
-// hundred dependent rounds of loads when the runs are short).  The block's sum replaces its own first token's first
-// partial maximum, which nobody else reads.
+// hundred dependent rounds of loads when the runs are short).  A maximum of -inf is left by no run at all (sum 0) and by a run
+// of NaN (sum NaN; maxima pass NaN over): both go into the sum with weight 0, so NaN stays.  The block's sum replaces its own
+// first token's first partial maximum, which nobody else reads.
 constexpr int FIN_T = 32;
 __global__ void __launch_bounds__(256) lce_finish_kernel(float* part_m, const float* part_l,
                                                          const float* zlab, const int* __restrict__ labels,
@@ -386,10 +387,9 @@ __global__ void __launch_bounds__(256) lce_finish_kernel(float* part_m, const fl
   if (t < T) {
 #pragma unroll 8
     for (int c = y0; c < n_runs; c += 8) m = fmaxf(m, part_m[(int64_t)c * ldp + t]);
-    if (m != -INFINITY) {
+    const float mb = m == -INFINITY ? 0.f : m;
 #pragma unroll 8
-      for (int c = y0; c < n_runs; c += 8) l += part_l[(int64_t)c * ldp + t] * exp2f(part_m[(int64_t)c * ldp + t] - m);
-    }
+    for (int c = y0; c < n_runs; c += 8) l += part_l[(int64_t)c * ldp + t] * exp2f(part_m[(int64_t)c * ldp + t] - mb);
   }
   sm_m[y0][x] = m; sm_l[y0][x] = l;
   __syncthreads();
@@ -399,8 +399,9 @@ __global__ void __launch_bounds__(256) lce_finish_kernel(float* part_m, const fl
     m = -INFINITY; l = 0.f;
 #pragma unroll
     for (int j = 0; j < 8; ++j) m = fmaxf(m, sm_m[j][x]);
+    const float mb = m == -INFINITY ? 0.f : m;
 #pragma unroll
-    for (int j = 0; j < 8; ++j) if (sm_m[j][x] != -INFINITY) l += sm_l[j][x] * exp2f(sm_m[j][x] - m);
+    for (int j = 0; j < 8; ++j) l += sm_l[j][x] * exp2f(sm_m[j][x] - mb);
     const float z = (m + log2f(l)) * LN2;
     const int y = labels[t];
     const float n = y >= 0 ? z - zlab[t] : 0.f;

@@ -175,3 +175,32 @@ def test_dh_of_a_token_does_not_depend_on_the_other_tokens(D):
         dh_n, _ = binding.bdlm_linear_ce_bwd(few[0], g["w"], few[1], lse[:n].contiguous(), few[2])
         torch.cuda.synchronize()
         assert torch.equal(dh_n, dh[:n]), n
+
+
+@pytest.mark.parametrize("V,least", [(512, False), (2048, False), (16384, True), (20008, True), (20008, False)])
+def test_nan_in_the_vocabulary_and_in_a_token_reaches_the_results(V, least):
+    T = 140
+    g = {k: v.cuda() for k, v in synth.make_lce_inputs(LceWorkload("nan", T, 64, V), "cpu").items()}
+    per, runs = (T * 4 + 255) // 256 * 256, (((V + 255) // 256) + 7) // 8
+    ws = torch.empty((2 * runs + 1) * per + 256, dtype=torch.uint8, device="cuda") if least else None
+    clean = [t.clone() for t in binding.bdlm_linear_ce_fwd(g["h"], g["w"], g["labels"], g["weight"], workspace=ws)]
+    # a token whose hidden state is NaN: its lse and the loss, and nobody else's lse
+    bad = 77
+    h = g["h"].clone()
+    h[bad] = float("nan")
+    labels = g["labels"].clone()
+    labels[bad] = 1
+    loss, nll, lse = binding.bdlm_linear_ce_fwd(h, g["w"], labels, g["weight"], workspace=ws)
+    assert bool(lse[bad].isnan()) and bool(nll[bad].isnan()) and bool(loss.isnan().all())
+    rest = torch.arange(T, device="cuda") != bad
+    assert torch.equal(lse[rest], clean[2][rest])
+    # a stretch of the vocabulary as long as the longest run: every token's lse, wherever its label lies
+    n = min(2048, V // 2)
+    for first in (0, V // n * n // 2 // n * n, V - n):
+        w = g["w"].clone()
+        w[first:first + n] = float("nan")
+        away = torch.full_like(labels, (first + n) % V if first + n < V else 0)
+        loss, nll, lse = binding.bdlm_linear_ce_fwd(g["h"], w, away, g["weight"], workspace=ws)
+        assert bool(lse.isnan().all()) and bool(nll.isnan().all()) and bool(loss.isnan().all()), first
+    torch.cuda.synchronize()
+    assert binding.bdlm_get_device_status() == 0
