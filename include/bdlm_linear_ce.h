@@ -51,14 +51,16 @@ enum { BDLM_LCE_WS_FWD = 0, BDLM_LCE_WS_BWD = 1 };
  * vocabulary run.  Backward: one chunk of dz, bf16 [token_chunk, V], plus -- when T needs more than one
  * chunk -- an fp32 dW accumulator [V, D].  Where the sizes call for it also: rows of dz padded to 128 bytes,
  * copies of W and h with padded rows (D no multiple of 64).  Without those extras a call
- * is still accepted and takes the plain path (same results up to the order of fp32 sums): forward
- * (2 r + 1) * a(4 T) + a(4 ceil(T / 256)) bytes with r = ceil(ceil(V / 256) / 8) and a() = rounding up to 256;
- * backward a(2 token_chunk V), plus a(4 V D) with several chunks. */
+ * is still accepted and takes the plain path (the forward's results are then the same up to the order of fp32
+ * sums: its vocabulary runs are eight times as long): forward (2 r + 1) * a(4 T) + a(4 ceil(T / 256)) bytes with
+ * r = ceil(ceil(V / 256) / 8) and a() = rounding up to 256; backward a(2 token_chunk V), plus a(4 V D) with
+ * several chunks. */
 size_t bdlm_linear_ce_workspace_bytes(const bdlm_lce_params* p, int32_t which);
 
 /*
  * Forward.  Writes lse [T] (natural log), nll [T] (may be NULL) and the scalar loss (one float in device
- * memory; summed in a fixed order, so bitwise reproducible).
+ * memory; summed in a fixed order, so bitwise reproducible).  A token's lse and nll do not depend on the other tokens
+ * of the call or on their number.
  */
 int bdlm_linear_ce_fwd(const bdlm_lce_params* p, const void* h, const void* w, const int32_t* labels,
                        const float* token_weight, float* loss, float* nll, float* lse,

@@ -57,7 +57,8 @@ struct GemmArgs {
   const float* weight;
   const float* lse;
   float grad;
-  float* part_m;   // [n_runs, ldp] running maxima (log2 units) per vocabulary run
+  int run_tiles;   // N tiles per vocabulary run (a divisor of n_run)
+  float* part_m;   // [vocabulary runs, ldp] running maxima (log2 units) per run
   float* part_l;   // [n_runs, ldp] sums of exponentials relative to that maximum
   float* zlab;     // [ldp] logit of the target
   int ldp;
@@ -97,8 +98,6 @@ struct TileWalk {
     nt_end = min(a->n_tiles, nt + a->n_run);
   }
   __device__ __forceinline__ bool valid() const { return item < items; }
-  __device__ __forceinline__ bool first_of_item() const { return nt == nrun * a->n_run; }
-  __device__ __forceinline__ bool last_of_item() const { return nt + 1 == nt_end; }
   __device__ __forceinline__ void next() {
     if (++nt < nt_end) return;
     item += gridDim.x;
@@ -208,7 +207,7 @@ lce_gemm_kernel(const __grid_constant__ GemmMaps maps, const GemmArgs a, int* __
     w.start(a);
     int tcnt = 0;
     bool ok = true;
-    // per-item row state of the forward
+    // row state of the forward over a vocabulary run
     float run_m = -INFINITY, run_l = 0.f;
     for (; w.valid() && ok; w.next(), ++tcnt) {
       const int buf = tcnt & 1;
@@ -226,7 +225,7 @@ lce_gemm_kernel(const __grid_constant__ GemmMaps maps, const GemmArgs a, int* __
           lse2 = a.lse[a.row0 + row] * LOG2E;
         }
       }
-      if (EPI == EPI_LSE && w.first_of_item()) { run_m = -INFINITY; run_l = 0.f; }
+      if (EPI == EPI_LSE && w.nt % a.run_tiles == 0) { run_m = -INFINITY; run_l = 0.f; }
       if (EPI == EPI_ADD) {
         // The fp32 sums of the earlier token chunks are requested two 32-column chunks ahead, the first ones before the
         // wait for the accumulator: requested where they are used, their round trips to memory took longer than the
@@ -300,7 +299,8 @@ lce_gemm_kernel(const __grid_constant__ GemmMaps maps, const GemmArgs a, int* __
           for (int e = 0; e < 32; ++e) mx = fmaxf(mx, __uint_as_float(x[e]));
           mx *= LOG2E;
           if (mx > run_m) { run_l *= exp2f(run_m - mx); run_m = mx; }
-          const uint64_t c2 = pack_f32x2(LOG2E, LOG2E), m2 = pack_f32x2(-run_m, -run_m);
+          const float mb = run_m == -INFINITY ? 0.f : run_m;   // (nothing but -inf so far: the sum is 0, not NaN)
+          const uint64_t c2 = pack_f32x2(LOG2E, LOG2E), m2 = pack_f32x2(-mb, -mb);
           uint64_t s2 = 0;
 #pragma unroll
           for (int e = 0; e < 32; e += 2) {
@@ -356,9 +356,10 @@ lce_gemm_kernel(const __grid_constant__ GemmMaps maps, const GemmArgs a, int* __
       }
       tc_fence_before();
       mbar_arrive(bar_acc_empty + 8 * buf);
-      if (EPI == EPI_LSE && w.last_of_item() && row_ok) {
-        a.part_m[(int64_t)w.nrun * a.ldp + a.row0 + row] = run_m;
-        a.part_l[(int64_t)w.nrun * a.ldp + a.row0 + row] = run_l;
+      if (EPI == EPI_LSE && ((w.nt + 1) % a.run_tiles == 0 || w.nt + 1 == a.n_tiles) && row_ok) {
+        const int64_t at = (int64_t)(w.nt / a.run_tiles) * a.ldp + a.row0 + row;
+        a.part_m[at] = run_m;
+        a.part_l[at] = run_l;
       }
     }
   }
@@ -465,19 +466,19 @@ struct Operand { const void* ptr; int64_t ld; int mn; bool whole; };
 // seven 8 columns wide).  The width of an N tile and the length of a run are chosen for the shortest launch: rounds of
 // items per SM times the clocks of one item.  A 16-deep slice of an M = 128 MMA takes bn / 2 clk, and no less than its
 // operands need from shared memory at 128 bytes per clk.  A
-// narrower tile or a shorter run has to promise 5 % (8192 x 4096 x 128256 would gain 3 % by this count and lost 1 %: more
-// partial results, and what bounds it is power).  A B operand
+// narrower tile or a shorter run has to promise 5 % (8192 x 4096 x 128256 would gain 3 % by this count and lost 1 %: what
+// bounds it is power).  The forward keeps 256 columns, where its runs end (see RUN_TILES).  A B operand
 // that lies MN-major keeps 256 columns where it has them (dH at T = 4096, D = 4096 in one piece: 5.7 ms with 240 or 192
 // columns against 3.4: its panels then start off the 128-byte lines, or a tile's rows off the 512 bytes they share).
 // Forward / dz at T = 1531, D = 1544, V = 32008: 234 -> 160 and 275 -> 188 us.
 struct Tiling { int bn, n_run; };
-Tiling choose_tiling(int M, int N, int K, int max_run, int epi_per_32, int b_mn) {
+Tiling choose_tiling(int M, int N, int K, int min_bn, int min_run, int max_run, int epi_per_32, int b_mn) {
   const long long m_tiles = (M + BM - 1) / BM, sms = device_sm_count();
   const int nk = (K + BK - 1) / BK;
   Tiling best = {BN, max_run};
   double t_best = 1e300;
   const int unit = b_mn ? 128 : 16;
-  for (int bn = BN; bn >= 128; bn -= unit) {
+  for (int bn = BN; bn >= min_bn; bn -= unit) {
     if (bn > 128 && bn - unit >= N) continue;              // a whole unit wider than the matrix
     if (b_mn && bn < BN && N > bn) break;
     const long long n_tiles = (N + bn - 1) / bn;
@@ -485,7 +486,7 @@ Tiling choose_tiling(int M, int N, int K, int max_run, int epi_per_32, int b_mn)
     const double epi = (double)epi_per_32 * ((bn + 31) / 32);
     const double mma = nk * (BK / 16) * slice;
     const double tile = mma > epi ? mma : epi;
-    for (int run = max_run; run >= 1; run /= 2) {
+    for (int run = max_run; run >= min_run; run /= 2) {
       const long long items = m_tiles * ((n_tiles + run - 1) / run);
       const double t = (double)((items + sms - 1) / sms) * (run < n_tiles ? run : n_tiles) * tile + epi;
       if (t < 0.95 * t_best) { t_best = t; best = {bn, run}; }
@@ -519,14 +520,21 @@ cudaError_t launch_gemm(GemmArgs a, const Operand& A, const Operand& B, cudaStre
   return launch_chained(kern, chained, grid, G_THREADS, G_SMEM, st, 1, maps, a, status);
 }
 
-constexpr int FWD_N_RUN = 8;   // most vocabulary tiles per work item: at most 2048 logits per partial (maximum, sum) pair
-constexpr Tiling FWD_COARSE = {BN, FWD_N_RUN};   // the fewest partial results: what the smallest accepted workspace holds
+constexpr int MAX_RUN = 8;   // most N tiles per work item of the forward and of dz
 
-int fwd_runs(int V, const Tiling& t) { const int nt = (V + t.bn - 1) / t.bn; return (nt + t.n_run - 1) / t.n_run; }
+// The forward's sums of exponentials: one running (maximum, sum) pair per token and vocabulary run, then the runs' pairs
+// together (lce_finish_kernel).  Where a run ends depends on nothing but the workspace, so that a token's lse is the same bit
+// for bit whatever other tokens are in the call; how many runs go into a work item is for the tiling to choose.  A run of one
+// tile leaves that choice free (T = 1531, D = 1544, V = 32008: forward 196 us, with 2048 logits a run 237; T = 149, D = 224,
+// V = 50912: 30 and 39) and costs 8 bytes written and read per token and 256 logits, which does not show (8192 x 4096 x
+// 128256: 6.35 and 6.42 ms, inside the noise).  The smallest workspace that is accepted holds the pairs of runs of eight tiles.
+constexpr int RUN_TILES = 1, RUN_TILES_LEAST = 8;
+
+int fwd_runs(int V, int run_tiles) { return ((V + BN - 1) / BN + run_tiles - 1) / run_tiles; }
 size_t align256(size_t x) { return (x + 255) / 256 * 256; }
-size_t fwd_part_bytes(const bdlm_lce_params* p, const Tiling& t) {
+size_t fwd_part_bytes(const bdlm_lce_params* p, int run_tiles) {
   const size_t per = align256((size_t)p->T * sizeof(float));
-  return (2 * (size_t)fwd_runs(p->V, t) + 1) * per;
+  return (2 * (size_t)fwd_runs(p->V, run_tiles) + 1) * per;
 }
 // Matrices whose rows are no whole number of 128-byte lines: every 128-byte row of a TMA box then straddles two lines,
 // and the products, which live on L2 bandwidth, take half as long again or more (T = 1531, V ~ 32000: D = 1536 against
@@ -548,12 +556,10 @@ cudaError_t pack(const bdlm_lce_params* p, char* at, Operand& h, Operand& w, cud
   h = Operand{h_out, up64(p->D), 0, true};
   return cudaGetLastError();
 }
-size_t fwd_bytes(const bdlm_lce_params* p, const Tiling& t) { return fwd_part_bytes(p, t) + (packs(p, PACK_FWD_T) ? pack_bytes(p) : 0); }
-Tiling fwd_tiling(const bdlm_lce_params* p) { return choose_tiling(p->T, p->V, p->D, FWD_N_RUN, EPI_CLK_LSE, 0); }
+size_t fwd_bytes(const bdlm_lce_params* p) { return fwd_part_bytes(p, RUN_TILES) + (packs(p, PACK_FWD_T) ? pack_bytes(p) : 0); }
 // the smallest workspace that is accepted (with room for loss sums that now lie elsewhere: the size is an old promise)
 size_t fwd_bytes_min(const bdlm_lce_params* p) {
-  const size_t per = align256((size_t)p->T * sizeof(float));
-  return (2 * (size_t)fwd_runs(p->V, FWD_COARSE) + 1) * per + align256(((size_t)p->T + 255) / 256 * sizeof(float));
+  return fwd_part_bytes(p, RUN_TILES_LEAST) + align256(((size_t)p->T + 255) / 256 * sizeof(float));
 }
 int default_chunk(const bdlm_lce_params* p) {
   if (p->token_chunk > 0) return p->token_chunk;
@@ -603,8 +609,8 @@ extern "C" {
 size_t bdlm_linear_ce_workspace_bytes(const bdlm_lce_params* p, int32_t which) {
   if (check(p) != BDLM_OK) return 0;
   if (which == BDLM_LCE_WS_FWD) {
-    const size_t fine = fwd_bytes(p, fwd_tiling(p)), least = fwd_bytes_min(p);
-    return fine > least ? fine : least;
+    const size_t full = fwd_bytes(p), least = fwd_bytes_min(p);
+    return full > least ? full : least;
   }
   if (which == BDLM_LCE_WS_BWD) return bwd_plan(p, false).bytes;
   return 0;
@@ -624,21 +630,20 @@ int bdlm_linear_ce_fwd(const bdlm_lce_params* p, const void* h, const void* w, c
   if (workspace_bytes < fwd_bytes_min(p)) return BDLM_ERR_WORKSPACE_TOO_SMALL;
   if (!sm100() || !tc_encoder_available()) return BDLM_ERR_UNSUPPORTED;
   cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
-  const Tiling fine = fwd_tiling(p);
-  const bool roomy = workspace_bytes >= fwd_bytes(p, fine);
-  const Tiling t = roomy ? fine : FWD_COARSE;
-  const int runs = fwd_runs(p->V, t);
+  const bool roomy = workspace_bytes >= fwd_bytes(p);
+  const int run_tiles = roomy ? RUN_TILES : RUN_TILES_LEAST, runs = fwd_runs(p->V, run_tiles);
   const size_t per = align256((size_t)p->T * sizeof(float));
   char* ws = static_cast<char*>(workspace);
   GemmArgs a = {};
-  a.M = p->T; a.N = p->V; a.K = p->D; a.bn = t.bn; a.n_run = t.n_run; a.m_inner = 1;
+  a.M = p->T; a.N = p->V; a.K = p->D; a.m_inner = 1; a.run_tiles = run_tiles;
+  a.bn = BN; a.n_run = choose_tiling(p->T, p->V, p->D, BN, run_tiles, MAX_RUN, EPI_CLK_LSE, 0).n_run;
   a.row0 = 0; a.labels = labels; a.weight = token_weight; a.ldp = (int)(per / sizeof(float));
   a.part_m = reinterpret_cast<float*>(ws);
   a.part_l = reinterpret_cast<float*>(ws + (size_t)runs * per);
   a.zlab = reinterpret_cast<float*>(ws + 2 * (size_t)runs * per);
   Operand oh{h, p->D, 0, false}, ow{w, p->D, 0, false};
   const bool packed = roomy && packs(p, PACK_FWD_T);
-  if (packed && pack(p, ws + fwd_part_bytes(p, t), oh, ow, st) != cudaSuccess) return BDLM_ERR_CUDA;
+  if (packed && pack(p, ws + fwd_part_bytes(p, run_tiles), oh, ow, st) != cudaSuccess) return BDLM_ERR_CUDA;
   if (launch_gemm<EPI_LSE>(a, oh, ow, st, packed) != cudaSuccess) return BDLM_ERR_CUDA;
   const int blocks = (p->T + FIN_T - 1) / FIN_T;
   if (launch_chained(lce_finish_kernel, true, blocks, 256, 0, st, 1, a.part_m, a.part_l, a.zlab, labels, token_weight, p->T, runs, a.ldp, lse, nll) != cudaSuccess)
@@ -678,19 +683,19 @@ int bdlm_linear_ce_bwd(const bdlm_lce_params* p, const void* h, const void* w, c
     const Operand odz{dz, ldz, 0, roomy};
     // dz of the chunk: logits again, softmax minus one-hot in the epilogue
     GemmArgs a = {};
-    const Tiling ta = choose_tiling(rows, V, D, FWD_N_RUN, EPI_CLK_DZ, 0);
+    const Tiling ta = choose_tiling(rows, V, D, 128, 1, MAX_RUN, EPI_CLK_DZ, 0);
     a.M = rows; a.N = V; a.K = D; a.bn = ta.bn; a.n_run = ta.n_run; a.m_inner = 1;
     a.row0 = t0; a.labels = labels; a.weight = token_weight; a.lse = lse; a.grad = p->grad_loss;
     a.dz = dz; a.ldz = (int)ldz;
     if (launch_gemm<EPI_DZ>(a, oh_c, ow, st, ci > 0 || plan.packed) != cudaSuccess) return BDLM_ERR_CUDA;
     // dH of the chunk = dz W   (contraction over the vocabulary; W as it lies is the MN-major B operand)
     GemmArgs b = {};
-    b.M = rows; b.N = D; b.K = V; b.bn = choose_tiling(rows, D, V, 1, EPI_CLK_STORE, 1).bn; b.n_run = 1; b.m_inner = 1;
+    b.M = rows; b.N = D; b.K = V; b.bn = choose_tiling(rows, D, V, 128, 1, 1, EPI_CLK_STORE, 1).bn; b.n_run = 1; b.m_inner = 1;
     b.c_mode = C_BF16; b.c16 = static_cast<bf16*>(dh) + (size_t)t0 * D; b.ldc = D;
     if (launch_gemm<EPI_STORE>(b, odz, mn(ow), st, true) != cudaSuccess) return BDLM_ERR_CUDA;
     // dW += dz^T H_c   (contraction over the chunk's tokens; both operands MN-major)
     GemmArgs c = {};
-    c.M = V; c.N = D; c.K = rows; c.bn = choose_tiling(V, D, rows, 1, EPI_CLK_STORE, 1).bn; c.n_run = 1; c.m_inner = 0;
+    c.M = V; c.N = D; c.K = rows; c.bn = choose_tiling(V, D, rows, 128, 1, 1, EPI_CLK_STORE, 1).bn; c.n_run = 1; c.m_inner = 0;
     c.c16 = static_cast<bf16*>(dw); c.c32 = dw32; c.ldc = D;
     c.c_mode = chunks == 1 ? C_BF16 : (ci == 0 ? C_F32_STORE : (ci + 1 < chunks ? C_F32_ADD : C_F32_ADD_TO_BF16));
     const Operand A = mn(odz), B = mn(oh_c);

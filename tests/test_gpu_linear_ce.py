@@ -204,3 +204,42 @@ def test_nan_in_the_vocabulary_and_in_a_token_reaches_the_results(V, least):
         assert bool(lse.isnan().all()) and bool(nll.isnan().all()) and bool(loss.isnan().all()), first
     torch.cuda.synchronize()
     assert binding.bdlm_get_device_status() == 0
+
+
+@pytest.mark.parametrize("D", [264, 256], ids=["copied_rows", "whole_rows"])
+def test_lse_of_a_token_does_not_depend_on_the_other_tokens(D):
+    """The same tokens by themselves and among many: every bit of their lse and nll (the vocabulary runs end at the same
+    places, whatever the tiling)."""
+    g = {k: v.cuda() for k, v in synth.make_lce_inputs(LceWorkload("among_others", 1531, D, 20008), "cpu").items()}
+    _, nll, lse = binding.bdlm_linear_ce_fwd(g["h"], g["w"], g["labels"], g["weight"])
+    for n in (1, 130, 700, 1100):
+        few = [g[k][:n].contiguous() for k in ("h", "labels", "weight")]
+        _, nll_n, lse_n = binding.bdlm_linear_ce_fwd(few[0], g["w"], few[1], few[2])
+        torch.cuda.synchronize()
+        assert torch.equal(lse_n, lse[:n]) and torch.equal(nll_n, nll[:n]), n
+
+
+@pytest.mark.parametrize("least", [False, True])
+def test_vocabulary_entries_of_minus_infinity_are_left_out(least):
+    """Logits of -inf (h positive, rows of W -inf): whole tiles, a whole run of the smallest workspace, single entries."""
+    T, D, V = 140, 64, 5000
+    gen = torch.Generator().manual_seed(1)
+    h = (torch.rand(T, D, generator=gen) + 0.1).to(torch.bfloat16)
+    w = (torch.randn(V, D, generator=gen) * 0.3).to(torch.bfloat16)
+    out = torch.zeros(V, dtype=torch.bool)
+    out[0:300] = True
+    out[2048:4096] = True
+    out[4990:] = True
+    out[700::97] = True
+    w[out] = float("-inf")
+    keep = torch.nonzero(~out)[:, 0]
+    labels = keep[torch.randint(len(keep), (T,), generator=gen)].int()
+    per, runs = (T * 4 + 255) // 256 * 256, (((V + 255) // 256) + 7) // 8
+    ws = torch.empty((2 * runs + 1) * per + 256, dtype=torch.uint8, device="cuda") if least else None
+    loss, nll, lse = binding.bdlm_linear_ce_fwd(h.cuda(), w.cuda(), labels.cuda(), workspace=ws)
+    where = {int(v): i for i, v in enumerate(keep)}
+    y = np.array([where[int(v)] for v in labels])
+    ref_loss, ref_nll, ref_lse = lce.linear_ce_forward(synth.to_f64(h), synth.to_f64(w[keep]), y)
+    assert np.abs(synth.to_f64(lse) - ref_lse).max() <= TOL_LSE
+    assert np.abs(synth.to_f64(nll) - ref_nll).max() <= TOL_NLL
+    assert abs(float(loss) - ref_loss) <= TOL_LOSS_REL * abs(ref_loss)
