@@ -141,7 +141,7 @@ lce_gemm_kernel(const __grid_constant__ GemmMaps maps, const GemmArgs a, int* __
     w.start(a);
     int ks = 0;
     bool ok = true;
-    const int stage_bytes = A_BYTES + (a.b_mn != K_MAJOR ? B_BYTES : a.bn * BK * 2);   // (MN-major: always all four panels, zeros past the end)
+    const int stage_bytes = A_BYTES + a.bn * BK * 2;
     for (; w.valid() && ok; w.next()) {
       const int m0 = w.mt * BM, n0 = w.nt * a.bn;
       for (int k = 0; k < nk; ++k, ++ks) {
@@ -160,7 +160,7 @@ lce_gemm_kernel(const __grid_constant__ GemmMaps maps, const GemmArgs a, int* __
         else if (a.b_mn == MN_PANELS) tma_load_panels_e(sB, &maps.b, bar, k * BK, n0 / 64, el);
         else {
 #pragma unroll
-          for (int p = 0; p < BN / 64; ++p) tma_load_2d_e(sB + p * MN_PANEL, &maps.b, bar, n0 + 64 * p, k * BK, el);
+          for (int p = 0; p < BN / 64; ++p) if (64 * p < a.bn) tma_load_2d_e(sB + p * MN_PANEL, &maps.b, bar, n0 + 64 * p, k * BK, el);
         }
       }
     }
@@ -469,7 +469,9 @@ struct Operand { const void* ptr; int64_t ld; int mn; bool whole; };
 // narrower tile or a shorter run has to promise 5 % (8192 x 4096 x 128256 would gain 3 % by this count and lost 1 %: what
 // bounds it is power).  The forward keeps 256 columns, where its runs end (see RUN_TILES).  A B operand
 // that lies MN-major keeps 256 columns where it has them (dH at T = 4096, D = 4096 in one piece: 5.7 ms with 240 or 192
-// columns against 3.4: its panels then start off the 128-byte lines, or a tile's rows off the 512 bytes they share).
+// columns against 3.4: its panels then start off the 128-byte lines, or a tile's rows off the 512 bytes they share),
+// unless its tiles leave SMs idle: dH (min_bn = 64) then takes 64 columns or more, which changes no bit of it (V = 32008: T = 1531,
+// D = 1536 backward 415 -> 380 us, T = 384, D = 1544 305 -> 264; T = 149, D = 224, V = 50912 280 -> 208).
 // Forward / dz at T = 1531, D = 1544, V = 32008: 234 -> 160 and 275 -> 188 us.
 struct Tiling { int bn, n_run; };
 Tiling choose_tiling(int M, int N, int K, int min_bn, int min_run, int max_run, int epi_per_32, int b_mn) {
@@ -477,10 +479,11 @@ Tiling choose_tiling(int M, int N, int K, int min_bn, int min_run, int max_run, 
   const int nk = (K + BK - 1) / BK;
   Tiling best = {BN, max_run};
   double t_best = 1e300;
-  const int unit = b_mn ? 128 : 16;
+  const int unit = b_mn ? min_bn : 16;
+  const bool few = b_mn && min_bn < 128 && m_tiles * ((N + BN - 1) / BN) < sms;
   for (int bn = BN; bn >= min_bn; bn -= unit) {
-    if (bn > 128 && bn - unit >= N) continue;              // a whole unit wider than the matrix
-    if (b_mn && bn < BN && N > bn) break;
+    if (bn > min_bn && bn - unit >= N) continue;           // a whole unit wider than the matrix
+    if (b_mn && bn < BN && N > bn && !few) break;
     const long long n_tiles = (N + bn - 1) / bn;
     const double slice = bn / 2 > 32 + bn / 4 ? bn / 2 : 32 + bn / 4;
     const double epi = (double)epi_per_32 * ((bn + 31) / 32);
@@ -505,7 +508,7 @@ cudaError_t launch_gemm(GemmArgs a, const Operand& A, const Operand& B, cudaStre
     layout = extent % 64 == 0 ? MN_PANELS : MN_BOXES;   // (a last panel that is not whole would reach past the matrix)
     return layout == MN_PANELS ? tc_make_map_panels(m, o.ptr, a.K, extent, o.ld, BK, box / 64) : tc_make_map_2d(m, o.ptr, a.K, extent, o.ld, 64);
   };
-  const bool okA = encode(&maps.a, A, a.M, BM, a.a_mn), okB = encode(&maps.b, B, a.N, B.mn ? BN : a.bn, a.b_mn);
+  const bool okA = encode(&maps.a, A, a.M, BM, a.a_mn), okB = encode(&maps.b, B, a.N, a.bn, a.b_mn);
   if (!okA || !okB) return cudaErrorInvalidValue;
   a.m_tiles = (a.M + BM - 1) / BM;
   a.n_tiles = (a.N + a.bn - 1) / a.bn;
@@ -690,7 +693,7 @@ int bdlm_linear_ce_bwd(const bdlm_lce_params* p, const void* h, const void* w, c
     if (launch_gemm<EPI_DZ>(a, oh_c, ow, st, ci > 0 || plan.packed) != cudaSuccess) return BDLM_ERR_CUDA;
     // dH of the chunk = dz W   (contraction over the vocabulary; W as it lies is the MN-major B operand)
     GemmArgs b = {};
-    b.M = rows; b.N = D; b.K = V; b.bn = choose_tiling(rows, D, V, 128, 1, 1, EPI_CLK_STORE, 1).bn; b.n_run = 1; b.m_inner = 1;
+    b.M = rows; b.N = D; b.K = V; b.bn = choose_tiling(rows, D, V, 64, 1, 1, EPI_CLK_STORE, 1).bn; b.n_run = 1; b.m_inner = 1;
     b.c_mode = C_BF16; b.c16 = static_cast<bf16*>(dh) + (size_t)t0 * D; b.ldc = D;
     if (launch_gemm<EPI_STORE>(b, odz, mn(ow), st, true) != cudaSuccess) return BDLM_ERR_CUDA;
     // dW += dz^T H_c   (contraction over the chunk's tokens; both operands MN-major)

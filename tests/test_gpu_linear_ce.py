@@ -243,3 +243,12 @@ def test_vocabulary_entries_of_minus_infinity_are_left_out(least):
     assert np.abs(synth.to_f64(lse) - ref_lse).max() <= TOL_LSE
     assert np.abs(synth.to_f64(nll) - ref_nll).max() <= TOL_NLL
     assert abs(float(loss) - ref_loss) <= TOL_LOSS_REL * abs(ref_loss)
+
+
+@pytest.mark.parametrize("w", [
+    LceWorkload("dh_64_columns", 130, 200, 3000, seed=1),      # whole panels, one past the matrix; and 64-column boxes
+    LceWorkload("dh_64_whole", 260, 320, 3000, seed=2),
+    LceWorkload("dh_192_columns", 1531, 1544, 1032, seed=3),
+], ids=lambda w: w.name)
+def test_dh_tiles_narrower_than_256_columns(w):
+    _check(w)
