@@ -65,11 +65,13 @@ typedef struct {
                                   BDLM_BWD_FUSED (1): one kernel produces dK, dV and dQ (5 GEMMs per tile pair instead of 7).
                                   Each CTA adds its dQ tiles into an fp32 accumulator in the workspace (bulk add-reductions),
                                   so dQ is reproducible only up to fp32 summation order; dK and dV are bitwise reproducible
-                                  (fixed order).  Needs the workspace bdlm_workspace_bytes[_packed] reports for this setting
+                                  (fixed order) from call to call of the same sizes, while their last bits may depend on
+                                  the batch size and the number of heads (on how many CTAs share a key tile).  Needs the workspace bdlm_workspace_bytes[_packed] reports for this setting
                                   (BDLM_ERR_WORKSPACE_TOO_SMALL otherwise); with impl = 1 (the mma.sync kernels) the
                                   two-pass path runs.
                                   BDLM_BWD_TWO_PASS (2): dK/dV pass + dQ pass, fixed summation order, every gradient
-                                  bitwise reproducible; needs only the D rows in the workspace.
+                                  bitwise reproducible and, for a batch element, independent of the rest of the batch;
+                                  needs only the D rows in the workspace.
                                   BDLM_BWD_AUTO (0, the default of a zeroed struct): the fused kernel when the workspace
                                   passed to the call is at least the size bdlm_workspace_bytes[_packed] reports for this
                                   setting (the fused size), the two-pass path when it is smaller (it must still hold the

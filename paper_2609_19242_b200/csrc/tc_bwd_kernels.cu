@@ -128,7 +128,7 @@ struct QStep { int qs, h, q0; };
 // slower: 4.7 against 3.3 ms on the sliding-window workload.)  Counters only, no division; the order is fixed, so
 // dK / dV stay bitwise reproducible.
 //
-// When a key tile is split over a cluster (see ClusterSplit), its steps are dealt out one by one: CTA `part` of `parts`
+// When a key tile is split over a cluster (see key_unit), its steps are dealt out one by one: CTA `part` of `parts`
 // takes steps part, part + parts, ... of the same order.
 struct StepWalk {
   int a1, na, b1, nb, G, h_first, qs_a, rows, part, parts;
@@ -161,6 +161,9 @@ struct StepWalk {
 // the partial tiles go to shared memory, each CTA adds up a share of the rows over its peers through distributed
 // shared memory, in the order of their ranks (so the sums stay reproducible), and stores it.  Noisy key tiles have a
 // few steps only (their own block's queries): in such a launch each CTA of a cluster takes one of its own.
+// Only the fused kernel does this.  How many CTAs share a tile depends on how full the launch makes the chip, so the last
+// bits of dK / dV depend on the batch size and the number of heads; the two-pass kernels, whose every gradient is
+// reproducible, keep one CTA per key tile and with it sums that depend on the sequence alone.
 struct KeyUnit { int bx, hk, ks, b, part, parts; bool none; };
 __device__ __forceinline__ KeyUnit key_unit(const TileGrid& tg) {
   KeyUnit u;
@@ -259,12 +262,12 @@ tc_dkdv_kernel(const __grid_constant__ BwdMaps maps, const KArgs a, const TileGr
   volatile int* abort_flag = reinterpret_cast<volatile int*>(sm + DKDV_BARS + 136);
 
   const KeyUnit unit = key_unit(tg);
-  const int ks = unit.ks, b = unit.b, hk = unit.hk, part = unit.part, parts = unit.parts;
+  const int ks = unit.ks, b = unit.b, hk = unit.hk;
   const int k0_row = unit.bx * TILE;   // the tile's first key in memory; key tile 0 has the most query tiles: started first
   const int k0 = ks == CLEAN ? clean_key_pos(a, k0_row) : k0_row;   // and its position
   const int warp = __shfl_sync(0xffffffffu, threadIdx.x >> 5, 0), lane = threadIdx.x & 31;   // warp index, provably uniform
   const int L = rows_k(a, ks), M = a.M;   // rows of this stream's K/V tensors
-  if (unit.none || k0_row >= L || a.dk[ks] == nullptr) return;
+  if (k0_row >= L || a.dk[ks] == nullptr) return;
 
   // query tiles that see this key tile: segment A (clean queries; noisy ones for a noisy key tile), then
   // segment B (noisy queries of a clean key tile), for each head of the group.  The visible-query interval of
@@ -288,8 +291,8 @@ tc_dkdv_kernel(const __grid_constant__ BwdMaps maps, const KArgs a, const TileGr
   }
   // the steps are walked in the same order by every role (see StepWalk)
   StepWalk walk;
-  walk.init(tA0, nA, tB0, nB, a.G, hk * a.G, ks == NOISY ? NOISY : CLEAN, TILE, part, parts);
-  const int nsteps = walk.count(), walk_total = walk.total();
+  walk.init(tA0, nA, tB0, nB, a.G, hk * a.G, ks == NOISY ? NOISY : CLEAN, TILE, 0, 1);
+  const int nsteps = walk.count();
   auto step_cur = [&]() { return walk.cur(); };
   auto step_next = [&]() { walk.next(); };
 
@@ -556,10 +559,7 @@ tc_dkdv_kernel(const __grid_constant__ BwdMaps maps, const KArgs a, const TileGr
       ok = mbar_wait_abortable(bar_done, 0, abort_flag);
       ok = __all_sync(0xffffffffu, ok);
     }
-    if (ok && parts > 1) {
-      tc_fence_after();
-      if (nsteps > 0) put_partial<D>(sm, w, r, tl + 256 + w * 128);
-    } else if (ok) {
+    if (ok) {
       tc_fence_after();
       constexpr int EW = 256 / DKDV_NWG;                       // accumulator columns per thread
       const int acol = w * EW;                                 // first of them, in [0, 256)
@@ -581,13 +581,6 @@ tc_dkdv_kernel(const __grid_constant__ BwdMaps maps, const KArgs a, const TileGr
   }
   tc_fence_before();
   __syncthreads();
-  if (parts > 1) {   // as in the fused kernel
-    cluster_sync();
-    if (warp < 8)
-      sum_partials<D>(sm, warp, lane, part, parts, min(parts, walk_total), (warp < 4 ? a.dv[ks] : a.dk[ks]) +
-                      (((int64_t)b * L + k0_row) * a.Hkv + hk) * D, (int64_t)a.Hkv * D, L - k0_row, warp < 4 ? 1.f : a.scale);
-    cluster_sync();
-  }
   if (threadIdx.x == 0 && *abort_flag) atomicExch(status, (int)BDLM_ERR_DEVICE_TIMEOUT);
   if (warp == DKDV_PRODUCER) tmem_dealloc(tmem, 512);
 }
@@ -1438,7 +1431,7 @@ void tc_bwd_place_dq(KArgs& a, void* extra_ws) {
   }
 }
 
-// How many CTAs share a clean key tile (1, 2 or 4), from two estimates in steps of `rows` query rows: `heavy` for the
+// How many CTAs share a clean key tile (1, 2 or 4), from two estimates in steps of HT query rows: `heavy` for the
 // first clean key tile and `mean` per SM; with a prefix table the blocks are taken to be spread evenly over the keys.
 // A launch cannot end before its heaviest CTA, so a split pays when that is well above the mean; below, longest-first
 // start order fills the chip and the exchange of the partial tiles (about 4 steps per CTA) is a loss.  Clusters of four
@@ -1451,7 +1444,8 @@ void tc_bwd_place_dq(KArgs& a, void* extra_ws) {
 //   L = 8192, H = 32 / 8        heavy 0.55 means  2755 / 3122 / 4237
 // Under MIN_HEAVY steps the exchange eats what the split gives (L = 256: 37 / 36 / 36).
 constexpr double MIN_HEAVY = 24, SPLIT_2 = 1.2, SPLIT_4 = 3.0;
-static int split_key_tiles(const KArgs& a, int rows) {
+static int split_key_tiles(const KArgs& a) {
+  constexpr int rows = HT;
   const double W = a.window > 0 ? a.window : 0;
   double heavy = 0, total = 0;
   for (int qs = CLEAN; qs <= NOISY; ++qs) {
@@ -1504,7 +1498,7 @@ static cudaError_t launch_tc_bwd_d(const KArgs& a, int passes, cudaStream_t st) 
       }
       auto kern = a.trace ? tc_bwdf_kernel<true, D> : tc_bwdf_kernel<false, D>;
       TileGrid tg = make_tile_grid((max(a.L, a.k[NOISY] != nullptr ? a.Ln : 0) + TILE - 1) / TILE, a.Hkv, a.batch * 2);
-      tg.parts = split_key_tiles(a, HT);
+      tg.parts = split_key_tiles(a);
       if ((e = launch_units(kern, tg, BF_THREADS, BF_SMEM, st, maps, a, status, after_rows)) != cudaSuccess) return e;
       ConvertArgs ca = {};
       long long blocks[2];
@@ -1521,8 +1515,7 @@ static cudaError_t launch_tc_bwd_d(const KArgs& a, int passes, cudaStream_t st) 
   }
   if (passes & BDLM_BWD_PASS_DKDV) {
     auto kern = a.trace ? tc_dkdv_kernel<true, D> : tc_dkdv_kernel<false, D>;
-    TileGrid tg = make_tile_grid((max(a.L, a.k[NOISY] != nullptr ? a.Ln : 0) + TILE - 1) / TILE, a.Hkv, a.batch * 2);
-    tg.parts = split_key_tiles(a, TILE);
+    const TileGrid tg = make_tile_grid((max(a.L, a.k[NOISY] != nullptr ? a.Ln : 0) + TILE - 1) / TILE, a.Hkv, a.batch * 2);
     if ((e = launch_units(kern, tg, DKDV_THREADS, DKDV_SMEM, st, maps, a, status, after_rows)) != cudaSuccess) return e;
   }
   if (passes & BDLM_BWD_PASS_DQ) {

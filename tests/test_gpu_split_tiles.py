@@ -1,6 +1,7 @@
 """Backward calls short enough that a cluster of CTAs shares each clean key tile: the partial dK / dV tiles are added up
-through distributed shared memory.  Two and four CTAs per tile, step counts that the CTAs do not divide, ragged last
-tiles, one head per group, key tiles only some of the CTAs have steps for (sliding window), both kernel paths."""
+through distributed shared memory (fused kernel).  Two and four CTAs per tile, step counts that the CTAs do not divide,
+ragged last tiles, one head per group, key tiles only some of the CTAs have steps for (sliding window).  The two-pass kernels,
+one CTA per key tile, at the same sizes: there a batch element's gradients do not depend on the batch."""
 import pytest
 import torch
 
@@ -30,3 +31,21 @@ def test_split_key_tiles_match_the_oracle_and_are_reproducible(w, single_pass):
     a, b = (pu.gpu_bwd(g, out, w.block_size, window=w.window, single_pass=single_pass) for _ in range(2))
     for i in (1, 2, 4, 5):   # dK, dV of both streams: a fixed order of summation
         assert torch.equal(a[i], b[i])
+
+
+@pytest.mark.parametrize("w", [
+    Workload("ten", 10, 8, 2, 128, 512, 32, seed=7),
+    Workload("odd_group_d64", 20, 3, 1, 64, 776, 8, seed=8),
+    Workload("window", 24, 8, 2, 128, 512, 16, window=130, seed=9),
+], ids=lambda w: w.name)
+def test_two_pass_gradients_of_a_batch_element_do_not_depend_on_the_batch(w):
+    g = synth.make_inputs(w, "cuda")
+    out = pu.gpu_fwd(g, w.block_size, window=w.window)
+    whole = pu.gpu_bwd(g, out, w.block_size, window=w.window, single_pass=False)
+    for i in (0, w.batch - 1):
+        gi = {k: (v[i:i + 1].contiguous() if v.dim() == 4 else v) for k, v in g.items()}
+        oi = pu.gpu_fwd(gi, w.block_size, window=w.window)
+        for a, b in zip(oi, out):
+            assert torch.equal(a[0], b[i])
+        for a, b in zip(pu.gpu_bwd(gi, oi, w.block_size, window=w.window, single_pass=False), whole):
+            assert torch.equal(a[0], b[i])
