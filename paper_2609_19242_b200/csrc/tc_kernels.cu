@@ -216,16 +216,21 @@ tc_fwdr_kernel(const __grid_constant__ FwdMaps maps, const KArgs a, const TileGr
         const bool two = a.q[CLEAN] != nullptr && a.q[NOISY] != nullptr;
         int index = blockIdx.x, g = 0, n_units = 0, n_q = 0, n_clc = 0;   // g: K/V tiles loaded so far
         bool ok = true, asked = false;
+        // The next unit is asked for three K/V tiles before the end of this one, and answered while those are loaded.  Asked
+        // for at the start of a unit, the next one would be taken long before it can begin: of 256 units on 148 SMs the
+        // heaviest, which start first, would take the second ones too (H = 8 / 1: L = 4096 87 us, now 65; L = 8192, H = 4 / 1
+        // 158, now 115; with one unit per CTA 72 and 131).
+        auto ask = [&]() { clc_request(clc_slot, bar_clc); asked = true; };
         while (ok) {
-          clc_request(clc_slot, bar_clc);   // answered while this unit is loaded
-          asked = true;
           int bx, by, bz;
           tile_grid_decode(tg, index, bx, by, bz);
           const int qs = two ? bz & 1 : (a.q[CLEAN] != nullptr ? CLEAN : NOISY), b = two ? bz >> 1 : bz;
           const int h0 = PAIRQ ? by : by * 2, hk = h0 / a.G;
           const int q0 = (tg.nx - 1 - bx) * QROWS;   // the last query tile sees the most keys: started first
           const int Lq = rows_q(a, qs);
-          if (q0 < Lq) {
+          if (q0 >= Lq) {
+            ask();
+          } else {
             TileSched sch;
             sch.init(qs, q0, min(q0 + QROWS, Lq) - 1, a);
             if (n_units >= 2) ok = mbar_wait_abortable(bar_unit_empty + 8 * (n_units & 1), ((n_units >> 1) - 1) & 1, abort_flag);
@@ -246,8 +251,10 @@ tc_fwdr_kernel(const __grid_constant__ FwdMaps maps, const KArgs a, const TileGr
               tma_load_3d(sQ + TILE_BYTES, &maps.q[qs], bar_q, (h0 + HSTEP) * D, q0 + QSTEP, b);
               if (D == 128) tma_load_3d(sQ + TILE_BYTES + PANEL_BYTES, &maps.q[qs], bar_q, (h0 + HSTEP) * D + 64, q0 + QSTEP, b);
             }
+            if (nt == 0) ask();
             for (int t = 0; t < nt; ++t, ++g) {
               const int s = g & 1;
+              if (t == max(nt - 3, 0)) ask();
               if (g >= 2) ok = mbar_wait_abortable(bar_kv_empty + 8 * s, ((g >> 1) - 1) & 1, abort_flag);
               if (!ok) break;
               const int ks = tile_ks(sch, t), k0 = tile_k0(sch, t);

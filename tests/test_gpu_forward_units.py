@@ -15,6 +15,7 @@ CASES = [
     Workload("even", 1, 16, 4, 128, 6144, 32, seed=1),
     Workload("odd_d64", 2, 6, 2, 64, 8192, 64, seed=2),
     Workload("ragged", 3, 8, 4, 128, 5000, 40, seed=3),
+    Workload("two_waves", 1, 8, 1, 128, 4096, 32, seed=5),
 ]
 
 
