@@ -3,6 +3,7 @@
 // accumulators in tensor memory; the online softmax runs in registers, one thread per query
 // row.  The tile schedule enumerates only the key tiles a query tile can see (Algorithm 1:
 // clean-prefix tiles, then the noisy-diagonal tiles); no mask is materialised.
+#include "fwd_issue.h"
 #include "tc_common.cuh"
 #include "tc_launch.h"
 
@@ -159,6 +160,10 @@ struct FwdUnit {
 constexpr int FWD_UNIT_BYTES = 64;
 static_assert(sizeof(FwdUnit) <= FWD_UNIT_BYTES, "unit slot");
 
+// What fwd_issue_loop works with: the issuing warp's waits and instructions, as closures over the kernel's state.
+template <class U, class Q, class K, class V, class P, class QK, class PV, class O, class KV>
+struct IssueOps { U& next_unit; Q& q_full; K& k_full; V& v_full; P& p_full; QK& qk; PV& pv; O& o_done; KV& kv_done; };
+
 // D = head dimension (128 or 64).  With D = 64 a tile is one 64-column panel: the second panel of every shared-memory
 // tile stays unused, Q K^T contracts over four k-slices and P V produces 64 output columns.
 template <bool TR, bool PAIRQ, int D>
@@ -176,7 +181,7 @@ tc_fwdr_kernel(const __grid_constant__ FwdMaps maps, const KArgs a, const TileGr
   const uint32_t bar_q = bars, bar_k_full = bars + 8 /*[2]*/, bar_v_full = bars + 24 /*[2]*/, bar_kv_empty = bars + 40 /*[2]*/,
                  bar_s = bars + 56 /*[2]*/, bar_o = bars + 72 /*[2]*/, bar_p = bars + 88 /*[head][key half]*/,
                  bar_q_empty = bars + 120, bar_unit_full = bars + 128 /*[2]*/, bar_unit_empty = bars + 144 /*[2]*/,
-                 bar_clc = bars + 160, clc_slot = bars + 176;
+                 bar_clc = bars + 160, bar_drain = bars + 168, clc_slot = bars + 176;
   volatile uint32_t* tmem_slot = reinterpret_cast<volatile uint32_t*>(sm + FWDR_BARS + 192);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(sm + FWDR_BARS + 200);
   auto unit_slot = [&](int k) { return reinterpret_cast<FwdUnit*>(sm + FWDR_BARS + 256 + (k & 1) * FWD_UNIT_BYTES); };
@@ -188,7 +193,7 @@ tc_fwdr_kernel(const __grid_constant__ FwdMaps maps, const KArgs a, const TileGr
   // The producer starts loading as soon as the barriers are set up; everyone else also needs tensor memory.
   if (warp == 8) {
     if (lane == 0) {
-      mbar_init(bar_q, 1); mbar_init(bar_q_empty, 1); mbar_init(bar_clc, 1);
+      mbar_init(bar_q, 1); mbar_init(bar_q_empty, 1); mbar_init(bar_clc, 1); mbar_init(bar_drain, 1);
       for (int i = 0; i < 2; ++i) {
         mbar_init(bar_k_full + 8 * i, 1); mbar_init(bar_v_full + 8 * i, 1); mbar_init(bar_kv_empty + 8 * i, 1);
         mbar_init(bar_s + 8 * i, 1); mbar_init(bar_o + 8 * i, 1);
@@ -277,9 +282,12 @@ tc_fwdr_kernel(const __grid_constant__ FwdMaps maps, const KArgs a, const TileGr
           if (!more) break;
           fence_async_smem();   // the answer has been read before the next request may overwrite it
         }
-        if (!ok && asked) {   // leaving early: not before the answer on its way has landed (bounded)
+        if (!ok) {   // leaving early: not before the answer and the loads on their way have landed (bounded)
           const long long t0 = clock64();
-          while (!mbar_try_wait(bar_clc, n_clc & 1) && clock64() - t0 < WAIT_LIMIT_TICKS) {}
+          auto landed = [&](uint32_t bar, int parity) { while (!mbar_try_wait(bar, parity) && clock64() - t0 < WAIT_LIMIT_TICKS) {} };
+          if (asked) landed(bar_clc, n_clc & 1);
+          if (n_q > 0) landed(bar_q, (n_q - 1) & 1);
+          for (int i = max(g - 2, 0); i < g; ++i) { landed(bar_k_full + 8 * (i & 1), (i >> 1) & 1); landed(bar_v_full + 8 * (i & 1), (i >> 1) & 1); }
         }
         if (ok && n_units >= 2) ok = mbar_wait_abortable(bar_unit_empty + 8 * (n_units & 1), ((n_units >> 1) - 1) & 1, abort_flag);
         if (ok) {
@@ -289,99 +297,53 @@ tc_fwdr_kernel(const __grid_constant__ FwdMaps maps, const KArgs a, const TileGr
       }
     } else if (warp == 9) {
       // ------------------------------------------------------------------ MMA issuer
-      // the whole warp walks the MMA loop; one elected lane issues (see elect_one).  A wait that fails only clears `ok`:
-      // the lanes of the warp stay together (later waits return at once when the abort flag is up) and leave with the
-      // next unit, whose tile count is broadcast so that the loop is provably uniform.
+      // the whole warp walks fwd_issue_loop; one elected lane issues (see elect_one).  The lanes vote on every wait, so that
+      // they leave together after one that failed in any of them.  (A vote is a few clocks of a tile's 2900; predicating the
+      // issue on a lane's own waits instead took the operands off the uniform datapath: 8 to 15 % of the forward.)  Tile
+      // counts are broadcast so that the loop is provably uniform.
       const uint32_t tmem = __shfl_sync(0xffffffffu, *tmem_slot, 0);   // broadcast: provably warp-uniform
       const uint32_t el = elect_one();
-      const uint32_t qa_lo = desc_lo_k(sQ), qb_lo = qa_lo + TILE_LO;
+      const uint32_t qa_lo = desc_lo_k(sQ);
       const uint32_t k_lo0 = desc_lo_k(sK0), v_lo0 = desc_lo_mn(sK0 + TILE_BYTES);
       int n_units = 0;
-      bool ok = true;
-      // tiles of the next unit (0: it sees no key), -1 when none is left
+      long long w_p = 0, w_v = 0, w_k = 0;
+      auto arrived = [&](uint32_t bar, int parity, long long& acc) { return __all_sync(0xffffffffu, mbar_wait_timed<TR>(bar, parity, abort_flag, acc)) != 0; };
       auto next_unit = [&]() {
-        ok = mbar_wait_abortable(bar_unit_full + 8 * (n_units & 1), (n_units >> 1) & 1, abort_flag) && ok;
+        if (!__all_sync(0xffffffffu, mbar_wait_abortable(bar_unit_full + 8 * (n_units & 1), (n_units >> 1) & 1, abort_flag))) return FWD_UNIT_FAILED;
         const volatile FwdUnit* u = unit_slot(n_units);
-        const int n = __shfl_sync(0xffffffffu, ok && u->more ? u->sch.nt0 + u->sch.nt1 : -1, 0);
+        const int n = __shfl_sync(0xffffffffu, u->more ? u->sch.nt0 + u->sch.nt1 : FWD_NO_UNIT, 0);
         if (lane == 0) mbar_arrive(bar_unit_empty + 8 * (n_units & 1));
         ++n_units;
         return n;
       };
+      auto q_full = [&](int n) { return arrived(bar_q, n & 1, w_k); };
+      auto k_full = [&](int g) { return arrived(bar_k_full + 8 * (g & 1), (g >> 1) & 1, w_k); };
+      auto v_full = [&](int g) { return arrived(bar_v_full + 8 * (g & 1), (g >> 1) & 1, w_v); };
+      // (P: bf16 pairs at columns [0,32) and [32,64) of the head's S region)
+      auto p_full = [&](int head, int half, int g) { return arrived(bar_p + 16 * head + 8 * half, g & 1, w_p); };
+      auto qk = [&](int head, int g, bool last_of_q) {
+        tc_fence_after();
+        gemm_ss_e<D / 16>(tmem + 128 * head, qa_lo + head * TILE_LO, k_lo0 + (g & 1) * 2 * TILE_LO, IDESC_QK, 0u, el);
+        mma_commit_e(bar_s + 8 * head, el);
+        if (last_of_q) mma_commit_e(bar_q_empty, el);
+      };
       // O += P V over key half j of the tile: four k-slices of 16 keys
-      auto pv_half = [&](uint32_t d, uint32_t p_tmem, uint32_t v_lo, int j, uint32_t acc_first) {
+      auto pv = [&](int head, int j, int g, uint32_t acc_first) {
+        tc_fence_after();
 #pragma unroll
         for (int kk = 0; kk < 4; ++kk)
-          mma_ts_e(d, p_tmem + (4 * j + kk) * 8, desc64(v_lo + moff(4 * j + kk)), IDESC_PV, kk == 0 ? acc_first : 1u, el);
+          mma_ts_e(tmem + 256 + 128 * head, tmem + 128 * head + (4 * j + kk) * 8, desc64(v_lo0 + (g & 1) * 2 * TILE_LO + moff(4 * j + kk)),
+                   IDESC_PV, kk == 0 ? acc_first : 1u, el);
       };
-      long long w_p = 0, w_v = 0, w_k = 0;
+      auto o_done = [&](int head) { mma_commit_e(bar_o + 8 * head, el); };
+      auto kv_done = [&](int g) { mma_commit_e(bar_kv_empty + 8 * (g & 1), el); };
       const long long tm0 = tick<TR>();
-      int nt = 0, g = 0, n_q = 0;   // g: tiles done so far, n_q: units whose Q has been waited for
-      while (nt >= 0) {
-        if (nt == 0) {   // the first unit, and after units that see no key: nothing in flight to overlap with
-          nt = next_unit();
-          if (nt <= 0) continue;
-          ok = mbar_wait_abortable(bar_q, n_q & 1, abort_flag) && ok;
-          ok = mbar_wait_abortable(bar_k_full + 8 * (g & 1), (g >> 1) & 1, abort_flag) && ok;
-          ++n_q;
-          tc_fence_after();
-          const uint32_t k_lo = k_lo0 + (g & 1) * 2 * TILE_LO;
-          gemm_ss_e<D / 16>(tmem, qa_lo, k_lo, IDESC_QK, 0u, el);
-          mma_commit_e(bar_s, el);
-          gemm_ss_e<D / 16>(tmem + 128, qb_lo, k_lo, IDESC_QK, 0u, el);
-          mma_commit_e(bar_s + 8, el);
-          if (nt == 1) mma_commit_e(bar_q_empty, el);
-        }
-        int nt_next = 0;
-        for (int t = 0; t < nt; ++t, ++g) {
-          const int s = g & 1;
-          const uint32_t cv_lo = v_lo0 + s * 2 * TILE_LO;
-          const uint32_t nk_lo = k_lo0 + (s ^ 1) * 2 * TILE_LO;
-          const uint32_t acc = t > 0 ? 1u : 0u;
-          // head A: P arrives in two halves of the keys (bf16 pairs at columns [0,32) and [32,64) of the head's S
-          // region), so P V over the first 64 keys runs while the softmax is still in the exponentials of the rest
-          ok = mbar_wait_timed<TR>(bar_p, g & 1, abort_flag, w_p) && ok;
-          ok = mbar_wait_timed<TR>(bar_v_full + 8 * s, (g >> 1) & 1, abort_flag, w_v) && ok;
-          tc_fence_after();
-          pv_half(tmem + 256, tmem, cv_lo, 0, acc);
-          ok = mbar_wait_timed<TR>(bar_p + 8, g & 1, abort_flag, w_p) && ok;
-          tc_fence_after();
-          pv_half(tmem + 256, tmem, cv_lo, 1, 1u);
-          mma_commit_e(bar_o, el);
-          // the next tile's scores: this unit's, or the first of the next unit (whose Q has been loaded meanwhile).
-          // Only one unit ahead: the one after it is announced when the softmax warps have left this one, and they
-          // still wait for head B's P V below.
-          bool more = t + 1 < nt, q_done = t + 2 == nt;   // q_done: they are the last that read Q
-          if (!more) {
-            nt_next = next_unit();
-            if (nt_next > 0) {
-              ok = mbar_wait_timed<TR>(bar_q, n_q & 1, abort_flag, w_k) && ok;
-              ++n_q;
-              more = true;
-              q_done = nt_next == 1;
-            }
-          }
-          if (more) {
-            ok = mbar_wait_timed<TR>(bar_k_full + 8 * (s ^ 1), ((g + 1) >> 1) & 1, abort_flag, w_k) && ok;
-            tc_fence_after();
-            gemm_ss_e<D / 16>(tmem, qa_lo, nk_lo, IDESC_QK, 0u, el);
-            mma_commit_e(bar_s, el);
-          }
-          // head B
-          ok = mbar_wait_timed<TR>(bar_p + 16, g & 1, abort_flag, w_p) && ok;
-          tc_fence_after();
-          pv_half(tmem + 384, tmem + 128, cv_lo, 0, acc);
-          ok = mbar_wait_timed<TR>(bar_p + 24, g & 1, abort_flag, w_p) && ok;
-          tc_fence_after();
-          pv_half(tmem + 384, tmem + 128, cv_lo, 1, 1u);
-          mma_commit_e(bar_o + 8, el);
-          mma_commit_e(bar_kv_empty + 8 * s, el);
-          if (more) {
-            gemm_ss_e<D / 16>(tmem + 128, qb_lo, nk_lo, IDESC_QK, 0u, el);
-            mma_commit_e(bar_s + 8, el);
-            if (q_done) mma_commit_e(bar_q_empty, el);
-          }
-        }
-        nt = nt_next;
+      IssueOps<decltype(next_unit), decltype(q_full), decltype(k_full), decltype(v_full), decltype(p_full), decltype(qk), decltype(pv),
+               decltype(o_done), decltype(kv_done)> ops = {next_unit, q_full, k_full, v_full, p_full, qk, pv, o_done, kv_done};
+      if (!fwd_issue_loop(ops)) {   // tensor memory is given back below: not before the MMAs already issued have landed (bounded)
+        mma_commit_e(bar_drain, el);
+        const long long t0 = clock64();
+        while (!mbar_try_wait(bar_drain, 0) && clock64() - t0 < WAIT_LIMIT_TICKS) {}
       }
       if (lane == 0) {
         trace_add(a.trace, 8, tick<TR>() - tm0); trace_add(a.trace, 9, w_p); trace_add(a.trace, 10, w_v); trace_add(a.trace, 11, w_k);
