@@ -8,6 +8,7 @@ from __future__ import annotations
 
 import ctypes
 import os
+import weakref
 
 import torch
 
@@ -212,7 +213,31 @@ def bdlm_attn_bwd_static_scratch(q_clean, k_clean, v_clean, q_noisy, k_noisy, v_
     return out
 
 
-_checked_prefix_tables = set()
+# Prefix tables that passed their check, by id: (weak reference, what it held when checked, rules it was checked against).
+# The entry goes when the tensor goes, so neither its id nor its address can vouch for a later one.
+_checked_prefix_tables = {}
+
+
+def _prefix_table_state(t):
+    return t.data_ptr(), t.numel(), t.device, t._version
+
+
+def _prefix_table_checked(t, state, rules):
+    entry = _checked_prefix_tables.get(id(t))
+    return entry is not None and entry[0]() is t and entry[1] == state and rules in entry[2]
+
+
+def _prefix_table_passed(t, state, rules):
+    key = id(t)
+    entry = _checked_prefix_tables.get(key)
+    if entry is not None and entry[0]() is t and entry[1] == state:
+        entry[2].add(rules)
+        return
+
+    def gone(ref):
+        if _checked_prefix_tables.get(key, (None,))[0] is ref:
+            del _checked_prefix_tables[key]
+    _checked_prefix_tables[key] = (weakref.ref(t, gone), state, {rules})
 
 
 def _packed_setup(q_clean, k_clean, q_noisy, block_size, block_prefix, clean_q_pos0, window, kv_chunks=None, **kw):
@@ -258,10 +283,10 @@ def _packed_setup(q_clean, k_clean, q_noisy, block_size, block_prefix, clean_q_p
             assert block_prefix.is_cuda and block_prefix.dtype == torch.int32 and block_prefix.is_contiguous()
             if block_prefix.numel() != g.n_blocks:
                 raise ValueError("block_prefix needs one entry per packed block")
-            # the host copy synchronises the device: a table that was checked once (same storage, same version
-            # counter, same rules) is not copied again on the calls of later steps
-            key = (block_prefix.data_ptr(), block_prefix.numel(), block_prefix._version, L, block_size, window > 0)
-            if key not in _checked_prefix_tables:
+            # the host copy synchronises the device (and cannot be captured): a tensor that was checked once is not copied
+            # again on later calls while it lives, unless it was written to (its version counter tells) or the rules differ
+            state, rules = _prefix_table_state(block_prefix), (L, block_size, window > 0)
+            if not _prefix_table_checked(block_prefix, state, rules):
                 host = block_prefix.cpu()
                 step = host[1:] - host[:-1]
                 if host.numel() and (int(host.min()) < 0 or int(host.max()) > L):
@@ -270,9 +295,7 @@ def _packed_setup(q_clean, k_clean, q_noisy, block_size, block_prefix, clean_q_p
                     raise ValueError("block_prefix must be non-decreasing (sort the packed blocks)")
                 if window > 0 and step.numel() and int(step.min()) < block_size:
                     raise ValueError("with a sliding window the packed blocks must not overlap in position")
-                if len(_checked_prefix_tables) >= 256:
-                    _checked_prefix_tables.clear()
-                _checked_prefix_tables.add(key)
+                _prefix_table_passed(block_prefix, state, rules)
             g.block_prefix = block_prefix.data_ptr()
     g._keep = keep
     return p, g

@@ -217,6 +217,51 @@ def test_binding_rejects_bad_prefix_tables():
         binding.bdlm_attn_fwd_packed(*args, block_prefix=mk([0, 64, 128]))            # wrong length
 
 
+def test_a_prefix_table_is_not_vouched_for_by_an_earlier_one():
+    """A good table passes its check and goes away; another one of the same length comes to lie at the same address."""
+    t = _cuda(_draw(16, 1, 256, 0, 128, 2, 1, 128))
+    args = (None, t["k_clean"], t["v_clean"], t["q_noisy"], t["k_noisy"], t["v_noisy"], 32)
+    good, bad = (torch.tensor(v, dtype=torch.int32, device="cuda") for v in ([0, 32, 64, 128], [0, 64, 32, 128]))
+    seen = 0
+    for _ in range(8):
+        first = good.clone()
+        binding.bdlm_attn_fwd_packed(*args, block_prefix=first)
+        at = first.data_ptr()
+        del first
+        second = bad.clone()
+        seen += second.data_ptr() == at
+        with pytest.raises(ValueError):
+            binding.bdlm_attn_fwd_packed(*args, block_prefix=second)
+        del second
+    assert seen > 0   # otherwise the allocator no longer does what this test is about
+    third = good.clone()
+    binding.bdlm_attn_fwd_packed(*args, block_prefix=third)
+    third.copy_(bad)
+    with pytest.raises(ValueError):   # written to in place
+        binding.bdlm_attn_fwd_packed(*args, block_prefix=third)
+    fourth = good.clone()
+    binding.bdlm_attn_fwd_packed(*args, block_prefix=fourth)
+    with pytest.raises(ValueError):   # the same table under other rules
+        binding.bdlm_attn_fwd_packed(None, t["k_clean"][:, :96].contiguous(), t["v_clean"][:, :96].contiguous(), *args[3:], block_prefix=fourth)
+    n = len(binding._checked_prefix_tables)
+    del third, fourth
+    assert len(binding._checked_prefix_tables) <= n - 2
+
+
+def test_a_checked_prefix_table_can_be_used_under_capture():
+    t = _cuda(_draw(16, 1, 256, 0, 128, 2, 1, 128))
+    args = (None, t["k_clean"], t["v_clean"], t["q_noisy"], t["k_noisy"], t["v_noisy"], 32)
+    table = torch.tensor([0, 32, 64, 128], dtype=torch.int32, device="cuda")
+    want = binding.bdlm_attn_fwd_packed(*args, block_prefix=table)
+    out = tuple(None if x is None else torch.zeros_like(x) for x in want)
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        binding.bdlm_attn_fwd_packed(*args, block_prefix=table, out=out)
+    graph.replay()
+    torch.cuda.synchronize()
+    assert torch.equal(out[2], want[2]) and torch.equal(out[3], want[3])
+
+
 @pytest.mark.parametrize("impl", IMPLS)
 @pytest.mark.parametrize("P", [2, 4])
 def test_clean_kv_in_gathered_order(P, impl):
