@@ -45,16 +45,18 @@ typedef struct {
   int32_t reserved[3];
 } bdlm_lce_params;
 
-enum { BDLM_LCE_WS_FWD = 0, BDLM_LCE_WS_BWD = 1 };
+enum { BDLM_LCE_WS_FWD = 0, BDLM_LCE_WS_BWD = 1, BDLM_LCE_WS_FWD_LEAST = 2, BDLM_LCE_WS_BWD_LEAST = 3 };
 
 /* Scratch bytes of a call (0 for invalid parameters).  Forward: partial (maximum, sum) pairs per token and
  * vocabulary run.  Backward: one chunk of dz, bf16 [token_chunk, V], plus -- when T needs more than one
  * chunk -- an fp32 dW accumulator [V, D].  Where the sizes call for it also: rows of dz padded to 128 bytes,
- * copies of W and h with padded rows (D no multiple of 64).  Without those extras a call
- * is still accepted and takes the plain path (the forward's results are then the same up to the order of fp32
- * sums: its vocabulary runs are eight times as long): forward (2 r + 1) * a(4 T) + a(4 ceil(T / 256)) bytes with
- * r = ceil(ceil(V / 256) / 8) and a() = rounding up to 256; backward a(2 token_chunk V), plus a(4 V D) with
- * several chunks. */
+ * and, with D no multiple of 64, copies of W and h with rows rounded up to 64 elements: 2 (V + T) D bytes and a little
+ * more (1.1 GB at T = 8192, D = 4104, V = 128256), in the forward from 1024 tokens on, in the backward from 384.
+ *
+ * Without those extras a call is still accepted and takes the plain path; the _LEAST values ask for that size.  The
+ * backward's results are the same bit for bit, the forward's up to the order of fp32 sums (its vocabulary runs are
+ * eight times as long): forward (2 r + 1) * a(4 T) + a(4 ceil(T / 256)) bytes with r = ceil(ceil(V / 256) / 8) and
+ * a() = rounding up to 256; backward a(2 token_chunk V), plus a(4 V D) with several chunks. */
 size_t bdlm_linear_ce_workspace_bytes(const bdlm_lce_params* p, int32_t which);
 
 /*

@@ -25,7 +25,7 @@ EXPORTS = ("bdlm_workspace_bytes", "bdlm_attn_fwd", "bdlm_attn_bwd", "bdlm_lse_m
            "bdlm_attn_bwd_static_scratch", "bdlm_workspace_bytes_packed", "bdlm_attn_fwd_packed",
            "bdlm_attn_bwd_packed", "bdlm_selftest_wait_timeout", "bdlm_linear_ce_workspace_bytes",
            "bdlm_linear_ce_fwd", "bdlm_linear_ce_bwd")
-LCE_WS_FWD, LCE_WS_BWD = 0, 1
+LCE_WS_FWD, LCE_WS_BWD, LCE_WS_FWD_LEAST, LCE_WS_BWD_LEAST = 0, 1, 2, 3
 STATIC_SCRATCH_ROWS = 1 << 20
 TRACE_SLOTS = 256
 
@@ -409,6 +409,15 @@ def bdlm_linear_ce_workspace_bytes(params: BdlmLceParams, which: int) -> int:
     return int(lib().bdlm_linear_ce_workspace_bytes(ctypes.byref(params), which))
 
 
+def _lce_workspace(p, which, least, device):
+    """The workspace with everything the library can use (copies of the matrices among it), or, where memory is short, the
+    smallest one that it accepts."""
+    try:
+        return torch.empty(max(bdlm_linear_ce_workspace_bytes(p, which), 16), dtype=torch.uint8, device=device)
+    except torch.OutOfMemoryError:
+        return torch.empty(max(bdlm_linear_ce_workspace_bytes(p, least), 16), dtype=torch.uint8, device=device)
+
+
 def bdlm_linear_ce_fwd(h, w, labels, token_weight=None, *, out=None, workspace=None):
     """Forward of the linear cross-entropy: h [T, D] bf16, w [V, D] bf16, labels [T] int32 (negative = ignored),
     token_weight [T] fp32 or None.  Returns (loss [1] fp32, nll [T] fp32, lse [T] fp32), all on the device."""
@@ -419,7 +428,7 @@ def bdlm_linear_ce_fwd(h, w, labels, token_weight=None, *, out=None, workspace=N
         out = (torch.empty(1, dtype=torch.float32, device=h.device), torch.empty(T, dtype=torch.float32, device=h.device),
                torch.empty(T, dtype=torch.float32, device=h.device))
     if workspace is None:
-        workspace = torch.empty(max(bdlm_linear_ce_workspace_bytes(p, LCE_WS_FWD), 16), dtype=torch.uint8, device=h.device)
+        workspace = _lce_workspace(p, LCE_WS_FWD, LCE_WS_FWD_LEAST, h.device)
     assert labels.dtype == torch.int32
     rc = lib().bdlm_linear_ce_fwd(ctypes.byref(p), _ptr(h), _ptr(w), _ptr(labels), _ptr(token_weight), _ptr(out[0]),
                                   _ptr(out[1]), _ptr(out[2]), _ptr(workspace), workspace.numel(), _stream())
@@ -437,7 +446,7 @@ def bdlm_linear_ce_bwd(h, w, labels, lse, token_weight=None, *, grad_loss=1.0, t
     if out is None:
         out = (torch.empty_like(h), torch.empty_like(w))
     if workspace is None:
-        workspace = torch.empty(max(bdlm_linear_ce_workspace_bytes(p, LCE_WS_BWD), 16), dtype=torch.uint8, device=h.device)
+        workspace = _lce_workspace(p, LCE_WS_BWD, LCE_WS_BWD_LEAST, h.device)
     assert labels.dtype == torch.int32
     rc = lib().bdlm_linear_ce_bwd(ctypes.byref(p), _ptr(h), _ptr(w), _ptr(labels), _ptr(token_weight), _ptr(lse),
                                   _ptr(out[0]), _ptr(out[1]), _ptr(workspace), workspace.numel(), _stream())

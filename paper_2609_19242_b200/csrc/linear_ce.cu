@@ -616,6 +616,8 @@ size_t bdlm_linear_ce_workspace_bytes(const bdlm_lce_params* p, int32_t which) {
     return full > least ? full : least;
   }
   if (which == BDLM_LCE_WS_BWD) return bwd_plan(p, false).bytes;
+  if (which == BDLM_LCE_WS_FWD_LEAST) return fwd_bytes_min(p);
+  if (which == BDLM_LCE_WS_BWD_LEAST) return bwd_plan(p, true).bytes;
   return 0;
 }
 

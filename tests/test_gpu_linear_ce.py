@@ -252,3 +252,29 @@ def test_vocabulary_entries_of_minus_infinity_are_left_out(least):
 ], ids=lambda w: w.name)
 def test_dh_tiles_narrower_than_256_columns(w):
     _check(w)
+
+
+def test_the_smallest_workspaces_serve_where_memory_is_short(monkeypatch):
+    """With no room for the copies of W and h a call does what it did without them: the backward to the bit."""
+    w = LceWorkload("short_of_memory", 1100, 264, 3000)
+    g = {k: v.cuda() for k, v in synth.make_lce_inputs(w, "cpu").items()}
+    p = binding.make_lce_params(w.T, w.D, w.V)
+    sizes = [binding.bdlm_linear_ce_workspace_bytes(p, i) for i in range(4)]
+    assert 0 < sizes[2] < sizes[0] and 0 < sizes[3] < sizes[1]
+    loss, nll, lse = binding.bdlm_linear_ce_fwd(g["h"], g["w"], g["labels"], g["weight"])
+    dh, dw = binding.bdlm_linear_ce_bwd(g["h"], g["w"], g["labels"], lse, g["weight"])
+    empty, refused = torch.empty, []
+
+    def short(*size, **kw):
+        if kw.get("dtype") == torch.uint8 and size[0] in sizes[:2]:
+            refused.append(size[0])
+            raise torch.OutOfMemoryError("no room")
+        return empty(*size, **kw)
+    monkeypatch.setattr(torch, "empty", short)
+    dh2, dw2 = binding.bdlm_linear_ce_bwd(g["h"], g["w"], g["labels"], lse, g["weight"])
+    loss2, nll2, lse2 = binding.bdlm_linear_ce_fwd(g["h"], g["w"], g["labels"], g["weight"])
+    monkeypatch.undo()
+    torch.cuda.synchronize()
+    assert refused == [sizes[1], sizes[0]]
+    assert torch.equal(dh, dh2) and torch.equal(dw, dw2)
+    assert float((lse - lse2).abs().max()) <= TOL_LSE and float((nll - nll2).abs().max()) <= TOL_NLL
