@@ -48,3 +48,45 @@ def test_forward_backward_replay_from_a_cuda_graph(fused):
     graph.replay()
     torch.cuda.synchronize()
     assert torch.equal(out[0], ref_o2[0]) and torch.equal(out[1], ref_o2[1])
+
+
+@pytest.mark.parametrize("T,D", [(300, 256), (1100, 264)], ids=["plain", "copied_rows"])
+def test_loss_head_replays_from_a_cuda_graph_and_runs_on_any_stream(T, D):
+    w = synth.LceWorkload("graph", T, D, 3000)
+    g = {k: v.cuda() for k, v in synth.make_lce_inputs(w, "cpu").items()}
+
+    def step(out=None, grads=None, ws=(None, None)):
+        out = binding.bdlm_linear_ce_fwd(g["h"], g["w"], g["labels"], g["weight"], out=out, workspace=ws[0])
+        return out, binding.bdlm_linear_ce_bwd(g["h"], g["w"], g["labels"], out[2], g["weight"], token_chunk=256, out=grads, workspace=ws[1])
+
+    def same(a, b):
+        return all(torch.equal(x, y) for x, y in zip(a[0] + a[1], b[0] + b[1]))
+    ref = step()
+    torch.cuda.synchronize()
+    # several streams at once, each with its own buffers
+    streams = [torch.cuda.Stream() for _ in range(3)]
+    got = []
+    for _ in range(3):
+        for s in streams:
+            with torch.cuda.stream(s):
+                got.append(step())
+    torch.cuda.synchronize()
+    assert all(same(x, ref) for x in got)
+    # one graph, replayed with other contents of the same buffers
+    out, grads = tuple(torch.zeros_like(t) for t in ref[0]), tuple(torch.zeros_like(t) for t in ref[1])
+    p = binding.make_lce_params(T, D, w.V, token_chunk=256)
+    ws = [torch.empty(binding.bdlm_linear_ce_workspace_bytes(p, i), dtype=torch.uint8, device="cuda") for i in (binding.LCE_WS_FWD, binding.LCE_WS_BWD)]
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        step(out, grads, ws)
+    for _ in range(2):
+        graph.replay()
+    torch.cuda.synchronize()
+    assert same((out, grads), ref)
+    g["h"].copy_(g["h"].flip(0))
+    g["labels"].copy_(g["labels"].flip(0))
+    ref = step()
+    graph.replay()
+    torch.cuda.synchronize()
+    assert same((out, grads), ref)
+    assert binding.bdlm_get_device_status() == 0

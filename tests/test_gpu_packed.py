@@ -366,3 +366,25 @@ def test_packed_form_with_head_dimension_64_on_the_tensor_core_kernels():
     _run_and_check(t, 32, binding.IMPL_TCGEN05, prefix=sorted(int(v) for v in rng.integers(0, 513, size=8)), pos0=128)
     _run_and_check(t, 32, binding.IMPL_TCGEN05, prefix=sorted(int(v) for v in rng.integers(0, 513, size=8)), pos0=128,
                    single_pass=True)
+
+
+def test_gathered_order_tables_of_calls_that_are_still_queued():
+    """Calls with different chunk orders one after the other on a busy stream: each has its own tables until it has run."""
+    t = _cuda(_draw(41, 1, 1024, 1024, 0, 4, 2, 128))
+    chunk, n = 128, 8
+    orders = [[(i * m + a) % n for i in range(n)] for m in (1, 3, 5, 7) for a in range(n)]
+    kv = []
+    for o in orders:
+        rows = torch.cat([torch.arange(c * chunk, (c + 1) * chunk) for c in o]).cuda()
+        kv.append((t["k_clean"][:, rows].contiguous(), t["v_clean"][:, rows].contiguous(), (chunk, [c * chunk for c in o])))
+    want = binding.bdlm_attn_fwd_packed(t["q_clean"], *kv[0][:2], None, None, None, 32, kv_chunks=kv[0][2])
+    busy = torch.randn(8192, 8192, device="cuda", dtype=torch.bfloat16)
+    torch.cuda.synchronize()
+    for stream in (torch.cuda.current_stream(), torch.cuda.Stream()):
+        with torch.cuda.stream(stream):
+            for _ in range(20):
+                busy @ busy
+            got = [binding.bdlm_attn_fwd_packed(t["q_clean"], k, v, None, None, None, 32, kv_chunks=c) for k, v, c in kv]
+        torch.cuda.synchronize()
+        for o, l, _, _ in got:
+            assert torch.equal(o, want[0]) and torch.equal(l, want[1])

@@ -49,3 +49,30 @@ def test_two_pass_gradients_of_a_batch_element_do_not_depend_on_the_batch(w):
             assert torch.equal(a[0], b[i])
         for a, b in zip(pu.gpu_bwd(gi, oi, w.block_size, window=w.window, single_pass=False), whole):
             assert torch.equal(a[0], b[i])
+
+
+@pytest.mark.parametrize("w", [
+    Workload("shared_tiles", 1, 4, 1, 128, 1000, 40, seed=10),
+    Workload("shared_tiles_d64", 2, 6, 2, 64, 776, 8, seed=11),
+    Workload("one_cta_per_tile", 1, 2, 2, 128, 296, 8, seed=12),
+    Workload("one_cta_per_tile_d64", 1, 2, 2, 64, 296, 8, seed=13),
+], ids=lambda w: w.name)
+def test_fused_passes_called_one_by_one_agree_with_the_whole_call(w):
+    """By themselves the passes clear the fp32 dQ accumulators in another launch than the whole call does, and are not
+    chained.  Nothing in the workspace may matter; lengths are no multiple of the 64-row step."""
+    g = synth.make_inputs(w, "cuda")
+    out = pu.gpu_fwd(g, w.block_size)
+    whole = pu.gpu_bwd(g, out, w.block_size, single_pass=True)
+    p = binding.make_params(w.batch, w.L, w.block_size, w.H, w.H_kv, w.d, bwd_single_pass=True)
+    ws = torch.empty(binding.bdlm_workspace_bytes(p, binding.BDLM_WS_BWD) // 4, dtype=torch.float32, device="cuda")
+    for order in ((binding.PASS_DSUM, binding.PASS_DKDV, binding.PASS_DQ), (binding.PASS_DSUM | binding.PASS_DKDV,),
+                  (binding.PASS_DSUM, binding.PASS_DKDV | binding.PASS_DQ)):
+        ws.fill_(float("nan"))
+        grads = tuple(torch.full_like(t, float("nan")) for t in whole)
+        for bits in order:
+            pu.gpu_bwd(g, out, w.block_size, single_pass=True, passes=bits, workspace=ws.view(torch.uint8), out=grads)
+        for i, (a, b) in enumerate(zip(grads, whole)):
+            if i in (0, 3):   # dQ: the order in which the key tiles' sums arrive, then one bf16 rounding
+                assert pu.rel_l2(synth.to_f64(a), synth.to_f64(b)) <= 1e-3
+            else:
+                assert torch.equal(a, b), (order, i)
