@@ -542,7 +542,9 @@ size_t fwd_part_bytes(const bdlm_lce_params* p, int run_tiles) {
 // Matrices whose rows are no whole number of 128-byte lines: every 128-byte row of a TMA box then straddles two lines,
 // and the products, which live on L2 bandwidth, take half as long again or more (T = 1531, V ~ 32000: D = 1536 against
 // 1544 forward 103 / 160 us, backward 346 / 600).  From PACK_*_T tokens on, W and h are copied to padded rows first
-// (W of 98 MB: 35 us); the rows of dz, which is ours, are padded in any case.
+// (W of 98 MB: 35 us); the rows of dz, which is ours, are padded in any case.  Without and with the copies at D = 1544, V = 32008
+// (us): forward T = 768 109 / 117, 1024 123 / 124, 1280 156 / 144; backward T = 128 225 / 233, 256 246 / 246, 384 278 / 265,
+// 768 358 / 316.  Where the matrices are small (D = 264, V = 8008) the forward's copies cost 3 us at 1024 tokens.
 constexpr int PACK_FWD_T = 1024, PACK_BWD_T = 384;
 int64_t up64(int64_t x) { return (x + 63) / 64 * 64; }
 bool packs(const bdlm_lce_params* p, int from) { return p->D % 64 != 0 && p->T >= from && ((int64_t)p->V + p->T) * (p->D / 8) < (1ll << 31); }

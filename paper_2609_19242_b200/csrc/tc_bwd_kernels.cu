@@ -1442,6 +1442,15 @@ void tc_bwd_place_dq(KArgs& a, void* extra_ws) {
 //   L = 16384, H = 8 / 1        heavy 2.3 means   4284 / 2717 / 2919
 //   L = 4096, H = 32 / 8        heavy 1.06 means   914 /  920 / 1050
 //   L = 8192, H = 32 / 8        heavy 0.55 means  2755 / 3122 / 4237
+// and at the thresholds:
+//   L = 4096, H = 32 / 8        heavy 1.09 means   806 /  798 /  972
+//   L = 3584, H = 32 / 8        heavy 1.23 means   682 /  639 /  790
+//   L = 3072, H = 32 / 8        heavy 1.42 means   571 /  470 /  585
+//   L = 1536, H = 32 / 8        heavy 2.64 means   248 /  151 /  174
+//   L = 14336, H = 8 / 1        heavy 2.60 means  3789 / 2302 / 2195
+//   L = 12288, H = 8 / 1        heavy 3.02 means  3193 / 1844 / 1625
+//   L = 1280, H = 32 / 8        heavy 3.08 means   200 /  123 /  138
+//   2 x 1024, H = 16 / 8, window 256   1.35 means, 28 steps: 74 / 82 / 121 (few steps: the estimate is rough there)
 // Under MIN_HEAVY steps the exchange eats what the split gives (L = 256: 37 / 36 / 36).
 constexpr double MIN_HEAVY = 24, SPLIT_2 = 1.2, SPLIT_4 = 3.0;
 static int split_key_tiles(const KArgs& a) {
