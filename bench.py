@@ -36,12 +36,12 @@ NAMES6 = ["q_clean", "k_clean", "v_clean", "q_noisy", "k_noisy", "v_noisy"]
 # DRAM traffic (dram__bytes_read.sum + dram__bytes_write.sum) per launch of a kernel from a one-pass ncu capture of
 # this command, keyed by (workload, kernel), each with the digest of the kernel sources it was captured on
 # (kernel_source_digest): a figure is reported only for the build it belongs to.
-_CAPTURED_ON = "4289fc252fec25f2"
+_CAPTURED_ON = "2abc69b5a1b0c168"
 NCU_TRAFFIC = {
-    ("32k", "fwd"): {"bytes": 967480576 + 528095488, "kernel_source": _CAPTURED_ON},
-    ("32k", "bwd_fused"): {"bytes": 5889652992 + 3375495168, "kernel_source": _CAPTURED_ON},
-    ("32k", "bwd_dkdv"): {"bytes": 2371290368 + 249625600, "kernel_source": _CAPTURED_ON},
-    ("32k", "bwd_dq"): {"bytes": 1543090432 + 519066880, "kernel_source": _CAPTURED_ON},
+    ("32k", "fwd"): {"bytes": 980136192 + 522032640, "kernel_source": _CAPTURED_ON},
+    ("32k", "bwd_fused"): {"bytes": 5856034560 + 3336947712, "kernel_source": _CAPTURED_ON},
+    ("32k", "bwd_dkdv"): {"bytes": 2386681088 + 249642752, "kernel_source": _CAPTURED_ON},
+    ("32k", "bwd_dq"): {"bytes": 1542742528 + 519323392, "kernel_source": _CAPTURED_ON},
 }
 TRAFFIC_NOTE = ("dram__bytes_read.sum + dram__bytes_write.sum per launch from a one-pass ncu capture of this command on "
                 "the 32k workload")
@@ -239,7 +239,7 @@ def kernel_source_digest():
     import hashlib
     h = hashlib.sha256()
     csrc = os.path.join(ROOT, "paper_2609_19242_b200", "csrc")
-    for f in ("bdlm_common.cuh", "tc_common.cuh", "tc_kernels.cu", "tc_bwd_kernels.cu"):
+    for f in ("bdlm_common.cuh", "fwd_issue.h", "tc_common.cuh", "tc_kernels.cu", "tc_bwd_kernels.cu"):
         with open(os.path.join(csrc, f), "rb") as fh:
             h.update(fh.read())
     return h.hexdigest()[:16]
@@ -306,8 +306,11 @@ class LayerRun:
         return ["fwd", "bwd_dsum", "bwd_fused" if self.fused else "bwd_dkdv", "bwd_dq"]
 
     def timed_steps(self, K, warmup, barrier, sampler=None):
-        """W warm-up steps, then K timed steps with events between the kernels of a step.  Returns the total time of
-        the K steps (ms, device clock), the per-step times and the mean time per kernel."""
+        """W warm-up steps, then K timed steps: the forward and the backward as a user calls them.  Returns the total time
+        of the K steps (ms, device clock), the per-step times and mean times: of the two calls ("fwd", "bwd_call") from
+        those steps, and of the backward's passes from a few more steps that call them one by one (where the fused
+        kernel's accumulators are cleared by a memset instead of the launch that forms the D rows, and nothing is
+        chained: the passes add up to a little more than the call)."""
         binding = self.binding
         for _ in range(warmup):
             self.run_fwd()
@@ -315,8 +318,7 @@ class LayerRun:
         torch.cuda.synchronize()
         if binding.bdlm_get_device_status() != 0:
             raise RuntimeError("device-side wait timed out during warm-up")
-        names = self.kernel_names()
-        ev = [[torch.cuda.Event(enable_timing=True) for _ in range(len(names) + 1)] for _ in range(K)]
+        ev = [[torch.cuda.Event(enable_timing=True) for _ in range(3)] for _ in range(K)]
         if sampler is not None:
             sampler.start()
             time.sleep(0.25)
@@ -327,20 +329,25 @@ class LayerRun:
             ev[i][0].record()
             self.run_fwd()
             ev[i][1].record()
-            self.run_bwd(passes=binding.PASS_DSUM)
+            self.run_bwd()
             ev[i][2].record()
-            self.run_bwd(passes=binding.PASS_DKDV)
-            ev[i][3].record()
-            self.run_bwd(passes=binding.PASS_DQ)
-            ev[i][4].record()
         e_stop.record()
         barrier()
         ms_total = e_start.elapsed_time(e_stop)
         clocks = sampler.stop() if sampler is not None else None
         if binding.bdlm_get_device_status() != 0:
             raise RuntimeError("device-side wait timed out during the timed region")
-        per_step = [ev[i][0].elapsed_time(ev[i][len(names)]) for i in range(K)]
-        per_kernel = {n: float(np.mean([ev[i][j].elapsed_time(ev[i][j + 1]) for i in range(K)])) for j, n in enumerate(names)}
+        per_step = [e[0].elapsed_time(e[2]) for e in ev]
+        per_kernel = {n: float(np.mean([e[j].elapsed_time(e[j + 1]) for e in ev])) for j, n in enumerate(("fwd", "bwd_call"))}
+        ev = [[torch.cuda.Event(enable_timing=True) for _ in range(4)] for _ in range(min(K, 5))]
+        for e in ev:
+            self.run_fwd()
+            e[0].record()
+            for j, bits in enumerate((binding.PASS_DSUM, binding.PASS_DKDV, binding.PASS_DQ)):
+                self.run_bwd(passes=bits)
+                e[j + 1].record()
+        torch.cuda.synchronize()
+        per_kernel.update({n: float(np.mean([e[j].elapsed_time(e[j + 1]) for e in ev])) for j, n in enumerate(self.kernel_names()[1:])})
         return ms_total, per_step, per_kernel, clocks
 
 
@@ -517,7 +524,9 @@ def run_ours(args, w):
     g, fwd_out, grads, ws = run.g, run.fwd_out, run.grads, run.ws
     like = run.like
 
-    # ---- timed region: K steps, device time, events between the kernels of a step -------------
+    # ---- timed region: K steps, device time, an event between forward and backward ------------
+    # (four launches of the library's kernels a step: forward, D rows, then the fused kernel and the conversion of its dQ or
+    # the two passes)
     K = args.steps
     names = run.kernel_names()
     sampler = ClockSampler(physical_gpu_index(local)) if rank == 0 else None
@@ -655,7 +664,7 @@ def run_ours(args, w):
                        "backward": "fused (one kernel; dQ through fp32 add-reductions)" if fused else "two-pass (dK/dV, then dQ)"},
             "pct_of_bf16_peak": {"measured_burst": 100 * pct["frac_burst"], "measured_sustained": 100 * pct["frac_sustained"],
                                  "nominal_2250": 100 * pct["frac_nominal_2250"], "source": peaks["source"]},
-            "clocks": clocks, "gclk_per_step": clock_normalised(ms_step, clocks), "e2e": e2e, "gpu_launches": (6 if fused else 5) * K, "roofline": roofline, "cpu_baseline": cpu,
+            "clocks": clocks, "gclk_per_step": clock_normalised(ms_step, clocks), "e2e": e2e, "gpu_launches": 4 * K, "roofline": roofline, "cpu_baseline": cpu,
             "other_configs": others}
     print(json.dumps(line), flush=True)
     if world > 1:

@@ -116,7 +116,8 @@ int bdlm_attn_fwd(const bdlm_params* p,
  * fp32 summation order when the fused kernel runs (see bdlm_params.bwd_single_pass for which one
  * does).  Requires the full clean key range.
  * The workspace holds D_i = sum_d dO_i,d * O_i,d and, for the fused kernel, an fp32 dQ accumulator
- * [batch, H, rows rounded up to 64, 128] per query stream; nothing in it has to be initialised or kept between calls.
+ * [batch, H, rows rounded up to 64, d] per query stream (for d = 64 the reported size still counts rows of 128); nothing
+ * in it has to be initialised or kept between calls.
  * bdlm_workspace_bytes(p, BDLM_WS_BWD) reports the size for p->bwd_single_pass; with the default
  * (BDLM_BWD_AUTO) that is the fused kernel's size, and a call given less than that -- but at least
  * the BDLM_BWD_TWO_PASS size -- runs the two-pass kernels.

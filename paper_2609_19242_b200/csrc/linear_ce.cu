@@ -10,12 +10,15 @@
 //                      dH_c = dz W          epilogue: bf16 store
 //                      dW  += dz^T H_c      epilogue: bf16 store, or fp32 accumulation over the chunks
 //
-// Tiles are 128 x 256 with 64-deep contraction steps: TMA (128-byte swizzle) fills a 4-stage ring of A (16 KB) and
-// B (32 KB) tiles, one warp issues tcgen05.mma (M = 128, N = 256, K = 16) into one of two 256-column accumulators in
-// tensor memory, and four epilogue warps (one thread per accumulator row) drain the other one meanwhile.  An operand
-// is either K-major (rows of the matrix = rows of the tile, contraction contiguous) or MN-major (rows of the matrix
-// = contraction index, M/N contiguous), so W, H and dz are used as they lie in memory, never transposed.
-// CTAs are persistent: work items (an M tile x a run of N tiles) are dealt round-robin in an order that keeps the
+// Tiles are 128 rows by at most 256 columns (the width is chosen per product, see choose_tiling) with 64-deep contraction
+// steps: TMA (128-byte swizzle) fills a 4-stage ring of A (16 KB) and B (up to 32 KB) tiles, one warp issues tcgen05.mma
+// (M = 128, N = the tile's width, K = 16) into one of two 256-column accumulators in tensor memory, and four epilogue warps
+// (one thread per accumulator row) drain the other one meanwhile.  An operand is either K-major (rows of the matrix = rows of
+// the tile, contraction contiguous) or MN-major (rows of the matrix = contraction index, M/N contiguous; one 3-D load per tile
+// where its 64-column panels are whole, a 64 x 64 box each otherwise), so W, H and dz are never transposed; W and H whose rows
+// are no whole number of 128-byte lines are copied to padded rows first where that pays.  An element of a product is one
+// accumulation over the whole contraction (dW: over a token chunk) whatever the tiling.
+// CTAs are persistent: work items (an M tile x some N tiles) are dealt round-robin in an order that keeps the
 // operand shared by concurrently running CTAs in L2.  Every wait is bounded and abortable.
 #include <math.h>
 

@@ -129,14 +129,14 @@ def test_all_positions_ignored_gives_zero_loss_and_zero_gradients():
 
 
 @pytest.mark.parametrize("w", [
-    LceWorkload("split_contraction", 150, 72, 8200),           # dH in eight pieces of the vocabulary, the last one short
+    LceWorkload("split_contraction", 150, 72, 8200),           # few dH tiles, each a long contraction
     LceWorkload("narrow_tiles", 520, 264, 9000),               # D one tile and 8 columns: tiles narrower than 256
     LceWorkload("odd_half_chunks", 390, 512, 5000),            # 144-column tiles: the last 32-column chunk reaches past them
-    LceWorkload("many_short_runs", 260, 64, 20008),            # more partial (maximum, sum) pairs than one per 2048 logits
+    LceWorkload("many_short_runs", 260, 64, 20008),            # 79 vocabulary runs with a full workspace, 10 with the smallest
 ], ids=lambda w: w.name)
 def test_tilings_and_split_contraction(w):
     one = _check(w)
-    # dH does not depend on the token chunks; the smallest accepted workspace takes the coarse tiling and one piece
+    # dH does not depend on the token chunks; the smallest accepted workspace has longer runs and no copies
     g = {k: v.cuda() for k, v in synth.make_lce_inputs(w, "cpu").items()}
     dh, _ = binding.bdlm_linear_ce_bwd(g["h"], g["w"], g["labels"], one[2], g["weight"], token_chunk=128)
     assert torch.equal(dh, one[3])
