@@ -66,7 +66,8 @@ typedef struct {
                                   Each CTA adds its dQ tiles into an fp32 accumulator in the workspace (bulk add-reductions),
                                   so dQ is reproducible only up to fp32 summation order; dK and dV are bitwise reproducible
                                   (fixed order) from call to call of the same sizes, while their last bits may depend on
-                                  the batch size and the number of heads (on how many CTAs share a key tile).  Needs the workspace bdlm_workspace_bytes[_packed] reports for this setting
+                                  the batch size and the number of heads (on how many CTAs share a key tile).
+                                  Needs the workspace bdlm_workspace_bytes[_packed] reports for this setting
                                   (BDLM_ERR_WORKSPACE_TOO_SMALL otherwise); with impl = 1 (the mma.sync kernels) the
                                   two-pass path runs.
                                   BDLM_BWD_TWO_PASS (2): dK/dV pass + dQ pass, fixed summation order, every gradient

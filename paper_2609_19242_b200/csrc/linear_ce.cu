@@ -466,16 +466,16 @@ struct Operand { const void* ptr; int64_t ld; int mn; bool whole; };
 
 // How a product is cut into tiles: with fixed 256-column tiles and runs of eight, a ragged or small product leaves a
 // part of the chip idle (T = 1531, D = 1544, V = 32008: 192 forward items on 148 SMs, dH 84 tiles, the last of every
-// seven 8 columns wide).  The width of an N tile and the length of a run are chosen for the shortest launch: rounds of
-// items per SM times the clocks of one item.  A 16-deep slice of an M = 128 MMA takes bn / 2 clk, and no less than its
-// operands need from shared memory at 128 bytes per clk.  A
-// narrower tile or a shorter run has to promise 5 % (8192 x 4096 x 128256 would gain 3 % by this count and lost 1 %: what
-// bounds it is power).  The forward keeps 256 columns, where its runs end (see RUN_TILES).  A B operand
-// that lies MN-major keeps 256 columns where it has them (dH at T = 4096, D = 4096 in one piece: 5.7 ms with 240 or 192
-// columns against 3.4: its panels then start off the 128-byte lines, or a tile's rows off the 512 bytes they share),
-// unless its tiles leave SMs idle: dH (min_bn = 64) then takes 64 columns or more, which changes no bit of it (V = 32008: T = 1531,
-// D = 1536 backward 415 -> 380 us, T = 384, D = 1544 305 -> 264; T = 149, D = 224, V = 50912 280 -> 208).
-// Forward / dz at T = 1531, D = 1544, V = 32008: 234 -> 160 and 275 -> 188 us.
+// seven 8 columns wide).  The width of an N tile and the number of tiles per item are chosen for the shortest launch: rounds
+// of items per SM times the clocks of one item.  A 16-deep slice of an M = 128 MMA takes bn / 2 clk, and no less than its
+// operands need from shared memory at 128 bytes per clk.  A narrower tile or fewer tiles have to promise 5 % (8192 x 4096 x
+// 128256 would gain 3 % by this count and lost 1 %: what bounds it is power).  No choice changes a bit of a result.
+//   forward   256 columns, where its vocabulary runs end (see RUN_TILES); 1 to 8 tiles per item
+//   dz        128 to 256 columns in steps of 16; 1 to 8 tiles per item.  T = 1531, D = 1544, V = 32008: 275 -> 188 us
+//   dH, dW    256 columns where the matrix has them (their B operand lies MN-major; dH at T = 4096, D = 4096: 5.7 ms with 240
+//             or 192 columns against 3.4: its panels then start off the 128-byte lines, or a tile's rows off the 512 bytes they
+//             share), unless dH's tiles leave SMs idle: then 64 columns or more (min_bn = 64; V = 32008: T = 1531, D = 1536
+//             backward 415 -> 380 us, T = 384, D = 1544 305 -> 264; T = 149, D = 224, V = 50912 280 -> 208)
 struct Tiling { int bn, n_run; };
 Tiling choose_tiling(int M, int N, int K, int min_bn, int min_run, int max_run, int epi_per_32, int b_mn) {
   const long long m_tiles = (M + BM - 1) / BM, sms = device_sm_count();
@@ -500,7 +500,9 @@ Tiling choose_tiling(int M, int N, int K, int min_bn, int min_run, int max_run, 
   }
   return best;
 }
-constexpr int EPI_CLK_LSE = 350, EPI_CLK_DZ = 500, EPI_CLK_STORE = 300;   // per 32 columns, rough
+// Clocks of an epilogue per 32 columns.  Rough, but they decide only where the contraction is short: 8 x 350 clk for a tile
+// against 512 per 64-deep step of its MMAs, which run under it.
+constexpr int EPI_CLK_LSE = 350, EPI_CLK_DZ = 500, EPI_CLK_STORE = 300;
 
 template <int EPI>
 cudaError_t launch_gemm(GemmArgs a, const Operand& A, const Operand& B, cudaStream_t st, bool chained) {

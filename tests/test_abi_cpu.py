@@ -136,6 +136,12 @@ def test_linear_ce_arguments_are_checked_without_a_device():
     assert binding.bdlm_linear_ce_workspace_bytes(good, binding.LCE_WS_BWD) == 256 * 512 * 2          # one chunk: dz only
     big = binding.make_lce_params(1000, 64, 512, token_chunk=256)
     assert binding.bdlm_linear_ce_workspace_bytes(big, binding.LCE_WS_BWD) == 256 * 512 * 2 + 512 * 64 * 4   # + fp32 dW
+    odd = binding.make_lce_params(1030, 72, 5000)
+    r, per = 3, 4352   # vocabulary runs of 2048, 4 bytes a token rounded up to 256
+    assert binding.bdlm_linear_ce_workspace_bytes(odd, binding.LCE_WS_FWD_LEAST) == (2 * r + 1) * per + 256
+    assert binding.bdlm_linear_ce_workspace_bytes(odd, binding.LCE_WS_BWD_LEAST) == 1152 * 5000 * 2
+    for full, least in ((binding.LCE_WS_FWD, binding.LCE_WS_FWD_LEAST), (binding.LCE_WS_BWD, binding.LCE_WS_BWD_LEAST)):
+        assert binding.bdlm_linear_ce_workspace_bytes(odd, full) > binding.bdlm_linear_ce_workspace_bytes(odd, least)
     for kw in (dict(T=0, D=64, V=512), dict(T=8, D=60, V=512), dict(T=8, D=64, V=500), dict(T=8, D=64, V=512, token_chunk=100),
                dict(T=8, D=64, V=512, grad_loss=float("nan"))):
         p = binding.make_lce_params(**kw)
