@@ -160,10 +160,11 @@ __global__ void __launch_bounds__(256) bwd_prepare_kernel(const PrepArgs pa) {
         ua[j] = make_uint4(0u, 0u, 0u, 0u); ub[j] = ua[j];
       }
     }
-    if (r0 == 0 && dq32 != nullptr) {   // the stores go out under the first loads
+    if (r0 == 0 && dq32 != nullptr) {   // the stores go out under the first loads; the last rows' block clears the padding too
+      const int nz = l0 + PREP_ROWS >= L ? dq32_rows - l0 : PREP_ROWS;
       for (int hi = 0; hi < nh; ++hi) {
         float4* z = reinterpret_cast<float4*>(dq32 + (((int64_t)b * H + h0 + hi) * dq32_rows + l0) * D);
-        for (int e = threadIdx.x; e < nl * D / 4; e += 256) z[e] = make_float4(0.f, 0.f, 0.f, 0.f);
+        for (int e = threadIdx.x; e < nz * D / 4; e += 256) z[e] = make_float4(0.f, 0.f, 0.f, 0.f);
       }
     }
 #pragma unroll

@@ -11,15 +11,15 @@
 //               (Eq. correctness-query-gradient).
 //   fused       the dK/dV unit with 64-query steps: the same CTA also forms dQ^T = K^T dS^T per step and a
 //               fourth warpgroup adds it into an fp32 dQ accumulator through TMA bulk reductions
-//               (5 GEMMs per pair instead of 7; selected with bwd_single_pass).
+//               (5 GEMMs per pair instead of 7; selected with bwd_single_pass).  Large calls of head dimension 128 run on
+//               pairs of CTAs instead (tc_bwd_pair.cu).
 //
 // All are warp-specialised: warp 8 issues TMA loads, warp 9 issues tcgen05.mma (the whole warp walks the
 // loop convergently, one elected lane issues), warps 0-7 (two warpgroups, each owning half of the 128
 // score columns of every TMEM lane) recompute P = exp(S - LSE) and dS = P * (dP - D) and hand them back
 // to the tensor core (dS as a TMEM-resident A operand; P^T of the dK/dV pass through a shared-memory tile).
 // Every wait is bounded and abortable.
-#include "tc_common.cuh"
-#include "tc_launch.h"
+#include "tc_bwd_common.cuh"
 
 namespace bdlm {
 namespace {
@@ -32,71 +32,7 @@ struct BwdMaps {
 };
 
 constexpr int BWD_THREADS = 320;
-constexpr int TILE_BYTES = 2 * PANEL_BYTES;
 constexpr uint32_t IDESC_KK = make_idesc(128, 128, false, false);   // A, B both K-major
-// B MN-major (a [k][n] tile as loaded) with N = the head dimension
-__host__ __device__ constexpr uint32_t idesc_km(int d) { return make_idesc(128, d, false, true); }
-
-// One operand tile of head `head`: D / 64 panels of 64 columns (D = head dimension, 128 or 64).
-template <int D>
-__device__ __forceinline__ void tma_tile(uint32_t dst, const CUtensorMap* map, uint32_t bar, int head, int row0, int b) {
-  tma_load_3d(dst, map, bar, head * D, row0, b);
-  if (D == 128) tma_load_3d(dst + PANEL_BYTES, map, bar, head * D + 64, row0, b);
-}
-
-// The elementwise work of a tile, two elements per instruction where the arithmetic allows it: the compute warps are bound
-// by instruction issue beside the exponential unit (L = 2048, H = 32: fused kernel 192 -> 189 us, windowed 32K 2.95 -> 2.85 ms,
-// dQ pass at L = 16K, H = 8 1169 -> 1107 us; at the power cap, 32K, no change).  Scores x become P = exp2(x * scale - lse); hidden elements (bits of
-// [lo, hi) clear) become zero.  nlse: minus the LSE rows in log2 units, one per element (-inf where there is no row).
-template <int N>
-__device__ __forceinline__ void exp_tile(uint32_t (&x)[N], uint64_t scale2, const float* nlse) {
-#pragma unroll
-  for (int c = 0; c < N; c += 4) {
-    const ulonglong2 z = *reinterpret_cast<const ulonglong2*>(nlse + c);
-    float p0, p1, p2, p3;
-    unpack_f32x2(fma_f32x2(pack_f32x2(__uint_as_float(x[c]), __uint_as_float(x[c + 1])), scale2, z.x), p0, p1);
-    unpack_f32x2(fma_f32x2(pack_f32x2(__uint_as_float(x[c + 2]), __uint_as_float(x[c + 3])), scale2, z.y), p2, p3);
-    x[c] = __float_as_uint(exp2f(p0)); x[c + 1] = __float_as_uint(exp2f(p1));
-    x[c + 2] = __float_as_uint(exp2f(p2)); x[c + 3] = __float_as_uint(exp2f(p3));
-  }
-}
-template <int N>
-__device__ __forceinline__ void hide_tile(uint32_t (&x)[N], int lo, int hi) {
-#pragma unroll
-  for (int g = 0; g < N / 32; ++g) {
-    const uint32_t seen = interval_bits(lo - 32 * g, hi - 32 * g);
-#pragma unroll
-    for (int e = 0; e < 32; ++e) x[32 * g + e] = (seen >> e) & 1u ? x[32 * g + e] : 0u;
-  }
-}
-// dS = P * (dP - D) as bf16 pairs; nd: minus the D of each element.
-template <int N>
-__device__ __forceinline__ void ds_tile(uint32_t (&pk)[N / 2], const uint32_t (&x)[N], const uint32_t (&y)[N], const float* nd) {
-#pragma unroll
-  for (int c = 0; c < N; c += 4) {
-    const ulonglong2 d = *reinterpret_cast<const ulonglong2*>(nd + c);
-    float d0, d1, d2, d3;
-    unpack_f32x2(mul_f32x2(pack_f32x2(__uint_as_float(x[c]), __uint_as_float(x[c + 1])),
-                           add_f32x2(pack_f32x2(__uint_as_float(y[c]), __uint_as_float(y[c + 1])), d.x)), d0, d1);
-    unpack_f32x2(mul_f32x2(pack_f32x2(__uint_as_float(x[c + 2]), __uint_as_float(x[c + 3])),
-                           add_f32x2(pack_f32x2(__uint_as_float(y[c + 2]), __uint_as_float(y[c + 3])), d.y)), d2, d3);
-    pk[c / 2] = pack_bf16(d0, d1);
-    pk[c / 2 + 1] = pack_bf16(d2, d3);
-  }
-}
-
-// Write a thread's 128 accumulator columns (4 x 32) as bf16 to a global row, scaled.
-__device__ __forceinline__ void store_row_chunk(bf16* dst, const uint32_t (&v)[32], float scale) {
-#pragma unroll
-  for (int e8 = 0; e8 < 4; ++e8) {
-    uint4 o;
-    uint32_t* po = reinterpret_cast<uint32_t*>(&o);
-#pragma unroll
-    for (int e = 0; e < 4; ++e)
-      po[e] = pack_bf16(__uint_as_float(v[e8 * 8 + 2 * e]) * scale, __uint_as_float(v[e8 * 8 + 2 * e + 1]) * scale);
-    *reinterpret_cast<uint4*>(dst + e8 * 8) = o;
-  }
-}
 
 // =============================================================================================
 // dK/dV pass
@@ -116,43 +52,6 @@ constexpr int DKDV_NWG = 2;                          // compute warpgroups; each
 constexpr int DKDV_CW = 128 / DKDV_NWG;
 constexpr int DKDV_THREADS = (4 * DKDV_NWG + 2) * 32;
 constexpr int DKDV_PRODUCER = 4 * DKDV_NWG, DKDV_ISSUER = 4 * DKDV_NWG + 1;
-
-struct QStep { int qs, h, q0; };
-
-// The steps of a key tile: every (query tile, query stream, head of the group) that sees it.  Segment A holds the
-// clean query tiles [a0, a1) (for a noisy key tile: the noisy ones), segment B the noisy query tiles [b0, b1) of a
-// clean key tile, both in units of the step's query rows.  Segment A is walked first, then segment B, each from its
-// last query tile down with all heads of the group inside a tile: CTAs that start together then meet the same
-// Q / dO tiles -- and, in the fused kernel, the same dQ accumulator tiles -- at the same time, so that those stay in
-// L2 between the CTAs that share them.  (Alternating the two streams tile by tile as well was measured and is
-// slower: 4.7 against 3.3 ms on the sliding-window workload.)  Counters only, no division; the order is fixed, so
-// dK / dV stay bitwise reproducible.
-//
-// When a key tile is split over a cluster (see key_unit), its steps are dealt out one by one: CTA `part` of `parts`
-// takes steps part, part + parts, ... of the same order.
-struct StepWalk {
-  int a1, na, b1, nb, G, h_first, qs_a, rows, part, parts;
-  int t, hh;   // tile counter over both segments, head within the group
-  __device__ __forceinline__ int total() const { return (na + nb) * G; }
-  __device__ __forceinline__ int count() const { return max(0, (total() - part + parts - 1) / parts); }
-  __device__ __forceinline__ void init(int a0, int na_, int b0, int nb_, int G_, int h_first_, int qs_a_, int rows_, int part_, int parts_) {
-    na = na_; nb = nb_; a1 = a0 + na_ - 1; b1 = b0 + nb_ - 1; G = G_; h_first = h_first_; qs_a = qs_a_; rows = rows_;
-    part = part_; parts = parts_;
-    t = 0; hh = part_;
-    while (hh >= G) { hh -= G; ++t; }
-  }
-  __device__ __forceinline__ QStep cur() const {
-    QStep s;
-    s.h = h_first + hh;
-    if (t < na) { s.qs = qs_a; s.q0 = (a1 - t) * rows; }
-    else { s.qs = NOISY; s.q0 = (b1 - (t - na)) * rows; }
-    return s;
-  }
-  __device__ __forceinline__ void next() {
-    hh += parts;
-    while (hh >= G) { hh -= G; ++t; }
-  }
-};
 
 // ---------------------------------------------------------------- key tiles split over a cluster
 // Short sequences have few key tiles and the first of them carries twice the mean work: with one CTA per key tile the
@@ -179,9 +78,6 @@ __device__ __forceinline__ KeyUnit key_unit(const TileGrid& tg) {
     u.part = 0; u.parts = 1;
   }
   return u;
-}
-__device__ __forceinline__ void cluster_sync() {
-  asm volatile("barrier.cluster.arrive.release;\n\tbarrier.cluster.wait.acquire;" ::: "memory");
 }
 __device__ __forceinline__ float4 ld_peer(uint32_t addr, int rank) {
   float4 v;
@@ -1369,6 +1265,7 @@ struct ConvertArgs {
   int rows[2], src_rows[2];
   int blocks_clean, H;
   float scale;
+  bool halves;   // D = 128: a block of 64 rows lies as two [64 x 64] halves of the head dimension (the pairs' kernel)
 };
 template <int D>
 __global__ void __launch_bounds__(256) dq_convert_kernel(const ConvertArgs ca) {
@@ -1381,13 +1278,15 @@ __global__ void __launch_bounds__(256) dq_convert_kernel(const ConvertArgs ca) {
   const int h = i % H;
   i /= H;
   const int l0 = (i % tiles) * 64 + (threadIdx.x >> 5) * U, b = i / tiles, lane = threadIdx.x & 31;
+  const int row = ca.halves ? D / 2 : D;
   const float* src = of(ca.src) + (((int64_t)b * H + h) * src_rows + l0) * D;
+  if (ca.halves) src += -(l0 & 63) * (D / 2) + (lane >> 4) * (64 * 64 - 64);
   bf16* dst = of(ca.dst) + (((int64_t)b * rows + l0) * H + h) * D;
   const int n = min(U, rows - l0);
   if (D == 128) {
     float4 u[U];
 #pragma unroll
-    for (int j = 0; j < U; ++j) if (j < n) u[j] = __ldcs(reinterpret_cast<const float4*>(src + j * D) + lane);
+    for (int j = 0; j < U; ++j) if (j < n) u[j] = __ldcs(reinterpret_cast<const float4*>(src + j * row) + lane);
 #pragma unroll
     for (int j = 0; j < U; ++j) {
       if (j < n) {
@@ -1453,7 +1352,8 @@ void tc_bwd_place_dq(KArgs& a, void* extra_ws) {
 //   2 x 1024, H = 16 / 8, window 256   1.35 means, 28 steps: 74 / 82 / 121 (few steps: the estimate is rough there)
 // Under MIN_HEAVY steps the exchange eats what the split gives (L = 256: 37 / 36 / 36).
 constexpr double MIN_HEAVY = 24, SPLIT_2 = 1.2, SPLIT_4 = 3.0;
-static int split_key_tiles(const KArgs& a) {
+struct KeyLoad { double heavy, mean, total; };   // steps of HT query rows: of the first clean key tile, per SM, of all clean key tiles of a KV head
+static KeyLoad key_load(const KArgs& a) {
   constexpr int rows = HT;
   const double W = a.window > 0 ? a.window : 0;
   double heavy = 0, total = 0;
@@ -1464,10 +1364,34 @@ static int split_key_tiles(const KArgs& a) {
     heavy += W > 0 ? min(nq, (W + TILE) / rows + 1) : nq;
     total += nq * ((W > 0 ? min(W, seen) : seen) / TILE + 1);
   }
-  heavy *= a.G;
-  const double mean = total * a.G * a.Hkv * a.batch / device_sm_count();
-  if (heavy < MIN_HEAVY || heavy < SPLIT_2 * mean) return 1;
-  return heavy < SPLIT_4 * mean ? 2 : 4;
+  total *= a.G;
+  return {heavy * a.G, total * a.Hkv * a.batch / device_sm_count(), total};
+}
+static int split_key_tiles(const KeyLoad& l) {
+  if (l.heavy < MIN_HEAVY || l.heavy < SPLIT_2 * l.mean) return 1;
+  return l.heavy < SPLIT_4 * l.mean ? 2 : 4;
+}
+
+// Whether pairs of CTAs (tc_bwd_pair_kernel) take the call: head dimension 128, key tiles not shared (a pair has two of them), and
+// enough work for what a pair does more.  In 128 x 128 tiles: its two key tiles see one query tile more in their hull than each by
+// itself wherever a query stream's limit passes them, noisy key tiles two (half as much again, as measured, for masking them),
+// and a unit's start and end cost it 3.6 tiles more than two CTAs'.  Fused backward, one CTA per tile / pairs (us, whole
+// call), by that extra over the tiles there are:
+//   0.015   L = 32768, H = 32 / 8                  40770 / 37860
+//   0.040   L = 12288, H = 32 / 8                   6400 /  6070
+//   0.051   L = 16384, H = 8 / 8                    2690 /  2640
+//   0.059   2 x 8192, H = 16 / 4                    2980 /  2850
+//   0.059   L = 32768, H = 32 / 8, window 4096     11540 / 11010
+//   0.078   L = 6144, H = 32 / 8                    1760 /  1730
+//   0.093   L = 5120, H = 32 / 8                    1230 /  1220
+//   0.100   L = 8192, H = 16 / 16                   1523 /  1540
+//   0.115   2 x 4096, H = 32 / 8                    1690 /  1710
+//   0.115   L = 32768, H = 32 / 8, window 2048      6390 /  6550
+//   0.132   3 x 6144, H = 8 / 8                     1367 /  1399
+constexpr double PAIR_EXTRA = 0.09, PAIR_MASKED = 1.5, PAIR_UNIT = 3.6;
+static bool pairs_pay(const KArgs& a, const KeyLoad& l) {
+  const double tiles = l.total * HT / TILE, pairs_c = a.q[CLEAN] != nullptr ? a.Lqc / 256.0 : 0, pairs_n = a.q[NOISY] != nullptr ? a.Ln / 256.0 : 0;
+  return PAIR_MASKED * a.G * (pairs_c + 3 * pairs_n) + PAIR_UNIT * (a.L / 256.0 + pairs_n) <= PAIR_EXTRA * tiles;
 }
 
 // One CTA, or one cluster of tg.parts CTAs, per unit of the grid.
@@ -1505,11 +1429,19 @@ static cudaError_t launch_tc_bwd_d(const KArgs& a, int passes, cudaStream_t st) 
         const size_t rows = (size_t)a.dq32_rows[CLEAN] + a.dq32_rows[NOISY];
         if ((e = cudaMemsetAsync(a.dq32[CLEAN], 0, rows * a.batch * a.H * D * sizeof(float), st)) != cudaSuccess) return e;
       }
-      auto kern = a.trace ? tc_bwdf_kernel<true, D> : tc_bwdf_kernel<false, D>;
-      TileGrid tg = make_tile_grid((max(a.L, a.k[NOISY] != nullptr ? a.Ln : 0) + TILE - 1) / TILE, a.Hkv, a.batch * 2);
-      tg.parts = split_key_tiles(a);
-      if ((e = launch_units(kern, tg, BF_THREADS, BF_SMEM, st, maps, a, status, after_rows)) != cudaSuccess) return e;
+      const KeyLoad load = key_load(a);
+      const int parts = split_key_tiles(load);
+      const bool pairs = D == 128 && parts == 1 && pairs_pay(a, load);
+      if (pairs) {
+        if ((e = launch_tc_bwd_pair(a, st, after_rows)) != cudaSuccess) return e;
+      } else {
+        auto kern = a.trace ? tc_bwdf_kernel<true, D> : tc_bwdf_kernel<false, D>;
+        TileGrid tg = make_tile_grid((max(a.L, a.k[NOISY] != nullptr ? a.Ln : 0) + TILE - 1) / TILE, a.Hkv, a.batch * 2);
+        tg.parts = parts;
+        if ((e = launch_units(kern, tg, BF_THREADS, BF_SMEM, st, maps, a, status, after_rows)) != cudaSuccess) return e;
+      }
       ConvertArgs ca = {};
+      ca.halves = pairs;
       long long blocks[2];
       for (int s2 = 0; s2 < 2; ++s2) {
         ca.src[s2] = a.dq32[s2]; ca.dst[s2] = a.dq[s2];
