@@ -10,9 +10,10 @@
 //                      dH_c = dz W          epilogue: bf16 store
 //                      dW  += dz^T H_c      epilogue: bf16 store, or fp32 accumulation over the chunks
 //
-// Tiles are 128 rows by at most 256 columns (the width is chosen per product, see choose_tiling) with 64-deep contraction
-// steps: TMA (128-byte swizzle) fills a 4-stage ring of A (16 KB) and B (up to 32 KB) tiles, one warp issues tcgen05.mma
-// (M = 128, N = the tile's width, K = 16) into one of two 256-column accumulators in tensor memory, and four epilogue warps
+// Tiles are 256 rows by at most 256 columns on a pair of CTAs, or 128 rows on one CTA (see choose_tiling), with 64-deep
+// contraction steps: TMA (128-byte swizzle) fills a ring of A (16 KB) and B (up to 32 KB; of a pair each CTA loads half) tiles, one
+// warp -- of a pair, that of rank 0 -- issues tcgen05.mma (M = 128 or 256, N = the tile's width, K = 16) into one of two
+// 256-column accumulators in tensor memory, and four epilogue warps
 // (one thread per accumulator row) drain the other one meanwhile.  An operand is either K-major (rows of the matrix = rows of
 // the tile, contraction contiguous) or MN-major (rows of the matrix = contraction index, M/N contiguous; one 3-D load per tile
 // where its 64-column panels are whole, a 64 x 64 box each otherwise), so W, H and dz are never transposed; W and H whose rows
@@ -33,12 +34,18 @@ using namespace tc;
 using bf16 = __nv_bfloat16;
 
 constexpr int BM = 128, BN = 256, BK = 64;
-constexpr int STAGES = 4;
 constexpr int A_BYTES = BM * BK * 2;
-constexpr int B_BYTES = BN * BK * 2;
-constexpr int STAGE_BYTES = A_BYTES + B_BYTES;
-constexpr int G_BARS = STAGES * STAGE_BYTES;
-constexpr int G_SMEM = G_BARS + 256 + 1024;      // barriers, TMEM slot, abort flag; slack for 1024-byte alignment
+// PAIR: two CTAs work on a tile of 256 rows, 128 each, and each holds half of B's columns: a third less through L2 and shared
+// memory per product, and the shorter stages make room for six.  The sums are the same bit for bit.  One CTA / pairs (us): 4096 x
+// 2048 x 50304 forward 613 / 601, backward 2070 / 1869; 2194 x 2816 x 107056 977 / 950 and 3622 / 3236; 1531 x 1544 x 32008 171 /
+// 158 and 494 / 465.  (MMAs of the pair run at the rate of one CTA's, 128 x 256 x 16 in 129 clk on each SM; what shrinks is the
+// energy, at the power cap, and the load on L2.)
+template <bool PAIR> struct Ring {
+  static constexpr int B_BYTES = BN * BK * 2 / (PAIR ? 2 : 1), STAGE_BYTES = A_BYTES + B_BYTES;
+  static constexpr int STAGES = PAIR ? 6 : 4;
+  static constexpr int BARS = STAGES * STAGE_BYTES;
+  static constexpr int SMEM = BARS + 256 + 1024;   // barriers, TMEM slot, abort flag; slack for 1024-byte alignment
+};
 constexpr int G_THREADS = 192;                   // warps 0-3 epilogue, warp 4 TMA, warp 5 MMA
 constexpr int MN_PANEL = BK * 128;               // an MN-major panel: 64 contraction rows x 64 M/N elements
 
@@ -50,7 +57,8 @@ enum { K_MAJOR = 0, MN_PANELS = 1, MN_BOXES = 2 };
 
 struct GemmArgs {
   int M, N, K;
-  int bn;                                // width of an N tile: a multiple of 16, at most BN
+  int bn;                                // width of an N tile: a multiple of 16 (of a pair 32), at most BN
+  bool pair;                             // a tile of 256 rows per pair of CTAs
   int m_tiles, n_tiles, n_run, n_runs;   // an item = one M tile x n_run consecutive N tiles; n_runs = ceil(n_tiles / n_run)
   int m_inner;                           // item order: 1 = consecutive items share the N run, 0 = share the M tile
   int a_mn, b_mn;                        // operand layouts: K_MAJOR, MN_PANELS (one load per tile), MN_BOXES (one per 64-column panel)
@@ -86,12 +94,25 @@ __device__ __forceinline__ void tma_load_panels_e(uint32_t dst, const CUtensorMa
       ::"r"(dst), "l"(reinterpret_cast<uint64_t>(map)), "r"(bar), "r"(row), "r"(panel), "r"(elected) : "memory");
 }
 
-// Walks the CTA's tiles in the order every role uses.
+__device__ __forceinline__ void tma_load_2d_pair_e(uint32_t dst, const CUtensorMap* map, uint32_t peer_bar, int x, int y, uint32_t elected) {
+  asm volatile(
+      "{\n\t.reg .pred q;\n\tsetp.ne.b32 q, %5, 0;\n\t"
+      "@q cp.async.bulk.tensor.2d.cta_group::2.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4}], [%2];\n\t}"
+      ::"r"(dst), "l"(reinterpret_cast<uint64_t>(map)), "r"(peer_bar), "r"(x), "r"(y), "r"(elected) : "memory");
+}
+__device__ __forceinline__ void tma_load_panels_pair_e(uint32_t dst, const CUtensorMap* map, uint32_t peer_bar, int row, int panel, uint32_t elected) {
+  asm volatile(
+      "{\n\t.reg .pred q;\n\tsetp.ne.b32 q, %5, 0;\n\t"
+      "@q cp.async.bulk.tensor.3d.cta_group::2.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {0, %3, %4}], [%2];\n\t}"
+      ::"r"(dst), "l"(reinterpret_cast<uint64_t>(map)), "r"(peer_bar), "r"(row), "r"(panel), "r"(elected) : "memory");
+}
+
+// Walks the CTA's (or the pair's) tiles in the order every role uses.
 struct TileWalk {
-  int item, items, mt, nrun, nt, nt_end;
+  int item, items, mt, nrun, nt, nt_end, stride;
   const GemmArgs* a;
-  __device__ __forceinline__ void start(const GemmArgs& args) {
-    a = &args; items = args.m_tiles * args.n_runs; item = blockIdx.x; nt = 0; nt_end = 0;
+  __device__ __forceinline__ void start(const GemmArgs& args, int first, int step) {
+    a = &args; items = args.m_tiles * args.n_runs; item = first; stride = step; nt = 0; nt_end = 0;
     if (item < items) open();
   }
   __device__ __forceinline__ void open() {
@@ -103,34 +124,42 @@ struct TileWalk {
   __device__ __forceinline__ bool valid() const { return item < items; }
   __device__ __forceinline__ void next() {
     if (++nt < nt_end) return;
-    item += gridDim.x;
+    item += stride;
     if (item < items) open();
   }
 };
 
-template <int EPI>
+template <int EPI, bool PAIR>
 __global__ void __launch_bounds__(G_THREADS, 1)
 lce_gemm_kernel(const __grid_constant__ GemmMaps maps, const GemmArgs a, int* __restrict__ status) {
+  constexpr int STAGES = Ring<PAIR>::STAGES, STAGE_BYTES = Ring<PAIR>::STAGE_BYTES, G_BARS = Ring<PAIR>::BARS;
   wait_for_predecessor();
   extern __shared__ uint8_t smem_raw[];
-  const uint32_t base = (smem_u32(smem_raw) + 1023u) & ~1023u;
+  const uint32_t base = (smem_u32(smem_raw) + 1023u) & ~1023u;   // (the same in both CTAs of a pair)
   uint8_t* sm = smem_raw + (base - smem_u32(smem_raw));
   const uint32_t bars = base + G_BARS;
+  // of a pair, full and acc_empty count in the CTA of rank 0, which issues for both; empty and acc_full are signalled to both
   const uint32_t bar_full = bars /*[STAGES]*/, bar_empty = bars + 8 * STAGES /*[STAGES]*/,
                  bar_acc_full = bars + 16 * STAGES /*[2]*/, bar_acc_empty = bars + 16 * STAGES + 16 /*[2]*/;
   volatile uint32_t* tmem_slot = reinterpret_cast<volatile uint32_t*>(sm + G_BARS + 16 * STAGES + 32);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(sm + G_BARS + 16 * STAGES + 40);
   const int warp = __shfl_sync(0xffffffffu, threadIdx.x >> 5, 0), lane = threadIdx.x & 31;
+  const int rank = PAIR ? (int)cluster_rank() : 0;
+  const int first = PAIR ? blockIdx.x >> 1 : blockIdx.x, step = PAIR ? gridDim.x >> 1 : gridDim.x;
 
   if (threadIdx.x == 0) {
     for (int s = 0; s < STAGES; ++s) { mbar_init(bar_full + 8 * s, 1); mbar_init(bar_empty + 8 * s, 1); }
-    for (int i = 0; i < 2; ++i) { mbar_init(bar_acc_full + 8 * i, 1); mbar_init(bar_acc_empty + 8 * i, 128); }
+    for (int i = 0; i < 2; ++i) { mbar_init(bar_acc_full + 8 * i, 1); mbar_init(bar_acc_empty + 8 * i, PAIR ? 8 : 128); }   // (of a pair: a warp each)
     *abort_flag = 0;
     fence_mbar_init();
   }
-  if (warp == 4) tmem_alloc(smem_u32(const_cast<uint32_t*>(tmem_slot)), 512);
+  if (warp == 4) {
+    if (PAIR) tmem_alloc_pair(smem_u32(const_cast<uint32_t*>(tmem_slot)), 512);
+    else tmem_alloc(smem_u32(const_cast<uint32_t*>(tmem_slot)), 512);
+  }
   tc_fence_before();
   __syncthreads();
+  if (PAIR) cluster_sync();   // the other CTA's barriers and tensor memory are there
   tc_fence_after();
   const uint32_t tmem = __shfl_sync(0xffffffffu, *tmem_slot, 0);
   const int nk = (a.K + BK - 1) / BK;
@@ -141,29 +170,46 @@ lce_gemm_kernel(const __grid_constant__ GemmMaps maps, const GemmArgs a, int* __
     // step, each from a lone lane): one load for all panels of a tile where the matrix allows it.
     const uint32_t el = elect_one();
     TileWalk w;
-    w.start(a);
+    w.start(a, first, step);
     int ks = 0;
     bool ok = true;
-    const int stage_bytes = A_BYTES + a.bn * BK * 2;
+    const int bn_own = PAIR ? a.bn / 2 : a.bn;   // this CTA's columns of B
+    const int stage_bytes = (A_BYTES + bn_own * BK * 2) * (PAIR ? 2 : 1);
     for (; w.valid() && ok; w.next()) {
-      const int m0 = w.mt * BM, n0 = w.nt * a.bn;
+      const int m0 = (PAIR ? 2 * w.mt + rank : w.mt) * BM, n0 = w.nt * a.bn + (PAIR ? rank * bn_own : 0);
       for (int k = 0; k < nk; ++k, ++ks) {
         const int s = ks % STAGES;
         if (ks >= STAGES) ok = mbar_wait_lean(bar_empty + 8 * s, ((ks / STAGES) - 1) & 1, abort_flag);
         if (!ok) break;
         const uint32_t sA = base + s * STAGE_BYTES, sB = sA + A_BYTES, bar = bar_full + 8 * s;
-        if (el) mbar_expect_tx(bar, stage_bytes);
-        if (a.a_mn == K_MAJOR) tma_load_2d_e(sA, &maps.a, bar, k * BK, m0, el);
-        else if (a.a_mn == MN_PANELS) tma_load_panels_e(sA, &maps.a, bar, k * BK, m0 / 64, el);
-        else {
+        if (el && rank == 0) mbar_expect_tx(bar, stage_bytes);
+        if constexpr (PAIR) {
+          const uint32_t pbar = peer_addr(bar, 0);
+          if (a.a_mn == K_MAJOR) tma_load_2d_pair_e(sA, &maps.a, pbar, k * BK, m0, el);
+          else if (a.a_mn == MN_PANELS) tma_load_panels_pair_e(sA, &maps.a, pbar, k * BK, m0 / 64, el);
+          else {
 #pragma unroll
-          for (int p = 0; p < BM / 64; ++p) tma_load_2d_e(sA + p * MN_PANEL, &maps.a, bar, m0 + 64 * p, k * BK, el);
-        }
-        if (a.b_mn == K_MAJOR) tma_load_2d_e(sB, &maps.b, bar, k * BK, n0, el);
-        else if (a.b_mn == MN_PANELS) tma_load_panels_e(sB, &maps.b, bar, k * BK, n0 / 64, el);
-        else {
+            for (int p = 0; p < BM / 64; ++p) tma_load_2d_pair_e(sA + p * MN_PANEL, &maps.a, pbar, m0 + 64 * p, k * BK, el);
+          }
+          if (a.b_mn == K_MAJOR) tma_load_2d_pair_e(sB, &maps.b, pbar, k * BK, n0, el);
+          else if (a.b_mn == MN_PANELS) tma_load_panels_pair_e(sB, &maps.b, pbar, k * BK, n0 / 64, el);
+          else {
 #pragma unroll
-          for (int p = 0; p < BN / 64; ++p) if (64 * p < a.bn) tma_load_2d_e(sB + p * MN_PANEL, &maps.b, bar, n0 + 64 * p, k * BK, el);
+            for (int p = 0; p < BN / 128; ++p) if (64 * p < bn_own) tma_load_2d_pair_e(sB + p * MN_PANEL, &maps.b, pbar, n0 + 64 * p, k * BK, el);
+          }
+        } else {
+          if (a.a_mn == K_MAJOR) tma_load_2d_e(sA, &maps.a, bar, k * BK, m0, el);
+          else if (a.a_mn == MN_PANELS) tma_load_panels_e(sA, &maps.a, bar, k * BK, m0 / 64, el);
+          else {
+#pragma unroll
+            for (int p = 0; p < BM / 64; ++p) tma_load_2d_e(sA + p * MN_PANEL, &maps.a, bar, m0 + 64 * p, k * BK, el);
+          }
+          if (a.b_mn == K_MAJOR) tma_load_2d_e(sB, &maps.b, bar, k * BK, n0, el);
+          else if (a.b_mn == MN_PANELS) tma_load_panels_e(sB, &maps.b, bar, k * BK, n0 / 64, el);
+          else {
+#pragma unroll
+            for (int p = 0; p < BN / 64; ++p) if (64 * p < a.bn) tma_load_2d_e(sB + p * MN_PANEL, &maps.b, bar, n0 + 64 * p, k * BK, el);
+          }
         }
       }
     }
@@ -171,16 +217,16 @@ lce_gemm_kernel(const __grid_constant__ GemmMaps maps, const GemmArgs a, int* __
     // ------------------------------------------------------------------ MMA issuer: the whole warp walks the loop,
     // one elected lane issues
     const uint32_t el = elect_one();
-    const uint32_t idesc = make_idesc(BM, a.bn, a.a_mn != 0, a.b_mn != 0);
+    const uint32_t idesc = make_idesc(PAIR ? 2 * BM : BM, a.bn, a.a_mn != 0, a.b_mn != 0);
     const uint32_t a_lo0 = a.a_mn ? (((base & 0x3FFFFu) >> 4) | (static_cast<uint32_t>(MN_PANEL >> 4) << 16)) : desc_lo_k(base);
     const uint32_t b_lo0 = a.b_mn ? ((((base + A_BYTES) & 0x3FFFFu) >> 4) | (static_cast<uint32_t>(MN_PANEL >> 4) << 16))
                                   : desc_lo_k(base + A_BYTES);
     const uint32_t a_step = a.a_mn ? 128u : 2u, b_step = a.b_mn ? 128u : 2u;   // low-word advance per 16-deep slice
     TileWalk w;
-    w.start(a);
+    w.start(a, first, step);
     int ks = 0, tcnt = 0;
     bool ok = true;
-    for (; w.valid() && ok; w.next(), ++tcnt) {
+    for (; rank == 0 && w.valid() && ok; w.next(), ++tcnt) {
       const int buf = tcnt & 1;
       if (tcnt >= 2) {
         ok = mbar_wait_abortable(bar_acc_empty + 8 * buf, ((tcnt >> 1) - 1) & 1, abort_flag);
@@ -196,25 +242,35 @@ lce_gemm_kernel(const __grid_constant__ GemmMaps maps, const GemmArgs a, int* __
         const uint32_t a_lo = a_lo0 + s * (STAGE_BYTES >> 4), b_lo = b_lo0 + s * (STAGE_BYTES >> 4);
 #pragma unroll
         for (int kk = 0; kk < BK / 16; ++kk)
-          mma_ss_e(d, desc64(a_lo + kk * a_step), desc64(b_lo + kk * b_step), idesc, (k > 0 || kk > 0) ? 1u : 0u, el);
-        mma_commit_e(bar_empty + 8 * s, el);
+          if (PAIR) mma_ss_pair_e(d, desc64(a_lo + kk * a_step), desc64(b_lo + kk * b_step), idesc, (k > 0 || kk > 0) ? 1u : 0u, el);
+          else mma_ss_e(d, desc64(a_lo + kk * a_step), desc64(b_lo + kk * b_step), idesc, (k > 0 || kk > 0) ? 1u : 0u, el);
+        if (PAIR) mma_commit_pair_e(bar_empty + 8 * s, el); else mma_commit_e(bar_empty + 8 * s, el);
       }
       if (!ok) break;
-      mma_commit_e(bar_acc_full + 8 * buf, el);
+      if (PAIR) mma_commit_pair_e(bar_acc_full + 8 * buf, el); else mma_commit_e(bar_acc_full + 8 * buf, el);
     }
   } else {
     // ------------------------------------------------------------------ epilogue: one thread per accumulator row
     const int r = warp * 32 + lane;
     const uint32_t tl = tmem + ((uint32_t)(warp * 32) << 16);
+    auto release = [&](int buf) {   // the accumulator's columns are read
+      tc_fence_before();
+      if (PAIR) {
+        __syncwarp();
+        if (lane == 0) mbar_arrive_peer(peer_addr(bar_acc_empty + 8 * buf, 0));
+      } else {
+        mbar_arrive(bar_acc_empty + 8 * buf);
+      }
+    };
     TileWalk w;
-    w.start(a);
+    w.start(a, first, step);
     int tcnt = 0;
     bool ok = true;
     // row state of the forward over a vocabulary run
     float run_m = -INFINITY, run_l = 0.f;
     for (; w.valid() && ok; w.next(), ++tcnt) {
       const int buf = tcnt & 1;
-      const int m0 = w.mt * BM, n0 = w.nt * a.bn;
+      const int m0 = (PAIR ? 2 * w.mt + rank : w.mt) * BM, n0 = w.nt * a.bn;
       const int row = m0 + r;
       const bool row_ok = row < a.M;
       const int ncols = min(a.bn, a.N - n0);        // valid columns of this tile (a multiple of 8)
@@ -276,8 +332,7 @@ lce_gemm_kernel(const __grid_constant__ GemmMaps maps, const GemmArgs a, int* __
           finish(c + 1, pre[1]);
           request(c + 3, pre[1]);
         }
-        tc_fence_before();
-        mbar_arrive(bar_acc_empty + 8 * buf);
+        release(buf);
         continue;
       }
       ok = mbar_wait_abortable(bar_acc_full + 8 * buf, (tcnt >> 1) & 1, abort_flag);
@@ -357,8 +412,7 @@ lce_gemm_kernel(const __grid_constant__ GemmMaps maps, const GemmArgs a, int* __
           }
         }
       }
-      tc_fence_before();
-      mbar_arrive(bar_acc_empty + 8 * buf);
+      release(buf);
       if (EPI == EPI_LSE && ((w.nt + 1) % a.run_tiles == 0 || w.nt + 1 == a.n_tiles) && row_ok) {
         const int64_t at = (int64_t)(w.nt / a.run_tiles) * a.ldp + a.row0 + row;
         a.part_m[at] = run_m;
@@ -368,8 +422,19 @@ lce_gemm_kernel(const __grid_constant__ GemmMaps maps, const GemmArgs a, int* __
   }
   tc_fence_before();
   __syncthreads();
-  if (threadIdx.x == 0 && *abort_flag) atomicExch(status, (int)BDLM_ERR_DEVICE_TIMEOUT);
-  if (warp == 4) tmem_dealloc(tmem, 512);
+  if (threadIdx.x == 0 && *abort_flag) {
+    atomicExch(status, (int)BDLM_ERR_DEVICE_TIMEOUT);
+    if (PAIR) {
+      // the other CTA waits for this one: it has to give up as well.  The copies on their way land first (all roles have left)
+      const long long t0 = clock64();
+      while (clock64() - t0 < (1ll << 18)) {}
+      asm volatile("st.shared::cluster.u32 [%0], %1;" ::"r"(peer_addr(smem_u32(const_cast<int*>(abort_flag)), rank ^ 1)), "r"(1) : "memory");
+    }
+  }
+  if (PAIR) cluster_sync();   // no CTA leaves while the other one still signals its barriers or reads its operands
+  if (warp == 4) {
+    if (PAIR) tmem_dealloc_pair(tmem, 512); else tmem_dealloc(tmem, 512);
+  }
 }
 
 // Combines the per-run partial (maximum, sum) pairs of every token (Eq. csbp-lse-merge's rule, in log2 units),
@@ -470,32 +535,41 @@ struct Operand { const void* ptr; int64_t ld; int mn; bool whole; };
 // of items per SM times the clocks of one item.  A 16-deep slice of an M = 128 MMA takes bn / 2 clk, and no less than its
 // operands need from shared memory at 128 bytes per clk.  A narrower tile or fewer tiles have to promise 5 % (8192 x 4096 x
 // 128256 would gain 3 % by this count and lost 1 %: what bounds it is power).  No choice changes a bit of a result.
+//   pairs     where rows in units of 256 fill the chip as well (a lone CTA's tiling has to promise 5 %) and the contraction has
+//             six steps or more: shorter ones are bound by the epilogue and the start (us, one CTA / pairs: T = 1000, D = 256,
+//             V = 32000 forward 34.9 / 36.8, backward 159 / 168; dW of 400 tokens, D = 2048, V = 50304, seven steps: the
+//             backward 431 / 415; of 300, five steps: 296 / 295)
 //   forward   256 columns, where its vocabulary runs end (see RUN_TILES); 1 to 8 tiles per item
-//   dz        128 to 256 columns in steps of 16; 1 to 8 tiles per item.  T = 1531, D = 1544, V = 32008: 275 -> 188 us
+//   dz        128 to 256 columns in steps of 16 (of a pair 32); 1 to 8 tiles per item.  T = 1531, D = 1544, V = 32008: 275 -> 188 us
 //   dH, dW    256 columns where the matrix has them (their B operand lies MN-major; dH at T = 4096, D = 4096: 5.7 ms with 240
 //             or 192 columns against 3.4: its panels then start off the 128-byte lines, or a tile's rows off the 512 bytes they
 //             share), unless dH's tiles leave SMs idle: then 64 columns or more (min_bn = 64; V = 32008: T = 1531, D = 1536
 //             backward 415 -> 380 us, T = 384, D = 1544 305 -> 264; T = 149, D = 224, V = 50912 280 -> 208)
-struct Tiling { int bn, n_run; };
+constexpr int PAIR_DEPTH = 6;
+struct Tiling { int bn, n_run; bool pair; };
 Tiling choose_tiling(int M, int N, int K, int min_bn, int min_run, int max_run, int epi_per_32, int b_mn) {
-  const long long m_tiles = (M + BM - 1) / BM, sms = device_sm_count();
   const int nk = (K + BK - 1) / BK;
-  Tiling best = {BN, max_run};
+  Tiling best = {BN, max_run, false};
   double t_best = 1e300;
-  const int unit = b_mn ? min_bn : 16;
-  const bool few = b_mn && min_bn < 128 && m_tiles * ((N + BN - 1) / BN) < sms;
-  for (int bn = BN; bn >= min_bn; bn -= unit) {
-    if (bn > min_bn && bn - unit >= N) continue;           // a whole unit wider than the matrix
-    if (b_mn && bn < BN && N > bn && !few) break;
-    const long long n_tiles = (N + bn - 1) / bn;
-    const double slice = bn / 2 > 32 + bn / 4 ? bn / 2 : 32 + bn / 4;
-    const double epi = (double)epi_per_32 * ((bn + 31) / 32);
-    const double mma = nk * (BK / 16) * slice;
-    const double tile = mma > epi ? mma : epi;
-    for (int run = max_run; run >= min_run; run /= 2) {
-      const long long items = m_tiles * ((n_tiles + run - 1) / run);
-      const double t = (double)((items + sms - 1) / sms) * (run < n_tiles ? run : n_tiles) * tile + epi;
-      if (t < 0.95 * t_best) { t_best = t; best = {bn, run}; }
+  for (int pair = nk >= PAIR_DEPTH; pair >= 0; --pair) {
+    const int rows = pair ? 2 * BM : BM, sms = device_sm_count() / (pair + 1);
+    const long long m_tiles = (M + rows - 1) / rows;
+    const int least = pair && b_mn && min_bn < 128 ? 128 : min_bn;   // (half of an MN-major tile is whole panels)
+    const int unit = b_mn ? least : pair ? 32 : 16;
+    const bool few = b_mn && least < 128 && m_tiles * ((N + BN - 1) / BN) < sms;
+    for (int bn = BN; bn >= least; bn -= unit) {
+      if (bn > least && bn - unit >= N) continue;           // a whole unit wider than the matrix
+      if (b_mn && bn < BN && N > bn && !few) break;
+      const long long n_tiles = (N + bn - 1) / bn;
+      const double oper = 32 + (pair ? bn / 8 : bn / 4), slice = bn / 2 > oper ? bn / 2 : oper;
+      const double epi = (double)epi_per_32 * ((bn + 31) / 32);
+      const double mma = nk * (BK / 16) * slice;
+      const double tile = mma > epi ? mma : epi;
+      for (int run = max_run; run >= min_run; run /= 2) {
+        const long long items = m_tiles * ((n_tiles + run - 1) / run);
+        const double t = (double)((items + sms - 1) / sms) * (run < n_tiles ? run : n_tiles) * tile + epi;
+        if (t < 0.95 * t_best) { t_best = t; best = {bn, run, pair != 0}; }
+      }
     }
   }
   return best;
@@ -513,19 +587,21 @@ cudaError_t launch_gemm(GemmArgs a, const Operand& A, const Operand& B, cudaStre
     layout = extent % 64 == 0 ? MN_PANELS : MN_BOXES;   // (a last panel that is not whole would reach past the matrix)
     return layout == MN_PANELS ? tc_make_map_panels(m, o.ptr, a.K, extent, o.ld, BK, box / 64) : tc_make_map_2d(m, o.ptr, a.K, extent, o.ld, 64);
   };
-  const bool okA = encode(&maps.a, A, a.M, BM, a.a_mn), okB = encode(&maps.b, B, a.N, a.bn, a.b_mn);
+  const bool okA = encode(&maps.a, A, a.M, BM, a.a_mn), okB = encode(&maps.b, B, a.N, a.pair ? a.bn / 2 : a.bn, a.b_mn);
   if (!okA || !okB) return cudaErrorInvalidValue;
-  a.m_tiles = (a.M + BM - 1) / BM;
+  const int tile_rows = a.pair ? 2 * BM : BM, ctas = a.pair ? 2 : 1;
+  a.m_tiles = (a.M + tile_rows - 1) / tile_rows;
   a.n_tiles = (a.N + a.bn - 1) / a.bn;
   a.n_runs = (a.n_tiles + a.n_run - 1) / a.n_run;
   int* status = device_status_ptr();
   if (status == nullptr) return cudaErrorUnknown;
-  auto kern = lce_gemm_kernel<EPI>;
-  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, G_SMEM);
+  auto kern = a.pair ? lce_gemm_kernel<EPI, true> : lce_gemm_kernel<EPI, false>;
+  const int smem = a.pair ? Ring<true>::SMEM : Ring<false>::SMEM;
+  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
   if (e != cudaSuccess) return e;
-  const int items = a.m_tiles * a.n_runs;
-  const int grid = items < device_sm_count() ? items : device_sm_count();
-  return launch_chained(kern, chained, grid, G_THREADS, G_SMEM, st, 1, maps, a, status);
+  const int items = a.m_tiles * a.n_runs, slots = device_sm_count() / ctas;
+  const int grid = (items < slots ? items : slots) * ctas;
+  return launch_chained(kern, chained, grid, G_THREADS, smem, st, ctas, maps, a, status);
 }
 
 constexpr int MAX_RUN = 8;   // most N tiles per work item of the forward and of dz
@@ -648,7 +724,8 @@ int bdlm_linear_ce_fwd(const bdlm_lce_params* p, const void* h, const void* w, c
   char* ws = static_cast<char*>(workspace);
   GemmArgs a = {};
   a.M = p->T; a.N = p->V; a.K = p->D; a.m_inner = 1; a.run_tiles = run_tiles;
-  a.bn = BN; a.n_run = choose_tiling(p->T, p->V, p->D, BN, run_tiles, MAX_RUN, EPI_CLK_LSE, 0).n_run;
+  const Tiling ta = choose_tiling(p->T, p->V, p->D, BN, run_tiles, MAX_RUN, EPI_CLK_LSE, 0);
+  a.bn = BN; a.n_run = ta.n_run; a.pair = ta.pair;
   a.row0 = 0; a.labels = labels; a.weight = token_weight; a.ldp = (int)(per / sizeof(float));
   a.part_m = reinterpret_cast<float*>(ws);
   a.part_l = reinterpret_cast<float*>(ws + (size_t)runs * per);
@@ -696,18 +773,20 @@ int bdlm_linear_ce_bwd(const bdlm_lce_params* p, const void* h, const void* w, c
     // dz of the chunk: logits again, softmax minus one-hot in the epilogue
     GemmArgs a = {};
     const Tiling ta = choose_tiling(rows, V, D, 128, 1, MAX_RUN, EPI_CLK_DZ, 0);
-    a.M = rows; a.N = V; a.K = D; a.bn = ta.bn; a.n_run = ta.n_run; a.m_inner = 1;
+    a.M = rows; a.N = V; a.K = D; a.bn = ta.bn; a.n_run = ta.n_run; a.pair = ta.pair; a.m_inner = 1;
     a.row0 = t0; a.labels = labels; a.weight = token_weight; a.lse = lse; a.grad = p->grad_loss;
     a.dz = dz; a.ldz = (int)ldz;
     if (launch_gemm<EPI_DZ>(a, oh_c, ow, st, ci > 0 || plan.packed) != cudaSuccess) return BDLM_ERR_CUDA;
     // dH of the chunk = dz W   (contraction over the vocabulary; W as it lies is the MN-major B operand)
     GemmArgs b = {};
-    b.M = rows; b.N = D; b.K = V; b.bn = choose_tiling(rows, D, V, 64, 1, 1, EPI_CLK_STORE, 1).bn; b.n_run = 1; b.m_inner = 1;
+    const Tiling tb = choose_tiling(rows, D, V, 64, 1, 1, EPI_CLK_STORE, 1);
+    b.M = rows; b.N = D; b.K = V; b.bn = tb.bn; b.n_run = 1; b.pair = tb.pair; b.m_inner = 1;
     b.c_mode = C_BF16; b.c16 = static_cast<bf16*>(dh) + (size_t)t0 * D; b.ldc = D;
     if (launch_gemm<EPI_STORE>(b, odz, mn(ow), st, true) != cudaSuccess) return BDLM_ERR_CUDA;
     // dW += dz^T H_c   (contraction over the chunk's tokens; both operands MN-major)
     GemmArgs c = {};
-    c.M = V; c.N = D; c.K = rows; c.bn = choose_tiling(V, D, rows, 128, 1, 1, EPI_CLK_STORE, 1).bn; c.n_run = 1; c.m_inner = 0;
+    const Tiling tw = choose_tiling(V, D, rows, 128, 1, 1, EPI_CLK_STORE, 1);
+    c.M = V; c.N = D; c.K = rows; c.bn = tw.bn; c.n_run = 1; c.pair = tw.pair; c.m_inner = 0;
     c.c16 = static_cast<bf16*>(dw); c.c32 = dw32; c.ldc = D;
     c.c_mode = chunks == 1 ? C_BF16 : (ci == 0 ? C_F32_STORE : (ci + 1 < chunks ? C_F32_ADD : C_F32_ADD_TO_BF16));
     const Operand A = mn(odz), B = mn(oh_c);

@@ -111,9 +111,6 @@ struct StepWalk {
   }
 };
 
-__device__ __forceinline__ void cluster_sync() {
-  asm volatile("barrier.cluster.arrive.release;\n\tbarrier.cluster.wait.acquire;" ::: "memory");
-}
 
 }  // namespace tc
 }  // namespace bdlm

@@ -241,6 +241,9 @@ __device__ __forceinline__ uint32_t cluster_rank() {
   asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
   return r;
 }
+__device__ __forceinline__ void cluster_sync() {
+  asm volatile("barrier.cluster.arrive.release;\n\tbarrier.cluster.wait.acquire;" ::: "memory");
+}
 // The address that `addr` of this CTA's shared memory has in the CTA of that rank.
 __device__ __forceinline__ uint32_t peer_addr(uint32_t addr, uint32_t rank) {
   uint32_t r;

@@ -153,6 +153,24 @@ def test_tilings_and_split_contraction(w):
 
 
 @pytest.mark.parametrize("w", [
+    LceWorkload("pairs_rank_1_without_rows", 640, 520, 20008),   # the last tile of 256 rows has 128, the last of V and D 8 columns
+    LceWorkload("pairs_rank_1_with_four_rows", 900, 384, 9000),
+    LceWorkload("pairs_whole_tiles", 1024, 512, 10240),
+    LceWorkload("pairs_several_rounds", 2000, 392, 16392),
+], ids=lambda w: w.name)
+def test_tiles_on_pairs_of_ctas(w):
+    one = _check(w)
+    # a token's results do not depend on the tile it is in: the same bits from calls of 128 tokens and from chunks of 128
+    g = {k: v.cuda() for k, v in synth.make_lce_inputs(w, "cpu").items()}
+    for t in (0, w.T // 256 * 128, (w.T - 1) // 128 * 128):
+        s = slice(t, t + 128)
+        _, nll, lse = binding.bdlm_linear_ce_fwd(g["h"][s].contiguous(), g["w"], g["labels"][s].contiguous(), g["weight"][s].contiguous())
+        assert torch.equal(lse, one[2][s]) and torch.equal(nll, one[1][s])
+    dh, _ = binding.bdlm_linear_ce_bwd(g["h"], g["w"], g["labels"], one[2], g["weight"], token_chunk=128)
+    assert torch.equal(dh, one[3])
+
+
+@pytest.mark.parametrize("w", [
     LceWorkload("copied_for_the_backward", 400, 72, 1032),
     LceWorkload("copied_for_both", 1030, 200, 1544),
     LceWorkload("copied_wide", 1100, 264, 1000),
