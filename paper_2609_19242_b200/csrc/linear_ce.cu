@@ -61,6 +61,7 @@ struct GemmArgs {
   bool pair;                             // a tile of 256 rows per pair of CTAs
   int m_tiles, n_tiles, n_run, n_runs;   // an item = one M tile x n_run consecutive N tiles; n_runs = ceil(n_tiles / n_run)
   int m_inner;                           // item order: 1 = consecutive items share the N run, 0 = share the M tile
+  int block;                             // and go through this many M tiles (N runs) before the next N run (M tile) begins
   int a_mn, b_mn;                        // operand layouts: K_MAJOR, MN_PANELS (one load per tile), MN_BOXES (one per 64-column panel)
   // EPI_LSE / EPI_DZ: rows are tokens row0 .. row0 + M - 1
   int row0;
@@ -116,8 +117,11 @@ struct TileWalk {
     if (item < items) open();
   }
   __device__ __forceinline__ void open() {
-    if (a->m_inner) { nrun = item / a->m_tiles; mt = item - nrun * a->m_tiles; }
-    else { mt = item / a->n_runs; nrun = item - mt * a->n_runs; }
+    const int inner = a->m_inner ? a->m_tiles : a->n_runs, outer = a->m_inner ? a->n_runs : a->m_tiles;
+    const int per_block = a->block * outer, blk = item / per_block, in_block = item - blk * per_block;
+    const int width = min(a->block, inner - blk * a->block), o = in_block / width, i = blk * a->block + in_block - o * width;
+    mt = a->m_inner ? i : o;
+    nrun = a->m_inner ? o : i;
     nt = nrun * a->n_run;
     nt_end = min(a->n_tiles, nt + a->n_run);
   }
@@ -578,6 +582,23 @@ Tiling choose_tiling(int M, int N, int K, int min_bn, int min_run, int max_run, 
 // against 512 per 64-deep step of its MMAs, which run under it.
 constexpr int EPI_CLK_LSE = 350, EPI_CLK_DZ = 500, EPI_CLK_STORE = 300;
 
+// How many tiles of the dimension that items walk first lie together before the other one advances: as many as keep
+// their operand in L2 (126 MB, in two halves) while the other operand streams past; where a few tiles' worth is too much (dH: a
+// contraction over the vocabulary), the block that lets the CTAs running together read the least of both operands.  All of them
+// / blocks: T = 12288, D = 4096 (h 100 MB), V = 64000 forward 5470 / 4870 us; T = 8192, D = 4096, V = 128256 forward 6500 /
+// 6500 (h 67 MB), backward 19800 / 19500; smaller ones have one block.
+constexpr double L2_KEEP = 40e6;
+int inner_block(const GemmArgs& a) {
+  const int rows = a.pair ? 2 * BM : BM, slots = device_sm_count() / (a.pair ? 2 : 1);
+  const int inner = a.m_inner ? a.m_tiles : a.n_runs;
+  const double in_elems = a.m_inner ? rows : (double)a.bn * a.n_run, out_elems = a.m_inner ? (double)a.bn : rows;
+  const double fit = L2_KEEP / (in_elems * a.K * 2), even = sqrt(slots * out_elems / in_elems);
+  const int most = (int)(fit > even ? fit : even);
+  if (inner <= most || most < 1) return inner;
+  const int blocks = (inner + most - 1) / most;
+  return (inner + blocks - 1) / blocks;
+}
+
 template <int EPI>
 cudaError_t launch_gemm(GemmArgs a, const Operand& A, const Operand& B, cudaStream_t st, bool chained) {
   GemmMaps maps;
@@ -599,6 +620,7 @@ cudaError_t launch_gemm(GemmArgs a, const Operand& A, const Operand& B, cudaStre
   const int smem = a.pair ? Ring<true>::SMEM : Ring<false>::SMEM;
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
   if (e != cudaSuccess) return e;
+  a.block = inner_block(a);
   const int items = a.m_tiles * a.n_runs, slots = device_sm_count() / ctas;
   const int grid = (items < slots ? items : slots) * ctas;
   return launch_chained(kern, chained, grid, G_THREADS, smem, st, ctas, maps, a, status);
