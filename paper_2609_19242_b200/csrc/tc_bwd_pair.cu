@@ -26,6 +26,8 @@
 // (1024 + 1700 clk and the signals between them) and, at the power cap, energy.  Handing P^T over in halves was slower (two more
 // waits of the issuing warp; 38.2 ms), so were read-out tiles of 32 queries and dS^T stored by the compute warps (40.4 ms).
 // The accumulators of dQ lie in blocks of 64 rows, each as two [64 rows x 64] halves of the head dimension.
+#include <type_traits>
+
 #include "tc_bwd_common.cuh"
 
 namespace bdlm {
@@ -56,14 +58,19 @@ constexpr int BP_ARR = BP_STG + 2 * STG_BYTES;       // lse_s[2][128], d_s[2][12
 constexpr int BP_BARS = BP_ARR + 2048;
 constexpr int BP_SMEM = BP_BARS + 256;
 // warps 0-7 compute, 8 TMA, 9 MMA issue (rank 0), 10 LSE / D rows, 11 idle, 12-15 dQ read-out, 16-19 dS^T to shared memory
-constexpr int BP_THREADS = 640;
-constexpr int BP_REGS_COMPUTE = 136, BP_REGS_MISC = 40, BP_REGS_READ = 88, BP_REGS_MOVE = 80;   // 256 x 136 + 128 x (40 + 88 + 80) = 640 x 96
+// (without dQ: 0-10 and one idle)
+__host__ __device__ constexpr int bp_threads(bool dq) { return dq ? 640 : 384; }
+// 256 x 136 + 128 x (40 + 88 + 80) = 640 x 96, without dQ 256 x 200 + 128 x 104 = 384 x 168
+__host__ __device__ constexpr int bp_regs_compute(bool dq) { return dq ? 136 : 200; }
+__host__ __device__ constexpr int bp_regs_misc(bool dq) { return dq ? 40 : 104; }
+constexpr int BP_REGS_READ = 88, BP_REGS_MOVE = 80;
 constexpr uint32_t IDESC_S = make_idesc(256, 128, false, false), IDESC_ACC = make_idesc(256, 128, false, true),
                    IDESC_DQT = make_idesc(128, 128, true, true);
 __host__ __device__ constexpr uint32_t koff_h(int kk) { return (kk >> 2) * (HPANEL_BYTES >> 4) + (kk & 3) * 2; }   // K-major slice of a 64-row tile
 
-template <bool TR>
-__global__ void __launch_bounds__(BP_THREADS, 1)
+// DQ = false: dK and dV only (the dK/dV pass of the two-pass backward).
+template <bool TR, bool DQ>
+__global__ void __launch_bounds__(bp_threads(DQ), 1)
 tc_bwd_pair_kernel(const __grid_constant__ PairMaps maps, const KArgs a, const TileGrid tg, int* __restrict__ status) {
   wait_for_predecessor();
   extern __shared__ __align__(1024) uint8_t sm[];
@@ -134,7 +141,7 @@ tc_bwd_pair_kernel(const __grid_constant__ PairMaps maps, const KArgs a, const T
     if (base & 1023u) *abort_flag = 1; else *abort_flag = 0;   // swizzled tiles need a 1024-byte aligned base
     // (a warp of each role of both CTAs counts once, the loads of both CTAs with rank 0's arrival)
     mbar_init(bar_kv, 1); mbar_init(bar_go_s, 1); mbar_init(bar_go_dv, 16 + 1); mbar_init(bar_go_dk, 16 + 1);
-    mbar_init(bar_go_dp, 8 + 8 + 1); mbar_init(bar_go_dq, 16 + 8 + 2);
+    mbar_init(bar_go_dp, DQ ? 8 + 8 + 1 : 1); mbar_init(bar_go_dq, 16 + 8 + 2);
     mbar_init(bar_st, 1); mbar_init(bar_dpt, 1); mbar_init(bar_dqf, 1); mbar_init(bar_doc_e, 1); mbar_init(bar_qc_e, 1); mbar_init(bar_done, 1);
     for (int i = 0; i < 2; ++i) { mbar_init(bar_rows_full + 8 * i, 1); mbar_init(bar_rows_empty + 8 * i, 8); }
     mbar_init(bar_dpl, 8); mbar_init(bar_dsl, 8); mbar_init(bar_rx, 1);
@@ -151,7 +158,7 @@ tc_bwd_pair_kernel(const __grid_constant__ PairMaps maps, const KArgs a, const T
   if (bad_base) {
     // fall through to the common exit
   } else if (warp >= 8 && warp < 12) {
-    reg_dec<BP_REGS_MISC>();
+    reg_dec<bp_regs_misc(DQ)>();
     if (warp == 8) {
       // ------------------------------------------------------------------ TMA loads of this CTA's share, counted by rank 0's
       // barriers
@@ -166,11 +173,11 @@ tc_bwd_pair_kernel(const __grid_constant__ PairMaps maps, const KArgs a, const T
         auto load_cols = [&](uint32_t dst, const CUtensorMap* map, uint32_t bar, const QStep& s) {
           tma_load_3d_pair(dst, map, peer_addr(bar, 0), s.h * D + rank * 64, s.q0, b);
         };
-        expect(bar_kv, 3 * TILE_BYTES + PANEL_BYTES);
+        expect(bar_kv, (DQ ? 3 : 2) * TILE_BYTES + PANEL_BYTES);
         for (int p = 0; p < 2; ++p) {
           tma_load_3d_pair(sK + p * PANEL_BYTES, &maps.k[ks], r_kv, hk * D + 64 * p, k0_row, b);
           tma_load_3d_pair(sV + p * PANEL_BYTES, &maps.v[ks], r_kv, hk * D + 64 * p, k0_row, b);
-          tma_load_3d_pair(sKT + p * PANEL_BYTES, &maps.k[ks], r_kv, hk * D + 64 * rank, pair_row + p * TILE, b);
+          if (DQ) tma_load_3d_pair(sKT + p * PANEL_BYTES, &maps.k[ks], r_kv, hk * D + 64 * rank, pair_row + p * TILE, b);
         }
         // (numbers: dOc(i) 4 i, Qr(i) 4 i - 3, Qc(i) 4 i + 2, dOr(i) 4 i - 1)
         auto buf = [&](int i, int p) { return sOP + oper_buf(i + p) * PANEL_BYTES; };
@@ -214,7 +221,7 @@ tc_bwd_pair_kernel(const __grid_constant__ PairMaps maps, const KArgs a, const T
           load_qc(i + 1, s1);
           s1 = s2;
         }
-        if (ok && rank == 0) mbar_arrive(bar_go_dp);   // in place of another step's load: dQ^T of the last step waits for it
+        if (DQ && ok && rank == 0) mbar_arrive(bar_go_dp);   // in place of another step's load: dQ^T of the last step waits for it
       }
     } else if (warp == 9) {
       // ------------------------------------------------------------------ MMA issue for both CTAs: the whole warp walks the
@@ -268,7 +275,7 @@ tc_bwd_pair_kernel(const __grid_constant__ PairMaps maps, const KArgs a, const T
             if (!ok) break;
             issue_st(b1);
           }
-          if (i > 0) {
+          if (DQ && i > 0) {
             ok = go(bar_go_dq, i - 1, w_dq);
             if (!ok) break;
             issue_dqt();
@@ -280,13 +287,13 @@ tc_bwd_pair_kernel(const __grid_constant__ PairMaps maps, const KArgs a, const T
           for (int kk = 0; kk < 8; ++kk)
             mma_ts_pair_e(tmem + 384, tmem + 128 + kk * 8, desc64(op_mn + b2 * (PANEL_BYTES >> 4) + moff(kk)), IDESC_ACC, kk == 0 ? acc : 1u, el);
           mma_commit_pair_e(bar_qc_e, el);
-          ok = go(bar_go_dp, i, w_dp);
+          if (DQ || more) ok = go(bar_go_dp, i, w_dp);
           if (!ok) break;
           if (more) issue_dpt(b0);   // i + 3
           const int t = b0;
           b0 = b1; b1 = b2; b2 = t;
         }
-        if (ok) {
+        if (DQ && ok) {
           ok = go(bar_go_dq, nsteps - 1, w_dq);
           if (ok) issue_dqt();
         }
@@ -338,7 +345,7 @@ tc_bwd_pair_kernel(const __grid_constant__ PairMaps maps, const KArgs a, const T
         __syncwarp();
         if (lane == 0) mbar_arrive(bar_rows_full + 8 * sr);
       }
-    } else if (lane == 0) {
+    } else if (DQ && lane == 0) {
       // ------------------------------------------------------------------ the rows of dS^T(i) that the other CTA has copied
       // here are complete: told rank 0
       const uint32_t r_go_dq = peer_addr(bar_go_dq, 0);
@@ -348,7 +355,7 @@ tc_bwd_pair_kernel(const __grid_constant__ PairMaps maps, const KArgs a, const T
         mbar_arrive_peer_smem(r_go_dq);
       }
     }
-  } else if (warp >= 16) {
+  } else if (DQ && warp >= 16) {
     // ------------------------------------------------------------------ dS^T out of tensor memory, where dK reads it, into the
     // shared memory of the CTAs whose dQ^T needs it: columns 0-63 (queries) to rank 0, 64-127 to rank 1; a lane is a key.  Not
     // done by the compute warps: their 64 columns each took 850 of 4000 clk per step.
@@ -387,7 +394,7 @@ tc_bwd_pair_kernel(const __grid_constant__ PairMaps maps, const KArgs a, const T
         }
       }
     }
-  } else if (warp >= 12) {
+  } else if (DQ && warp >= 12) {
     // ------------------------------------------------------------------ dQ read-out: warps 12, 13 the first 64 queries of the
     // step, 14, 15 the other 64; a lane is a head-dimension index of this CTA's half
     reg_dec<BP_REGS_READ>();
@@ -446,7 +453,7 @@ tc_bwd_pair_kernel(const __grid_constant__ PairMaps maps, const KArgs a, const T
     }
   } else {
     // ------------------------------------------------------------------ compute: warpgroup w has queries 64 w .. of every step
-    reg_inc<BP_REGS_COMPUTE>();
+    reg_inc<bp_regs_compute(DQ)>();
     const int w = warp >> 2;
     const int r = (warp & 3) * 32 + lane;                      // TMEM lane = key row of the tile
     const int j = k0 + r;
@@ -496,16 +503,22 @@ tc_bwd_pair_kernel(const __grid_constant__ PairMaps maps, const KArgs a, const T
         tmem_ld32(tl + c0, c[0]); tmem_ld32(tl + c0 + 32, c[1]);
         tmem_wait_ld();
       }
-      exp_tile<64>(x, scale2, lse_s + sr * 128 + c0);
-      if (need_mask)   // visible columns of this thread's key row inside the step
-        hide_tile<64>(x, (st.qs == CLEAN ? vqc_lo : vqn_lo) - st.q0 - c0, (st.qs == CLEAN ? vqc_hi : vqn_hi) - st.q0 - c0);
-      {
-        uint32_t pk[32];
+      // (no branch between the exponentials and the packing of an unmasked tile, so that they overlap)
+      auto p_tile = [&](auto masked) {
+        const int lo = (st.qs == CLEAN ? vqc_lo : vqn_lo) - st.q0 - c0, hi = (st.qs == CLEAN ? vqc_hi : vqn_hi) - st.q0 - c0;   // visible columns of this thread's key row
 #pragma unroll
-        for (int e = 0; e < 32; ++e) pk[e] = pack_bf16(__uint_as_float(x[2 * e]), __uint_as_float(x[2 * e + 1]));
-        tmem_st32(tl + c0, pk);
+        for (int half = 0; half < 2; ++half) {
+          uint32_t (&xh)[32] = reinterpret_cast<uint32_t (&)[32]>(x[32 * half]);
+          exp_tile<32>(xh, scale2, lse_s + sr * 128 + c0 + 32 * half);
+          if (decltype(masked)::value) hide_tile<32>(xh, lo - 32 * half, hi - 32 * half);
+          uint32_t pk[16];
+#pragma unroll
+          for (int e = 0; e < 16; ++e) pk[e] = pack_bf16(__uint_as_float(xh[2 * e]), __uint_as_float(xh[2 * e + 1]));
+          tmem_st16(tl + c0 + 16 * half, pk);
+        }
         tmem_wait_st();
-      }
+      };
+      if (need_mask) p_tile(std::true_type{}); else p_tile(std::false_type{});
       tc_fence_before();
       __syncwarp();
       if (lane == 0) mbar_arrive_peer(r_go_dv);
@@ -528,7 +541,7 @@ tc_bwd_pair_kernel(const __grid_constant__ PairMaps maps, const KArgs a, const T
           __syncwarp();
           if (lane == 0) {   // the other warpgroup's dS^T and dQ^T go over columns of this one's dP^T
             mbar_arrive(bar_dpl);
-            if (i > 0) mbar_arrive_peer(r_go_dq);
+            if (DQ && i > 0) mbar_arrive_peer(r_go_dq);
           }
         }
         ds_tile<32>(pk[half], reinterpret_cast<const uint32_t (&)[32]>(x[32 * half]), y, d_s + sr * 128 + c0 + 32 * half);
@@ -541,10 +554,10 @@ tc_bwd_pair_kernel(const __grid_constant__ PairMaps maps, const KArgs a, const T
       tmem_wait_st();
       tc_fence_before();
       __syncwarp();
-      if (lane == 0) { mbar_arrive_peer(r_go_dk); mbar_arrive(bar_dsl); mbar_arrive(bar_rows_empty + 8 * sr); }   // this warp is done with the stage's LSE / D rows
+      if (lane == 0) { mbar_arrive_peer(r_go_dk); if (DQ) mbar_arrive(bar_dsl); mbar_arrive(bar_rows_empty + 8 * sr); }   // this warp is done with the stage's LSE / D rows
       c_ds += tick<TR>() - t2;
     }
-    if (ok && lane == 0 && nsteps > 0) mbar_arrive_peer(r_go_dq);   // dQ^T of the last step waits for no dP^T
+    if (DQ && ok && lane == 0 && nsteps > 0) mbar_arrive_peer(r_go_dq);   // dQ^T of the last step waits for no dP^T
     if (warp == 0 && lane == 0 && rank == 0) {
       trace_add(a.trace, 16 + 0, nsteps); trace_add(a.trace, 16 + 1, w_st); trace_add(a.trace, 16 + 2, w_dpt);
       trace_add(a.trace, 16 + 3, w_dsf); trace_add(a.trace, 16 + 4, c_exp); trace_add(a.trace, 16 + 5, c_ds);
@@ -606,7 +619,8 @@ tc_bwd_pair_kernel(const __grid_constant__ PairMaps maps, const KArgs a, const T
 
 }  // namespace
 
-cudaError_t launch_tc_bwd_pair(const KArgs& a, cudaStream_t st, bool chained) {
+template <bool DQ>
+static cudaError_t launch_pair(const KArgs& a, cudaStream_t st, bool chained) {
   PairMaps maps;
   for (int s = 0; s < 2; ++s) {
     // a stream that is left out gets the other stream's tensors as placeholders: its maps are never used
@@ -626,10 +640,14 @@ cudaError_t launch_tc_bwd_pair(const KArgs& a, cudaStream_t st, bool chained) {
   const TileGrid tg = make_tile_grid((max(a.L, a.k[NOISY] != nullptr ? a.Ln : 0) + 2 * TILE - 1) / (2 * TILE), a.Hkv, a.batch * 2);
   const long long blocks = 2LL * tile_grid_blocks(tg);
   if (blocks == 0 || blocks > 0x7fffffffLL) return cudaErrorInvalidValue;
-  auto kern = a.trace ? tc_bwd_pair_kernel<true> : tc_bwd_pair_kernel<false>;
+  auto kern = a.trace ? tc_bwd_pair_kernel<true, DQ> : tc_bwd_pair_kernel<false, DQ>;
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, BP_SMEM);
   if (e != cudaSuccess) return e;
-  return launch_chained(kern, chained, (unsigned)blocks, BP_THREADS, BP_SMEM, st, 2, maps, a, tg, status);
+  return launch_chained(kern, chained, (unsigned)blocks, bp_threads(DQ), BP_SMEM, st, 2, maps, a, tg, status);
+}
+
+cudaError_t launch_tc_bwd_pair(const KArgs& a, bool dq, cudaStream_t st, bool chained) {
+  return dq ? launch_pair<true>(a, st, chained) : launch_pair<false>(a, st, chained);
 }
 
 }  // namespace bdlm

@@ -30,7 +30,7 @@ cudaError_t launch_tc_fwd(const KArgs& a, cudaStream_t st);
 // Lays the fused backward's dQ accumulators out in the workspace (a.dq32, a.dq32_rows).
 void tc_bwd_place_dq(KArgs& a, void* extra_ws);
 cudaError_t launch_tc_bwd(const KArgs& a, int passes, cudaStream_t st);
-// The fused backward on pairs of CTAs (head dimension 128): dK, dV and the sums for dQ.
-cudaError_t launch_tc_bwd_pair(const KArgs& a, cudaStream_t st, bool chained);
+// The backward on pairs of CTAs (head dimension 128): dK, dV and, with dq, the sums for dQ.
+cudaError_t launch_tc_bwd_pair(const KArgs& a, bool dq, cudaStream_t st, bool chained);
 
 }  // namespace bdlm

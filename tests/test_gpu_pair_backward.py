@@ -1,5 +1,5 @@
-"""The fused backward on pairs of CTAs (large calls of head dimension 128) against the two-pass kernels, which other tests
-compare with the oracle: an odd number of key tiles, ragged lengths with rows that are not 16-byte aligned, windows, blocks of
+"""The backward on pairs of CTAs (large calls of head dimension 128): the fused one against the two-pass one, that one against
+the oracle on sampled rows.  An odd number of key tiles, ragged lengths with rows that are not 16-byte aligned, windows, blocks of
 several tiles, both mask modes, the packed form with repeated and empty prefixes, a clean run by itself, gathered K/V in chunks
 of an odd number of tiles."""
 import pytest
@@ -59,6 +59,16 @@ def test_plain_layer(w, mode):
         _close(got[i], want[i], i)
     for i in (1, 2, 4, 5):   # dK, dV: a fixed order of summation
         assert torch.equal(got[i], again[i]), i
+
+
+@pytest.mark.parametrize("w", [
+    Workload("two_pass", 1, 24, 6, 128, 6016, 32, seed=1),
+    Workload("two_pass_ragged", 2, 12, 3, 128, 6040, 40, seed=2),
+    Workload("two_pass_window", 1, 16, 4, 128, 12000, 96, seed=6, window=3500),
+], ids=lambda w: w.name)
+def test_two_pass_gradients(w):
+    """The two-pass backward's dK/dV pass runs on pairs as well: the gradients of sampled rows against the oracle."""
+    pu.check_sampled(w, binding.IMPL_TCGEN05, n_rows=96, single_pass=False)
 
 
 @pytest.mark.parametrize("case", ["blocks", "blocks_and_clean", "clean_run", "gathered"])
