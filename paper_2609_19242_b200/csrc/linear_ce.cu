@@ -133,6 +133,14 @@ struct TileWalk {
   }
 };
 
+// Columns that the MMAs of a tile compute: the last tile of a row of tiles only those that the matrix has, in whole units of what
+// the operand's layout allows (16 columns; of a pair 32, or a panel per CTA).  With D = 1544 the last of seven tiles is 8 wide.
+template <bool PAIR>
+__device__ __forceinline__ int mma_columns(const GemmArgs& a, int nt) {
+  const int unit = PAIR ? (a.b_mn == K_MAJOR ? 32 : 128) : 16;
+  return min(a.bn, (a.N - nt * a.bn + unit - 1) / unit * unit);
+}
+
 template <int EPI, bool PAIR>
 __global__ void __launch_bounds__(G_THREADS, 1)
 lce_gemm_kernel(const __grid_constant__ GemmMaps maps, const GemmArgs a, int* __restrict__ status) {
@@ -180,7 +188,7 @@ lce_gemm_kernel(const __grid_constant__ GemmMaps maps, const GemmArgs a, int* __
     const int bn_own = PAIR ? a.bn / 2 : a.bn;   // this CTA's columns of B
     const int stage_bytes = (A_BYTES + bn_own * BK * 2) * (PAIR ? 2 : 1);
     for (; w.valid() && ok; w.next()) {
-      const int m0 = (PAIR ? 2 * w.mt + rank : w.mt) * BM, n0 = w.nt * a.bn + (PAIR ? rank * bn_own : 0);
+      const int m0 = (PAIR ? 2 * w.mt + rank : w.mt) * BM, n0 = w.nt * a.bn + (PAIR ? rank * (mma_columns<PAIR>(a, w.nt) / 2) : 0);
       for (int k = 0; k < nk; ++k, ++ks) {
         const int s = ks % STAGES;
         if (ks >= STAGES) ok = mbar_wait_lean(bar_empty + 8 * s, ((ks / STAGES) - 1) & 1, abort_flag);
@@ -221,7 +229,6 @@ lce_gemm_kernel(const __grid_constant__ GemmMaps maps, const GemmArgs a, int* __
     // ------------------------------------------------------------------ MMA issuer: the whole warp walks the loop,
     // one elected lane issues
     const uint32_t el = elect_one();
-    const uint32_t idesc = make_idesc(PAIR ? 2 * BM : BM, a.bn, a.a_mn != 0, a.b_mn != 0);
     const uint32_t a_lo0 = a.a_mn ? (((base & 0x3FFFFu) >> 4) | (static_cast<uint32_t>(MN_PANEL >> 4) << 16)) : desc_lo_k(base);
     const uint32_t b_lo0 = a.b_mn ? ((((base + A_BYTES) & 0x3FFFFu) >> 4) | (static_cast<uint32_t>(MN_PANEL >> 4) << 16))
                                   : desc_lo_k(base + A_BYTES);
@@ -237,7 +244,7 @@ lce_gemm_kernel(const __grid_constant__ GemmMaps maps, const GemmArgs a, int* __
         if (!ok) break;
         tc_fence_after();
       }
-      const uint32_t d = tmem + buf * BN;
+      const uint32_t d = tmem + buf * BN, idesc = make_idesc(PAIR ? 2 * BM : BM, mma_columns<PAIR>(a, w.nt), a.a_mn != 0, a.b_mn != 0);
       for (int k = 0; k < nk; ++k, ++ks) {
         const int s = ks % STAGES;
         ok = mbar_wait_lean(bar_full + 8 * s, (ks / STAGES) & 1, abort_flag);
