@@ -36,12 +36,12 @@ NAMES6 = ["q_clean", "k_clean", "v_clean", "q_noisy", "k_noisy", "v_noisy"]
 # DRAM traffic (dram__bytes_read.sum + dram__bytes_write.sum) per launch of a kernel from a one-pass ncu capture of
 # this command, keyed by (workload, kernel), each with the digest of the kernel sources it was captured on
 # (kernel_source_digest): a figure is reported only for the build it belongs to.
-_CAPTURED_ON = "2abc69b5a1b0c168"
+_CAPTURED_ON = "151b29bf182d6b68"
 NCU_TRAFFIC = {
-    ("32k", "fwd"): {"bytes": 980136192 + 522032640, "kernel_source": _CAPTURED_ON},
-    ("32k", "bwd_fused"): {"bytes": 5856034560 + 3336947712, "kernel_source": _CAPTURED_ON},
-    ("32k", "bwd_dkdv"): {"bytes": 2386681088 + 249642752, "kernel_source": _CAPTURED_ON},
-    ("32k", "bwd_dq"): {"bytes": 1542742528 + 519323392, "kernel_source": _CAPTURED_ON},
+    ("32k", "fwd"): {"bytes": 981373696 + 521526272, "kernel_source": _CAPTURED_ON},
+    ("32k", "bwd_fused"): {"bytes": 5656973056 + 3099851776, "kernel_source": _CAPTURED_ON},
+    ("32k", "bwd_dkdv"): {"bytes": 2405314304 + 266414848, "kernel_source": _CAPTURED_ON},
+    ("32k", "bwd_dq"): {"bytes": 1542419200 + 518608896, "kernel_source": _CAPTURED_ON},
 }
 TRAFFIC_NOTE = ("dram__bytes_read.sum + dram__bytes_write.sum per launch from a one-pass ncu capture of this command on "
                 "the 32k workload")
@@ -239,7 +239,8 @@ def kernel_source_digest():
     import hashlib
     h = hashlib.sha256()
     csrc = os.path.join(ROOT, "paper_2609_19242_b200", "csrc")
-    for f in ("bdlm_common.cuh", "fwd_issue.h", "tc_common.cuh", "tc_kernels.cu", "tc_bwd_kernels.cu"):
+    for f in ("bdlm_common.cuh", "fwd_issue.h", "tc_common.cuh", "tc_kernels.cu", "tc_bwd_common.cuh", "tc_bwd_kernels.cu",
+              "tc_bwd_pair.cu"):
         with open(os.path.join(csrc, f), "rb") as fh:
             h.update(fh.read())
     return h.hexdigest()[:16]

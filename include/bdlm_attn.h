@@ -266,7 +266,9 @@ int bdlm_attn_bwd_static_scratch(const bdlm_params* p,
  *   6 total; 7 in the fused backward: the MMA warp's wait for Q tiles), 8..11 to the MMA warp (8 total,
  *   9..11 waits), 12..13 to the producer (12 total or, fused, the MMA warp's wait for dO tiles; 13 wait
  *   for a free stage), 14..15 kernel-specific (dK/dV pass: S^T load and exponent arithmetic; fused: the
- *   read-out warpgroup's wait for dQ^T and its busy time).
+ *   read-out warpgroup's wait for dQ^T and its busy time).  Where pairs of CTAs run the backward, the counters are those of
+ *   the first CTA of each pair, a step is 256 keys x 128 queries (otherwise 128 x 128, fused 128 x 64), 7 and 9..12 are the MMA
+ *   warp's waits for the products S, dV, dP, dK and dQ, and 13 is not used.
  * The buffer is set per device (the device current at the call) and applies to every later launch on
  * that device from any thread.  Pass NULL to switch tracing off (the default).  The caller zeroes and
  * reads the buffer.

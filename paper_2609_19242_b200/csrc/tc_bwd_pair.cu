@@ -1,4 +1,4 @@
-// Fused backward on pairs of CTAs: dK, dV and dQ in one kernel for head dimension 128.
+// Backward on pairs of CTAs for head dimension 128: dK, dV and dQ in one kernel (or dK and dV alone, see DQ).
 //
 // A unit is two neighbouring 128-key tiles of one KV head, one per CTA of a cluster of two; the pair walks every 128-row query
 // tile that sees either of them (all heads of the group, clean then noisy queries).  Every product is one tcgen05.mma of the
@@ -68,7 +68,8 @@ constexpr uint32_t IDESC_S = make_idesc(256, 128, false, false), IDESC_ACC = mak
                    IDESC_DQT = make_idesc(128, 128, true, true);
 __host__ __device__ constexpr uint32_t koff_h(int kk) { return (kk >> 2) * (HPANEL_BYTES >> 4) + (kk & 3) * 2; }   // K-major slice of a 64-row tile
 
-// DQ = false: dK and dV only (the dK/dV pass of the two-pass backward).
+// DQ = false: dK and dV only (the dK/dV pass of the two-pass backward), the same sums as tc_dkdv_kernel.  A step is then bound by
+// the same chain; L = 16384, H = 8 / 8: two-pass backward 3239 -> 3177 us.
 template <bool TR, bool DQ>
 __global__ void __launch_bounds__(bp_threads(DQ), 1)
 tc_bwd_pair_kernel(const __grid_constant__ PairMaps maps, const KArgs a, const TileGrid tg, int* __restrict__ status) {

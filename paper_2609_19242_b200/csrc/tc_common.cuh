@@ -251,8 +251,9 @@ __device__ __forceinline__ uint32_t peer_addr(uint32_t addr, uint32_t rank) {
   return r;
 }
 // Arrivals at a barrier of either CTA (an address from peer_addr).  mbar_arrive_peer is relaxed: execution order only, for what
-// lies in tensor memory (ordered by tcgen05.wait and the tcgen05 fences).  mbar_arrive_peer_smem goes after a proxy fence, for
-// shared memory of the arriving CTA that an MMA is about to read.  (A release to the cluster costs a thread a thousand clocks.)
+// lies in tensor memory (ordered by tcgen05.wait and the tcgen05 fences).  mbar_arrive_peer_smem is for shared memory of the
+// arriving CTA that an MMA of the pair is about to read there: after a proxy fence of the threads that wrote it, which makes it
+// visible to the reader, the async proxy of the same SM.  (A release to the cluster costs a thread a thousand clocks.)
 __device__ __forceinline__ void mbar_arrive_peer(uint32_t peer_bar) {
   asm volatile("mbarrier.arrive.relaxed.cluster.shared::cluster.b64 _, [%0];" ::"r"(peer_bar) : "memory");
 }
