@@ -5,6 +5,7 @@
 #include <stdint.h>
 
 #include "../../include/bdlm_attn.h"
+#include "dispatch_rules.h"
 
 namespace bdlm {
 
@@ -140,20 +141,16 @@ int device_sm_count();
 //                    Q / dO / K / V tiles (and, in the fused backward, the same dQ accumulator tiles) together;
 //   tile_major = 1   x slowest: the heaviest tiles of every head, batch element and stream start first -- longest job
 //                    first over the whole launch.  Chosen by the launchers when the heaviest tile is a sizeable part of
-//                    the ideal duration of the launch (short sequences), where the first order would start the heavy
-//                    tiles of the second and later batch elements too late.
+//                    the ideal duration of the launch (short sequences; dispatch_rules.h), where the first order would
+//                    start the heavy tiles of the second and later batch elements too late.
 // parts: CTAs that share one unit (the backward's key tiles: a cluster of that size), index i = unit * parts + part.
 struct TileGrid { int nx, ny, nz, tile_major, parts; };
 __device__ __forceinline__ void tile_grid_decode(const TileGrid& g, int i, int& x, int& y, int& z) {
   if (!g.tile_major) { x = i % g.nx; i /= g.nx; y = i % g.ny; z = i / g.ny; }
   else { const int c = g.ny * g.nz; x = i / c; i -= x * c; y = i % g.ny; z = i / g.ny; }
 }
-inline TileGrid make_tile_grid(int nx, int ny, int nz) {
-  TileGrid g = {nx, ny, nz, 0, 1};
-  // heaviest tile ~ nx units, whole launch ~ ny nz nx (nx + 1) / 2 units over the device's SMs: tile-major when the
-  // heaviest tile exceeds a fifth of the ideal duration
-  g.tile_major = (10LL * device_sm_count() > (long long)ny * nz * (nx + 1)) ? 1 : 0;
-  return g;
+inline TileGrid make_tile_grid(int nx, int ny, int nz) {   // one CTA per unit, one on an SM
+  return {nx, ny, nz, tile_major_pays(nx, ny, nz, nx, device_sm_count(), ORDER_RATIO) ? 1 : 0, 1};
 }
 // Number of CTAs, or 0 if it does not fit a grid dimension.
 inline unsigned tile_grid_blocks(const TileGrid& g) {

@@ -1,0 +1,16 @@
+// Asks the rules that choose a launch: the first argument names the rule, the others are its sizes.  Prints the answer.
+#include <cstdio>
+#include <cstdlib>
+#include <cstring>
+
+#include "dispatch_rules.h"
+
+using namespace bdlm;
+
+int main(int argc, char** argv) {
+  auto num = [&](int i) { return i + 2 < argc ? std::atoi(argv[i + 2]) : 0; };
+  const char* rule = argv[1];
+  if (!std::strcmp(rule, "order")) std::printf("%d\n", tile_major_pays(num(0), num(1), num(2), num(0), num(3), ORDER_RATIO));
+  else if (!std::strcmp(rule, "order_pairs")) std::printf("%d\n", pairs_tile_major_pay(num(0), num(1), num(2), num(3), num(4), num(5) != 0));
+  else return 1;
+}
