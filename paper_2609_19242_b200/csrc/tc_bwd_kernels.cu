@@ -1330,68 +1330,9 @@ void tc_bwd_place_dq(KArgs& a, void* extra_ws) {
   }
 }
 
-// How many CTAs share a clean key tile (1, 2 or 4), from two estimates in steps of HT query rows: `heavy` for the
-// first clean key tile and `mean` per SM; with a prefix table the blocks are taken to be spread evenly over the keys.
-// A launch cannot end before its heaviest CTA, so a split pays when that is well above the mean; below, longest-first
-// start order fills the chip and the exchange of the partial tiles (about 4 steps per CTA) is a loss.  Clusters of four
-// only reach 132 of the 148 SMs.  Fused backward with 1 / 2 / 4 CTAs per tile (us, all kernels of the call):
-//   L = 2048, H = 32 / 8        heavy 1.9 means    386 /  308 /  343
-//   L = 1024, H = 32 / 8        heavy 3.4 means    236 /  176 /  174
-//   L = 8192, H = 8 / 1         heavy 4.4 means   2097 / 1098 /  740
-//   L = 16384, H = 8 / 1        heavy 2.3 means   4284 / 2717 / 2919
-//   L = 4096, H = 32 / 8        heavy 1.06 means   914 /  920 / 1050
-//   L = 8192, H = 32 / 8        heavy 0.55 means  2755 / 3122 / 4237
-// and at the thresholds:
-//   L = 4096, H = 32 / 8        heavy 1.09 means   806 /  798 /  972
-//   L = 3584, H = 32 / 8        heavy 1.23 means   682 /  639 /  790
-//   L = 3072, H = 32 / 8        heavy 1.42 means   571 /  470 /  585
-//   L = 1536, H = 32 / 8        heavy 2.64 means   248 /  151 /  174
-//   L = 14336, H = 8 / 1        heavy 2.60 means  3789 / 2302 / 2195
-//   L = 12288, H = 8 / 1        heavy 3.02 means  3193 / 1844 / 1625
-//   L = 1280, H = 32 / 8        heavy 3.08 means   200 /  123 /  138
-//   2 x 1024, H = 16 / 8, window 256   1.35 means, 28 steps: 74 / 82 / 121 (few steps: the estimate is rough there)
-// Under MIN_HEAVY steps the exchange eats what the split gives (L = 256: 37 / 36 / 36).
-constexpr double MIN_HEAVY = 24, SPLIT_2 = 1.2, SPLIT_4 = 3.0;
-struct KeyLoad { double heavy, mean, total; };   // steps of HT query rows: of the first clean key tile, per SM, of all clean key tiles of a KV head
-static KeyLoad key_load(const KArgs& a) {
-  constexpr int rows = HT;
-  const double W = a.window > 0 ? a.window : 0;
-  double heavy = 0, total = 0;
-  for (int qs = CLEAN; qs <= NOISY; ++qs) {
-    if (a.q[qs] == nullptr) continue;
-    const double nq = (rows_q(a, qs) + rows - 1) / rows;
-    const double seen = qs == CLEAN ? a.cq_pos0 + 0.5 * a.Lqc : 0.5 * a.L;   // keys a query sees on average
-    heavy += W > 0 ? min(nq, (W + TILE) / rows + 1) : nq;
-    total += nq * ((W > 0 ? min(W, seen) : seen) / TILE + 1);
-  }
-  total *= a.G;
-  return {heavy * a.G, total * a.Hkv * a.batch / device_sm_count(), total};
-}
-static int split_key_tiles(const KeyLoad& l) {
-  if (l.heavy < MIN_HEAVY || l.heavy < SPLIT_2 * l.mean) return 1;
-  return l.heavy < SPLIT_4 * l.mean ? 2 : 4;
-}
-
-// Whether pairs of CTAs (tc_bwd_pair_kernel) take the call: head dimension 128, key tiles not shared (a pair has two of them), and
-// enough work for what a pair does more.  In 128 x 128 tiles: its two key tiles see one query tile more in their hull than each by
-// itself wherever a query stream's limit passes them, noisy key tiles two (half as much again, as measured, for masking them),
-// and a unit's start and end cost it 3.6 tiles more than two CTAs'.  Fused backward, one CTA per tile / pairs (us, whole
-// call), by that extra over the tiles there are:
-//   0.015   L = 32768, H = 32 / 8                  40770 / 37860
-//   0.040   L = 12288, H = 32 / 8                   6400 /  6070
-//   0.051   L = 16384, H = 8 / 8                    2690 /  2640
-//   0.059   2 x 8192, H = 16 / 4                    2980 /  2850
-//   0.059   L = 32768, H = 32 / 8, window 4096     11540 / 11010
-//   0.078   L = 6144, H = 32 / 8                    1760 /  1730
-//   0.093   L = 5120, H = 32 / 8                    1230 /  1220
-//   0.100   L = 8192, H = 16 / 16                   1523 /  1540
-//   0.115   2 x 4096, H = 32 / 8                    1690 /  1710
-//   0.115   L = 32768, H = 32 / 8, window 2048      6390 /  6550
-//   0.132   3 x 6144, H = 8 / 8                     1367 /  1399
-constexpr double PAIR_EXTRA = 0.09, PAIR_MASKED = 1.5, PAIR_UNIT = 3.6;
-static bool pairs_pay(const KArgs& a, const KeyLoad& l) {
-  const double tiles = l.total * HT / TILE, pairs_c = a.q[CLEAN] != nullptr ? a.Lqc / 256.0 : 0, pairs_n = a.q[NOISY] != nullptr ? a.Ln / 256.0 : 0;
-  return PAIR_MASKED * a.G * (pairs_c + 3 * pairs_n) + PAIR_UNIT * (a.L / 256.0 + pairs_n) <= PAIR_EXTRA * tiles;
+static_assert(TILE_KEYS == TILE && STEP_ROWS == HT, "the rules count these tiles and steps");
+static BwdSizes bwd_sizes(const KArgs& a) {
+  return {a.batch, a.L, a.q[CLEAN] != nullptr ? a.Lqc : 0, a.cq_pos0, a.q[NOISY] != nullptr ? a.Ln : 0, a.Hkv, a.G, a.window, a.kv_chunk_len};
 }
 
 // One CTA, or one cluster of tg.parts CTAs, per unit of the grid.
@@ -1429,9 +1370,10 @@ static cudaError_t launch_tc_bwd_d(const KArgs& a, int passes, cudaStream_t st) 
         const size_t rows = (size_t)a.dq32_rows[CLEAN] + a.dq32_rows[NOISY];
         if ((e = cudaMemsetAsync(a.dq32[CLEAN], 0, rows * a.batch * a.H * D * sizeof(float), st)) != cudaSuccess) return e;
       }
-      const KeyLoad load = key_load(a);
+      const BwdSizes z = bwd_sizes(a);
+      const KeyLoad load = key_load(z, device_sm_count());
       const int parts = split_key_tiles(load);
-      const bool pairs = D == 128 && parts == 1 && pairs_pay(a, load);
+      const bool pairs = D == 128 && parts == 1 && pairs_pay(z, load);
       if (pairs) {
         if ((e = launch_tc_bwd_pair(a, true, st, after_rows)) != cudaSuccess) return e;
       } else {
@@ -1458,7 +1400,8 @@ static cudaError_t launch_tc_bwd_d(const KArgs& a, int passes, cudaStream_t st) 
     // (the rule knows nothing of the batch or the number of KV heads; the sums are the same bit for bit either way.  One CTA per
     // tile / pairs, whole two-pass backward: L = 16384, H = 8 / 8 3239 / 3177 us, H = 32 / 8 12720 / 12390; L = 6016, H = 24 / 6
     // 1467 / 1441)
-    if (D == 128 && pairs_pay(a, key_load(a))) {
+    const BwdSizes z = bwd_sizes(a);
+    if (D == 128 && pairs_pay(z, key_load(z, device_sm_count()))) {
       if ((e = launch_tc_bwd_pair(a, false, st, after_rows)) != cudaSuccess) return e;
     } else {
       auto kern = a.trace ? tc_dkdv_kernel<true, D> : tc_dkdv_kernel<false, D>;

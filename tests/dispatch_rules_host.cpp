@@ -12,5 +12,9 @@ int main(int argc, char** argv) {
   const char* rule = argv[1];
   if (!std::strcmp(rule, "order")) std::printf("%d\n", tile_major_pays(num(0), num(1), num(2), num(0), num(3), ORDER_RATIO));
   else if (!std::strcmp(rule, "order_pairs")) std::printf("%d\n", pairs_tile_major_pay(num(0), num(1), num(2), num(3), num(4), num(5) != 0));
-  else return 1;
+  else if (!std::strcmp(rule, "pairs")) {
+    const BwdSizes z = {num(0), num(1), num(2), num(3), num(4), num(5), num(6), num(7), num(8)};
+    const KeyLoad load = key_load(z, num(9));
+    std::printf("%d %d\n", split_key_tiles(load), pairs_pay(z, load));
+  } else return 1;
 }

@@ -50,3 +50,29 @@ def test_start_order_of_one_cta_per_tile(ask, nx, stacks, want):
     """Exactly 10 SMs > stacks (nx + 1)."""
     assert (10 * SMS > stacks * (nx + 1)) == bool(want)
     assert ask("order", nx, stacks, 1, SMS) == [want]
+
+
+@pytest.mark.parametrize("L,H,H_kv,window,want", [
+    (32768, 32, 8, 0, 1), (6144, 32, 8, 0, 1), (16384, 8, 8, 0, 1), (32768, 32, 8, 4096, 1),
+    (4096, 32, 8, 0, 0), (8192, 16, 16, 0, 0), (32768, 32, 8, 2048, 0), (32768, 32, 8, 1024, 0),
+])
+def test_calls_that_pairs_take(ask, L, H, H_kv, window, want):
+    assert ask("pairs", 1, L, L, 0, L, H_kv, H // H_kv, window, 0, SMS) == [1, want]
+
+
+@pytest.mark.parametrize("L,chunk_tiles,rank_of,blocks,want", [
+    (32768, 1, None, True, 0), (16128, 3, None, True, 0), (32640, 3, None, True, 0), (16000, 5, None, True, 0),
+    (16128, 7, None, True, 1), (32256, 9, None, True, 1),
+    (32768, 16, None, True, 1),                              # an even number of tiles: a pair stays within a chunk
+    (11264, 11, (3, 4), True, 0), (26624, 13, (4, 8), True, 1), (65536, 32, (3, 8), True, 1),
+    (22528, 11, (7, 8), False, 1), (10240, 5, (7, 8), False, 0),
+])
+def test_pairs_whose_tiles_stand_far_apart(ask, L, chunk_tiles, rank_of, blocks, want):
+    """Gathered K/V: whole-sequence calls (rank_of None), and one rank's first run of clean queries with its blocks or its second
+    run by itself."""
+    if rank_of is None:
+        pos0, Lq, Ln = 0, L, L
+    else:
+        r, P = rank_of
+        pos0, Lq, Ln = ((r if blocks else 2 * P - 1 - r) * L // (2 * P), L // (2 * P), L // P if blocks else 0)
+    assert ask("pairs", 1, L, Lq, pos0, Ln, 8, 4, 0, 128 * chunk_tiles, SMS) == [1, want]
