@@ -10,7 +10,7 @@
 //                      dH_c = dz W          epilogue: bf16 store
 //                      dW  += dz^T H_c      epilogue: bf16 store, or fp32 accumulation over the chunks
 //
-// Tiles are 256 rows by at most 256 columns on a pair of CTAs, or 128 rows on one CTA (see choose_tiling), with 64-deep
+// Tiles are 256 rows by at most 256 columns on a pair of CTAs, or 128 rows on one CTA (lce_rules.h), with 64-deep
 // contraction steps: TMA (128-byte swizzle) fills a ring of A (16 KB) and B (up to 32 KB; of a pair each CTA loads half) tiles, one
 // warp -- of a pair, that of rank 0 -- issues tcgen05.mma (M = 128 or 256, N = the tile's width, K = 16) into one of two
 // 256-column accumulators in tensor memory, and four epilogue warps
@@ -24,6 +24,7 @@
 #include <math.h>
 
 #include "../../include/bdlm_linear_ce.h"
+#include "lce_rules.h"
 #include "tc_common.cuh"
 #include "tc_launch.h"
 
@@ -33,7 +34,6 @@ namespace {
 using namespace tc;
 using bf16 = __nv_bfloat16;
 
-constexpr int BM = 128, BN = 256, BK = 64;
 constexpr int A_BYTES = BM * BK * 2;
 // PAIR: two CTAs work on a tile of 256 rows, 128 each, and each holds half of B's columns: a third less through L2 and shared
 // memory per product, and the shorter stages make room for six.  The sums are the same bit for bit.  One CTA / pairs (us): 4096 x
@@ -540,55 +540,6 @@ __global__ void __launch_bounds__(256) lce_pack_kernel(const uint4* __restrict__
 // whole: rows may be read up to the next multiple of 64 elements (a copy of our own).
 struct Operand { const void* ptr; int64_t ld; int mn; bool whole; };
 
-// How a product is cut into tiles: with fixed 256-column tiles and runs of eight, a ragged or small product leaves a
-// part of the chip idle (T = 1531, D = 1544, V = 32008: 192 forward items on 148 SMs, dH 84 tiles, the last of every
-// seven 8 columns wide).  The width of an N tile and the number of tiles per item are chosen for the shortest launch: rounds
-// of items per SM times the clocks of one item.  A 16-deep slice of an M = 128 MMA takes bn / 2 clk, and no less than its
-// operands need from shared memory at 128 bytes per clk.  A narrower tile or fewer tiles have to promise 5 % (8192 x 4096 x
-// 128256 would gain 3 % by this count and lost 1 %: what bounds it is power).  No choice changes a bit of a result.
-//   pairs     where rows in units of 256 fill the chip as well (a lone CTA's tiling has to promise 5 %) and the contraction has
-//             six steps or more: shorter ones are bound by the epilogue and the start (us, one CTA / pairs: T = 1000, D = 256,
-//             V = 32000 forward 34.9 / 36.8, backward 159 / 168; dW of 400 tokens, D = 2048, V = 50304, seven steps: the
-//             backward 431 / 415; of 300, five steps: 296 / 295)
-//   forward   256 columns, where its vocabulary runs end (see RUN_TILES); 1 to 8 tiles per item
-//   dz        128 to 256 columns in steps of 16 (of a pair 32); 1 to 8 tiles per item.  T = 1531, D = 1544, V = 32008: 275 -> 188 us
-//   dH, dW    256 columns where the matrix has them (their B operand lies MN-major; dH at T = 4096, D = 4096: 5.7 ms with 240
-//             or 192 columns against 3.4: its panels then start off the 128-byte lines, or a tile's rows off the 512 bytes they
-//             share), unless dH's tiles leave SMs idle: then 64 columns or more (min_bn = 64; V = 32008: T = 1531, D = 1536
-//             backward 415 -> 380 us, T = 384, D = 1544 305 -> 264; T = 149, D = 224, V = 50912 280 -> 208)
-constexpr int PAIR_DEPTH = 6;
-struct Tiling { int bn, n_run; bool pair; };
-Tiling choose_tiling(int M, int N, int K, int min_bn, int min_run, int max_run, int epi_per_32, int b_mn) {
-  const int nk = (K + BK - 1) / BK;
-  Tiling best = {BN, max_run, false};
-  double t_best = 1e300;
-  for (int pair = nk >= PAIR_DEPTH; pair >= 0; --pair) {
-    const int rows = pair ? 2 * BM : BM, sms = device_sm_count() / (pair + 1);
-    const long long m_tiles = (M + rows - 1) / rows;
-    const int least = pair && b_mn && min_bn < 128 ? 128 : min_bn;   // (half of an MN-major tile is whole panels)
-    const int unit = b_mn ? least : pair ? 32 : 16;
-    const bool few = b_mn && least < 128 && m_tiles * ((N + BN - 1) / BN) < sms;
-    for (int bn = BN; bn >= least; bn -= unit) {
-      if (bn > least && bn - unit >= N) continue;           // a whole unit wider than the matrix
-      if (b_mn && bn < BN && N > bn && !few) break;
-      const long long n_tiles = (N + bn - 1) / bn;
-      const double oper = 32 + (pair ? bn / 8 : bn / 4), slice = bn / 2 > oper ? bn / 2 : oper;
-      const double epi = (double)epi_per_32 * ((bn + 31) / 32);
-      const double mma = nk * (BK / 16) * slice;
-      const double tile = mma > epi ? mma : epi;
-      for (int run = max_run; run >= min_run; run /= 2) {
-        const long long items = m_tiles * ((n_tiles + run - 1) / run);
-        const double t = (double)((items + sms - 1) / sms) * (run < n_tiles ? run : n_tiles) * tile + epi;
-        if (t < 0.95 * t_best) { t_best = t; best = {bn, run, pair != 0}; }
-      }
-    }
-  }
-  return best;
-}
-// Clocks of an epilogue per 32 columns.  Rough, but they decide only where the contraction is short: 8 x 350 clk for a tile
-// against 512 per 64-deep step of its MMAs, which run under it.
-constexpr int EPI_CLK_LSE = 350, EPI_CLK_DZ = 500, EPI_CLK_STORE = 300;
-
 // How many tiles of the dimension that items walk first lie together before the other one advances: as many as keep
 // their operand in L2 (126 MB, in two halves) while the other operand streams past; where a few tiles' worth is too much (dH: a
 // contraction over the vocabulary), the block that lets the CTAs running together read the least of both operands.  All of them
@@ -632,8 +583,6 @@ cudaError_t launch_gemm(GemmArgs a, const Operand& A, const Operand& B, cudaStre
   const int grid = (items < slots ? items : slots) * ctas;
   return launch_chained(kern, chained, grid, G_THREADS, smem, st, ctas, maps, a, status);
 }
-
-constexpr int MAX_RUN = 8;   // most N tiles per work item of the forward and of dz
 
 // The forward's sums of exponentials: one running (maximum, sum) pair per token and vocabulary run, then the runs' pairs
 // together (lce_finish_kernel).  Where a run ends depends on nothing but the workspace, so that a token's lse is the same bit
@@ -753,7 +702,7 @@ int bdlm_linear_ce_fwd(const bdlm_lce_params* p, const void* h, const void* w, c
   char* ws = static_cast<char*>(workspace);
   GemmArgs a = {};
   a.M = p->T; a.N = p->V; a.K = p->D; a.m_inner = 1; a.run_tiles = run_tiles;
-  const Tiling ta = choose_tiling(p->T, p->V, p->D, BN, run_tiles, MAX_RUN, EPI_CLK_LSE, 0);
+  const Tiling ta = forward_tiling(device_sm_count(), p->T, p->D, p->V, run_tiles);
   a.bn = BN; a.n_run = ta.n_run; a.pair = ta.pair;
   a.row0 = 0; a.labels = labels; a.weight = token_weight; a.ldp = (int)(per / sizeof(float));
   a.part_m = reinterpret_cast<float*>(ws);
@@ -801,20 +750,20 @@ int bdlm_linear_ce_bwd(const bdlm_lce_params* p, const void* h, const void* w, c
     const Operand odz{dz, ldz, 0, roomy};
     // dz of the chunk: logits again, softmax minus one-hot in the epilogue
     GemmArgs a = {};
-    const Tiling ta = choose_tiling(rows, V, D, 128, 1, MAX_RUN, EPI_CLK_DZ, 0);
+    const Tiling ta = choose_tiling(device_sm_count(), rows, V, D, 128, 1, MAX_RUN, EPI_CLK_DZ, 0);
     a.M = rows; a.N = V; a.K = D; a.bn = ta.bn; a.n_run = ta.n_run; a.pair = ta.pair; a.m_inner = 1;
     a.row0 = t0; a.labels = labels; a.weight = token_weight; a.lse = lse; a.grad = p->grad_loss;
     a.dz = dz; a.ldz = (int)ldz;
     if (launch_gemm<EPI_DZ>(a, oh_c, ow, st, ci > 0 || plan.packed) != cudaSuccess) return BDLM_ERR_CUDA;
     // dH of the chunk = dz W   (contraction over the vocabulary; W as it lies is the MN-major B operand)
     GemmArgs b = {};
-    const Tiling tb = choose_tiling(rows, D, V, 64, 1, 1, EPI_CLK_STORE, 1);
+    const Tiling tb = choose_tiling(device_sm_count(), rows, D, V, 64, 1, 1, EPI_CLK_STORE, 1);
     b.M = rows; b.N = D; b.K = V; b.bn = tb.bn; b.n_run = 1; b.pair = tb.pair; b.m_inner = 1;
     b.c_mode = C_BF16; b.c16 = static_cast<bf16*>(dh) + (size_t)t0 * D; b.ldc = D;
     if (launch_gemm<EPI_STORE>(b, odz, mn(ow), st, true) != cudaSuccess) return BDLM_ERR_CUDA;
     // dW += dz^T H_c   (contraction over the chunk's tokens; both operands MN-major)
     GemmArgs c = {};
-    const Tiling tw = choose_tiling(V, D, rows, 128, 1, 1, EPI_CLK_STORE, 1);
+    const Tiling tw = choose_tiling(device_sm_count(), V, D, rows, 128, 1, 1, EPI_CLK_STORE, 1);
     c.M = V; c.N = D; c.K = rows; c.bn = tw.bn; c.n_run = 1; c.pair = tw.pair; c.m_inner = 0;
     c.c16 = static_cast<bf16*>(dw); c.c32 = dw32; c.ldc = D;
     c.c_mode = chunks == 1 ? C_BF16 : (ci == 0 ? C_F32_STORE : (ci + 1 < chunks ? C_F32_ADD : C_F32_ADD_TO_BF16));

@@ -4,6 +4,7 @@
 #include <cstring>
 
 #include "dispatch_rules.h"
+#include "lce_rules.h"
 
 using namespace bdlm;
 
@@ -16,5 +17,8 @@ int main(int argc, char** argv) {
     const BwdSizes z = {num(0), num(1), num(2), num(3), num(4), num(5), num(6), num(7), num(8)};
     const KeyLoad load = key_load(z, num(9));
     std::printf("%d %d\n", split_key_tiles(load), pairs_pay(z, load));
+  } else if (!std::strcmp(rule, "lce_forward")) {
+    const Tiling t = forward_tiling(num(4), num(0), num(1), num(2), num(3));
+    std::printf("%d %d %d\n", t.bn, t.n_run, t.pair);
   } else return 1;
 }

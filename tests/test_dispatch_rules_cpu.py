@@ -76,3 +76,18 @@ def test_pairs_whose_tiles_stand_far_apart(ask, L, chunk_tiles, rank_of, blocks,
         r, P = rank_of
         pos0, Lq, Ln = ((r if blocks else 2 * P - 1 - r) * L // (2 * P), L // (2 * P), L // P if blocks else 0)
     assert ask("pairs", 1, L, Lq, pos0, Ln, 8, 4, 0, 128 * chunk_tiles, SMS) == [1, want]
+
+
+@pytest.mark.parametrize("T,D,V,n_run,pair", [
+    (8192, 4096, 128256, 1, 1), (12288, 4096, 64000, 1, 1), (8192, 1024, 50304, 1, 1), (1531, 1544, 32008, 1, 1),
+    (300, 2048, 100000, 1, 0),           # three tiles of 128 rows, two of 256
+    (8192, 512, 50304, 8, 1), (2048, 384, 128256, 8, 1),
+])
+def test_forward_items_of_the_loss_head(ask, T, D, V, n_run, pair):
+    assert ask("lce_forward", T, D, V, 1, SMS) == [256, n_run, pair]
+
+
+@pytest.mark.parametrize("D", [256, 1024, 4096])
+def test_forward_items_hold_whole_vocabulary_runs(ask, D):
+    """With the smallest workspace a vocabulary run is eight tiles, and an item never less."""
+    assert ask("lce_forward", 8192, D, 128256, 8, SMS)[1] == 8
