@@ -1346,23 +1346,37 @@ static cudaError_t launch_units(Kern kern, const TileGrid& tg, int threads, size
   return launch_chained(kern, chained, (unsigned)blocks, threads, smem, st, tg.parts, maps, a, tg, status);
 }
 
+// Tensor maps of the kernels with one CTA per unit; the pairs' launcher encodes its own.
 template <int D>
-static cudaError_t launch_tc_bwd_d(const KArgs& a, int passes, cudaStream_t st) {
-  BwdMaps maps;
+static bool encode_maps(BwdMaps& maps, const KArgs& a) {
   for (int s = 0; s < 2; ++s) {
     // a stream that is left out gets the other stream's tensors as placeholders: its maps are never used
     const int sq = a.q[s] != nullptr ? s : 1 - s;
     const int sk = a.k[s] != nullptr ? s : CLEAN;
     const int qbox = a.single_pass ? HT : TILE;   // the fused kernel loads 64 query rows per step
-    if (!tc_make_map(&maps.q[s], a.q[sq], a.H, rows_q(a, sq), a.batch, qbox, D)) return cudaErrorInvalidValue;
-    if (!tc_make_map(&maps.dout[s], a.dout[sq], a.H, rows_q(a, sq), a.batch, qbox, D)) return cudaErrorInvalidValue;
-    if (!tc_make_map(&maps.k[s], a.k[sk], a.Hkv, rows_k(a, sk), a.batch, TILE, D)) return cudaErrorInvalidValue;
-    if (!tc_make_map(&maps.v[s], a.v[sk], a.Hkv, rows_k(a, sk), a.batch, TILE, D)) return cudaErrorInvalidValue;
+    if (!tc_make_map(&maps.q[s], a.q[sq], a.H, rows_q(a, sq), a.batch, qbox, D)) return false;
+    if (!tc_make_map(&maps.dout[s], a.dout[sq], a.H, rows_q(a, sq), a.batch, qbox, D)) return false;
+    if (!tc_make_map(&maps.k[s], a.k[sk], a.Hkv, rows_k(a, sk), a.batch, TILE, D)) return false;
+    if (!tc_make_map(&maps.v[s], a.v[sk], a.Hkv, rows_k(a, sk), a.batch, TILE, D)) return false;
   }
+  return true;
+}
+
+template <int D>
+static cudaError_t launch_tc_bwd_d(const KArgs& a, int passes, cudaStream_t st) {
   int* status = device_status_ptr();
   if (status == nullptr) return cudaErrorUnknown;
   cudaError_t e;
   const bool after_rows = (passes & BDLM_BWD_PASS_DSUM) != 0;   // the launch that forms the D rows is this call's predecessor
+  const BwdSizes sizes = bwd_sizes(a);
+  const KeyLoad load = key_load(sizes, device_sm_count());
+  const int parts = a.single_pass ? split_key_tiles(load) : 1;
+  // (for the two-pass kernels the rule knows nothing of the batch or the number of KV heads; the sums are the same bit for bit
+  // either way.  One CTA per tile / pairs, whole two-pass backward: L = 16384, H = 8 / 8 3239 / 3177 us, H = 32 / 8 12720 / 12390;
+  // L = 6016, H = 24 / 6 1467 / 1441)
+  const bool pairs = D == 128 && parts == 1 && pairs_pay(sizes, load);
+  BwdMaps maps;
+  if (!(a.single_pass && pairs) && !encode_maps<D>(maps, a)) return cudaErrorInvalidValue;
   if (a.single_pass) {
     // one kernel produces dK, dV and (through fp32 add-reductions) dQ; it runs for the DKDV pass bit, the DQ bit is a no-op
     if (passes & BDLM_BWD_PASS_DKDV) {
@@ -1370,10 +1384,6 @@ static cudaError_t launch_tc_bwd_d(const KArgs& a, int passes, cudaStream_t st) 
         const size_t rows = (size_t)a.dq32_rows[CLEAN] + a.dq32_rows[NOISY];
         if ((e = cudaMemsetAsync(a.dq32[CLEAN], 0, rows * a.batch * a.H * D * sizeof(float), st)) != cudaSuccess) return e;
       }
-      const BwdSizes z = bwd_sizes(a);
-      const KeyLoad load = key_load(z, device_sm_count());
-      const int parts = split_key_tiles(load);
-      const bool pairs = D == 128 && parts == 1 && pairs_pay(z, load);
       if (pairs) {
         if ((e = launch_tc_bwd_pair(a, true, st, after_rows)) != cudaSuccess) return e;
       } else {
@@ -1397,11 +1407,7 @@ static cudaError_t launch_tc_bwd_d(const KArgs& a, int passes, cudaStream_t st) 
     return cudaSuccess;
   }
   if (passes & BDLM_BWD_PASS_DKDV) {
-    // (the rule knows nothing of the batch or the number of KV heads; the sums are the same bit for bit either way.  One CTA per
-    // tile / pairs, whole two-pass backward: L = 16384, H = 8 / 8 3239 / 3177 us, H = 32 / 8 12720 / 12390; L = 6016, H = 24 / 6
-    // 1467 / 1441)
-    const BwdSizes z = bwd_sizes(a);
-    if (D == 128 && pairs_pay(z, key_load(z, device_sm_count()))) {
+    if (pairs) {
       if ((e = launch_tc_bwd_pair(a, false, st, after_rows)) != cudaSuccess) return e;
     } else {
       auto kern = a.trace ? tc_dkdv_kernel<true, D> : tc_dkdv_kernel<false, D>;
