@@ -280,10 +280,11 @@ int bdlm_set_trace_buffer(void* device_counters, size_t bytes);
  * Self-test of the bounded device-side waits (no counterpart in the paper).  Every wait inside the
  * kernels gives up after a limit of clock ticks, raises its CTA's abort flag so that the other roles
  * leave their loops too, and the kernel reports BDLM_ERR_DEVICE_TIMEOUT through the device status
- * word instead of hanging the GPU.  This call launches a one-CTA kernel without any copy or
+ * word instead of hanging the GPU.  This call launches a kernel of one pair of CTAs without any copy or
  * tensor-core work in which one warp waits, with a limit of `limit_ticks` clock ticks (1 .. 2^31), on
- * a barrier that nothing will ever complete, and a second warp waits on the same barrier with the
- * kernels' regular limit (about a second) and leaves as soon as the first warp has raised the flag.  Afterwards bdlm_get_device_status returns
+ * a barrier that nothing will ever complete, a second warp waits on the same barrier with the
+ * kernels' regular limit (about a second) and leaves as soon as the first warp has raised the flag, and
+ * the warps of the other CTA wait likewise and leave once the first CTA has raised theirs.  Afterwards bdlm_get_device_status returns
  * BDLM_ERR_DEVICE_TIMEOUT once, and BDLM_OK on the next call.  The kernel always terminates.
  */
 int bdlm_selftest_wait_timeout(int64_t limit_ticks, void* cuda_stream);

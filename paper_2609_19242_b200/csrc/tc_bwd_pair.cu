@@ -607,13 +607,7 @@ tc_bwd_pair_kernel(const __grid_constant__ PairMaps maps, const KArgs a, const T
   }
   tc_fence_before();
   __syncthreads();
-  if (threadIdx.x == 0 && *abort_flag) {
-    atomicExch(status, (int)BDLM_ERR_DEVICE_TIMEOUT);
-    // the other CTA waits for this one: it has to give up as well.  The copies on their way land first (all roles have left)
-    const long long t0 = clock64();
-    while (clock64() - t0 < (1ll << 18)) {}
-    asm volatile("st.shared::cluster.u32 [%0], %1;" ::"r"(peer_addr(smem_u32(const_cast<int*>(abort_flag)), rank ^ 1)), "r"(1) : "memory");
-  }
+  if (threadIdx.x == 0 && *abort_flag) give_up_pair(abort_flag, status, rank);
   cluster_sync();   // no CTA leaves while the other one still writes to its shared memory or signals its barriers
   if (warp == 8) tmem_dealloc_pair(tmem, 512);
 }

@@ -7,6 +7,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include "../../include/bdlm_attn.h"
+
 namespace bdlm {
 namespace tc {
 
@@ -249,6 +251,14 @@ __device__ __forceinline__ uint32_t peer_addr(uint32_t addr, uint32_t rank) {
   uint32_t r;
   asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(addr), "r"(rank));
   return r;
+}
+// A CTA of a pair whose waits have given up, one thread after all its roles have left: reports it and makes the other CTA, which
+// waits for this one, give up as well.  The copies on their way land first.  Both CTAs then meet in cluster_sync.
+__device__ __forceinline__ void give_up_pair(volatile int* abort_flag, int* status, uint32_t rank) {
+  atomicExch(status, (int)BDLM_ERR_DEVICE_TIMEOUT);
+  const long long t0 = clock64();
+  while (clock64() - t0 < (1ll << 18)) {}
+  asm volatile("st.shared::cluster.u32 [%0], %1;" ::"r"(peer_addr(smem_u32(const_cast<int*>(abort_flag)), rank ^ 1)), "r"(1) : "memory");
 }
 // Arrivals at a barrier of either CTA (an address from peer_addr).  mbar_arrive_peer is relaxed: execution order only, for what
 // lies in tensor memory (ordered by tcgen05.wait and the tcgen05 fences).  mbar_arrive_peer_smem is for shared memory of the

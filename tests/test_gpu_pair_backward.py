@@ -104,3 +104,18 @@ def test_packed_form(case):
             _close(a, b, i)
     for i in (1, 2):
         assert torch.equal(got[i], again[i])
+
+
+def test_a_cta_that_gives_up_makes_the_other_one_of_its_pair_give_up():
+    """The self-test kernel is a pair of CTAs: one wait of the first runs out after about a millisecond of clock ticks, the other
+    CTA's waits have a limit of a second or more and nothing that would complete them.  They have to end because of the flag the
+    first CTA raises in the other one's shared memory."""
+    binding.bdlm_selftest_wait_timeout(1_000)   # (loads the kernel)
+    assert binding.bdlm_get_device_status() == -5
+    begin, end = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+    begin.record()
+    binding.bdlm_selftest_wait_timeout(2_000_000)
+    end.record()
+    assert binding.bdlm_get_device_status() == -5
+    assert binding.bdlm_get_device_status() == 0
+    assert 0.5 < begin.elapsed_time(end) < 200.0   # ms; 2e6 + 2^18 ticks (twice) at 1 to 2 GHz, the other CTA's own limit is 2^31
