@@ -66,7 +66,8 @@ typedef struct {
                                   Each CTA adds its dQ tiles into an fp32 accumulator in the workspace (bulk add-reductions),
                                   so dQ is reproducible only up to fp32 summation order; dK and dV are bitwise reproducible
                                   (fixed order) from call to call of the same sizes, while their last bits may depend on
-                                  the batch size and the number of heads (on how many CTAs share a key tile).
+                                  the batch size, the number of heads and the chunk length of gathered K/V (on how many
+                                  CTAs share a key tile, and on whether pairs of CTAs take two).
                                   Needs the workspace bdlm_workspace_bytes[_packed] reports for this setting
                                   (BDLM_ERR_WORKSPACE_TOO_SMALL otherwise); with impl = 1 (the mma.sync kernels) the
                                   two-pass path runs.
@@ -116,6 +117,12 @@ int bdlm_attn_fwd(const bdlm_params* p,
  * is fixed, so they are bitwise reproducible; dQ is too on the two-pass path, and reproducible up to
  * fp32 summation order when the fused kernel runs (see bdlm_params.bwd_single_pass for which one
  * does).  Requires the full clean key range.
+ * NaN and infinities among the inputs: hidden elements with finite values have no effect, but the products run over
+ * whole tiles, and there a hidden zero times a NaN is NaN.  A NaN in a query's row (q, do, o, lse) can reach dK / dV of
+ * keys that the row does not see, and one in a key's row dQ of queries that do not see it, up to 256 positions away
+ * (128 where one CTA takes each key tile: short calls, head dimension 64).  With gathered K/V (kv_chunk_len, an odd
+ * number of 128-row tiles) a pair of CTAs may join the end of one chunk and the beginning of the next in memory; for
+ * those two tiles it is as far as their positions are apart.
  * The workspace holds D_i = sum_d dO_i,d * O_i,d and, for the fused kernel, an fp32 dQ accumulator
  * [batch, H, rows rounded up to 64, d] per query stream (for d = 64 the reported size still counts rows of 128); nothing
  * in it has to be initialised or kept between calls.
