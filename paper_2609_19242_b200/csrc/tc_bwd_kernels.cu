@@ -60,9 +60,10 @@ constexpr int DKDV_PRODUCER = 4 * DKDV_NWG, DKDV_ISSUER = 4 * DKDV_NWG + 1;
 // the partial tiles go to shared memory, each CTA adds up a share of the rows over its peers through distributed
 // shared memory, in the order of their ranks (so the sums stay reproducible), and stores it.  Noisy key tiles have a
 // few steps only (their own block's queries): in such a launch each CTA of a cluster takes one of its own.
-// Only the fused kernel does this.  How many CTAs share a tile depends on how full the launch makes the chip, so the last
-// bits of dK / dV depend on the batch size and the number of heads; the two-pass kernels, whose every gradient is
-// reproducible, keep one CTA per key tile and with it sums that depend on the sequence alone.
+// Only the fused kernel does this (split_key_tiles).  How many CTAs share a tile depends on how full the launch makes the
+// chip, so the last bits of dK / dV depend on the batch size and the number of heads; the two-pass kernels, whose every
+// gradient is reproducible, sum a key tile in one CTA (of a pair in large calls: the same sums), so that they depend on the
+// sequence alone.
 struct KeyUnit { int bx, hk, ks, b, part, parts; bool none; };
 __device__ __forceinline__ KeyUnit key_unit(const TileGrid& tg) {
   KeyUnit u;
