@@ -239,8 +239,8 @@ def kernel_source_digest():
     import hashlib
     h = hashlib.sha256()
     csrc = os.path.join(ROOT, "paper_2609_19242_b200", "csrc")
-    for f in ("bdlm_common.cuh", "fwd_issue.h", "tc_common.cuh", "tc_kernels.cu", "tc_bwd_common.cuh", "tc_bwd_kernels.cu",
-              "tc_bwd_pair.cu"):
+    for f in ("bdlm_common.cuh", "dispatch_rules.h", "fwd_issue.h", "tc_common.cuh", "tc_kernels.cu", "tc_bwd_common.cuh",
+              "tc_bwd_kernels.cu", "tc_bwd_pair.cu"):
         with open(os.path.join(csrc, f), "rb") as fh:
             h.update(fh.read())
     return h.hexdigest()[:16]

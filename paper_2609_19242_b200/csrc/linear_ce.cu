@@ -537,8 +537,8 @@ struct Operand { const void* ptr; int64_t ld; int mn; bool whole; };
 // How many tiles of the dimension that items walk first lie together before the other one advances: as many as keep
 // their operand in L2 (126 MB, in two halves) while the other operand streams past; where a few tiles' worth is too much (dH: a
 // contraction over the vocabulary), the block that lets the CTAs running together read the least of both operands.  All of them
-// / blocks: T = 12288, D = 4096 (h 100 MB), V = 64000 forward 5470 / 4870 us; T = 8192, D = 4096, V = 128256 forward 6500 /
-// 6500 (h 67 MB), backward 19800 / 19500; smaller ones have one block.
+// / blocks: T = 12288, D = 4096 (h 100 MB), V = 64000 forward 5270 / 4560 us; T = 8192, D = 4096, V = 128256 forward 6425 /
+// 6000 (h 67 MB), backward 19800 / 19500; smaller ones have one block.
 constexpr double L2_KEEP = 40e6;
 int inner_block(const GemmArgs& a) {
   const int rows = a.pair ? 2 * BM : BM, slots = device_sm_count() / (a.pair ? 2 : 1);
