@@ -56,15 +56,19 @@ inline Tiling choose_tiling(int sms, int M, int N, int K, int min_bn, int min_ru
   return best;
 }
 
-// The forward: items of one tile where the contraction has DEEP steps or more.  The tiles of an item share nothing on chip, and
-// the CTAs that run together read the same few W tiles only while they keep step, which eight deep tiles in a row do not:
-// 8192 x 4096 x 128256 reads 8.6 GB from memory with items of eight, 5.6 with items of one.  Items of eight / one, on pairs (us):
-// 8192 x 4096 x 128256 6450 / 5960; 12288 x 4096 x 64000 4890 / 4465; 4096 x 4096 x 128256 3058 / 2957; 8192 x 1280 x 50304
-// 742 / 728; 8192 x 1024 x 50304 591 / 588; 8192 x 768 x 50304 450 / 449; shorter ones are bound by the epilogue, and all CTAs on
-// the same W tile at once cost more there: 8192 x 512 x 50304 339 / 349, 2048 x 384 x 128256 211 / 218.
-constexpr int DEEP = 16;
+// The forward: items of one tile where the contraction has DEEP steps or more, the token tiles share W's and there are ROUNDS rounds of
+// items.  The tiles of an item share nothing on chip, and the CTAs that run together read the same few W tiles only while they keep
+// step, which eight deep tiles in a row do not: 8192 x 4096 x 128256 reads 8.6 GB from memory with items of eight, 5.6 with items of
+// one.  Items of eight / one, on pairs (us): 8192 x 4096 x 128256 6450 / 5960; 12288 x 4096 x 64000 4890 / 4465; 4096 x 4096 x
+// 128256 3058 / 2957; 8192 x 1280 x 50304 742 / 728; 8192 x 1024 x 50304 591 / 588; 8192 x 768 x 50304 450 / 449; shorter ones are
+// bound by the epilogue, and all CTAs on the same W tile at once cost more there: 8192 x 512 x 50304 339 / 349, 2048 x 384 x 128256
+// 211 / 218.  In few rounds the last one counts, which choose_tiling weighs (items of two / one: 123 x 1048 x 49664 37 / 40, 137 x
+// 4000 x 20272 54 / 58).
+constexpr int DEEP = 16, ROUNDS = 4;
 inline Tiling forward_tiling(int sms, int T, int D, int V, int run_tiles) {
-  return choose_tiling(sms, T, V, D, BN, run_tiles, (D + BK - 1) / BK >= DEEP ? run_tiles : MAX_RUN, EPI_CLK_LSE, 0);
+  const long long items = (long long)((T + 2 * BM - 1) / (2 * BM)) * ((V + BN - 1) / BN);
+  const bool one = (D + BK - 1) / BK >= DEEP && T > 2 * BM && items >= ROUNDS * (sms / 2);
+  return choose_tiling(sms, T, V, D, BN, run_tiles, one ? run_tiles : MAX_RUN, EPI_CLK_LSE, 0);
 }
 
 }  // namespace bdlm

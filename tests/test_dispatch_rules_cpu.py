@@ -81,6 +81,7 @@ def test_pairs_whose_tiles_stand_far_apart(ask, L, chunk_tiles, rank_of, blocks,
 @pytest.mark.parametrize("T,D,V,n_run,pair", [
     (8192, 4096, 128256, 1, 1), (12288, 4096, 64000, 1, 1), (8192, 1024, 50304, 1, 1), (1531, 1544, 32008, 1, 1),
     (300, 2048, 100000, 1, 0),           # three tiles of 128 rows, two of 256
+    (123, 1048, 49664, 2, 0), (137, 4000, 20272, 2, 1),   # few rounds of items: as even as they get
     (8192, 512, 50304, 8, 1), (2048, 384, 128256, 8, 1),
 ])
 def test_forward_items_of_the_loss_head(ask, T, D, V, n_run, pair):
