@@ -193,6 +193,11 @@ __device__ __forceinline__ uint32_t pack_bf16(float lo, float hi) {
   return *reinterpret_cast<uint32_t*>(&v);
 }
 
+// The call as the rules on sizes see it.
+inline BwdSizes bwd_sizes(const KArgs& a) {
+  return {a.batch, a.L, a.q[CLEAN] != nullptr ? a.Lqc : 0, a.cq_pos0, a.q[NOISY] != nullptr ? a.Ln : 0, a.Hkv, a.G, a.window, a.kv_chunk_len};
+}
+
 // Launchers (host).  Each enqueues on `st` and returns the launch's cudaError_t.
 cudaError_t launch_portable_fwd(const KArgs& a, cudaStream_t st);
 cudaError_t launch_portable_bwd(const KArgs& a, int passes, cudaStream_t st);

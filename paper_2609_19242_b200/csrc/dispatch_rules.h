@@ -5,6 +5,12 @@
 
 namespace bdlm {
 
+// What a backward call looks like to the rules below.
+struct BwdSizes {
+  int batch, L, Lqc, cq_pos0, Ln;   // clean keys, clean query rows (0: none) from this position on, noisy rows (0: none)
+  int Hkv, G, window, kv_chunk_len;
+};
+
 // Whether the units of a launch start tile-major (see TileGrid).  A stack (one head of one batch element and stream; ny nz of
 // them) has nx units; work grows by one from the lightest unit up to `heavy` (nx without a window) and stays there; `at_once`
 // units run at one time.  Tile-major when the heaviest unit takes more than 1 / ratio of the launch's ideal duration.
@@ -36,16 +42,15 @@ constexpr double ORDER_RATIO = 5;   // one CTA per tile: 10 SMs > ny nz (nx + 1)
 //   1280   2 x 12000, H = 16 / 4, window 3500   3296 / 3773        2232 / 2330
 // The fused kernel turns earlier than dK/dV alone, and under a window earlier still: its dQ accumulators leave L2 when the tiles of
 // all heads run together, while neighbouring tiles of one head complete them (3 x 6144, H = 32 / 8: one CTA per tile 5107).
-inline bool pairs_tile_major_pay(int nx, int ny, int nz, int window, int sms, bool dq) {
-  const double keys = window > 0 ? window / 256.0 + 1 : nx, heavy = keys < nx ? keys : nx;
-  return tile_major_pays(nx, ny, nz, heavy, sms / 2, !dq ? 20.0 / 3 : heavy < nx ? 4.2 : 6);
+// Tiles are counted over the clean keys: noisy ones have a few steps each.  With 32 query heads or more the fused kernel counts the
+// longer of the two streams, as its accumulators then need the other order all the more (blocks without clean queries, fused,
+// x-fastest / tile-major: L = 9984, 19712 rows, H = 24 / 8 3147 / 3094; L = 12288, 32768 rows, H = 32 / 8 8228 / 8660; L = 8192,
+// 20480 rows, H = 64 / 8 7814 / 8316).
+inline bool pairs_tile_major_pay(const BwdSizes& z, int sms, bool dq) {
+  const int keys = dq && z.Hkv * z.G * z.batch >= 32 ? std::max(z.L, z.Ln) : z.L, nx = (keys + 255) / 256;
+  const double band = z.window > 0 ? z.window / 256.0 + 1 : nx, heavy = band < nx ? band : nx;
+  return tile_major_pays(nx, z.Hkv, 2 * z.batch, heavy, sms / 2, !dq ? 20.0 / 3 : heavy < nx ? 4.2 : 6);
 }
-
-// What a backward call looks like to the rules below.
-struct BwdSizes {
-  int batch, L, Lqc, cq_pos0, Ln;   // clean keys, clean query rows (0: none) from this position on, noisy rows (0: none)
-  int Hkv, G, window, kv_chunk_len;
-};
 
 // How many CTAs share a clean key tile (1, 2 or 4), from two estimates in steps of STEP_ROWS query rows: `heavy` for the
 // first clean key tile and `mean` per SM; with a prefix table the blocks are taken to be spread evenly over the keys.

@@ -1332,10 +1332,6 @@ void tc_bwd_place_dq(KArgs& a, void* extra_ws) {
 }
 
 static_assert(TILE_KEYS == TILE && STEP_ROWS == HT, "the rules count these tiles and steps");
-static BwdSizes bwd_sizes(const KArgs& a) {
-  return {a.batch, a.L, a.q[CLEAN] != nullptr ? a.Lqc : 0, a.cq_pos0, a.q[NOISY] != nullptr ? a.Ln : 0, a.Hkv, a.G, a.window, a.kv_chunk_len};
-}
-
 // One CTA, or one cluster of tg.parts CTAs, per unit of the grid.
 template <class Kern>
 static cudaError_t launch_units(Kern kern, const TileGrid& tg, int threads, size_t smem, cudaStream_t st, const BwdMaps& maps,

@@ -633,7 +633,7 @@ static cudaError_t launch_pair(const KArgs& a, cudaStream_t st, bool chained) {
   int* status = device_status_ptr();
   if (status == nullptr) return cudaErrorUnknown;
   TileGrid tg = {(max(a.L, a.k[NOISY] != nullptr ? a.Ln : 0) + 2 * TILE - 1) / (2 * TILE), a.Hkv, a.batch * 2, 0, 1};
-  tg.tile_major = pairs_tile_major_pay(tg.nx, tg.ny, tg.nz, a.window, device_sm_count(), DQ) ? 1 : 0;
+  tg.tile_major = pairs_tile_major_pay(bwd_sizes(a), device_sm_count(), DQ) ? 1 : 0;
   const long long blocks = 2LL * tile_grid_blocks(tg);
   if (blocks == 0 || blocks > 0x7fffffffLL) return cudaErrorInvalidValue;
   auto kern = a.trace ? tc_bwd_pair_kernel<true, DQ> : tc_bwd_pair_kernel<false, DQ>;

@@ -12,7 +12,10 @@ int main(int argc, char** argv) {
   auto num = [&](int i) { return i + 2 < argc ? std::atoi(argv[i + 2]) : 0; };
   const char* rule = argv[1];
   if (!std::strcmp(rule, "order")) std::printf("%d\n", tile_major_pays(num(0), num(1), num(2), num(0), num(3), ORDER_RATIO));
-  else if (!std::strcmp(rule, "order_pairs")) std::printf("%d\n", pairs_tile_major_pay(num(0), num(1), num(2), num(3), num(4), num(5) != 0));
+  else if (!std::strcmp(rule, "order_pairs")) {
+    const BwdSizes z = {num(0), num(1), num(2), num(3), num(4), num(5), num(6), num(7), num(8)};
+    std::printf("%d %d\n", pairs_tile_major_pay(z, num(9), true), pairs_tile_major_pay(z, num(9), false));
+  }
   else if (!std::strcmp(rule, "pairs")) {
     const BwdSizes z = {num(0), num(1), num(2), num(3), num(4), num(5), num(6), num(7), num(8)};
     const KeyLoad load = key_load(z, num(9));

@@ -40,9 +40,16 @@ def ask(tmp_path_factory):
     (1, 8192, 8, 8192, 1, 1),     # one that cuts nothing off
 ])
 def test_start_order_of_pairs(ask, batch, L, H_kv, window, fused, dkdv):
-    units = (-(-L // 256), H_kv, 2 * batch, window, SMS)
-    assert ask("order_pairs", *units, 1) == [fused]
-    assert ask("order_pairs", *units, 0) == [dkdv]
+    assert ask("order_pairs", batch, L, L, 0, L, H_kv, 4, window, 0, SMS) == [fused, dkdv]
+
+
+@pytest.mark.parametrize("L,H_kv,G,Lq,Ln,fused,dkdv", [
+    (9984, 8, 3, 0, 19712, 1, 1), (10240, 8, 2, 8000, 19200, 1, 1),   # more noisy rows than clean keys
+    (12288, 8, 4, 0, 32768, 0, 1), (8192, 8, 8, 0, 20480, 0, 1), (16384, 8, 4, 0, 32768, 0, 0),
+    (20480, 8, 4, 0, 9600, 0, 0),
+])
+def test_start_order_of_pairs_in_the_packed_form(ask, L, H_kv, G, Lq, Ln, fused, dkdv):
+    assert ask("order_pairs", 1, L, Lq, 2000 if Lq else 0, Ln, H_kv, G, 0, 0, SMS) == [fused, dkdv]
 
 
 @pytest.mark.parametrize("nx,stacks,want", [(64, 16, 1), (91, 16, 1), (92, 16, 0), (256, 16, 0)])
