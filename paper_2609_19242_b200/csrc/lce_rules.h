@@ -26,6 +26,9 @@ constexpr int EPI_CLK_LSE = 350, EPI_CLK_DZ = 500, EPI_CLK_STORE = 300;
 //             or 192 columns against 3.4: its panels then start off the 128-byte lines, or a tile's rows off the 512 bytes they
 //             share), unless dH's tiles leave SMs idle: then 64 columns or more (min_bn = 64; V = 32008: T = 1531, D = 1536
 //             backward 415 -> 380 us, T = 384, D = 1544 305 -> 264; T = 149, D = 224, V = 50912 280 -> 208)
+//             Matrices of 129 to 240 columns in one round of items: one CTA's MMAs cover them in units of 16, a pair's in units of
+//             128 (dW, pairs / one CTA, whole backward: 2609 x 224 x 4488 53.1 / 50.0 us, 11177 x 224 x 5192 220 / 209, 4096 x 144 x
+//             8000 92.2 / 89.5; in more rounds memory bounds them: 3000 x 176 x 30000 266.5 / 268.4)
 constexpr int PAIR_DEPTH = 6;
 struct Tiling { int bn, n_run; bool pair; };
 inline Tiling choose_tiling(int sms, int M, int N, int K, int min_bn, int min_run, int max_run, int epi_per_32, int b_mn) {
@@ -42,7 +45,11 @@ inline Tiling choose_tiling(int sms, int M, int N, int K, int min_bn, int min_ru
       if (bn > least && bn - unit >= N) continue;           // a whole unit wider than the matrix
       if (b_mn && bn < BN && N > bn && !few) break;
       const long long n_tiles = (N + bn - 1) / bn;
-      const double oper = 32 + (pair ? bn / 8 : bn / 4), slice = bn / 2 > oper ? bn / 2 : oper;
+      // the columns that MMAs compute: of a lone tile wider than the matrix those that its layout's units cover
+      const int cover = pair ? (b_mn ? 128 : 32) : 16;
+      const bool narrow = bn == BN && n_tiles == 1 && m_tiles <= slots;
+      const int cols = narrow ? (N + cover - 1) / cover * cover : bn;
+      const double oper = 32 + (pair ? bn / 8 : bn / 4), slice = cols / 2 > oper ? cols / 2 : oper;
       const double epi = (double)epi_per_32 * ((bn + 31) / 32);
       const double mma = nk * (BK / 16) * slice;
       const double tile = mma > epi ? mma : epi;

@@ -23,5 +23,8 @@ int main(int argc, char** argv) {
   } else if (!std::strcmp(rule, "lce_forward")) {
     const Tiling t = forward_tiling(num(4), num(0), num(1), num(2), num(3));
     std::printf("%d %d %d\n", t.bn, t.n_run, t.pair);
+  } else if (!std::strcmp(rule, "lce_dw")) {
+    const Tiling t = choose_tiling(num(3), num(2), num(1), num(0), 128, 1, 1, EPI_CLK_STORE, 1);
+    std::printf("%d %d\n", t.bn, t.pair);
   } else return 1;
 }

@@ -99,3 +99,12 @@ def test_forward_items_of_the_loss_head(ask, T, D, V, n_run, pair):
 def test_forward_items_hold_whole_vocabulary_runs(ask, D):
     """With the smallest workspace a vocabulary run is eight tiles, and an item never less."""
     assert ask("lce_forward", 8192, D, 128256, 8, SMS)[1] == 8
+
+
+@pytest.mark.parametrize("T,D,V,bn,pair", [
+    (2609, 224, 4488, 256, 0), (2146, 240, 8992, 256, 0), (4096, 144, 8000, 256, 0),   # one round of narrow matrices
+    (3000, 176, 30000, 256, 1), (4096, 256, 8000, 256, 1), (4096, 248, 8000, 256, 1), (4096, 128, 16000, 128, 1), (4000, 72, 9000, 128, 1),
+    (4096, 2048, 50304, 256, 1), (300, 2048, 50304, 256, 0),
+])
+def test_weight_gradient_of_the_loss_head(ask, T, D, V, bn, pair):
+    assert ask("lce_dw", T, D, V, SMS) == [bn, pair]
