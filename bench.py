@@ -36,12 +36,12 @@ NAMES6 = ["q_clean", "k_clean", "v_clean", "q_noisy", "k_noisy", "v_noisy"]
 # DRAM traffic (dram__bytes_read.sum + dram__bytes_write.sum) per launch of a kernel from a one-pass ncu capture of
 # this command, keyed by (workload, kernel), each with the digest of the kernel sources it was captured on
 # (kernel_source_digest): a figure is reported only for the build it belongs to.
-_CAPTURED_ON = "151b29bf182d6b68"
+_CAPTURED_ON = "2f31cc4ed154cebe"
 NCU_TRAFFIC = {
-    ("32k", "fwd"): {"bytes": 981373696 + 521526272, "kernel_source": _CAPTURED_ON},
-    ("32k", "bwd_fused"): {"bytes": 5656973056 + 3099851776, "kernel_source": _CAPTURED_ON},
-    ("32k", "bwd_dkdv"): {"bytes": 2405314304 + 266414848, "kernel_source": _CAPTURED_ON},
-    ("32k", "bwd_dq"): {"bytes": 1542419200 + 518608896, "kernel_source": _CAPTURED_ON},
+    ("32k", "fwd"): {"bytes": 980215296 + 521339904, "kernel_source": _CAPTURED_ON},
+    ("32k", "bwd_fused"): {"bytes": 5519783936 + 3002078976, "kernel_source": _CAPTURED_ON},
+    ("32k", "bwd_dkdv"): {"bytes": 2408756992 + 265991424, "kernel_source": _CAPTURED_ON},
+    ("32k", "bwd_dq"): {"bytes": 1539036672 + 518338560, "kernel_source": _CAPTURED_ON},
 }
 TRAFFIC_NOTE = ("dram__bytes_read.sum + dram__bytes_write.sum per launch from a one-pass ncu capture of this command on "
                 "the 32k workload")
